@@ -222,6 +222,22 @@ __global__ void k_sub(const float* __restrict__ a, const float* __restrict__ b, 
     out[i] = a[i] - b[i];
 }
 
+// A plan's pass table: entry off + (t - 1) Ns + k of a stage is
+// exp(-2 pi i t k / (Ns R)), from tw[m] = exp(-2 pi i m / (L step)).
+__global__ void k_pass_table(float2* __restrict__ tab, FftPlan p, int n, const float2* __restrict__ tw, int step) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= n) return;
+  for (int s = p.nst - 1; s >= 1; --s) {
+    const FftStage& g = p.st[s];
+    if (e >= g.off) {
+      const int t = 1 + (e - g.off) / g.Ns, k = (e - g.off) % g.Ns;
+      tab[e] = tw[t * k * (p.L / (g.Ns * g.R)) * step];
+      return;
+    }
+  }
+  tab[e] = make_float2(1.f, 0.f);  // a single-stage plan reads no table
+}
+
 int grid_for(long long n, int threads, int cap = 4096) {
   long long g = (n + threads - 1) / threads;
   if (g < 1) g = 1;
@@ -246,23 +262,22 @@ bool make_geo(int H, int W, int J, Geo* g) {
   g->eta = (1 << (J + 2)) - 3;
   g->L = W / 2;
   g->Wh = W / 2 + 1;
-  if (!make_plan(H, &g->planH) || !make_plan(g->L, &g->planL)) return false;
+  g->Wy = (g->Wh + 7) & ~7;  // row segments of a column tile on 64-byte boundaries
+  if (!make_plan(H, &g->planH) || !make_plan(g->L, &g->planL) || !make_plan(g->L, &g->planLr, true)) return false;
   int tc = pow2_floor(4096 / H);
   if (tc < 4) tc = 4;
   if (tc > 16) tc = 16;
   if (tc > g->Wh) tc = g->Wh;
   g->TC = tc;
   g->ntiles = (g->Wh + tc - 1) / tc;
-  const int E = H * tc;
-  const int per = (E + kColThreads - 1) / kColThreads;
-  g->maxe = per <= 8 ? 8 : (per <= 16 ? 16 : 32);
-  if (per > 32) return false;
+  if ((H * tc + kColThreads - 1) / kColThreads > 32) return false;
   int rb = 4096 / g->L;
   if (rb < 1) rb = 1;
   if (rb > H) rb = H;
   g->RB = rb;
   g->twH = nullptr;
   g->twW = nullptr;
+  g->ptH = g->ptL = g->ptLr = nullptr;
   g->bank = nullptr;
   g->ranges = nullptr;
   return true;
@@ -284,6 +299,28 @@ int filter_descs(int J, FilterDesc* out) {
 cudaError_t launch_twiddles(float2* tw, int N, cudaStream_t st) {
   k_twiddles<<<grid_for(N, 256), 256, 0, st>>>(tw, N);
   return cudaGetLastError();
+}
+
+size_t pass_table_entries(const Geo& g) {
+  return static_cast<size_t>(plan_table(g.planH)) + 2 * static_cast<size_t>(plan_table(g.planL));
+}
+
+cudaError_t launch_pass_tables(Geo* g, float2* tab, cudaStream_t st) {
+  struct {
+    const FftPlan* p;
+    const float2* tw;
+    int step;
+    const float2** out;
+  } const parts[] = {{&g->planH, g->twH, 1, &g->ptH}, {&g->planL, g->twW, 2, &g->ptL}, {&g->planLr, g->twW, 2, &g->ptLr}};
+  for (const auto& q : parts) {
+    const int n = plan_table(*q.p);
+    k_pass_table<<<grid_for(n, 256), 256, 0, st>>>(tab, *q.p, n, q.tw, q.step);
+    cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+    *q.out = tab;
+    tab += n;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t launch_build_bank(float* bank, const Geo& g, const FilterDesc* descs_dev, cudaStream_t st) {

@@ -65,8 +65,15 @@ struct shf_bank {
   int2* ranges = nullptr;
   float2* twH = nullptr;
   float2* twW = nullptr;
+  float2* pt = nullptr;  // the plans' pass tables
   shf::FilterDesc* descs = nullptr;
   int device = 0;
+  // Temporaries of the transforms.  A pool of the bank's own keeps up to
+  // kPoolKeep bytes between calls: the device's default pool gives its memory
+  // back whenever the device is waited for, and a call after that pays for
+  // mapping it again (a 64 x 64 analysis: 256 us against 30 us in a row).
+  cudaMemPool_t pool = nullptr;
+  static constexpr unsigned long long kPoolKeep = 512ull << 20;
 };
 
 struct seg_state {
@@ -88,8 +95,8 @@ struct seg_state {
   int* labels = nullptr;
   int* flag = nullptr;
   double* red = nullptr;
-  int red_len = 0;
   int groups = 1;
+  std::vector<shf::FilterWave> waves;  // general path: the waves of `groups` filter groups
   cudaGraphExec_t exec = nullptr;        // one iteration
   cudaGraphExec_t exec_timed = nullptr;  // the same with an event before every launch
   bool graph_tried = false;
@@ -112,9 +119,10 @@ struct seg_state {
   // unrolled mode (reverse-mode differentiation): generic-path scratch and
   // the states kept every un_ck iterations
   int un_T = 0, un_ck = 0;
-  float2* un_Y = nullptr;        // [K][eta][H][Wh]
+  float2* un_Y = nullptr;        // a wave's spectra [planes][H][Wy]
   float2* un_partial = nullptr;  // [un_groups][K][H][Wh]
   int un_groups = 0;
+  std::vector<shf::FilterWave> un_waves;
   std::vector<float*> ck_bv, ck_w, ck_bw;
   std::vector<float2*> ck_T;
   // the forward and reverse sweeps captured as graphs for (T, ckpt) = un_key;
@@ -131,9 +139,38 @@ struct seg_state {
 
 namespace shf {
 void bank_geo(const shf_bank* b, Geo* g) { *g = b->g; }
+
 int bank_device(const shf_bank* b) { return b->device; }
 int set_error(int code, const std::string& msg) { return fail(code, msg); }
 }  // namespace shf
+
+namespace {
+
+// Stream-ordered temporary memory from the bank's pool.
+cudaError_t scratch_alloc(const shf_bank* b, float2** p, size_t count, cudaStream_t st) {
+  const size_t bytes = sizeof(float2) * count;
+  return b->pool ? cudaMallocFromPoolAsync(reinterpret_cast<void**>(p), bytes, b->pool, st)
+                 : cudaMallocAsync(reinterpret_cast<void**>(p), bytes, st);
+}
+
+// The bank's pool; without one (an older driver) the default pool serves.
+void make_pool(shf_bank* b) {
+  cudaMemPoolProps props = {};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.handleTypes = cudaMemHandleTypeNone;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = b->device;
+  unsigned long long keep = shf_bank::kPoolKeep;
+  if (cudaMemPoolCreate(&b->pool, &props) != cudaSuccess) {
+    b->pool = nullptr;
+  } else if (cudaMemPoolSetAttribute(b->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+    cudaMemPoolDestroy(b->pool);
+    b->pool = nullptr;
+  }
+  cudaGetLastError();
+}
+
+}  // namespace
 
 extern "C" {
 
@@ -159,10 +196,12 @@ int shfilters_build(int H, int W, int J, void* stream, shf_bank** out) {
   auto* b = new shf_bank();
   b->g = g;
   b->device = device;
+  make_pool(b);
   std::vector<shf::FilterDesc> d(g.eta);
   shf::filter_descs(J, d.data());
   if ((rc = dev_alloc(&b->bank, static_cast<size_t>(g.eta) * H * g.Wh, "bank")) ||
       (rc = dev_alloc(&b->twH, H, "twH")) || (rc = dev_alloc(&b->twW, W, "twW")) ||
+      (rc = dev_alloc(&b->pt, shf::pass_table_entries(g), "pass tables")) ||
       (rc = dev_alloc(&b->descs, g.eta, "descs")) || (rc = dev_alloc(&b->ranges, g.eta, "ranges"))) {
     shfilters_destroy(b);
     return rc;
@@ -174,6 +213,7 @@ int shfilters_build(int H, int W, int J, void* stream, shf_bank** out) {
   cudaError_t e = cudaMemcpyAsync(b->descs, d.data(), sizeof(shf::FilterDesc) * g.eta, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = shf::launch_twiddles(b->twH, H, st);
   if (e == cudaSuccess) e = shf::launch_twiddles(b->twW, W, st);
+  if (e == cudaSuccess) e = shf::launch_pass_tables(&b->g, b->pt, st);
   if (e == cudaSuccess) e = shf::launch_build_bank(b->bank, b->g, b->descs, st);
   if (e == cudaSuccess) e = shf::launch_filter_ranges(b->bank, b->g, b->ranges, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // d is a host temporary
@@ -191,6 +231,8 @@ int shfilters_destroy(shf_bank* b) {
   cudaFree(b->bank);
   cudaFree(b->twH);
   cudaFree(b->twW);
+  cudaFree(b->pt);
+  if (b->pool) cudaMemPoolDestroy(b->pool);
   cudaFree(b->descs);
   cudaFree(b->ranges);
   delete b;
@@ -219,14 +261,18 @@ int shearlet_analyze(const shf_bank* b, const float* u, int nch, float* coef, vo
   const Geo& g = b->g;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const size_t ph = static_cast<size_t>(g.H) * g.Wh;
+  const std::vector<shf::FilterWave> waves = shf::general_waves(g, nch, shf::default_groups(g, nch));
   float2* tmp = nullptr;
-  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&tmp), sizeof(float2) * ph * nch * (1 + g.eta), st);
+  cudaError_t e = scratch_alloc(b, &tmp, ph * nch + shf::wave_planes(waves) * g.H * g.Wy, st);
   if (e != cudaSuccess) return fail(SHF_ERR_OOM, std::string("shearlet_analyze: ") + cudaGetErrorString(e));
-  float2* Ur = tmp;
-  float2* Y = tmp + ph * nch;
+  float2* Ur = tmp + shf::wave_planes(waves) * g.H * g.Wy;
+  float2* Y = tmp;
   e = shf::run_row_r2c(g, u, Ur, nch, 1.f, st);
-  if (e == cudaSuccess) e = shf::run_col_fan(g, Ur, Y, nch, shf::default_groups(g, nch), st);
-  if (e == cudaSuccess) e = shf::run_row_c2r(g, Y, coef, nch * g.eta, 1.f / (static_cast<float>(g.H) * g.W), st);
+  if (e == cudaSuccess) e = shf::run_col_fwd(g, Ur, nch, st);
+  for (const shf::FilterWave& wv : waves) {
+    if (e == cudaSuccess) e = shf::run_wave_fan(g, Ur, Y, wv, st);
+    if (e == cudaSuccess) e = shf::run_wave_c2r(g, Y, coef, wv, 1.f / (static_cast<float>(g.H) * g.W), st);
+  }
   cudaError_t e2 = cudaFreeAsync(tmp, st);
   if (e != cudaSuccess || e2 != cudaSuccess)
     return fail(SHF_ERR_CUDA, std::string("shearlet_analyze: ") + cudaGetErrorString(e != cudaSuccess ? e : e2));
@@ -235,16 +281,21 @@ int shearlet_analyze(const shf_bank* b, const float* u, int nch, float* coef, vo
 
 namespace {
 // T[nch][H][Wh] = column-inverse of sum_f W_f * fft2(coef_f) (unscaled).
-cudaError_t synthesis_spectrum(const Geo& g, const float* coef, int nch, float2* T, cudaStream_t st) {
+cudaError_t synthesis_spectrum(const shf_bank* b, const Geo& g, const float* coef, int nch, float2* T,
+                               cudaStream_t st) {
   const size_t ph = static_cast<size_t>(g.H) * g.Wh;
   const int groups = shf::default_groups(g, nch);
+  const std::vector<shf::FilterWave> waves = shf::general_waves(g, nch, groups);
+  const size_t ny = shf::wave_planes(waves) * g.H * g.Wy;
   float2* tmp = nullptr;
-  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&tmp), sizeof(float2) * ph * nch * (g.eta + groups), st);
+  cudaError_t e = scratch_alloc(b, &tmp, ny + ph * nch * static_cast<size_t>(groups), st);
   if (e != cudaSuccess) return e;
   float2* Z = tmp;
-  float2* part = tmp + ph * nch * g.eta;
-  e = shf::run_row_r2c(g, coef, Z, nch * g.eta, 1.f, st);
-  if (e == cudaSuccess) e = shf::run_col_gather(g, Z, part, nch, groups, st);
+  float2* part = tmp + ny;
+  for (const shf::FilterWave& wv : waves) {
+    if (e == cudaSuccess) e = shf::run_wave_r2c(g, coef, Z, wv, st);
+    if (e == cudaSuccess) e = shf::run_wave_gather(g, Z, part, nch, groups, wv, st);
+  }
   if (e == cudaSuccess) e = shf::run_col_reduce_inv(g, part, T, nch, groups, st);
   cudaError_t e2 = cudaFreeAsync(tmp, st);
   return e != cudaSuccess ? e : e2;
@@ -259,9 +310,9 @@ int shearlet_synthesize(const shf_bank* b, const float* coef, int nch, float* u,
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const size_t ph = static_cast<size_t>(g.H) * g.Wh;
   float2* T = nullptr;
-  cudaError_t e = cudaMallocAsync(reinterpret_cast<void**>(&T), sizeof(float2) * ph * nch, st);
+  cudaError_t e = scratch_alloc(b, &T, ph * nch, st);
   if (e != cudaSuccess) return fail(SHF_ERR_OOM, std::string("shearlet_synthesize: ") + cudaGetErrorString(e));
-  e = synthesis_spectrum(g, coef, nch, T, st);
+  e = synthesis_spectrum(b, g, coef, nch, T, st);
   if (e == cudaSuccess) e = shf::run_row_c2r(g, T, u, nch, 1.f / (static_cast<float>(g.H) * g.W), st);
   cudaError_t e2 = cudaFreeAsync(T, st);
   if (e != cudaSuccess || e2 != cudaSuccess)
@@ -329,7 +380,7 @@ int restart(seg_state* st, const float* codebook) {
 
 // Launches of one iteration, plus the closing mark.
 int marks_needed(const seg_state* st) {
-  if (!st->fast) return 8;
+  if (!st->fast) return 4 + 3 * static_cast<int>(st->waves.size());
   int n = 4;  // u/w-step, column forward, reduction, end
   n += 3 * static_cast<int>(st->plan.wave_f0.size());  // fan, v-step, gather per wave
   return n;
@@ -398,12 +449,16 @@ cudaError_t enqueue_iteration(seg_state* st, bool timed, signed char* code = nul
       e = shf::run_fast_iteration_body(g, st->plan, st->Ur, st->uhat, st->Y, st->bv, st->thr, st->partial, st->T,
                                        st->K, scale, s, hook, code);
   } else {
-    hook.mark(shf::kKindFan);
-    if (e == cudaSuccess) e = shf::run_col_fan(g, st->Ur, st->Y, st->K, st->groups, s);
-    hook.mark(shf::kKindShrink);
-    if (e == cudaSuccess) e = shf::run_row_shrink(g, st->Y, st->bv, st->thr, st->K * g.eta, scale, s);
-    hook.mark(shf::kKindGather);
-    if (e == cudaSuccess) e = shf::run_col_gather(g, st->Y, st->partial, st->K, st->groups, s);
+    hook.mark(shf::kKindColFwd);
+    if (e == cudaSuccess) e = shf::run_col_fwd(g, st->Ur, st->K, s);
+    for (const shf::FilterWave& wv : st->waves) {
+      hook.mark(shf::kKindFan);
+      if (e == cudaSuccess) e = shf::run_wave_fan(g, st->Ur, st->Y, wv, s);
+      hook.mark(shf::kKindShrink);
+      if (e == cudaSuccess) e = shf::run_wave_shrink(g, st->Y, st->bv, st->thr, wv, scale, s);
+      hook.mark(shf::kKindGather);
+      if (e == cudaSuccess) e = shf::run_wave_gather(g, st->Y, st->partial, st->K, st->groups, wv, s);
+    }
     hook.mark(shf::kKindReduce);
     if (e == cudaSuccess) e = shf::run_col_reduce_inv(g, st->partial, st->T, st->K, st->groups, s);
   }
@@ -419,9 +474,12 @@ cudaError_t enqueue_generic_iteration(seg_state* st, float* gout) {
   cudaStream_t s = st->stream;
   cudaError_t e =
       shf::run_row_ustep(g, st->T, st->s, st->w, st->bw, st->u, st->Ur, nullptr, st->K, st->gamma, scale, s);
-  if (e == cudaSuccess) e = shf::run_col_fan(g, st->Ur, st->un_Y, st->K, st->groups, s);
-  if (e == cudaSuccess) e = shf::run_row_shrink(g, st->un_Y, st->bv, st->thr, st->K * g.eta, scale, s, gout);
-  if (e == cudaSuccess) e = shf::run_col_gather(g, st->un_Y, st->un_partial, st->K, st->un_groups, s);
+  if (e == cudaSuccess) e = shf::run_col_fwd(g, st->Ur, st->K, s);
+  for (const shf::FilterWave& wv : st->un_waves) {
+    if (e == cudaSuccess) e = shf::run_wave_fan(g, st->Ur, st->un_Y, wv, s);
+    if (e == cudaSuccess) e = shf::run_wave_shrink(g, st->un_Y, st->bv, st->thr, wv, scale, s, gout);
+    if (e == cudaSuccess) e = shf::run_wave_gather(g, st->un_Y, st->un_partial, st->K, st->un_groups, wv, s);
+  }
   if (e == cudaSuccess) e = shf::run_col_reduce_inv(g, st->un_partial, st->T, st->K, st->un_groups, s);
   return e;
 }
@@ -589,19 +647,28 @@ int install_generic_plan(seg_state* st, int TC, int RB, int groups) {
   if (!shf::set_generic_tiles(&g, TC, RB, st->K, optin))
     return fail(SHF_ERR_ARG, "tile shape not supported for this image size");
   groups = normalise_groups(g.eta, groups);
-  float2* partial = nullptr;
+  std::vector<shf::FilterWave> waves = shf::general_waves(g, st->K, groups);
+  float2 *partial = nullptr, *Y = nullptr;
   int rc = dev_alloc(&partial, st->Ph() * st->K * static_cast<size_t>(groups), "partial");
-  if (rc) return rc;
+  if (!rc) rc = dev_alloc(&Y, shf::wave_planes(waves) * g.H * g.Wy, "Y");
+  if (rc) {
+    cudaFree(partial);
+    return rc;
+  }
   cudaError_t e = cudaStreamSynchronize(st->stream);
   if (e != cudaSuccess) {
     cudaFree(partial);
+    cudaFree(Y);
     return fail(SHF_ERR_CUDA, std::string("install_generic_plan: ") + cudaGetErrorString(e));
   }
   drop_graphs(st);
   cudaFree(st->partial);
+  cudaFree(st->Y);
   st->partial = partial;
+  st->Y = Y;
   st->g = g;
   st->groups = groups;
+  st->waves = std::move(waves);
   return SHF_OK;
 }
 
@@ -611,22 +678,27 @@ int energy_of_w(seg_state* st, double* out_host) {
   const float scale = 1.f / (static_cast<float>(g.H) * g.W);
   // <w, s>
   SHF_CK(shf::launch_dot(st->w, st->s, static_cast<long>(P * st->K), st->red + 2, 512, st->red, st->stream));
-  // sum_f Lambda_f ||(S w)_f||_1: row-forward of w, fan-out over all filters,
-  // l1 of the row-inverse; the spectra of all K*eta planes go to stream-ordered
-  // temporaries (the state's scratch holds one wave of filters on the fast path).
+  // sum_f Lambda_f ||(S w)_f||_1: row- and column-forward of w, then per wave
+  // the fan-out and the l1 of the row-inverse, in stream-ordered temporaries
   const size_t ph = st->Ph();
+  const std::vector<shf::FilterWave> waves = shf::general_waves(g, st->K, shf::default_groups(g, st->K));
+  const size_t ny = shf::wave_planes(waves) * g.H * g.Wy;
+  const int nb = shf::l1_blocks(g, st->K);
   float2* tmp = nullptr;
-  SHF_CK(cudaMallocAsync(reinterpret_cast<void**>(&tmp), sizeof(float2) * ph * st->K * (1 + g.eta), st->stream));
-  float2* Uw = tmp;
-  float2* Yw = tmp + ph * st->K;
+  SHF_CK(scratch_alloc(st->bank, &tmp, ph * st->K + ny + static_cast<size_t>(nb), st->stream));
+  float2* Yw = tmp;
+  float2* Uw = Yw + ny;
+  double* part = reinterpret_cast<double*>(Uw + ph * st->K);  // float2 units: 8-byte aligned
   cudaError_t e = shf::run_row_r2c(g, st->w, Uw, st->K, 1.f, st->stream);
-  if (e == cudaSuccess) e = shf::run_col_fan(g, Uw, Yw, st->K, st->groups, st->stream);
-  int nb = 0;
-  if (e == cudaSuccess) e = shf::run_row_l1(g, Yw, st->lam, st->K * g.eta, scale, st->red + 2 + 512, &nb, st->stream);
+  if (e == cudaSuccess) e = shf::run_col_fwd(g, Uw, st->K, st->stream);
+  for (const shf::FilterWave& wv : waves) {
+    if (e == cudaSuccess) e = shf::run_wave_fan(g, Uw, Yw, wv, st->stream);
+    if (e == cudaSuccess) e = shf::run_wave_l1(g, Yw, st->lam, wv, scale, part, st->stream);
+  }
+  if (e == cudaSuccess) e = shf::launch_sum_partials(part, nb, st->red + 1, st->stream);
   cudaError_t e2 = cudaFreeAsync(tmp, st->stream);
   SHF_CK(e);
   SHF_CK(e2);
-  SHF_CK(shf::launch_sum_partials(st->red + 2 + 512, nb, st->red + 1, st->stream));
   double h[2];
   SHF_CK(cudaMemcpyAsync(h, st->red, sizeof(h), cudaMemcpyDeviceToHost, st->stream));
   SHF_CK(cudaStreamSynchronize(st->stream));
@@ -708,8 +780,7 @@ int seg_admm_init(const shf_bank* b, const float* f, int C, const float* codeboo
       return fail(SHF_ERR_CUDA, std::string("seg_admm_init: ") + cudaGetErrorString(e));
     }
   }
-  const int l1_blocks = ((g.H + g.RB - 1) / g.RB) * K * g.eta;
-  st->red_len = 2 + 512 + l1_blocks;
+  if (!st->fast) st->waves = shf::general_waves(g, K, st->groups);
   int rc;
   if ((rc = dev_alloc(&st->f, P * C, "f")) || (rc = dev_alloc(&st->s, P * K, "s")) ||
       (rc = dev_alloc(&st->bv, P * K * g.eta, "b_v")) || (rc = dev_alloc(&st->w, P * K, "w")) ||
@@ -717,14 +788,14 @@ int seg_admm_init(const shf_bank* b, const float* f, int C, const float* codeboo
       (rc = dev_alloc(&st->stv, P * K, "stv")) || (rc = dev_alloc(&st->Ur, Ph * K, "Ur")) ||
       (rc = dev_alloc(&st->T, Ph * K, "T")) ||
       (st->fast && (rc = dev_alloc(&st->uhat, static_cast<size_t>(g.H) * shf::fast_pitch(g) * K, "uhat"))) ||
-      // coefficient spectra of the whole label set and one partial sum per
-      // filter group on the general path (the fast path's come with its plan)
-      (!st->fast && (rc = dev_alloc(&st->Y, Ph * K * g.eta, "Y"))) ||
+      // one wave's coefficient spectra and one partial sum per filter group on
+      // the general path (the fast path's come with its plan)
+      (!st->fast && (rc = dev_alloc(&st->Y, shf::wave_planes(st->waves) * g.H * g.Wy, "Y"))) ||
       (!st->fast && (rc = dev_alloc(&st->partial, Ph * K * static_cast<size_t>(st->groups), "partial"))) ||
       (st->fast && (rc = install_fast_plan(st, shf::kDefaultWaveMiB, 0))) ||
       (rc = dev_alloc(&st->thr, g.eta, "thr")) || (rc = dev_alloc(&st->lam, g.eta, "lam")) ||
       (rc = dev_alloc(&st->gap, P, "gap")) || (rc = dev_alloc(&st->labels, P, "labels")) ||
-      (rc = dev_alloc(&st->flag, 1, "flag")) || (rc = dev_alloc(&st->red, st->red_len, "red"))) {
+      (rc = dev_alloc(&st->flag, 1, "flag")) || (rc = dev_alloc(&st->red, 2 + 512, "red"))) {
     free_state(st);
     return rc;
   }
@@ -1119,7 +1190,7 @@ int seg_admm_set(seg_state* st, int what, const void* src, int on_host) {
       cudaError_t e = cudaMemcpyAsync(d, src, sizeof(float) * KP * g.eta,
                                       on_host ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice, st->stream);
       if (e == cudaSuccess) e = shf::launch_sub(d, st->bv, d, static_cast<long>(KP * g.eta), st->stream);
-      if (e == cudaSuccess) e = synthesis_spectrum(g, d, st->K, st->T, st->stream);
+      if (e == cudaSuccess) e = synthesis_spectrum(st->bank, g, d, st->K, st->T, st->stream);
       cudaError_t e2 = cudaFreeAsync(d, st->stream);
       if (e == cudaSuccess) e = e2;
       if (e == cudaSuccess && on_host) e = cudaStreamSynchronize(st->stream);
@@ -1372,13 +1443,18 @@ cudaError_t enqueue_unrolled_bwd(seg_state* st, const UnLayout& U) {
       } else {
         // dbar = S Qbar
         ok(shf::run_row_r2c(g, Qbar, Uw, K, 1.f, s));
-        ok(shf::run_col_fan(g, Uw, st->un_Y, K, st->groups, s));
-        ok(shf::run_row_c2r(g, st->un_Y, dbar, K * eta, scale, s));
+        ok(shf::run_col_fwd(g, Uw, K, s));
+        for (const shf::FilterWave& wv : st->un_waves) {
+          ok(shf::run_wave_fan(g, Uw, st->un_Y, wv, s));
+          ok(shf::run_wave_c2r(g, st->un_Y, dbar, wv, scale, s));
+        }
         ok(shf::launch_adj_shrink(grec + static_cast<size_t>(i) * NC, dbar, bvbar, st->thr, K, eta,
                                   static_cast<long>(P), tpart, tbar, s));
         // stv = S^T bvbar
-        ok(shf::run_row_r2c(g, bvbar, st->un_Y, K * eta, 1.f, s));
-        ok(shf::run_col_gather(g, st->un_Y, st->un_partial, K, st->un_groups, s));
+        for (const shf::FilterWave& wv : st->un_waves) {
+          ok(shf::run_wave_r2c(g, bvbar, st->un_Y, wv, s));
+          ok(shf::run_wave_gather(g, st->un_Y, st->un_partial, K, st->un_groups, wv, s));
+        }
         ok(shf::run_col_reduce_inv(g, st->un_partial, Tt, K, st->un_groups, s));
       }
       ok(shf::run_row_c2r(g, Tt, stv, K, scale, s));
@@ -1401,7 +1477,8 @@ int seg_admm_unrolled_fwd(seg_state* st, int T, int ckpt_every) {
   // the general path keeps the spectra of every filter; the fast path
   // iterates with its own wave scratch
   if (!st->fast && !st->un_Y) {
-    if ((rc = dev_alloc(&st->un_Y, Ph * st->K * g.eta, "unrolled scratch")) ||
+    st->un_waves = shf::general_waves(g, st->K, st->groups);
+    if ((rc = dev_alloc(&st->un_Y, shf::wave_planes(st->un_waves) * g.H * g.Wy, "unrolled scratch")) ||
         (rc = dev_alloc(&st->un_partial, Ph * st->K * st->groups, "unrolled partials")))
       return rc;
     st->un_groups = st->groups;

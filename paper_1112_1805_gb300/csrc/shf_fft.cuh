@@ -1,6 +1,7 @@
-// Shared-memory FFT building blocks for sm_103a: mixed-radix (2, 3, 4, 5, 8)
-// Stockham stages on float2 data, and the packing that turns a length-W real
-// transform into a length-W/2 complex one.  Conventions follow the paper's
+// FFT building blocks for sm_103a: complex helpers, the small DFTs, the stage
+// plans of the general lengths (the transforms themselves are in shf_gfft.cuh),
+// and the packing that turns a length-W real transform into a length-W/2
+// complex one.  Conventions follow the paper's
 // fft2/ifft2 (Sec. 2): forward exponent -1 without scaling, inverse exponent
 // +1 (the 1/(H W) factor is applied by the caller).
 #pragma once
@@ -9,14 +10,33 @@
 
 namespace shf {
 
-constexpr int kMaxStages = 16;
+constexpr int kMaxStages = 6;
 
-// Radix sequence of one transform length L (product of the radices).
+// One Stockham stage of a transform of length L: radix, span (product of the
+// radices before it), butterflies L / radix, the offset of its twiddles in the
+// pass table ([t - 1][j mod span], t = 1..radix - 1), and multipliers that
+// divide small integers by the span and by the butterfly count (0: divisor 1).
+struct FftStage {
+  int R, Ns, nb, off;
+  unsigned mNs, mNb;
+};
 struct FftPlan {
   int L;
   int nst;
-  int radix[kMaxStages];
+  FftStage st[kMaxStages];
 };
+
+// x / d for x d < 2^32, from fdiv_mul(d) = floor(2^32 / d) + 1 (d > 1).
+__host__ __device__ __forceinline__ unsigned fdiv_mul(unsigned d) {
+  return d <= 1 ? 0u : static_cast<unsigned>((1ull << 32) / d) + 1u;
+}
+__host__ __device__ __forceinline__ unsigned fdiv(unsigned x, unsigned m) {
+#ifdef __CUDA_ARCH__
+  return m ? __umulhi(x, m) : x;
+#else
+  return m ? static_cast<unsigned>((static_cast<unsigned long long>(x) * m) >> 32) : x;
+#endif
+}
 
 // Complex sums on the device use the packed FP32x2 adds of sm_100-class GPUs
 // (one instruction for both components, IEEE round-to-nearest per component,
@@ -179,82 +199,6 @@ __host__ __device__ __forceinline__ void dft_small(float2* v) {
   if (R == 8) dft8<S>(v);
 }
 
-// One butterfly of a Stockham stage of length L, radix R, sub-transform span
-// Ns (product of the radices of the earlier stages).  Element (i, b) of the
-// batch lives at ptr[i*istride + b*bstride].  Reads in(j + t L/R), applies
-// the twiddles exp(S 2 pi i t (j mod Ns) / (Ns R)), an R-point DFT, and writes
-// out((j / Ns) Ns R + (j mod Ns) + q Ns).  tw[m] = exp(-2 pi i m / (L twstep)).
-template <int R, int S>
-__host__ __device__ __forceinline__ void stockham_bfly(const float2* in, float2* out, int L, int Ns, int j, int b,
-                                                       int istride, int bstride, const float2* tw, int twstep) {
-  const int nb = L / R;
-  float2 v[R];
-#pragma unroll
-  for (int t = 0; t < R; ++t) v[t] = in[(j + t * nb) * istride + b * bstride];
-  const int k = j % Ns;
-  if (Ns > 1) {
-    const int base = k * (L / (Ns * R)) * twstep;
-#pragma unroll
-    for (int t = 1; t < R; ++t) {
-      float2 w = tw[t * base];
-      if (S > 0) w.y = -w.y;
-      v[t] = c_mul(v[t], w);
-    }
-  }
-  dft_small<R, S>(v);
-  const int o = (j / Ns) * Ns * R + k;
-#pragma unroll
-  for (int q = 0; q < R; ++q) out[(o + q * Ns) * istride + b * bstride] = v[q];
-}
-
-// Work item `idx` of a stage: BATCH_FAST maps consecutive items to
-// consecutive batch members (column transforms of a row-major tile),
-// otherwise to consecutive butterflies of one sequence (row transforms).
-template <int S, bool BATCH_FAST>
-__host__ __device__ __forceinline__ void stockham_item(const float2* in, float2* out, int L, int R, int Ns, int idx,
-                                                       int B, int istride, int bstride, const float2* tw,
-                                                       int twstep) {
-  const int nb = L / R;
-  int j, b;
-  if (BATCH_FAST) {
-    b = idx % B;
-    j = idx / B;
-  } else {
-    j = idx % nb;
-    b = idx / nb;
-  }
-  switch (R) {
-    case 2: stockham_bfly<2, S>(in, out, L, Ns, j, b, istride, bstride, tw, twstep); break;
-    case 3: stockham_bfly<3, S>(in, out, L, Ns, j, b, istride, bstride, tw, twstep); break;
-    case 4: stockham_bfly<4, S>(in, out, L, Ns, j, b, istride, bstride, tw, twstep); break;
-    case 5: stockham_bfly<5, S>(in, out, L, Ns, j, b, istride, bstride, tw, twstep); break;
-    default: stockham_bfly<8, S>(in, out, L, Ns, j, b, istride, bstride, tw, twstep); break;
-  }
-}
-
-#ifdef __CUDACC__
-// A batch of B transforms of length p.L in shared memory, ping-ponging
-// between a and b; returns the buffer holding the natural-order result.
-// All threads of the block must call it (it synchronises after each stage).
-template <int S, bool BATCH_FAST>
-__device__ __forceinline__ float2* stockham(float2* a, float2* b, const FftPlan& p, int B, int istride, int bstride,
-                                            const float2* __restrict__ tw, int twstep) {
-  int Ns = 1;
-  for (int s = 0; s < p.nst; ++s) {
-    const int R = p.radix[s];
-    const int total = (p.L / R) * B;
-    for (int idx = threadIdx.x; idx < total; idx += blockDim.x)
-      stockham_item<S, BATCH_FAST>(a, b, p.L, R, Ns, idx, B, istride, bstride, tw, twstep);
-    __syncthreads();
-    float2* t = a;
-    a = b;
-    b = t;
-    Ns *= R;
-  }
-  return a;
-}
-#endif
-
 // Real transforms of length W = 2L through one complex transform of length L.
 // twW[m] = exp(-2 pi i m / W).
 //
@@ -278,40 +222,55 @@ __host__ __device__ __forceinline__ float2 r2c_unpack(const float2* Z, int L, in
   return unpack_combine(s, d, twW[k]);
 }
 
-// Radix sequence for L = 2^a 3^b 5^c (8s first, then a 4 or 2, then 3s and
-// 5s); returns false when L has another prime factor or too many stages.
-inline bool make_plan(int L, FftPlan* p) {
-  p->L = L;
-  p->nst = 0;
-  int n = L, a = 0;
-  while (n % 2 == 0) {
-    n /= 2;
-    ++a;
-  }
-  int b = 0, c = 0;
-  while (n % 3 == 0) {
-    n /= 3;
-    ++b;
-  }
-  while (n % 5 == 0) {
-    n /= 5;
-    ++c;
-  }
-  if (n != 1 || L < 1) return false;
-  auto push = [&](int r) {
-    if (p->nst >= kMaxStages) return false;
-    p->radix[p->nst++] = r;
-    return true;
+// Stage plan for L = 2^a 3^b 5^c: the fewest stages of radices up to 16, then
+// the smallest sum of radices (registers and twiddles), in increasing order or,
+// for `reversed`, in decreasing order (the forward transform of the v-step,
+// whose first stage takes over the last stage's registers of the inverse one).
+// False when L has another prime factor.
+inline bool make_plan(int L, FftPlan* p, bool reversed = false) {
+  constexpr int kRadices[] = {2, 3, 4, 5, 6, 8, 9, 10, 12, 15, 16};
+  if (L < 1) return false;
+  int best[kMaxStages], nbest = kMaxStages + 1, sbest = 0, cur[kMaxStages];
+  auto search = [&](auto&& self, int rest, int depth, int from, int sum) -> void {
+    if (rest == 1) {
+      if (depth >= 1 && (depth < nbest || (depth == nbest && sum < sbest))) {
+        nbest = depth;
+        sbest = sum;
+        for (int i = 0; i < depth; ++i) best[i] = cur[i];
+      }
+      return;
+    }
+    if (depth >= kMaxStages || depth >= nbest) return;
+    for (int i = from; i < 11; ++i)
+      if (rest % kRadices[i] == 0) {
+        cur[depth] = kRadices[i];
+        self(self, rest / kRadices[i], depth + 1, i, sum + kRadices[i]);
+      }
   };
-  for (int i = 0; i < a / 3; ++i)
-    if (!push(8)) return false;
-  if (a % 3 == 2 && !push(4)) return false;
-  if (a % 3 == 1 && !push(2)) return false;
-  for (int i = 0; i < b; ++i)
-    if (!push(3)) return false;
-  for (int i = 0; i < c; ++i)
-    if (!push(5)) return false;
+  search(search, L, 0, 0, 0);
+  if (nbest > kMaxStages) return false;
+  p->L = L;
+  p->nst = nbest;
+  int Ns = 1, off = 0;
+  for (int s = 0; s < nbest; ++s) {
+    FftStage& g = p->st[s];
+    g.R = best[reversed ? nbest - 1 - s : s];
+    g.Ns = Ns;
+    g.nb = L / g.R;
+    g.off = off;
+    g.mNs = fdiv_mul(static_cast<unsigned>(Ns));
+    g.mNb = fdiv_mul(static_cast<unsigned>(g.nb));
+    if (s > 0) off += (g.R - 1) * Ns;
+    Ns *= g.R;
+  }
   return true;
+}
+
+// Entries of a plan's pass table.
+inline int plan_table(const FftPlan& p) {
+  int n = 0;
+  for (int s = 1; s < p.nst; ++s) n += (p.st[s].R - 1) * p.st[s].Ns;
+  return n > 0 ? n : 1;
 }
 
 }  // namespace shf

@@ -24,11 +24,13 @@ struct Geo {
   int H, W, J, eta;
   int L;   // W / 2, length of the packed complex row transform
   int Wh;  // W / 2 + 1, columns of the half spectrum
-  FftPlan planH, planL;
+  int Wy;  // row pitch (complex) of the coefficient spectra of a wave
+  // stage plans: columns, rows, and the rows' reversed one with their pass tables
+  FftPlan planH, planL, planLr;
+  const float2 *ptH, *ptL, *ptLr;
   int TC;       // columns per column-transform tile
   int ntiles;   // ceil(Wh / TC)
   int RB;       // rows per row-transform block
-  int maxe;     // per-thread register elements of a column tile (8, 16 or 32)
   const float2* twH;  // exp(-2 pi i m / H), m < H
   const float2* twW;  // exp(-2 pi i m / W), m < W
   const float* bank;  // [eta][H][Wh]
@@ -46,6 +48,10 @@ int filter_descs(int J, FilterDesc* out);  // returns eta
 
 // Filter bank and tables (shf_bank.cu).
 cudaError_t launch_twiddles(float2* tw, int N, cudaStream_t st);
+// The pass tables of g's plans from its twiddles twH, twW: entries in all, and
+// their construction in `tab` (sets g's ptH, ptL, ptLr).
+size_t pass_table_entries(const Geo& g);
+cudaError_t launch_pass_tables(Geo* g, float2* tab, cudaStream_t st);
 cudaError_t launch_build_bank(float* bank, const Geo& g, const FilterDesc* descs_dev, cudaStream_t st);
 cudaError_t launch_filter_ranges(const float* bank, const Geo& g, int2* ranges, cudaStream_t st);
 cudaError_t launch_data_term(const float* f, int C, const float* codebook_host, int K, float* s, int P,
@@ -59,24 +65,46 @@ cudaError_t launch_sqdiff(const float* a, const float* b, long n, double* partia
                           cudaStream_t st);
 cudaError_t launch_sum_partials(const double* partial, int n, double* out, cudaStream_t st);
 
-// Transform kernels (shf_transform.cu).
+// Transform kernels of the general lengths (rows: shf_transform.cu, columns:
+// shf_gcol.cu).
 // Real rows [planes][H][W] -> half spectra [planes][H][Wh] (row transforms).
 cudaError_t run_row_r2c(const Geo& g, const float* in, float2* out, int planes, float scale, cudaStream_t st);
 // Half spectra -> real rows, times `scale`.
 cudaError_t run_row_c2r(const Geo& g, const float2* in, float* out, int planes, float scale, cudaStream_t st);
-// ADMM v-step on coefficient spectra Y [nch*eta][H][Wh] (in place) and b_v.
-// gout (optional): receives g = b_v + S u before the clipping, [planes][H][W].
-cudaError_t run_row_shrink(const Geo& g, float2* Y, float* bv, const float* thr, int planes, float scale,
-                           cudaStream_t st, float* gout = nullptr);
-// sum_f lam[f] * ||ifft rows of Y_f||_1 into partial[nblocks] (nblocks returned).
-cudaError_t run_row_l1(const Geo& g, const float2* Y, const float* lam, int planes, float scale, double* partial,
-                       int* nblocks, cudaStream_t st);
-// Column transform, fan-out over filters: in [nch][H][Wh] (row spectra) ->
-// out [nch][eta][H][Wh] = column-inverse( W_f * column-forward(in) ).
-cudaError_t run_col_fan(const Geo& g, const float2* in, float2* out, int nch, int groups, cudaStream_t st);
-// Column transform, gather over filters: partial[grp][nch][H][Wh] =
-// sum_{f in grp} W_f * column-forward(in[ch][f]).
-cudaError_t run_col_gather(const Geo& g, const float2* in, float2* partial, int nch, int groups, cudaStream_t st);
+// A wave: filters [f0, f0 + nf) of channels [c0, c0 + nc).  Its spectra are
+// planes Y_p [H][Wy], p = (c - c0) nf + (f - f0), of which only the filters'
+// column ranges are written and read; coefficients are planes c eta + f.
+struct FilterWave {
+  int c0, nc, f0, nf;
+};
+// The waves of nch channels with the synthesis summed in `groups` filter
+// groups (each group inside one wave), and the planes of the largest.
+std::vector<FilterWave> general_waves(const Geo& g, int nch, int groups);
+size_t wave_planes(const std::vector<FilterWave>& waves);
+// Column-forward of row spectra U [nch][H][Wh], in place.
+cudaError_t run_col_fwd(const Geo& g, float2* U, int nch, cudaStream_t st);
+// out = column-inverse( g.bank * column-forward(in) ), planes [nch][H][Wh], one
+// filter [H][Wh].
+cudaError_t run_col_filter(const Geo& g, const float2* in, float2* out, int nch, cudaStream_t st);
+// Y = column-inverse( W_f * uhat[c] ) over the wave.
+cudaError_t run_wave_fan(const Geo& g, const float2* uhat, float2* Y, const FilterWave& wv, cudaStream_t st);
+// Row transforms of the wave's coefficient planes, both ways.
+cudaError_t run_wave_r2c(const Geo& g, const float* coef, float2* Y, const FilterWave& wv, cudaStream_t st);
+cudaError_t run_wave_c2r(const Geo& g, const float2* Y, float* coef, const FilterWave& wv, float scale,
+                         cudaStream_t st);
+// ADMM v-step on the wave's spectra (in place) and b_v [nch][eta][H][W].
+// gout (optional): receives g = b_v + S u before the clipping, laid out as b_v.
+cudaError_t run_wave_shrink(const Geo& g, float2* Y, float* bv, const float* thr, const FilterWave& wv, float scale,
+                            cudaStream_t st, float* gout = nullptr);
+// lam[f] * ||row-inverse of Y||_1 of the wave's planes, one FP64 partial per
+// block of the l1_blocks(g, nch) of all planes.
+cudaError_t run_wave_l1(const Geo& g, const float2* Y, const float* lam, const FilterWave& wv, float scale,
+                        double* partial, cudaStream_t st);
+int l1_blocks(const Geo& g, int nch);
+// partial[grp][nch][H][Wh] = sum_{f in grp} W_f * column-forward(Y) for the
+// wave's groups and channels.
+cudaError_t run_wave_gather(const Geo& g, const float2* Y, float2* partial, int nch, int groups, const FilterWave& wv,
+                            cudaStream_t st);
 // out[nch][H][Wh] = column-inverse( sum_grp partial[grp] ).
 cudaError_t run_col_reduce_inv(const Geo& g, const float2* partial, float2* out, int nch, int groups,
                                cudaStream_t st);

@@ -80,9 +80,14 @@ int shearlet_analyze_noalloc(const shf_bank* bank, const float* u, int nch, floa
   float2* Y = Ur + ph * nch;
   // Every scratch element read below is first written by this call, so nothing
   // has to be cleared between calls.
+  // (the spectra at the pitch Wh: a wave holds at most nch eta planes)
+  g.Wy = g.Wh;
   cudaError_t e = shf::run_row_r2c(g, u, Ur, nch, 1.f, st);
-  if (e == cudaSuccess) e = shf::run_col_fan(g, Ur, Y, nch, shf::default_groups(g, nch), st);
-  if (e == cudaSuccess) e = shf::run_row_c2r(g, Y, coef, nch * eta, 1.f / (static_cast<float>(H) * W), st);
+  if (e == cudaSuccess) e = shf::run_col_fwd(g, Ur, nch, st);
+  for (const shf::FilterWave& wv : shf::general_waves(g, nch, shf::default_groups(g, nch))) {
+    if (e == cudaSuccess) e = shf::run_wave_fan(g, Ur, Y, wv, st);
+    if (e == cudaSuccess) e = shf::run_wave_c2r(g, Y, coef, wv, 1.f / (static_cast<float>(H) * W), st);
+  }
   if (e != cudaSuccess)
     return shf::set_error(SHF_ERR_CUDA, std::string("shearlet_analyze_noalloc: ") + cudaGetErrorString(e));
   return SHF_OK;

@@ -1,27 +1,42 @@
-// Shearlet transform and ADMM kernels (Haeuser & Steidl, arXiv:1112.1805).
+// Row kernels of the general lengths (Haeuser & Steidl, arXiv:1112.1805): sizes
+// H, W/2 = 2^a 3^b 5^c that the register-FFT path (shf_fast_*.cu) does not
+// take, and the transforms of single planes at any size.
 //
 // A 2-D transform of an H x W real plane is split into row transforms (real
 // length W, packed into complex length W/2) and column transforms (complex
 // length H) over the W/2+1 columns of the half spectrum.  The filters are real
 // and even, so every product of a filter with the spectrum of a real plane is
-// again the half spectrum of a real plane.
+// again the half spectrum of a real plane.  They also vanish outside a column
+// range (compact support, Sec. 2, Remark 1): coefficient spectra are computed,
+// stored and read on that range only.
 //
-// Analysis S (eq. wichtig), for each channel:
-//   row-forward -> [k_col_fan: column-forward, then per filter f:
-//                   multiply by W_f, column-inverse] -> row-inverse.
-// Synthesis S^T (Fourier-domain form after the Theorem), for each channel:
-//   row-forward of every coefficient plane -> [k_col_gather: column-forward,
-//   multiply by W_f, sum over a filter group] -> [k_col_reduce_inv: sum over
-//   groups in fixed order, column-inverse] -> row-inverse.
+// Analysis S (eq. wichtig) in waves of (channel, filter) pairs whose spectra
+// stay near the L2 between the launches:
+//   row-forward -> column-forward (in place) -> per wave [fan: times W_f,
+//   column-inverse] -> row-inverse.
+// Synthesis S^T (Fourier-domain form after the Theorem), per wave:
+//   row-forward of the coefficient planes -> [gather: column-forward, times
+//   W_f, sum over a filter group]; then [reduce: sum over groups in fixed
+//   order, column-inverse] -> row-inverse.
 // ADMM iteration (Sec. 3), state (b_v, T = column-inverse of the synthesis
 // spectrum of v - b_v, w, b_w):
 //   k_row_ustep   : T -> S^T(v-b_v); u-step; w-step; b_w; row-forward of u
-//   k_col_fan     : u spectra -> per-filter coefficient spectra
-//   k_row_shrink  : row-inverse -> g = b_v + Su; b_v <- clip(g); d = soft(g) - clip(g)
-//                   = v - b_v; row-forward of d (in place)
-//   k_col_gather + k_col_reduce_inv : synthesis spectrum of d -> T
+//   column-forward of u's row spectra
+//   per wave: fan; k_row_shrink: row-inverse -> g = b_v + Su; b_v <- clip(g);
+//     d = soft(g) - clip(g) = v - b_v; row-forward of d (in place); gather
+//   reduce        : synthesis spectrum of d -> T
+// Every transform runs on the staged FFTs of shf_gfft.cuh.  Measured against
+// full-width spectra of all channels at once and radix-2/3/4/5/8 stages that
+// each crossed shared memory: an iteration at 480 x 640, K = 5, J = 4 3.14 ->
+// 1.09 ms (u/w-step 70 -> 59 us, fan 776 -> 157, v-step 955 -> 613, gather
+// 1213 -> 200, reduce 34 -> 26, column-forward 12); synthesis of three 1080 x
+// 1920 channels 7.8 -> 2.5 ms (row-forward 2224 -> 1200 us, gather 5227 ->
+// 1180).  The v-step and the row transforms are bound by instruction issue and
+// latency (issue slots 40% busy, 127 registers, two CTAs per SM).
 #include <algorithm>
 
+#include "shf_fast.h"
+#include "shf_gfft.cuh"
 #include "shf_internal.h"
 #include "shf_simplex.cuh"
 
@@ -29,281 +44,268 @@ namespace shf {
 
 namespace {
 
+using fast::launch_pdl;
+using fast::pdl_trigger;
+using fast::pdl_wait;
+
 // ---------------------------------------------------------------------------
-// Column kernels: one CTA owns a tile of TC consecutive half-spectrum columns
-// over all H rows, stored row-major [H][TC] in shared memory (coalesced
-// loads; consecutive threads work on consecutive columns).
+// One CTA owns RB consecutive rows of one plane.  A real row of length W = 2L
+// is handled as the complex row z[n] = x[2n] + i x[2n+1].
 // ---------------------------------------------------------------------------
 
-template <int MAXE>
-__global__ void __launch_bounds__(kColThreads)
-    k_col_fan(const float2* __restrict__ in, const float* __restrict__ bank, float2* __restrict__ out, int H, int Wh,
-              int eta, int TC, int fg, FftPlan pH, const float2* __restrict__ twH) {
+// A plane of a launch: its index, and where its data and its filter are.  A
+// plain launch has planes 0, 1, ...; a wave's plane p is filter f0 + p mod nf of
+// channel c0 + p / nf, whose coefficients are plane c eta + f.
+struct Plane {
+  size_t data;  // plane of the real data
+  int f;        // filter (waves)
+  int c0, c1;   // columns of the half spectrum that are not zero by construction
+};
+template <bool FILT>
+__device__ __forceinline__ Plane plane_of(const Geo& g, const FilterWave& wv) {
+  Plane p{blockIdx.y, 0, 0, g.L};
+  if constexpr (FILT) {
+    const int q = static_cast<int>(blockIdx.y) / wv.nf;
+    p.f = wv.f0 + static_cast<int>(blockIdx.y) - q * wv.nf;
+    p.data = static_cast<size_t>(wv.c0 + q) * g.eta + p.f;
+    if (g.ranges) {
+      const int2 r = g.ranges[p.f];
+      p.c0 = r.x;
+      p.c1 = min(r.y, g.L);
+    }
+  }
+  return p;
+}
+
+// Element k of the inverse packing of half-spectrum row X, zero outside [c0, c1].
+__device__ __forceinline__ float2 packed(const float2* X, int L, int k, int c0, int c1, const float2* __restrict__ twW) {
+  const int m = L - k;
+  const float2 a = (k >= c0 && k <= c1) ? X[k] : make_float2(0.f, 0.f);
+  const float2 b = (m >= c0 && m <= c1) ? c_conj(X[m]) : make_float2(0.f, 0.f);
+  const float2 s = c_add(a, b), d = c_sub(a, b);
+  return pack_combine(s, d, twW[k]);
+}
+
+// Writes columns [c0, c1] of the half spectra of RB rows from their complex
+// transforms Z (rows of L), times `scale`.
+__device__ __forceinline__ void store_half(const float2* Z, float2* dst, int pitch, int L, int row0, int rows, int c0,
+                                           int c1, float scale, const float2* __restrict__ twW) {
+  const int n = c1 - c0 + 1;
+  if (n <= 0) return;
+  const unsigned m = fdiv_mul(static_cast<unsigned>(n));
+  for (int e = threadIdx.x; e < rows * n; e += blockDim.x) {
+    const int r = static_cast<int>(fdiv(static_cast<unsigned>(e), m)), k = c0 + e - r * n;
+    dst[static_cast<size_t>(row0 + r) * pitch + k] = c_scale(r2c_unpack(Z + r * L, L, k, twW), scale);
+  }
+}
+
+template <bool FILT>
+__global__ void __launch_bounds__(kRowThreads, 2)
+    k_row_r2c(const __grid_constant__ Geo g, const float* __restrict__ in, float2* __restrict__ out, int pitch, int RB,
+              const __grid_constant__ gf::Batch ba, int bufn, const FilterWave wv, float scale) {
   extern __shared__ float2 sm[];
-  const int E = H * TC;
-  float2* A = sm;
-  float2* B = sm + E;
-  const int col0 = blockIdx.x * TC, ch = blockIdx.y;
-  const int f_begin = blockIdx.z * fg, f_end = min(eta, f_begin + fg);
-  const float2* src = in + static_cast<size_t>(ch) * H * Wh;
-  for (int e = threadIdx.x; e < E; e += kColThreads) {
-    const int r = e / TC, col = col0 + (e - r * TC);
-    A[e] = col < Wh ? src[static_cast<size_t>(r) * Wh + col] : make_float2(0.f, 0.f);
-  }
+  gf::Exchange x{{sm, sm + bufn}};
+  const int L = g.L, row0 = blockIdx.x * RB, rows = min(RB, g.H - row0);
+  pdl_wait();
+  pdl_trigger();
+  const Plane p = plane_of<FILT>(g, wv);
+  if (p.c1 < p.c0) return;  // an empty filter: nothing reads its spectrum
+  const float2* src = reinterpret_cast<const float2*>(in) + p.data * g.H * L + static_cast<size_t>(row0) * L;
+  const auto ld = [&](int i, int b) { return b < rows ? src[static_cast<size_t>(b) * L + i] : make_float2(0.f, 0.f); };
+  const float2* y = gf::fft_head<-1, false>(g.planL, ba, x, g.ptL, ld);
+  float2* Z = x.next();
+  const auto st = [&](int i, int b, float2 v) { Z[b * L + i] = v; };
+  gf::NoLd nl;
+  if (g.planL.nst == 1)
+    gf::run_stage<-1, false, gf::kOnly>(g.planL, 0, ba, nullptr, nullptr, g.ptL, ld, st, threadIdx.x, blockDim.x);
+  else
+    gf::run_stage<-1, false, gf::kLast>(g.planL, g.planL.nst - 1, ba, y, nullptr, g.ptL, nl, st, threadIdx.x, blockDim.x);
   __syncthreads();
-  const float2* U = stockham<-1, true>(A, B, pH, TC, TC, 1, twH, 1);
-  float2 uh[MAXE];
+  store_half(Z, out + static_cast<size_t>(blockIdx.y) * g.H * pitch, pitch, L, row0, rows, p.c0, p.c1, scale, g.twW);
+}
+
+template <bool FILT>
+__global__ void __launch_bounds__(kRowThreads, 2)
+    k_row_c2r(const __grid_constant__ Geo g, const float2* __restrict__ in, float* __restrict__ out, int pitch, int RB,
+              const __grid_constant__ gf::Batch ba, int bufn, const FilterWave wv, float scale) {
+  extern __shared__ float2 sm[];
+  gf::Exchange x{{sm, sm + bufn}};
+  const int L = g.L, row0 = blockIdx.x * RB, rows = min(RB, g.H - row0);
+  pdl_wait();
+  pdl_trigger();
+  const Plane p = plane_of<FILT>(g, wv);
+  const float2* src = in + (static_cast<size_t>(blockIdx.y) * g.H + row0) * pitch;
+  float2* dst = reinterpret_cast<float2*>(out) + p.data * g.H * L + static_cast<size_t>(row0) * L;
+  gf::fft<+1, false>(
+      g.planL, ba, x, g.ptL,
+      [&](int i, int b) {
+        return b < rows ? packed(src + static_cast<size_t>(b) * pitch, L, i, p.c0, p.c1, g.twW) : make_float2(0.f, 0.f);
+      },
+      [&](int i, int b, float2 v) {
+        if (b < rows) {
+          if constexpr (FILT)
+            __stcs(dst + static_cast<size_t>(b) * L + i, c_scale(v, scale));
+          else
+            dst[static_cast<size_t>(b) * L + i] = c_scale(v, scale);
+        }
+      });
+}
+
+// The v-step's middle: the inverse transform's last stage, the shrinkage on
+// its results and the forward transform's first stage, on the same registers
+// (the forward plan is the inverse one reversed, so both stages have the same
+// radix and hold the values j + q L/R of a row).
+struct Turn {
+  const Geo& g;
+  const gf::Batch &bi, &bf;
+  const float2* in;
+  float2* out;
+  const float2* src;  // spectra rows (single-stage plans)
+  int pitch, rows, c0, c1;
+  float2 *b2, *gout;  // b_v rows, optional g rows (pitch L)
+  float t, scale;
+  template <int R>
+  __device__ __forceinline__ void run() {
+    const FftStage& gi = g.planL.st[g.planL.nst - 1];
+    const FftStage& gfw = g.planLr.st[0];
+    const int total = gi.nb * bi.B, L = g.L;
+    for (int idx = threadIdx.x; idx < total; idx += blockDim.x) {
+      int j, b, k = 0;
+      gf::item_of<false>(gi, bi, idx, j, b);
+      const bool live = b < rows;
+      float2* br = b2 + static_cast<size_t>(live ? b : 0) * L;
+      float2 bo[R], v[R];
 #pragma unroll
-  for (int m = 0; m < MAXE; ++m) {
-    const int e = threadIdx.x + m * kColThreads;
-    uh[m] = e < E ? U[e] : make_float2(0.f, 0.f);
-  }
-  __syncthreads();
-  for (int f = f_begin; f < f_end; ++f) {
-    const float* wf = bank + static_cast<size_t>(f) * H * Wh;
+      for (int q = 0; q < R; ++q) bo[q] = live ? __ldcs(br + j + q * gi.nb) : make_float2(0.f, 0.f);
+      if (g.planL.nst == 1) {
 #pragma unroll
-    for (int m = 0; m < MAXE; ++m) {
-      const int e = threadIdx.x + m * kColThreads;
-      if (e < E) {
-        const int r = e / TC, col = col0 + (e - r * TC);
-        const float w = col < Wh ? __ldg(wf + static_cast<size_t>(r) * Wh + col) : 0.f;
-        A[e] = c_scale(uh[m], w);
+        for (int q = 0; q < R; ++q)
+          v[q] = live ? packed(src + static_cast<size_t>(b) * pitch, L, j + q * gi.nb, c0, c1, g.twW) : make_float2(0.f, 0.f);
+      } else {
+        gf::stage_in<R, +1, false>(gi, bi, g.planL.nst == 2, j, b, in, g.ptL, v, k);
       }
-    }
-    __syncthreads();
-    const float2* Y = stockham<+1, true>(A, B, pH, TC, TC, 1, twH, 1);
-    float2* dst = out + (static_cast<size_t>(ch) * eta + f) * H * Wh;
-    for (int e = threadIdx.x; e < E; e += kColThreads) {
-      const int r = e / TC, col = col0 + (e - r * TC);
-      if (col < Wh) dst[static_cast<size_t>(r) * Wh + col] = Y[e];
-    }
-    __syncthreads();
-  }
-}
-
-template <int MAXE>
-__global__ void __launch_bounds__(kColThreads)
-    k_col_gather(const float2* __restrict__ in, const float* __restrict__ bank, float2* __restrict__ partial, int H,
-                 int Wh, int eta, int nch, int TC, int fg, FftPlan pH, const float2* __restrict__ twH) {
-  extern __shared__ float2 sm[];
-  const int E = H * TC;
-  float2* A = sm;
-  float2* B = sm + E;
-  const int col0 = blockIdx.x * TC, ch = blockIdx.y, grp = blockIdx.z;
-  const int f_begin = grp * fg, f_end = min(eta, f_begin + fg);
-  float2 acc[MAXE];
+      gf::dft<R, +1>(v);
 #pragma unroll
-  for (int m = 0; m < MAXE; ++m) acc[m] = make_float2(0.f, 0.f);
-  for (int f = f_begin; f < f_end; ++f) {
-    const float2* src = in + (static_cast<size_t>(ch) * eta + f) * H * Wh;
-    for (int e = threadIdx.x; e < E; e += kColThreads) {
-      const int r = e / TC, col = col0 + (e - r * TC);
-      A[e] = col < Wh ? src[static_cast<size_t>(r) * Wh + col] : make_float2(0.f, 0.f);
-    }
-    __syncthreads();
-    const float2* Z = stockham<-1, true>(A, B, pH, TC, TC, 1, twH, 1);
-    const float* wf = bank + static_cast<size_t>(f) * H * Wh;
-#pragma unroll
-    for (int m = 0; m < MAXE; ++m) {
-      const int e = threadIdx.x + m * kColThreads;
-      if (e < E) {
-        const int r = e / TC, col = col0 + (e - r * TC);
-        const float w = col < Wh ? __ldg(wf + static_cast<size_t>(r) * Wh + col) : 0.f;
-        acc[m].x = fmaf(w, Z[e].x, acc[m].x);
-        acc[m].y = fmaf(w, Z[e].y, acc[m].y);
+      for (int q = 0; q < R; ++q) {
+        const float2 gv = c_fma2(make_float2(scale, scale), v[q], bo[q]);
+        const float2 c = make_float2(fminf(fmaxf(gv.x, -t), t), fminf(fmaxf(gv.y, -t), t));
+        if (live) {
+          __stcs(br + j + q * gi.nb, c);
+          if (gout) gout[static_cast<size_t>(b) * L + j + q * gi.nb] = gv;
+        }
+        v[q] = c_fma2(make_float2(-2.f, -2.f), c, gv);  // g - 2 clip(g)
       }
-    }
-    __syncthreads();
-  }
-  float2* dst = partial + (static_cast<size_t>(grp) * nch + ch) * H * Wh;
-#pragma unroll
-  for (int m = 0; m < MAXE; ++m) {
-    const int e = threadIdx.x + m * kColThreads;
-    if (e < E) {
-      const int r = e / TC, col = col0 + (e - r * TC);
-      if (col < Wh) dst[static_cast<size_t>(r) * Wh + col] = acc[m];
+      gf::dft<R, -1>(v);
+      gf::stage_out<R, false>(gfw, bf, true, j, b, 0, out, v);
     }
   }
-}
-
-__global__ void __launch_bounds__(kColThreads)
-    k_col_reduce_inv(const float2* __restrict__ partial, float2* __restrict__ out, int H, int Wh, int nch, int groups,
-                     int TC, FftPlan pH, const float2* __restrict__ twH) {
-  extern __shared__ float2 sm[];
-  const int E = H * TC;
-  float2* A = sm;
-  float2* B = sm + E;
-  const int col0 = blockIdx.x * TC, ch = blockIdx.y;
-  const size_t plane = static_cast<size_t>(H) * Wh;
-  for (int e = threadIdx.x; e < E; e += kColThreads) {
-    const int r = e / TC, col = col0 + (e - r * TC);
-    float2 s = make_float2(0.f, 0.f);
-    if (col < Wh) {
-      const size_t off = static_cast<size_t>(r) * Wh + col;
-      for (int g = 0; g < groups; ++g) s = c_add(s, partial[(static_cast<size_t>(g) * nch + ch) * plane + off]);
-    }
-    A[e] = s;
-  }
-  __syncthreads();
-  const float2* Y = stockham<+1, true>(A, B, pH, TC, TC, 1, twH, 1);
-  float2* dst = out + static_cast<size_t>(ch) * plane;
-  for (int e = threadIdx.x; e < E; e += kColThreads) {
-    const int r = e / TC, col = col0 + (e - r * TC);
-    if (col < Wh) dst[static_cast<size_t>(r) * Wh + col] = Y[e];
-  }
-}
-
-// ---------------------------------------------------------------------------
-// Row kernels: one CTA owns RB consecutive rows of one plane.  A real row of
-// length W = 2L is handled as the complex row z[n] = x[2n] + i x[2n+1].
-// ---------------------------------------------------------------------------
-
-__global__ void __launch_bounds__(kRowThreads)
-    k_row_r2c(const float* __restrict__ in, float2* __restrict__ out, int H, int L, int RB, FftPlan pL,
-              const float2* __restrict__ twW, float scale) {
-  extern __shared__ float2 sm[];
-  const int E = RB * L, Wh = L + 1;
-  float2* A = sm;
-  float2* B = sm + E;
-  const int row0 = blockIdx.x * RB;
-  const size_t plane = blockIdx.y;
-  const float2* src = reinterpret_cast<const float2*>(in) + plane * H * L;
-  for (int e = threadIdx.x; e < E; e += kRowThreads) {
-    const int r = e / L, row = row0 + r;
-    A[e] = row < H ? src[static_cast<size_t>(row) * L + (e - r * L)] : make_float2(0.f, 0.f);
-  }
-  __syncthreads();
-  const float2* Z = stockham<-1, false>(A, B, pL, RB, 1, L, twW, 2);
-  float2* dst = out + plane * H * Wh;
-  for (int e = threadIdx.x; e < RB * Wh; e += kRowThreads) {
-    const int r = e / Wh, k = e - r * Wh, row = row0 + r;
-    if (row < H) dst[static_cast<size_t>(row) * Wh + k] = c_scale(r2c_unpack(Z + r * L, L, k, twW), scale);
-  }
-}
-
-// Loads RB packed rows of a half-spectrum plane for the inverse row transform.
-__device__ __forceinline__ void load_c2r(const float2* __restrict__ src, float2* A, int H, int L, int row0, int RB,
-                                         const float2* __restrict__ twW) {
-  const int E = RB * L, Wh = L + 1;
-  for (int e = threadIdx.x; e < E; e += kRowThreads) {
-    const int r = e / L, row = row0 + r;
-    A[e] = row < H ? c2r_pack(src + static_cast<size_t>(row) * Wh, L, e - r * L, twW) : make_float2(0.f, 0.f);
-  }
-}
-
-__global__ void __launch_bounds__(kRowThreads)
-    k_row_c2r(const float2* __restrict__ in, float* __restrict__ out, int H, int L, int RB, FftPlan pL,
-              const float2* __restrict__ twW, float scale) {
-  extern __shared__ float2 sm[];
-  const int E = RB * L, Wh = L + 1;
-  float2* A = sm;
-  float2* B = sm + E;
-  const int row0 = blockIdx.x * RB;
-  const size_t plane = blockIdx.y;
-  load_c2r(in + plane * H * Wh, A, H, L, row0, RB, twW);
-  __syncthreads();
-  const float2* Z = stockham<+1, false>(A, B, pL, RB, 1, L, twW, 2);
-  float2* dst = reinterpret_cast<float2*>(out) + plane * H * L;
-  for (int e = threadIdx.x; e < E; e += kRowThreads) {
-    const int r = e / L, row = row0 + r;
-    if (row < H) dst[static_cast<size_t>(row) * L + (e - r * L)] = c_scale(Z[e], scale);
-  }
-}
+};
 
 // v-step and b_v update (Sec. 3): with c = (S u)_f on this row,
 // g = b_v + c, b_v <- clip(g, -t, t) = g - soft(g, t), d = soft(g) - clip(g);
 // d (= v - b_v of the new iterate) is transformed back in place.
-__global__ void __launch_bounds__(kRowThreads)
-    k_row_shrink(float2* __restrict__ Y, float* __restrict__ bv, const float* __restrict__ thr, int eta, int H, int L,
-                 int RB, FftPlan pL, const float2* __restrict__ twW, float scale, float* __restrict__ gout) {
+__global__ void __launch_bounds__(kRowThreads, 2)
+    k_row_shrink(const __grid_constant__ Geo g, float2* __restrict__ Y, float* __restrict__ bv,
+                 const float* __restrict__ thr, int pitch, int RB, const __grid_constant__ gf::Batch bi,
+                 const __grid_constant__ gf::Batch bf, int bufn, const FilterWave wv, float scale,
+                 float* __restrict__ gout) {
   extern __shared__ float2 sm[];
-  const int E = RB * L, Wh = L + 1;
-  float2* A = sm;
-  float2* B = sm + E;
-  const int row0 = blockIdx.x * RB;
-  const size_t plane = blockIdx.y;
-  float2* X = Y + plane * H * Wh;
-  load_c2r(X, A, H, L, row0, RB, twW);
+  gf::Exchange x{{sm, sm + bufn}};
+  const int L = g.L, row0 = blockIdx.x * RB, rows = min(RB, g.H - row0);
+  pdl_wait();
+  pdl_trigger();
+  const Plane p = plane_of<true>(g, wv);
+  float2* X = Y + (static_cast<size_t>(blockIdx.y) * g.H + row0) * pitch;
+  const size_t off = (p.data * g.H + row0) * L;
+  const float2* y = gf::fft_head<+1, false>(g.planL, bi, x, g.ptL, [&](int i, int b) {
+    return b < rows ? packed(X + static_cast<size_t>(b) * pitch, L, i, p.c0, p.c1, g.twW) : make_float2(0.f, 0.f);
+  });
+  float2* z = x.next();
+  Turn turn{g,  bi,     bf,   y,    z,    X, pitch, rows, p.c0, p.c1, reinterpret_cast<float2*>(bv) + off,
+            gout ? reinterpret_cast<float2*>(gout) + off : nullptr, thr[p.f], scale};
+  gf::with_radix(g.planL.st[g.planL.nst - 1].R, turn);
   __syncthreads();
-  float2* Z = stockham<+1, false>(A, B, pL, RB, 1, L, twW, 2);
-  const float t = thr[plane % eta];
-  float2* b2 = reinterpret_cast<float2*>(bv) + plane * H * L;
-  for (int e = threadIdx.x; e < E; e += kRowThreads) {
-    const int r = e / L, row = row0 + r;
-    float2 d = make_float2(0.f, 0.f);
-    if (row < H) {
-      const size_t off = static_cast<size_t>(row) * L + (e - r * L);
-      const float2 b = b2[off];
-      const float gx = b.x + scale * Z[e].x, gy = b.y + scale * Z[e].y;
-      const float cx = fminf(fmaxf(gx, -t), t), cy = fminf(fmaxf(gy, -t), t);
-      b2[off] = make_float2(cx, cy);
-      if (gout) reinterpret_cast<float2*>(gout)[plane * H * L + off] = make_float2(gx, gy);
-      d = make_float2(gx - 2.f * cx, gy - 2.f * cy);
-    }
-    Z[e] = d;
+  gf::NoLd nl;
+  gf::NoSt ns;
+  const float2* in = z;
+  for (int s = 1; s + 1 < g.planLr.nst; ++s) {
+    float2* o = x.next();
+    gf::run_stage<-1, false, gf::kMid>(g.planLr, s, bf, in, o, g.ptLr, nl, ns, threadIdx.x, blockDim.x);
+    __syncthreads();
+    in = o;
   }
-  __syncthreads();
-  float2* other = (Z == A) ? B : A;
-  const float2* D = stockham<-1, false>(Z, other, pL, RB, 1, L, twW, 2);
-  for (int e = threadIdx.x; e < RB * Wh; e += kRowThreads) {
-    const int r = e / Wh, k = e - r * Wh, row = row0 + r;
-    if (row < H) X[static_cast<size_t>(row) * Wh + k] = r2c_unpack(D + r * L, L, k, twW);
+  if (g.planLr.nst > 1) {
+    float2* Z = x.next();
+    const auto st = [&](int i, int b, float2 v) { Z[b * L + i] = v; };
+    gf::run_stage<-1, false, gf::kLast>(g.planLr, g.planLr.nst - 1, bf, in, nullptr, g.ptLr, nl, st, threadIdx.x,
+                                        blockDim.x);
+    __syncthreads();
+    in = Z;
   }
+  store_half(in, X - static_cast<size_t>(row0) * pitch, pitch, L, row0, rows, p.c0, p.c1, 1.f, g.twW);
 }
 
 constexpr int kL1Threads = kRowThreads;
 
 // Weighted l1 norm of the real planes behind the half spectra: one FP64
 // partial per block, fixed summation order.
-__global__ void __launch_bounds__(kRowThreads)
-    k_row_l1(const float2* __restrict__ in, const float* __restrict__ lam, int eta, int H, int L, int RB, FftPlan pL,
-             const float2* __restrict__ twW, float scale, double* __restrict__ partial) {
+__global__ void __launch_bounds__(kRowThreads, 2)
+    k_row_l1(const __grid_constant__ Geo g, const float2* __restrict__ in, const float* __restrict__ lam, int pitch,
+             int RB, const __grid_constant__ gf::Batch ba, int bufn, const FilterWave wv, float scale,
+             double* __restrict__ partial) {
   extern __shared__ float2 sm[];
   __shared__ double red[kL1Threads];
-  const int E = RB * L, Wh = L + 1;
-  float2* A = sm;
-  float2* B = sm + E;
-  const int row0 = blockIdx.x * RB;
-  const size_t plane = blockIdx.y;
-  load_c2r(in + plane * H * Wh, A, H, L, row0, RB, twW);
-  __syncthreads();
-  const float2* Z = stockham<+1, false>(A, B, pL, RB, 1, L, twW, 2);
+  gf::Exchange x{{sm, sm + bufn}};
+  const int L = g.L, row0 = blockIdx.x * RB, rows = min(RB, g.H - row0);
+  pdl_wait();
+  pdl_trigger();
+  const Plane p = plane_of<true>(g, wv);
+  const float2* src = in + (static_cast<size_t>(blockIdx.y) * g.H + row0) * pitch;
   double acc = 0.0;
-  for (int e = threadIdx.x; e < E; e += kRowThreads) {
-    const int r = e / L, row = row0 + r;
-    if (row < H) acc += static_cast<double>(fabsf(scale * Z[e].x)) + static_cast<double>(fabsf(scale * Z[e].y));
-  }
-  red[threadIdx.x] = acc * static_cast<double>(lam[plane % eta]);
+  gf::fft<+1, false>(
+      g.planL, ba, x, g.ptL,
+      [&](int i, int b) {
+        return b < rows ? packed(src + static_cast<size_t>(b) * pitch, L, i, p.c0, p.c1, g.twW) : make_float2(0.f, 0.f);
+      },
+      [&](int, int b, float2 v) {
+        if (b < rows) acc += static_cast<double>(fabsf(scale * v.x)) + static_cast<double>(fabsf(scale * v.y));
+      });
+  red[threadIdx.x] = acc * static_cast<double>(lam[p.f]);
   __syncthreads();
   for (int s = kL1Threads / 2; s > 0; s >>= 1) {
     if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
     __syncthreads();
   }
-  if (threadIdx.x == 0) partial[plane * gridDim.x + blockIdx.x] = red[0];
+  if (threadIdx.x == 0) partial[p.data * gridDim.x + blockIdx.x] = red[0];
 }
 
 // u-step (u = 1/2 [S^T(v - b_v) + (w - b_w) - gamma s], A^T A = 2I), w-step
 // (pixelwise projection of g_w = b_w + u onto the simplex), b_w = g_w - w,
 // and the row-forward transform of u for the next analysis.  Shared memory:
-// A, B (RB x L complex each) and U (K x RB x L complex).
+// the exchange buffers and U (K x RB x L complex).
 __global__ void __launch_bounds__(kRowThreads)
-    k_row_ustep(const float2* __restrict__ T, const float* __restrict__ s, float* __restrict__ w,
-                float* __restrict__ bw, float* __restrict__ u, float2* __restrict__ Ur, float* __restrict__ stv, int K,
-                int H, int L, int RB, FftPlan pL, const float2* __restrict__ twW, float scale, float gamma) {
+    k_row_ustep(const __grid_constant__ Geo g, const float2* __restrict__ T, const float* __restrict__ s,
+                float* __restrict__ w, float* __restrict__ bw, float* __restrict__ u, float2* __restrict__ Ur,
+                float* __restrict__ stv, int K, int RB, const __grid_constant__ gf::Batch ba, int bufn, float scale,
+                float gamma) {
   extern __shared__ float2 sm[];
-  const int E = RB * L, Wh = L + 1;
-  float2* A = sm;
-  float2* B = sm + E;
-  float2* U = sm + 2 * E;
-  const int row0 = blockIdx.x * RB;
-  const size_t HL = static_cast<size_t>(H) * L, HWh = static_cast<size_t>(H) * Wh;
+  gf::Exchange x{{sm, sm + bufn}};
+  float2* U = sm + 2 * bufn;
+  const int L = g.L, E = RB * L, Wh = g.Wh, row0 = blockIdx.x * RB, rows = min(RB, g.H - row0);
+  const size_t HL = static_cast<size_t>(g.H) * L, HWh = static_cast<size_t>(g.H) * Wh;
+  pdl_wait();
+  pdl_trigger();
   for (int k = 0; k < K; ++k) {
-    load_c2r(T + k * HWh, A, H, L, row0, RB, twW);
-    __syncthreads();
-    const float2* Z = stockham<+1, false>(A, B, pL, RB, 1, L, twW, 2);
-    for (int e = threadIdx.x; e < E; e += kRowThreads) U[k * E + e] = c_scale(Z[e], scale);
-    __syncthreads();
+    const float2* src = T + k * HWh + static_cast<size_t>(row0) * Wh;
+    float2* Uk = U + k * E;
+    gf::fft<+1, false>(
+        g.planL, ba, x, g.ptL,
+        [&](int i, int b) {
+          return b < rows ? packed(src + static_cast<size_t>(b) * Wh, L, i, 0, L, g.twW) : make_float2(0.f, 0.f);
+        },
+        [&](int i, int b, float2 v) { Uk[b * L + i] = c_scale(v, scale); });
   }
+  __syncthreads();
   const float2* s2 = reinterpret_cast<const float2*>(s);
   float2* w2 = reinterpret_cast<float2*>(w);
   float2* bw2 = reinterpret_cast<float2*>(bw);
@@ -311,12 +313,11 @@ __global__ void __launch_bounds__(kRowThreads)
   float2* stv2 = reinterpret_cast<float2*>(stv);
   const float hg = 0.5f * gamma;
   for (int e = threadIdx.x; e < E; e += kRowThreads) {
-    const int r = e / L, row = row0 + r;
-    if (row >= H) {
+    if (e >= rows * L) {
       for (int k = 0; k < K; ++k) U[k * E + e] = make_float2(0.f, 0.f);
       continue;
     }
-    const size_t off = static_cast<size_t>(row) * L + (e - r * L);
+    const size_t off = static_cast<size_t>(row0) * L + e;
     float gx[kMaxK], gy[kMaxK];
 #pragma unroll
     for (int k = 0; k < kMaxK; ++k) {
@@ -352,13 +353,19 @@ __global__ void __launch_bounds__(kRowThreads)
   }
   __syncthreads();
   for (int k = 0; k < K; ++k) {
-    const float2* Z = stockham<-1, false>(U + k * E, A, pL, RB, 1, L, twW, 2);
-    float2* dst = Ur + k * HWh;
-    for (int e = threadIdx.x; e < RB * Wh; e += kRowThreads) {
-      const int r = e / Wh, kk = e - r * Wh, row = row0 + r;
-      if (row < H) dst[static_cast<size_t>(row) * Wh + kk] = r2c_unpack(Z + r * L, L, kk, twW);
-    }
+    const float2* Uk = U + k * E;
+    const auto ld = [&](int i, int b) { return Uk[b * L + i]; };
+    const float2* y = gf::fft_head<-1, false>(g.planL, ba, x, g.ptL, ld);
+    float2* Z = x.next();
+    const auto st = [&](int i, int b, float2 v) { Z[b * L + i] = v; };
+    gf::NoLd nl;
+    if (g.planL.nst == 1)
+      gf::run_stage<-1, false, gf::kOnly>(g.planL, 0, ba, nullptr, nullptr, g.ptL, ld, st, threadIdx.x, blockDim.x);
+    else
+      gf::run_stage<-1, false, gf::kLast>(g.planL, g.planL.nst - 1, ba, y, nullptr, g.ptL, nl, st, threadIdx.x,
+                                          blockDim.x);
     __syncthreads();
+    store_half(Z, Ur + k * HWh, Wh, L, row0, rows, 0, L, 1.f, g.twW);
   }
 }
 
@@ -374,7 +381,28 @@ int ustep_rows(const Geo& g, int K) {
   return rb;
 }
 
+// Padding of the first exchange of a row plan: only even first radices need
+// it, and only where the padded buffers still fit.
+constexpr size_t kRowSmemMax = 227 * 1024 - sizeof(double) * kL1Threads;
+int row_pad(const FftPlan& p, int rb, int extra) {
+  const size_t need = sizeof(float2) * (2 * static_cast<size_t>(gf::buf_elems(p, rb, 1)) + static_cast<size_t>(extra));
+  return p.nst > 1 && p.st[0].R % 2 == 0 && need <= kRowSmemMax ? 1 : 0;
+}
+
+// Launch shape of a row kernel: the batch of the plan and its buffers.
+struct RowShape {
+  gf::Batch ba;
+  int bufn;
+  size_t smem;
+};
+RowShape row_shape(const FftPlan& p, int rb) {
+  const int pad = row_pad(p, rb, 0), n = gf::buf_elems(p, rb, pad);
+  return RowShape{gf::make_batch(p, rb, pad), n, sizeof(float2) * 2 * static_cast<size_t>(n)};
+}
+
 }  // namespace
+
+cudaError_t prepare_col_general(int optin);
 
 // Raises the dynamic shared-memory limit of every kernel to the device's
 // opt-in maximum (an upper bound only), once per device, outside any capture.
@@ -385,11 +413,10 @@ cudaError_t prepare_kernels() {
   e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
   if (e != cudaSuccess) return e;
   const cudaError_t errs[] = {
-      set_smem(k_row_r2c, optin),          set_smem(k_row_c2r, optin),        set_smem(k_row_shrink, optin),
+      set_smem(k_row_r2c<false>, optin), set_smem(k_row_r2c<true>, optin), set_smem(k_row_c2r<false>, optin),
+      set_smem(k_row_c2r<true>, optin),  set_smem(k_row_shrink, optin),
       set_smem(k_row_l1, optin - static_cast<int>(sizeof(double)) * kL1Threads),
-      set_smem(k_col_fan<8>, optin),       set_smem(k_col_fan<16>, optin),    set_smem(k_col_fan<32>, optin),
-      set_smem(k_col_gather<8>, optin),    set_smem(k_col_gather<16>, optin), set_smem(k_col_gather<32>, optin),
-      set_smem(k_col_reduce_inv, optin),   set_smem(k_row_ustep, optin)};
+      set_smem(k_row_ustep, optin),      prepare_col_general(optin)};
   for (cudaError_t x : errs)
     if (x != cudaSuccess) return x;
   return cudaSuccess;
@@ -409,7 +436,6 @@ bool set_generic_tiles(Geo* g, int TC, int RB, int K, int smem_limit) {
   Geo t = *g;
   t.TC = TC;
   t.ntiles = (t.Wh + TC - 1) / TC;
-  t.maxe = per <= 8 ? 8 : (per <= 16 ? 16 : 32);
   t.RB = RB;
   const size_t col = 2 * sizeof(float2) * static_cast<size_t>(t.H) * t.TC;
   const size_t row = 2 * sizeof(float2) * static_cast<size_t>(t.RB) * t.L;
@@ -420,93 +446,55 @@ bool set_generic_tiles(Geo* g, int TC, int RB, int K, int smem_limit) {
   return true;
 }
 
-int default_groups(const Geo& g, int nch) {
-  const int base = g.ntiles * nch;
-  int G = (4 * 152 + base - 1) / base;
-  if (G < 1) G = 1;
-  if (G > g.eta) G = g.eta;
-  const int fg = (g.eta + G - 1) / G;
-  return (g.eta + fg - 1) / fg;
-}
-
 cudaError_t run_row_r2c(const Geo& g, const float* in, float2* out, int planes, float scale, cudaStream_t st) {
-  const size_t smem = 2 * sizeof(float2) * g.RB * g.L;
-  dim3 grid((g.H + g.RB - 1) / g.RB, planes);
-  k_row_r2c<<<grid, kRowThreads, smem, st>>>(in, out, g.H, g.L, g.RB, g.planL, g.twW, scale);
-  return cudaGetLastError();
+  const RowShape s = row_shape(g.planL, g.RB);
+  return launch_pdl(k_row_r2c<false>, dim3((g.H + g.RB - 1) / g.RB, planes), dim3(kRowThreads), s.smem, st, g, in, out,
+                    g.Wh, g.RB, s.ba, s.bufn, FilterWave{}, scale);
 }
 
 cudaError_t run_row_c2r(const Geo& g, const float2* in, float* out, int planes, float scale, cudaStream_t st) {
-  const size_t smem = 2 * sizeof(float2) * g.RB * g.L;
-  dim3 grid((g.H + g.RB - 1) / g.RB, planes);
-  k_row_c2r<<<grid, kRowThreads, smem, st>>>(in, out, g.H, g.L, g.RB, g.planL, g.twW, scale);
-  return cudaGetLastError();
+  const RowShape s = row_shape(g.planL, g.RB);
+  return launch_pdl(k_row_c2r<false>, dim3((g.H + g.RB - 1) / g.RB, planes), dim3(kRowThreads), s.smem, st, g, in, out,
+                    g.Wh, g.RB, s.ba, s.bufn, FilterWave{}, scale);
 }
 
-cudaError_t run_row_shrink(const Geo& g, float2* Y, float* bv, const float* thr, int planes, float scale,
-                           cudaStream_t st, float* gout) {
-  const size_t smem = 2 * sizeof(float2) * g.RB * g.L;
-  dim3 grid((g.H + g.RB - 1) / g.RB, planes);
-  k_row_shrink<<<grid, kRowThreads, smem, st>>>(Y, bv, thr, g.eta, g.H, g.L, g.RB, g.planL, g.twW, scale, gout);
-  return cudaGetLastError();
+cudaError_t run_wave_r2c(const Geo& g, const float* coef, float2* Y, const FilterWave& wv, cudaStream_t st) {
+  const RowShape s = row_shape(g.planL, g.RB);
+  return launch_pdl(k_row_r2c<true>, dim3((g.H + g.RB - 1) / g.RB, wv.nc * wv.nf), dim3(kRowThreads), s.smem, st, g,
+                    coef, Y, g.Wy, g.RB, s.ba, s.bufn, wv, 1.f);
 }
 
-cudaError_t run_row_l1(const Geo& g, const float2* Y, const float* lam, int planes, float scale, double* partial,
-                       int* nblocks, cudaStream_t st) {
-  const size_t smem = 2 * sizeof(float2) * g.RB * g.L;
-  dim3 grid((g.H + g.RB - 1) / g.RB, planes);
-  k_row_l1<<<grid, kRowThreads, smem, st>>>(Y, lam, g.eta, g.H, g.L, g.RB, g.planL, g.twW, scale, partial);
-  *nblocks = grid.x * grid.y;
-  return cudaGetLastError();
+cudaError_t run_wave_c2r(const Geo& g, const float2* Y, float* coef, const FilterWave& wv, float scale,
+                         cudaStream_t st) {
+  const RowShape s = row_shape(g.planL, g.RB);
+  return launch_pdl(k_row_c2r<true>, dim3((g.H + g.RB - 1) / g.RB, wv.nc * wv.nf), dim3(kRowThreads), s.smem, st, g, Y,
+                    coef, g.Wy, g.RB, s.ba, s.bufn, wv, scale);
 }
 
-template <int MAXE>
-static cudaError_t fan_t(const Geo& g, const float2* in, float2* out, int nch, int groups, cudaStream_t st) {
-  const size_t smem = 2 * sizeof(float2) * g.H * g.TC;
-  const int fg = (g.eta + groups - 1) / groups;
-  dim3 grid(g.ntiles, nch, (g.eta + fg - 1) / fg);
-  k_col_fan<MAXE><<<grid, kColThreads, smem, st>>>(in, g.bank, out, g.H, g.Wh, g.eta, g.TC, fg, g.planH, g.twH);
-  return cudaGetLastError();
+cudaError_t run_wave_shrink(const Geo& g, float2* Y, float* bv, const float* thr, const FilterWave& wv, float scale,
+                            cudaStream_t st, float* gout) {
+  const RowShape s = row_shape(g.planL, g.RB), r = row_shape(g.planLr, g.RB);
+  const int bufn = std::max(s.bufn, r.bufn);
+  return launch_pdl(k_row_shrink, dim3((g.H + g.RB - 1) / g.RB, wv.nc * wv.nf), dim3(kRowThreads),
+                    2 * sizeof(float2) * static_cast<size_t>(bufn), st, g, Y, bv, thr, g.Wy, g.RB, s.ba, r.ba, bufn, wv,
+                    scale, gout);
 }
 
-cudaError_t run_col_fan(const Geo& g, const float2* in, float2* out, int nch, int groups, cudaStream_t st) {
-  if (g.maxe == 8) return fan_t<8>(g, in, out, nch, groups, st);
-  if (g.maxe == 16) return fan_t<16>(g, in, out, nch, groups, st);
-  return fan_t<32>(g, in, out, nch, groups, st);
+cudaError_t run_wave_l1(const Geo& g, const float2* Y, const float* lam, const FilterWave& wv, float scale,
+                        double* partial, cudaStream_t st) {
+  const RowShape s = row_shape(g.planL, g.RB);
+  return launch_pdl(k_row_l1, dim3((g.H + g.RB - 1) / g.RB, wv.nc * wv.nf), dim3(kRowThreads), s.smem, st, g, Y, lam,
+                    g.Wy, g.RB, s.ba, s.bufn, wv, scale, partial);
 }
 
-template <int MAXE>
-static cudaError_t gather_t(const Geo& g, const float2* in, float2* partial, int nch, int groups, cudaStream_t st) {
-  const size_t smem = 2 * sizeof(float2) * g.H * g.TC;
-  const int fg = (g.eta + groups - 1) / groups;
-  dim3 grid(g.ntiles, nch, (g.eta + fg - 1) / fg);
-  k_col_gather<MAXE><<<grid, kColThreads, smem, st>>>(in, g.bank, partial, g.H, g.Wh, g.eta, nch, g.TC, fg,
-                                                      g.planH, g.twH);
-  return cudaGetLastError();
-}
-
-cudaError_t run_col_gather(const Geo& g, const float2* in, float2* partial, int nch, int groups, cudaStream_t st) {
-  if (g.maxe == 8) return gather_t<8>(g, in, partial, nch, groups, st);
-  if (g.maxe == 16) return gather_t<16>(g, in, partial, nch, groups, st);
-  return gather_t<32>(g, in, partial, nch, groups, st);
-}
-
-cudaError_t run_col_reduce_inv(const Geo& g, const float2* partial, float2* out, int nch, int groups,
-                               cudaStream_t st) {
-  const size_t smem = 2 * sizeof(float2) * g.H * g.TC;
-  dim3 grid(g.ntiles, nch);
-  k_col_reduce_inv<<<grid, kColThreads, smem, st>>>(partial, out, g.H, g.Wh, nch, groups, g.TC, g.planH, g.twH);
-  return cudaGetLastError();
-}
+int l1_blocks(const Geo& g, int nch) { return ((g.H + g.RB - 1) / g.RB) * nch * g.eta; }
 
 cudaError_t run_row_ustep(const Geo& g, const float2* T, const float* s, float* w, float* bw, float* u, float2* Ur,
                           float* stv, int K, float gamma, float scale, cudaStream_t st) {
-  const int rb = ustep_rows(g, K);
-  const size_t smem = sizeof(float2) * static_cast<size_t>(rb) * g.L * (2 + K);
-  dim3 grid((g.H + rb - 1) / rb);
-  k_row_ustep<<<grid, kRowThreads, smem, st>>>(T, s, w, bw, u, Ur, stv, K, g.H, g.L, rb, g.planL, g.twW, scale,
-                                               gamma);
-  return cudaGetLastError();
+  const int rb = ustep_rows(g, K), pad = row_pad(g.planL, rb, K * rb * g.L), n = gf::buf_elems(g.planL, rb, pad);
+  return launch_pdl(k_row_ustep, dim3((g.H + rb - 1) / rb), dim3(kRowThreads),
+                    sizeof(float2) * (2 * static_cast<size_t>(n) + static_cast<size_t>(K) * rb * g.L), st, g, T, s, w, bw,
+                    u, Ur, stv, K, rb, gf::make_batch(g.planL, rb, pad), n, scale, gamma);
 }
 
 }  // namespace shf

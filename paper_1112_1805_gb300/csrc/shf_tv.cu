@@ -36,7 +36,7 @@ struct tv_state {
   bool own_stream = false;
   float *f = nullptr, *s = nullptr, *u = nullptr, *bv = nullptr, *d = nullptr, *w = nullptr, *bw = nullptr;
   float *q = nullptr, *rhs = nullptr, *sym = nullptr, *gap = nullptr;
-  float2 *twH = nullptr, *twW = nullptr, *Ur = nullptr, *Y = nullptr;
+  float2 *twH = nullptr, *twW = nullptr, *pt = nullptr, *Ur = nullptr, *Y = nullptr;
   int* labels = nullptr;
   int* flag = nullptr;
   double* red = nullptr;
@@ -246,7 +246,7 @@ void free_tv(tv_state* st) {
   if (st->stream) cudaStreamSynchronize(st->stream);
   if (st->exec) cudaGraphExecDestroy(st->exec);
   void* bufs[] = {st->f, st->s, st->u, st->bv, st->d, st->w, st->bw, st->q, st->rhs, st->sym, st->gap,
-                  st->twH, st->twW, st->Ur, st->Y, st->labels, st->flag, st->red};
+                  st->twH, st->twW, st->pt, st->Ur, st->Y, st->labels, st->flag, st->red};
   for (void* b : bufs) cudaFree(b);
   if (st->own_stream && st->stream) cudaStreamDestroy(st->stream);
   delete st;
@@ -304,7 +304,7 @@ cudaError_t enqueue_tv_iteration(tv_state* st, cudaEvent_t* ev) {
   cudaError_t e = mark(kTvRowFwd);
   if (e == cudaSuccess) e = shf::run_row_r2c(g, st->rhs, st->Ur, st->K, 1.f, ss);
   if (e == cudaSuccess) e = mark(kTvCol);
-  if (e == cudaSuccess) e = shf::run_col_fan(g, st->Ur, st->Y, st->K, 1, ss);
+  if (e == cudaSuccess) e = shf::run_col_filter(g, st->Ur, st->Y, st->K, ss);
   if (e == cudaSuccess) e = mark(kTvRowInv);
   if (e == cudaSuccess) e = shf::run_row_c2r(g, st->Y, st->u, st->K, 1.f / (static_cast<float>(g.H) * g.W), ss);
   if (e == cudaSuccess) e = mark(kTvProx);
@@ -412,7 +412,8 @@ int tv_admm_init(int H, int W, const float* f, int C, const float* codebook, int
       (rc = tv_alloc(&st->bw, P * K, "b_w")) || (rc = tv_alloc(&st->q, P * K, "q")) ||
       (rc = tv_alloc(&st->rhs, P * K, "rhs")) || (rc = tv_alloc(&st->sym, Ph, "symbol")) ||
       (rc = tv_alloc(&st->gap, P, "gap")) || (rc = tv_alloc(&st->twH, H, "twH")) ||
-      (rc = tv_alloc(&st->twW, W, "twW")) || (rc = tv_alloc(&st->Ur, Phs * K, "Ur")) ||
+      (rc = tv_alloc(&st->twW, W, "twW")) ||
+      (rc = tv_alloc(&st->pt, shf::pass_table_entries(g), "pass tables")) || (rc = tv_alloc(&st->Ur, Phs * K, "Ur")) ||
       (rc = tv_alloc(&st->Y, Phs * K, "Y")) || (rc = tv_alloc(&st->labels, P, "labels")) ||
       (rc = tv_alloc(&st->flag, 1, "flag")) || (rc = tv_alloc(&st->red, 2 * kRedBlocks + 2, "red"))) {
     free_tv(st);
@@ -425,6 +426,7 @@ int tv_admm_init(int H, int W, const float* f, int C, const float* codebook, int
   st->g = g;
   cudaError_t e = shf::launch_twiddles(st->twH, H, st->stream);
   if (e == cudaSuccess) e = shf::launch_twiddles(st->twW, W, st->stream);
+  if (e == cudaSuccess) e = shf::launch_pass_tables(&st->g, st->pt, st->stream);
   if (e == cudaSuccess) {
     k_poisson_symbol<<<grid_for(Ph), kThreads, 0, st->stream>>>(st->sym, H, W, g.Wh);
     e = cudaGetLastError();
