@@ -6,9 +6,9 @@
 // patch of G_a(t) sum_ch (f(i + t) - f(j + t))^2 (G_a the Gaussian of
 // standard deviation a normalised to sum 1, f mirrored at the border) for
 // every candidate j of the varpi x varpi search window (clipped to the image)
-// is computed on the GPU in FP64 with every product and sum rounded
-// separately, and each pixel's candidates are ranked by (distance, raster
-// index).  The selection itself is sequential in the paper (pixels in
+// is computed on the GPU (in FP32, and in FP64 with every product and sum
+// rounded separately where that decides the order), and each pixel's
+// candidates are ranked by (distance, raster index).  The selection itself is sequential in the paper (pixels in
 // raster order pick min(mt, 2 mt - l) new neighbours, l the neighbours they
 // already have, and links are symmetric), so it runs on the host over the
 // ranked lists; a candidate already linked or holding 2 mt neighbours is
@@ -39,19 +39,26 @@ struct nl_state {
   float gamma = 1.f, lambda = 0.f;
   nl_params prm{};
   std::vector<float> codebook;
-  std::vector<int> nbr_host, deg_host;  // [P][m] (increasing index, -1 padded), [P]
+  // pinned: the links [P][m] in the order of selection, their counts, the first ranks
+  int* nbr_host = nullptr;
+  unsigned char *deg_host = nullptr, *head_host = nullptr;
   std::vector<float> cheb_a, cheb_c;    // Chebyshev coefficients per step
   cudaStream_t stream = nullptr;
   bool own_stream = false;
-  float *f = nullptr, *s = nullptr, *u = nullptr, *bv = nullptr, *d = nullptr;
-  float *w = nullptr, *bw = nullptr, *q = nullptr, *gap = nullptr;
-  // the u-step's vectors pixel-major, four labels per float4 ([P][Q], Q = ceil(K/4)):
-  // two Chebyshev iterates, the Chebyshev direction and the right-hand side
-  float4 *xa = nullptr, *xb = nullptr, *cd = nullptr, *rhs = nullptr;
+  float *f = nullptr, *s = nullptr, *u = nullptr, *w = nullptr, *bw = nullptr, *gap = nullptr;
+  // four labels per float4, Q = ceil(K/4), labels past K zero: pixel-major
+  // ([P][Q]) the u-step's vectors (two Chebyshev iterates, the Chebyshev
+  // direction, the right-hand side) and q = (w - b_w) - gamma s; [Q][m][P] the
+  // pair b_v and d = v - b_v of the differences to the m neighbours
+  float4 *xa = nullptr, *xb = nullptr, *cd = nullptr, *rhs = nullptr, *q = nullptr, *bv = nullptr, *d = nullptr;
   int Q = 0;
   int* nbr = nullptr;                   // [m][P]
   short* off = nullptr;                 // [m][P] neighbour minus pixel index (|off| <= 7 W + 7)
   unsigned char *rev = nullptr, *deg = nullptr;
+  // the graph's construction: patch weights, the first ranks, the selected links
+  double* gw = nullptr;
+  unsigned char* head = nullptr;
+  int* list = nullptr;
   int* labels = nullptr;
   int* flag = nullptr;
   double* red = nullptr;
@@ -74,60 +81,262 @@ constexpr int kRedBlocks = 512;
 constexpr int kMaxM = 16;       // neighbours per pixel (2 mt, mt <= 8)
 constexpr int kMaxWin = 15;     // search window side: (2r + 1)^2 <= 225 window codes
 constexpr int kMaxPatch = 9;    // patch side
-constexpr int kRankWarps = 4;   // warps (pixels) per CTA of the ranking kernel
+constexpr int kRankWarps = 8;   // warps per CTA of the ranking kernel
 
 __device__ __forceinline__ int mirror_idx(int x, int n) {
   while (x < 0 || x >= n) x = x < 0 ? -x : 2 * (n - 1) - x;
   return x;
 }
 
-// One warp per pixel: the patch distances to every window code c = (dy + r)
-// (2r + 1) + (dx + r) (the centre and codes outside the image excluded) and
-// their ranks by (distance, code); rank[i][pos] = code of position pos, 255
-// for the unused positions at the end.  Codes in increasing order are
-// candidates in increasing raster index, so this is the order (distance,
-// raster index).  G: the patch weights [(2h+1)^2] in FP64.
-__global__ void __launch_bounds__(32 * kRankWarps) k_nl_rank(const float* __restrict__ f, int H, int W, int C,
-                                                             const double* __restrict__ G, int h, int r,
-                                                             unsigned char* __restrict__ rank) {
-  __shared__ double key[kRankWarps][(2 * (kMaxWin / 2) + 1) * (2 * (kMaxWin / 2) + 1)];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int i = blockIdx.x * kRankWarps + wid;
-  const int side = 2 * r + 1, NW = side * side;
-  const size_t P = static_cast<size_t>(H) * W;
-  if (i >= H * W) return;  // whole warps leave together
-  const int ri = i / W, ci = i - ri * W;
+// Ranks of the window candidates of every pixel by (distance, code), code c =
+// (dy + r)(2r + 1) + (dx + r) (the centre and codes outside the image
+// excluded): codes in increasing order are candidates in increasing raster
+// index, so this is the order (distance, raster index) of the FP64 distances
+// with every product and sum rounded separately.
+//
+// GB300's FP64 rate is a 64th of its FP32 rate, and the exact distances are
+// only needed where they decide the order.  A warp takes a pixel: FP32
+// distances from a shared-memory tile of the image (7 candidates per lane),
+// a bitonic sort of (distance, code) keys over the warp's registers, and then,
+// for the candidates whose FP32 distance is within twice its error bound of a
+// neighbour's in the sorted order, the FP64 distances, by which each run of
+// such candidates is ordered.  The bound: with the weights and the image
+// in the range checked below, a distance is a sum of n positive terms, each
+// with four rounding errors, so its relative error is at most (n + 4) 2^-24
+// (the caller's `delta` doubles it) plus what underflow costs (kTiny).
+constexpr int kRankTX = 32, kRankTY = 4;  // pixels per CTA
+constexpr int kMaxHalo = kMaxWin / 2 + kMaxPatch / 2;
+constexpr int kRankRows = kRankTY + 2 * kMaxHalo, kRankCols = kRankTX + 2 * kMaxHalo;
+constexpr float kRankMax = 1e4f;  // largest |f| of a tile for the FP32 distances
+constexpr float kTiny = 1e-36f;
+// ranks copied to the host for every pixel; a pixel needs more only when its
+// nearest 64 candidates are nearly all full (1 pixel in 10^4 of the textured
+// images, 3 in 10^3 would need more than 32)
+constexpr int kRankHead = 64;
+
+// FP64 distance of the pixel at tile position (y, x) to the candidate (dy, dx).
+__device__ __forceinline__ double nl_exact(const float (*tile)[kRankRows][kRankCols], int C, const double* __restrict__ G,
+                                           int h, int y, int x, int dy, int dx) {
   const int n = 2 * h + 1;
-  for (int c = lane; c < NW; c += 32) {
-    const int dy = c / side - r, dx = c % side - r;
-    const int rj = ri + dy, cj = ci + dx;
-    double acc = INFINITY;
-    if ((dy != 0 || dx != 0) && rj >= 0 && rj < H && cj >= 0 && cj < W) {
-      acc = 0.0;
-      for (int t1 = -h; t1 <= h; ++t1)
-        for (int t2 = -h; t2 <= h; ++t2) {
-          const size_t a = static_cast<size_t>(mirror_idx(ri + t1, H)) * W + mirror_idx(ci + t2, W);
-          const size_t b = static_cast<size_t>(mirror_idx(rj + t1, H)) * W + mirror_idx(cj + t2, W);
-          double sum = 0.0;
-          for (int ch = 0; ch < C; ++ch) {
-            const double dd = __dsub_rn(static_cast<double>(f[ch * P + a]), static_cast<double>(f[ch * P + b]));
-            sum = __dadd_rn(sum, __dmul_rn(dd, dd));
-          }
-          acc = __dadd_rn(acc, __dmul_rn(G[(t1 + h) * n + (t2 + h)], sum));
-        }
+  double acc = 0.0;
+  for (int t1 = -h; t1 <= h; ++t1)
+    for (int t2 = -h; t2 <= h; ++t2) {
+      double sum = 0.0;
+      for (int ch = 0; ch < C; ++ch) {
+        const double dd = __dsub_rn(static_cast<double>(tile[ch][y + t1][x + t2]),
+                                    static_cast<double>(tile[ch][y + dy + t1][x + dx + t2]));
+        sum = __dadd_rn(sum, __dmul_rn(dd, dd));
+      }
+      acc = __dadd_rn(acc, __dmul_rn(G[(t1 + h) * n + (t2 + h)], sum));
     }
-    key[wid][c] = acc;
+  return acc;
+}
+
+// The rows from ystrip on.  rank (optional) holds every code of those rows'
+// pixels in order, 255 for the unused positions at the end; head[i] (optional)
+// the first kRankHead of pixel i.  G: the patch weights [(2h+1)^2].
+// Bound by instruction issue (about 3000 warp instructions a pixel: distances
+// 900, sort 1500); 512 x 512, 5 x 5 patches, 15 x 15 window: 79.3 ms with FP64
+// distances and ranks counted over all pairs, 1.2 ms so.
+template <int C>
+__global__ void __launch_bounds__(32 * kRankWarps)
+    k_nl_rank(const float* __restrict__ f, int H, int W, const double* __restrict__ G, int h, int r, float delta,
+              int ystrip, unsigned char* __restrict__ rank, unsigned char* __restrict__ head) {
+  __shared__ float tile[C][kRankRows][kRankCols];
+  __shared__ float sG[kMaxPatch * kMaxPatch];
+  __shared__ double ex[kRankWarps][256];
+  __shared__ unsigned char code[kRankWarps][256], out[kRankWarps][256], list[kRankWarps][256], near_next[kRankWarps][256];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int side = 2 * r + 1, NW = side * side, cen = NW / 2, n = 2 * h + 1, halo = r + h;
+  const size_t P = static_cast<size_t>(H) * W;
+  const int y0 = ystrip + blockIdx.y * kRankTY, x0 = blockIdx.x * kRankTX;
+  for (int e = threadIdx.x; e < n * n; e += blockDim.x) sG[e] = static_cast<float>(G[e]);
+  // the image around the CTA's pixels, mirrored at the borders
+  const int rows = kRankTY + 2 * halo, cols = kRankTX + 2 * halo;
+  bool wide = false;
+  for (int e = threadIdx.x; e < rows * cols; e += blockDim.x) {
+    const int y = e / cols, x = e - y * cols;
+    const size_t src = static_cast<size_t>(mirror_idx(y0 - halo + y, H)) * W + mirror_idx(x0 - halo + x, W);
+#pragma unroll
+    for (int ch = 0; ch < C; ++ch) {
+      const float v = f[ch * P + src];
+      tile[ch][y][x] = v;
+      wide = wide || !(fabsf(v) <= kRankMax);
+    }
   }
-  __syncwarp();
-  unsigned char* out = rank + static_cast<size_t>(i) * NW;
-  for (int c = lane; c < NW; c += 32) {
-    const double kc = key[wid][c];
-    int pos = 0;
-    for (int c2 = 0; c2 < NW; ++c2) {
-      const double k2 = key[wid][c2];
-      pos += (k2 < kc || (k2 == kc && c2 < c)) ? 1 : 0;
+  // delta < 0: weights too small for the bound; then, and for large values,
+  // every candidate takes its FP64 distance
+  const bool all_exact = __syncthreads_or(wide ? 1 : 0) != 0 || delta < 0.f;
+  // the lane's candidates: number lane + 32 q of the window without its centre
+  int dy[7], dx[7];
+#pragma unroll
+  for (int q = 0; q < 7; ++q) {
+    const int m = lane + 32 * q, c = m < cen ? m : m + 1;
+    dy[q] = m < NW - 1 ? c / side - r : 0;
+    dx[q] = m < NW - 1 ? c % side - r : 0;
+  }
+  for (int px = wid; px < kRankTX * kRankTY; px += kRankWarps) {
+    const int ri = y0 + px / kRankTX, ci = x0 + px % kRankTX;
+    if (ri >= H || ci >= W) continue;  // the whole warp
+    const int y = px / kRankTX + halo, x = px % kRankTX + halo;
+    float acc[7];
+    const float* base[7];
+#pragma unroll
+    for (int q = 0; q < 7; ++q) {
+      acc[q] = 0.f;
+      base[q] = &tile[0][y + dy[q] - h][x + dx[q] - h];
     }
-    out[pos] = kc == INFINITY ? 255 : static_cast<unsigned char>(c);
+    const float* own = &tile[0][y - h][x - h];
+#pragma unroll
+    for (int ch = 0; ch < C; ++ch)
+      for (int t1 = 0; t1 < n; ++t1)
+        for (int t2 = 0; t2 < n; ++t2) {
+          const int o = (ch * kRankRows + t1) * kRankCols + t2;
+          const float a = own[o], g = sG[t1 * n + t2];
+#pragma unroll
+          for (int q = 0; q < 7; ++q) {
+            const float d = a - base[q][o];
+            acc[q] = fmaf(d * g, d, acc[q]);
+          }
+        }
+    // keys: distance bits (non-negative floats order as integers) and code
+    unsigned long long key[8];
+    int nv = 0;  // valid candidates
+#pragma unroll
+    for (int q = 0; q < 7; ++q) {
+      const int m = lane + 32 * q, c = m < cen ? m : m + 1;
+      const int rj = ri + dy[q], cj = ci + dx[q];
+      const bool ok = m < NW - 1 && rj >= 0 && rj < H && cj >= 0 && cj < W;
+      const unsigned bits = all_exact ? 0u : __float_as_uint(acc[q]);
+      key[q] = ok ? (static_cast<unsigned long long>(bits) << 32) | static_cast<unsigned>(c) : ~0ull;
+      nv += __popc(__ballot_sync(0xffffffffu, ok));
+    }
+    key[7] = ~0ull;
+    // bitonic sort of the 256 keys, element lane * 8 + i in key[i]
+#pragma unroll
+    for (int k = 2; k <= 256; k <<= 1)
+#pragma unroll
+      for (int j = k >> 1; j > 0; j >>= 1) {
+        if (j >= 8) {
+          const bool up = ((lane * 8) & k) == 0, lower = (lane & (j / 8)) == 0;
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            const unsigned long long o = __shfl_xor_sync(0xffffffffu, key[i], j / 8);
+            key[i] = ((o < key[i]) == (up == lower)) ? o : key[i];
+          }
+        } else {
+#pragma unroll
+          for (int i = 0; i < 8; ++i)
+            if ((i & j) == 0) {
+              const bool up = ((lane * 8 + i) & k) == 0;
+              const unsigned long long a = key[i], b = key[i | j];
+              const bool sw = (b < a) == up;
+              key[i] = sw ? b : a;
+              key[i | j] = sw ? a : b;
+            }
+        }
+      }
+    // which neighbours in the order are closer than the bound
+    const unsigned long long first_next = __shfl_down_sync(0xffffffffu, key[0], 1);
+    unsigned close = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int e = lane * 8 + i;
+      const float a = __uint_as_float(static_cast<unsigned>(key[i] >> 32));
+      const float b = __uint_as_float(static_cast<unsigned>((i < 7 ? key[i < 7 ? i + 1 : 0] : first_next) >> 32));
+      const bool c = e + 1 < nv && !(b > fmaf(a, delta, a) + kTiny);
+      close |= (c ? 1u : 0u) << i;
+      code[wid][e] = static_cast<unsigned char>(key[i]);
+      out[wid][e] = e < nv ? static_cast<unsigned char>(key[i]) : 255;
+      near_next[wid][e] = c ? 1 : 0;
+    }
+    const unsigned before = __shfl_up_sync(0xffffffffu, close, 1) >> 7;
+    const unsigned amb = close | ((close << 1) & 0xffu) | (lane > 0 ? before & 1u : 0u);
+    if (__any_sync(0xffffffffu, amb != 0u)) {
+      // positions of the undecided candidates
+      int at = __popc(amb), total = at;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, at, o);
+        at += lane >= o ? v : 0;
+      }
+      total = __shfl_sync(0xffffffffu, at, 31);
+      at -= __popc(amb);
+      for (int i = 0; i < 8; ++i)
+        if (amb >> i & 1u) list[wid][at++] = static_cast<unsigned char>(lane * 8 + i);
+      __syncwarp();
+      for (int q = lane; q < total; q += 32) {
+        const int e = list[wid][q], c = code[wid][e];
+        ex[wid][e] = nl_exact(tile, C, G, h, y, x, c / side - r, c % side - r);
+      }
+      __syncwarp();
+      for (int q = lane; q < total; q += 32) {
+        const int e = list[wid][q];
+        const double me = ex[wid][e];
+        const int c = code[wid][e];
+        int pos = e;
+        for (int o = e - 1; o >= 0 && near_next[wid][o]; --o) {
+          const double v = ex[wid][o];
+          pos -= (v > me || (v == me && code[wid][o] > c)) ? 1 : 0;
+        }
+        for (int o = e + 1; near_next[wid][o - 1]; ++o) {
+          const double v = ex[wid][o];
+          pos += (v < me || (v == me && code[wid][o] < c)) ? 1 : 0;
+        }
+        out[wid][pos] = static_cast<unsigned char>(c);
+      }
+    }
+    __syncwarp();
+    const size_t i = static_cast<size_t>(ri) * W + ci;
+    if (rank)
+      for (int c = lane; c < NW; c += 32) rank[(i - static_cast<size_t>(ystrip) * W) * NW + c] = out[wid][c];
+    if (head)
+      for (int c = lane; c < kRankHead; c += 32) head[i * kRankHead + c] = c < NW ? out[wid][c] : 255;
+    __syncwarp();
+  }
+}
+
+// The device tables of the selected links, list [P][m] with deg[i] entries:
+// sorted neighbour lists nbr [m][P] (-1 padded) and offsets off [m][P].
+__global__ void __launch_bounds__(kThreads) k_nl_tables(const int* __restrict__ list, const unsigned char* __restrict__ deg,
+                                                        int m, size_t P, int* __restrict__ nbr, short* __restrict__ off) {
+  const size_t i = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x;
+  if (i >= P) return;
+  const int dg = deg[i];
+  int v[kMaxM];
+#pragma unroll
+  for (int b = 0; b < kMaxM; ++b) v[b] = b < dg ? list[i * m + b] : 0x7fffffff;
+  // odd-even transposition
+#pragma unroll
+  for (int t = 0; t < kMaxM; ++t)
+#pragma unroll
+    for (int b = t & 1; b + 1 < kMaxM; b += 2) {
+      const int a = min(v[b], v[b + 1]), c = max(v[b], v[b + 1]);
+      v[b] = a;
+      v[b + 1] = c;
+    }
+#pragma unroll
+  for (int b = 0; b < kMaxM; ++b)
+    if (b < m) {
+      nbr[b * P + i] = b < dg ? v[b] : -1;
+      off[b * P + i] = b < dg ? static_cast<short>(v[b] - static_cast<long long>(i)) : static_cast<short>(0);
+    }
+}
+
+// rev[b][i]: the position of pixel i in the list of its b-th neighbour.
+__global__ void __launch_bounds__(kThreads) k_nl_reverse(const int* __restrict__ nbr, const unsigned char* __restrict__ deg,
+                                                         int m, size_t P, unsigned char* __restrict__ rev) {
+  const size_t i = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x;
+  if (i >= P) return;
+  const int dg = deg[i];
+  for (int b = 0; b < m; ++b) {
+    int pos = 0;
+    if (b < dg) {
+      const size_t j = static_cast<size_t>(nbr[b * P + i]);
+      const int dj = deg[j];
+      while (pos + 1 < dj && nbr[pos * P + j] != static_cast<int>(i)) ++pos;
+    }
+    rev[b * P + i] = static_cast<unsigned char>(pos);
   }
 }
 
@@ -145,7 +354,7 @@ __device__ __forceinline__ int load_nbrs(const int* __restrict__ nbr, const unsi
 // The iterates, the direction and the right-hand side are pixel-major, four
 // labels per float4, so that each neighbour is one 16-byte load per four
 // labels; the first step reads u label-major ([K][P], IN_LM) and the last
-// writes it back label-major (OUT_LM).
+// also writes it back label-major (OUT_LM).
 __device__ __forceinline__ float4 f4_axpy(float a, float4 x, float4 y) {
   return make_float4(fmaf(a, x.x, y.x), fmaf(a, x.y, y.y), fmaf(a, x.z, y.z), fmaf(a, x.w, y.w));
 }
@@ -198,9 +407,8 @@ __global__ void __launch_bounds__(kThreads) k_nl_cheb(const float* __restrict__ 
         if (k0 + 1 < K) xout_lm[(k0 + 1) * P + i] = xo.y;
         if (k0 + 2 < K) xout_lm[(k0 + 2) * P + i] = xo.z;
         if (k0 + 3 < K) xout_lm[(k0 + 3) * P + i] = xo.w;
-      } else {
-        xout[i * Q + qd] = xo;
       }
+      xout[i * Q + qd] = xo;
     }
   }
 }
@@ -346,6 +554,7 @@ __global__ void __launch_bounds__(kChebThreads, 1) k_nl_cheb_all(float* __restri
   for (int p = 0; p < kChebPPT; ++p) {
     const size_t i = base + p * kChebThreads + threadIdx.x;
     if (i >= P) continue;
+    xout[i] = xi[p];  // nobody reads that buffer in the last step
     u[i] = xi[p].x;
     if (K > 1) u[P + i] = xi[p].y;
     if (K > 2) u[2 * P + i] = xi[p].z;
@@ -366,111 +575,165 @@ size_t cheb_all_smem(int R, int MM) {
 
 // The v-, w- and b-updates after the u-step: g_b = b_v,b + u(nbr_b) - u(i)
 // (b < deg; b_v,b for the zero rows), group clip over the m K values,
-// d = g - 2 b_v; w-step and q = (w - b_w) - gamma s.
-template <int KM>
-__global__ void __launch_bounds__(kThreads) k_nl_prox(const float* __restrict__ u, float* __restrict__ bv,
-                                                      float* __restrict__ d, float* __restrict__ w,
+// d = g - 2 b_v; w-step and q = (w - b_w) - gamma s.  xu: u pixel-major.
+// With four labels per float4 a neighbour is one 16-byte load (the labels one
+// by one took four 4-byte loads each, of sectors that held nothing else), and
+// for K <= 4 (ONE) all g of a pixel stay in registers between the norm and the
+// update; otherwise they are formed twice.  MM: at most m neighbours (10 for
+// the paper's five picked per pixel).  Bound by memory: per pixel 3 m Q 16 B of
+// b_v and d, 150 MB at 512 x 512, K = 4, m = 10: 112 -> 44 us.
+template <int KM, int MM, bool ONE>
+__global__ void __launch_bounds__(kThreads) k_nl_prox(const float4* __restrict__ xu, float4* __restrict__ bv,
+                                                      float4* __restrict__ d, float* __restrict__ w,
                                                       float* __restrict__ bw, const float* __restrict__ s,
-                                                      float* __restrict__ q, const int* __restrict__ nbr,
-                                                      const unsigned char* __restrict__ deg, int K, int m, size_t P,
-                                                      float t, float gamma) {
+                                                      float4* __restrict__ q, const short* __restrict__ off,
+                                                      const unsigned char* __restrict__ deg, int K, int Q, int m,
+                                                      size_t P, float t, float gamma) {
   shf::fast::pdl_wait();  // u comes from the last Chebyshev step
   shf::fast::pdl_trigger();
   for (size_t i = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; i < P;
        i += static_cast<size_t>(gridDim.x) * blockDim.x) {
-    int nb[kMaxM];
-    const int dg = load_nbrs(nbr, deg, P, i, m, nb);
-    // the group norm over the m K values of g (the label loop is not unrolled:
-    // only the neighbour indices stay in registers)
-    float n2 = 0.f;
-    for (int k = 0; k < K; ++k) {
-      const float* up = u + k * P;
-      const float ui = up[i];
-      const float* bk = bv + static_cast<size_t>(k) * m * P;
+    const int dg = deg[i];
+    int nb[MM];
 #pragma unroll
-      for (int b = 0; b < kMaxM; ++b) {
+    for (int b = 0; b < MM; ++b) nb[b] = b < dg ? static_cast<int>(i) + off[b * P + i] : static_cast<int>(i);
+    auto diff = [&](int b, int qd, float4 ui) {  // g_b; the pixel itself stands in for a missing neighbour
+      const float4 x = xu[static_cast<size_t>(nb[b]) * Q + qd];
+      const float4 o = bv[(static_cast<size_t>(qd) * m + b) * P + i];
+      return make_float4(o.x + (x.x - ui.x), o.y + (x.y - ui.y), o.z + (x.z - ui.z), o.w + (x.w - ui.w));
+    };
+    float4 g[ONE ? MM : 1];
+    float n2 = 0.f;
+    for (int qd = 0; qd < (ONE ? 1 : Q); ++qd) {
+      const float4 ui = xu[i * Q + qd];
+#pragma unroll
+      for (int b = 0; b < MM; ++b) {
         if (b < m) {
-          const float g = bk[b * P + i] + (b < dg ? up[nb[b]] - ui : 0.f);
-          n2 = fmaf(g, g, n2);
+          const float4 v = diff(b, qd, ui);
+          if (ONE) g[ONE ? b : 0] = v;
+          n2 = fmaf(v.x, v.x, n2);
+          n2 = fmaf(v.y, v.y, n2);
+          n2 = fmaf(v.z, v.z, n2);
+          n2 = fmaf(v.w, v.w, n2);
         }
       }
     }
     const float nrm = sqrtf(n2);
     const float fac = nrm > t ? t / nrm : 1.f;
-    for (int k = 0; k < K; ++k) {
-      const float* up = u + k * P;
-      const float ui = up[i];
-      float* bk = bv + static_cast<size_t>(k) * m * P;
-      float* dk = d + static_cast<size_t>(k) * m * P;
+    for (int qd = 0; qd < (ONE ? 1 : Q); ++qd) {
+      const float4 ui = xu[i * Q + qd];
 #pragma unroll
-      for (int b = 0; b < kMaxM; ++b) {
+      for (int b = 0; b < MM; ++b) {
         if (b < m) {
-          const float g = bk[b * P + i] + (b < dg ? up[nb[b]] - ui : 0.f);
-          const float bn = fac * g;
-          bk[b * P + i] = bn;
-          dk[b * P + i] = g - 2.f * bn;
+          const float4 v = ONE ? g[ONE ? b : 0] : diff(b, qd, ui);
+          const float4 bn = make_float4(fac * v.x, fac * v.y, fac * v.z, fac * v.w);
+          bv[(static_cast<size_t>(qd) * m + b) * P + i] = bn;
+          d[(static_cast<size_t>(qd) * m + b) * P + i] =
+              make_float4(v.x - 2.f * bn.x, v.y - 2.f * bn.y, v.z - 2.f * bn.z, v.w - 2.f * bn.w);
         }
       }
     }
     float gw[KM], wk[KM];
 #pragma unroll
-    for (int k = 0; k < KM; ++k) {
-      gw[k] = k < K ? bw[k * P + i] + u[k * P + i] : 0.f;
-      wk[k] = gw[k];
+    for (int k = 0; k < KM; k += 4) {
+      const float4 ui = k < K ? xu[i * Q + k / 4] : make_float4(0.f, 0.f, 0.f, 0.f);
+      const float uk[4] = {ui.x, ui.y, ui.z, ui.w};
+#pragma unroll
+      for (int c = 0; c < 4; ++c) {
+        gw[k + c] = k + c < K ? bw[(k + c) * P + i] + uk[c] : 0.f;
+        wk[k + c] = gw[k + c];
+      }
     }
     shf::simplex_project<KM>(wk, K);
 #pragma unroll
-    for (int k = 0; k < KM; ++k) {
-      if (k < K) {
-        const float bn = gw[k] - wk[k];
-        w[k * P + i] = wk[k];
-        bw[k * P + i] = bn;
-        q[k * P + i] = (wk[k] - bn) - gamma * s[k * P + i];
-      }
+    for (int k = 0; k < KM; k += 4) {
+      float qv[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+      for (int c = 0; c < 4; ++c)
+        if (k + c < K) {
+          const float bn = gw[k + c] - wk[k + c];
+          w[(k + c) * P + i] = wk[k + c];
+          bw[(k + c) * P + i] = bn;
+          qv[c] = (wk[k + c] - bn) - gamma * s[(k + c) * P + i];
+        }
+      if (k < K) q[i * Q + k / 4] = make_float4(qv[0], qv[1], qv[2], qv[3]);
     }
   }
 }
 
 // rhs = q + D^T d: (D^T d)(j) = sum_{b < deg(j)} [d_rev(j,b)(nbr_b(j)) - d_b(j)],
-// written pixel-major ([P][4 Q], labels K..4Q-1 zero) for the Chebyshev steps.
-__global__ void __launch_bounds__(kThreads) k_nl_rhs(const float* __restrict__ q, const float* __restrict__ d,
-                                                     float* __restrict__ rhs, const int* __restrict__ nbr,
+// pixel-major as the Chebyshev steps read it (512 x 512, K = 4: 47 -> 27 us with
+// one 16-byte load per neighbour).
+template <int MM>
+__global__ void __launch_bounds__(kThreads) k_nl_rhs(const float4* __restrict__ q, const float4* __restrict__ d,
+                                                     float4* __restrict__ rhs, const short* __restrict__ off,
                                                      const unsigned char* __restrict__ rev,
-                                                     const unsigned char* __restrict__ deg, int K, int Q, int m,
-                                                     size_t P) {
+                                                     const unsigned char* __restrict__ deg, int Q, int m, size_t P) {
   shf::fast::pdl_wait();  // q and d come from the prox kernel
   shf::fast::pdl_trigger();
   for (size_t j = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; j < P;
        j += static_cast<size_t>(gridDim.x) * blockDim.x) {
-    int nb[kMaxM];
-    const int dg = load_nbrs(nbr, deg, P, j, m, nb);
-    int rv[kMaxM];
+    const int dg = deg[j];
+    size_t at[MM];  // where the neighbour keeps its difference to j
 #pragma unroll
-    for (int b = 0; b < kMaxM; ++b) rv[b] = b < dg ? rev[b * P + j] : 0;
-    for (int k = 0; k < K; ++k) {
-      const float* dk = d + static_cast<size_t>(k) * m * P;
-      float acc = 0.f;
+    for (int b = 0; b < MM; ++b)
+      at[b] = b < dg ? static_cast<size_t>(rev[b * P + j]) * P + (static_cast<long long>(j) + off[b * P + j]) : 0;
+    for (int qd = 0; qd < Q; ++qd) {
+      const float4* dq = d + static_cast<size_t>(qd) * m * P;
+      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-      for (int b = 0; b < kMaxM; ++b)
-        if (b < dg) acc += dk[rv[b] * P + nb[b]] - dk[b * P + j];
-      rhs[j * 4 * Q + k] = q[k * P + j] + acc;  // pixel-major, four labels per float4
+      for (int b = 0; b < MM; ++b)
+        if (b < dg) {
+          const float4 x = dq[at[b]], y = dq[b * P + j];
+          acc = make_float4(acc.x + (x.x - y.x), acc.y + (x.y - y.y), acc.z + (x.z - y.z), acc.w + (x.w - y.w));
+        }
+      const float4 qv = q[j * Q + qd];
+      rhs[j * Q + qd] = make_float4(qv.x + acc.x, qv.y + acc.y, qv.z + acc.z, qv.w + acc.w);
     }
-    for (int k = K; k < 4 * Q; ++k) rhs[j * 4 * Q + k] = 0.f;
   }
 }
 
+// q from label-major planes, pixel-major.
 __global__ void k_nl_q(const float* __restrict__ w, const float* __restrict__ bw, const float* __restrict__ s,
-                       float* __restrict__ q, float gamma, size_t n) {
-  for (size_t i = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; i < n;
-       i += static_cast<size_t>(gridDim.x) * blockDim.x)
-    q[i] = (w[i] - bw[i]) - gamma * s[i];
+                       float* __restrict__ q, float gamma, int K, int Q, size_t P) {
+  const size_t n = P * 4 * Q;
+  for (size_t e = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; e < n;
+       e += static_cast<size_t>(gridDim.x) * blockDim.x) {
+    const size_t i = e / (4 * Q), k = e - i * 4 * Q;
+    q[e] = k < static_cast<size_t>(K) ? (w[k * P + i] - bw[k * P + i]) - gamma * s[k * P + i] : 0.f;
+  }
 }
 
-// out = a + sb b (out may alias a).
-__global__ void k_nl_axpb(const float* a, const float* __restrict__ b, float* out, float sb, size_t n) {
-  for (size_t i = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; i < n;
-       i += static_cast<size_t>(gridDim.x) * blockDim.x)
-    out[i] = a[i] + sb * b[i];
+// The neighbour pairs of the state ([Q][m][P] float4) as label-major planes
+// [K][m][P]: out = a + sb b (b optional), and back: out = a + sb b with a
+// label-major, labels past K zero.
+__global__ void k_nl_unpack(const float4* __restrict__ a, const float4* __restrict__ b, float* __restrict__ out, float sb,
+                            int K, int Q, size_t mP) {
+  for (size_t e = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; e < mP * Q;
+       e += static_cast<size_t>(gridDim.x) * blockDim.x) {
+    const size_t qd = e / mP, i = e - qd * mP;
+    const float4 x = a[e], y = b ? b[e] : make_float4(0.f, 0.f, 0.f, 0.f);
+    const float v[4] = {x.x + sb * y.x, x.y + sb * y.y, x.z + sb * y.z, x.w + sb * y.w};
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+      if (4 * qd + c < static_cast<size_t>(K)) out[(4 * qd + c) * mP + i] = v[c];
+  }
+}
+__global__ void k_nl_pack(const float* __restrict__ a, const float4* __restrict__ b, float4* __restrict__ out, float sb,
+                          int K, int Q, size_t mP) {
+  for (size_t e = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; e < mP * Q;
+       e += static_cast<size_t>(gridDim.x) * blockDim.x) {
+    const size_t qd = e / mP, i = e - qd * mP;
+    const float4 y = b ? b[e] : make_float4(0.f, 0.f, 0.f, 0.f);
+    const float o[4] = {y.x, y.y, y.z, y.w};
+    float v[4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const size_t k = 4 * qd + c;
+      v[c] = k < static_cast<size_t>(K) ? a[k * mP + i] + sb * o[c] : 0.f;
+    }
+    out[e] = make_float4(v[0], v[1], v[2], v[3]);
+  }
 }
 
 // FP64 energy partials: <w, s> and sum_i (sum_k sum_b ((D w_k)_b(i))^2)^(1/2).
@@ -547,6 +810,21 @@ int nl_alloc(T** p, size_t count, const char* what) {
   return SHF_OK;
 }
 
+// Pinned host memory: the graph's copies run at the link's rate and touch no new
+// pages on a reset.
+template <typename T>
+int nl_alloc_host(T** p, size_t count, const char* what) {
+  *p = nullptr;
+  cudaError_t e = cudaMallocHost(reinterpret_cast<void**>(p), count * sizeof(T));
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    *p = nullptr;
+    return nl_fail(e == cudaErrorMemoryAllocation ? SHF_ERR_OOM : SHF_ERR_CUDA,
+                   std::string("cudaMallocHost(") + what + "): " + cudaGetErrorString(e));
+  }
+  return SHF_OK;
+}
+
 int grid_for(size_t n) {
   const size_t b = (n + kThreads - 1) / kThreads;
   return static_cast<int>(b < 8192 ? (b ? b : 1) : 8192);
@@ -557,9 +835,13 @@ void free_nl(nl_state* st) {
   if (st->stream) cudaStreamSynchronize(st->stream);
   if (st->exec) cudaGraphExecDestroy(st->exec);
   void* bufs[] = {st->f, st->s, st->u, st->xa, st->xb, st->cd, st->bv, st->d, st->w, st->bw, st->q, st->rhs,
-                  st->gap, st->nbr, st->off, st->rev, st->deg, st->labels, st->flag, st->red,
+                  st->gap, st->nbr, st->off, st->rev, st->deg, st->gw, st->head, st->list, st->labels, st->flag,
+                  st->red,
                   st->cbar, st->cerr, st->cheb_ac};
   for (void* b : bufs) cudaFree(b);
+  cudaFreeHost(st->nbr_host);
+  cudaFreeHost(st->deg_host);
+  cudaFreeHost(st->head_host);
   if (st->own_stream && st->stream) cudaStreamDestroy(st->stream);
   delete st;
 }
@@ -587,68 +869,80 @@ int build_graph(nl_state* st) {
   const int h = st->prm.patch / 2, r = st->prm.window / 2, side = 2 * r + 1, NW = side * side;
   const size_t P = st->P();
   const auto G = patch_weights(h, st->prm.a);
-  double* dG = nullptr;
-  unsigned char* drank = nullptr;
-  NL_CK(cudaMallocAsync(reinterpret_cast<void**>(&dG), sizeof(double) * G.size(), st->stream));
-  NL_CK(cudaMallocAsync(reinterpret_cast<void**>(&drank), P * NW, st->stream));
-  std::vector<unsigned char> rank(P * NW);
-  cudaError_t e = cudaMemcpyAsync(dG, G.data(), sizeof(double) * G.size(), cudaMemcpyHostToDevice, st->stream);
-  if (e == cudaSuccess) {
-    k_nl_rank<<<static_cast<unsigned>((P + kRankWarps - 1) / kRankWarps), 32 * kRankWarps, 0, st->stream>>>(
-        st->f, H, W, st->C, dG, h, r, drank);
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess) e = cudaMemcpyAsync(rank.data(), drank, P * NW, cudaMemcpyDeviceToHost, st->stream);
-  cudaError_t e2 = cudaFreeAsync(dG, st->stream);
-  cudaError_t e3 = cudaFreeAsync(drank, st->stream);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st->stream);
-  if (e == cudaSuccess) e = e2 != cudaSuccess ? e2 : e3;
-  NL_CK(e);
+  // twice the FP32 distances' relative error bound; negative when a weight is
+  // too small for it
+  double gmin = G[0];
+  for (double g : G) gmin = std::min(gmin, g);
+  const float bound = gmin < 1e-30 ? -1.f : static_cast<float>(2.02 * (static_cast<double>(G.size()) * st->C + 4) / 16777216.0);
+  NL_CK(cudaMemcpyAsync(st->gw, G.data(), sizeof(double) * G.size(), cudaMemcpyHostToDevice, st->stream));
+  auto launch_rank = [&](int y, int strips, unsigned char* rank, unsigned char* head) {
+    const dim3 grid((W + kRankTX - 1) / kRankTX, strips);
+    if (st->C == 1)
+      k_nl_rank<1><<<grid, 32 * kRankWarps, 0, st->stream>>>(st->f, H, W, st->gw, h, r, bound, y, rank, head);
+    else
+      k_nl_rank<3><<<grid, 32 * kRankWarps, 0, st->stream>>>(st->f, H, W, st->gw, h, r, bound, y, rank, head);
+    return cudaGetLastError();
+  };
+  // every rank of the strip of kRankTY rows that holds row y (for the few
+  // pixels that need more than the first ones)
+  std::vector<unsigned char> strip;
+  int strip_y = -1;
+  auto fetch_strip = [&](int y) -> int {
+    const int y0 = y / kRankTY * kRankTY;
+    if (y0 == strip_y) return SHF_OK;
+    const size_t bytes = static_cast<size_t>(std::min(kRankTY, H - y0)) * W * NW;
+    unsigned char* drank = nullptr;
+    strip.resize(bytes);
+    NL_CK(cudaMallocAsync(reinterpret_cast<void**>(&drank), bytes, st->stream));
+    cudaError_t e = launch_rank(y0, 1, drank, nullptr);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(strip.data(), drank, bytes, cudaMemcpyDeviceToHost, st->stream);
+    const cudaError_t e2 = cudaFreeAsync(drank, st->stream);
+    if (e == cudaSuccess) e = e2;
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st->stream);
+    NL_CK(e);
+    strip_y = y0;
+    return SHF_OK;
+  };
+  NL_CK(launch_rank(0, (H + kRankTY - 1) / kRankTY, nullptr, st->head));
+  NL_CK(cudaMemcpyAsync(st->head_host, st->head, P * kRankHead, cudaMemcpyDeviceToHost, st->stream));
+  NL_CK(cudaStreamSynchronize(st->stream));
   // selection in raster order over the ranked candidates
-  std::vector<int>& nb = st->nbr_host;
-  std::vector<int>& dg = st->deg_host;
-  nb.assign(P * m, -1);
-  dg.assign(P, 0);
+  int* const nb = st->nbr_host;
+  unsigned char* const dg = st->deg_host;
+  std::fill(dg, dg + P, static_cast<unsigned char>(0));
+  std::vector<int> step(NW);
+  for (int c = 0; c < NW; ++c) step[c] = (c / side - r) * W + (c % side - r);
   for (size_t i = 0; i < P; ++i) {
-    const int ri = static_cast<int>(i / W), ci = static_cast<int>(i % W);
-    const int k = std::min(mt, m - dg[i]);
-    int taken = 0;
-    for (int pos = 0; pos < NW && taken < k; ++pos) {
-      const int c = rank[i * NW + pos];
+    int left = std::min(mt, m - static_cast<int>(dg[i]));
+    int* mine = nb + i * m;
+    const unsigned char* rk = st->head_host + i * kRankHead;
+    for (int pos = 0; pos < NW && left > 0; ++pos) {
+      if (pos == kRankHead) {  // beyond the ranks copied for every pixel (rare)
+        const int rc = fetch_strip(static_cast<int>(i / W));
+        if (rc) return rc;
+        rk = strip.data() + (i - static_cast<size_t>(strip_y) * W) * NW;
+      }
+      const int c = rk[pos];
       if (c == 255) break;  // the rest lie outside the image
-      const int j = (ri + c / side - r) * W + (ci + c % side - r);
+      const int j = static_cast<int>(i) + step[c];
       if (dg[j] >= m) continue;
       bool linked = false;
-      for (int b = 0; b < dg[i]; ++b) linked = linked || nb[i * m + b] == j;
+      for (int b = 0; b < dg[i]; ++b) linked = linked || mine[b] == j;
       if (linked) continue;
-      nb[i * m + dg[i]++] = j;
+      mine[dg[i]++] = j;
       nb[static_cast<size_t>(j) * m + dg[j]++] = static_cast<int>(i);
-      ++taken;
+      --left;
     }
   }
   st->deg_max = 0;
-  std::vector<int> nbt(P * m, -1);
-  std::vector<unsigned char> rev(P * m, 0), deg8(P);
-  for (size_t i = 0; i < P; ++i) {
-    std::sort(nb.begin() + i * m, nb.begin() + i * m + dg[i]);
-    st->deg_max = std::max(st->deg_max, dg[i]);
-    deg8[i] = static_cast<unsigned char>(dg[i]);
-    for (int b = 0; b < dg[i]; ++b) nbt[static_cast<size_t>(b) * P + i] = nb[i * m + b];
-  }
-  for (size_t i = 0; i < P; ++i)
-    for (int b = 0; b < dg[i]; ++b) {  // position of i in the list of its b-th neighbour
-      const int j = nb[i * m + b];
-      int pos = 0;
-      while (nb[static_cast<size_t>(j) * m + pos] != static_cast<int>(i)) ++pos;
-      rev[static_cast<size_t>(b) * P + i] = static_cast<unsigned char>(pos);
-    }
-  std::vector<short> offs(P * m, 0);
-  for (size_t e = 0; e < P * m; ++e)
-    if (nbt[e] >= 0) offs[e] = static_cast<short>(nbt[e] - static_cast<long long>(e % P));
-  NL_CK(cudaMemcpy(st->nbr, nbt.data(), sizeof(int) * P * m, cudaMemcpyHostToDevice));
-  NL_CK(cudaMemcpy(st->off, offs.data(), sizeof(short) * P * m, cudaMemcpyHostToDevice));
-  NL_CK(cudaMemcpy(st->rev, rev.data(), P * m, cudaMemcpyHostToDevice));
-  NL_CK(cudaMemcpy(st->deg, deg8.data(), P, cudaMemcpyHostToDevice));
+  for (size_t i = 0; i < P; ++i) st->deg_max = std::max(st->deg_max, static_cast<int>(dg[i]));
+  NL_CK(cudaMemcpyAsync(st->list, nb, sizeof(int) * P * m, cudaMemcpyHostToDevice, st->stream));
+  NL_CK(cudaMemcpyAsync(st->deg, dg, P, cudaMemcpyHostToDevice, st->stream));
+  const unsigned tgrid = static_cast<unsigned>((P + kThreads - 1) / kThreads);
+  k_nl_tables<<<tgrid, kThreads, 0, st->stream>>>(st->list, st->deg, m, P, st->nbr, st->off);
+  NL_CK(cudaGetLastError());
+  k_nl_reverse<<<tgrid, kThreads, 0, st->stream>>>(st->nbr, st->deg, m, P, st->rev);
+  NL_CK(cudaGetLastError());
   // Chebyshev iteration on [1, 1 + 4 deg_max]: theta = centre, delta = half width
   const double lo = 1.0, hi = 1.0 + 4.0 * st->deg_max;
   const double theta = 0.5 * (hi + lo), delta = 0.5 * (hi - lo);
@@ -707,25 +1001,25 @@ int build_graph(nl_state* st) {
 enum NlKind { kNlSolve = 0, kNlProx = 1, kNlRhs = 2, kNlKinds = 3 };
 const char* const kNlNames[kNlKinds] = {"nl_solve", "nl_prox", "nl_rhs"};
 
+// u pixel-major after the solve: the buffer its last step wrote.
+const float4* solved(const nl_state* st) { return st->cheb_grid > 0 ? st->xa : st->xb; }
+
+template <int KM, bool ONE>
+cudaError_t launch_prox_t(nl_state* st) {
+  const auto kern = st->m <= 10 ? k_nl_prox<KM, 10, ONE> : k_nl_prox<KM, kMaxM, ONE>;
+  return shf::fast::launch_pdl(kern, dim3(grid_for(st->P())), dim3(kThreads), 0, st->stream, solved(st), st->bv, st->d,
+                               st->w, st->bw, st->s, st->q, st->off, st->deg, st->K, st->Q, st->m, st->P(),
+                               st->gamma * st->lambda, st->gamma);
+}
+
 cudaError_t launch_prox(nl_state* st) {
-  const size_t P = st->P();
-  const float t = st->gamma * st->lambda;
-  const int grid = grid_for(P);
-  if (st->K <= 4)
-    return shf::fast::launch_pdl(k_nl_prox<4>, dim3(grid), dim3(kThreads), 0, st->stream, st->u, st->bv, st->d, st->w,
-                                 st->bw, st->s, st->q, st->nbr, st->deg, st->K, st->m, P, t, st->gamma);
-  else if (st->K <= 8)
-    return shf::fast::launch_pdl(k_nl_prox<8>, dim3(grid), dim3(kThreads), 0, st->stream, st->u, st->bv, st->d, st->w,
-                                 st->bw, st->s, st->q, st->nbr, st->deg, st->K, st->m, P, t, st->gamma);
-  else
-    return shf::fast::launch_pdl(k_nl_prox<16>, dim3(grid), dim3(kThreads), 0, st->stream, st->u, st->bv, st->d, st->w,
-                                 st->bw, st->s, st->q, st->nbr, st->deg, st->K, st->m, P, t, st->gamma);
+  if (st->K <= 4) return launch_prox_t<4, true>(st);
+  return st->K <= 8 ? launch_prox_t<8, false>(st) : launch_prox_t<16, false>(st);
 }
 
 cudaError_t launch_rhs(nl_state* st) {
-  return shf::fast::launch_pdl(k_nl_rhs, dim3(grid_for(st->P())), dim3(kThreads), 0, st->stream, st->q, st->d,
-                               reinterpret_cast<float*>(st->rhs), st->nbr, st->rev, st->deg, st->K, st->Q, st->m,
-                               st->P());
+  return shf::fast::launch_pdl(st->m <= 10 ? k_nl_rhs<10> : k_nl_rhs<kMaxM>, dim3(grid_for(st->P())), dim3(kThreads), 0,
+                               st->stream, st->q, st->d, st->rhs, st->off, st->rev, st->deg, st->Q, st->m, st->P());
 }
 
 // One iteration; ev (nullable, kNlKinds + 1 events) recorded before each
@@ -764,12 +1058,11 @@ cudaError_t enqueue_nl_iteration(nl_state* st, cudaEvent_t* ev) {
     const float* none = nullptr;
     float* none_out = nullptr;
     const float4* none4 = nullptr;
-    float4* none4_out = nullptr;
     if (k == 0)  // from u (label-major)
       e = shf::fast::launch_pdl(k_nl_cheb<true, false>, grid, block, 0, ss, st->u, none4, none_out, x0, st->cd,
                                 st->rhs, st->off, st->deg, st->K, st->Q, st->m, P, a, c);
     else if (k == n - 1)  // back into u
-      e = shf::fast::launch_pdl(k_nl_cheb<false, true>, grid, block, 0, ss, none, x0, st->u, none4_out, st->cd,
+      e = shf::fast::launch_pdl(k_nl_cheb<false, true>, grid, block, 0, ss, none, x0, st->u, x1, st->cd,
                                 st->rhs, st->off, st->deg, st->K, st->Q, st->m, P, a, c);
     else {
       e = shf::fast::launch_pdl(k_nl_cheb<false, false>, grid, block, 0, ss, none, x0, none_out, x1, st->cd,
@@ -786,8 +1079,8 @@ cudaError_t enqueue_nl_iteration(nl_state* st, cudaEvent_t* ev) {
 }
 
 cudaError_t rebuild_rhs(nl_state* st) {
-  const size_t n = st->P() * st->K;
-  k_nl_q<<<grid_for(n), kThreads, 0, st->stream>>>(st->w, st->bw, st->s, st->q, st->gamma, n);
+  k_nl_q<<<grid_for(st->P() * 4 * st->Q), kThreads, 0, st->stream>>>(st->w, st->bw, st->s, reinterpret_cast<float*>(st->q),
+                                                                     st->gamma, st->K, st->Q, st->P());
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? launch_rhs(st) : e;
 }
@@ -812,8 +1105,8 @@ int nl_restart(nl_state* st) {
   NL_CK(cudaMemsetAsync(st->u, 0, sizeof(float) * P * K, st->stream));
   NL_CK(cudaMemsetAsync(st->w, 0, sizeof(float) * P * K, st->stream));
   NL_CK(cudaMemsetAsync(st->bw, 0, sizeof(float) * P * K, st->stream));
-  NL_CK(cudaMemsetAsync(st->bv, 0, sizeof(float) * m * P * K, st->stream));
-  NL_CK(cudaMemsetAsync(st->d, 0, sizeof(float) * m * P * K, st->stream));
+  NL_CK(cudaMemsetAsync(st->bv, 0, sizeof(float4) * m * P * st->Q, st->stream));
+  NL_CK(cudaMemsetAsync(st->d, 0, sizeof(float4) * m * P * st->Q, st->stream));
   NL_CK(cudaMemsetAsync(st->cd, 0, sizeof(float4) * P * st->Q, st->stream));
   NL_CK(rebuild_rhs(st));
   NL_CK(cudaStreamSynchronize(st->stream));
@@ -881,12 +1174,15 @@ int nl_admm_init(int H, int W, const float* f, int C, const float* codebook, int
   if ((rc = nl_alloc(&st->f, P * C, "f")) || (rc = nl_alloc(&st->s, P * K, "s")) ||
       (rc = nl_alloc(&st->u, P * K, "u")) || (rc = nl_alloc(&st->xa, P * st->Q, "chebyshev x")) ||
       (rc = nl_alloc(&st->xb, P * st->Q, "chebyshev x")) || (rc = nl_alloc(&st->cd, P * st->Q, "chebyshev d")) ||
-      (rc = nl_alloc(&st->bv, m * P * K, "b_v")) ||
-      (rc = nl_alloc(&st->d, m * P * K, "d")) || (rc = nl_alloc(&st->w, P * K, "w")) ||
-      (rc = nl_alloc(&st->bw, P * K, "b_w")) || (rc = nl_alloc(&st->q, P * K, "q")) ||
+      (rc = nl_alloc(&st->bv, m * P * st->Q, "b_v")) ||
+      (rc = nl_alloc(&st->d, m * P * st->Q, "d")) || (rc = nl_alloc(&st->w, P * K, "w")) ||
+      (rc = nl_alloc(&st->bw, P * K, "b_w")) || (rc = nl_alloc(&st->q, P * st->Q, "q")) ||
       (rc = nl_alloc(&st->rhs, P * st->Q, "rhs")) || (rc = nl_alloc(&st->gap, P, "gap")) ||
       (rc = nl_alloc(&st->nbr, P * m, "neighbours")) || (rc = nl_alloc(&st->off, P * m, "offsets")) ||
-      (rc = nl_alloc(&st->rev, P * m, "reverse")) ||
+      (rc = nl_alloc(&st->rev, P * m, "reverse")) || (rc = nl_alloc(&st->gw, kMaxPatch * kMaxPatch, "weights")) ||
+      (rc = nl_alloc(&st->head, P * kRankHead, "ranks")) || (rc = nl_alloc(&st->list, P * m, "links")) ||
+      (rc = nl_alloc_host(&st->nbr_host, P * m, "links")) || (rc = nl_alloc_host(&st->deg_host, P, "counts")) ||
+      (rc = nl_alloc_host(&st->head_host, P * kRankHead, "ranks")) ||
       (rc = nl_alloc(&st->deg, P, "counts")) || (rc = nl_alloc(&st->labels, P, "labels")) ||
       (rc = nl_alloc(&st->flag, 1, "flag")) || (rc = nl_alloc(&st->red, 2 * kRedBlocks + 2, "red")) ||
       (rc = nl_alloc(&st->cbar, 1, "barrier")) || (rc = nl_alloc(&st->cerr, 1, "barrier flag"))) {
@@ -921,8 +1217,16 @@ int nl_admm_reset(nl_state* st, const float* f, int f_on_host) {
 
 int nl_admm_graph(const nl_state* st, int* nbr, int* deg, int* solve_steps) {
   if (!st) return nl_fail(SHF_ERR_ARG, "nl_admm_graph: NULL state");
-  if (nbr) std::copy(st->nbr_host.begin(), st->nbr_host.end(), nbr);
-  if (deg) std::copy(st->deg_host.begin(), st->deg_host.end(), deg);
+  if (nbr) {  // the selection's links, sorted, -1 padded
+    const size_t P = st->P(), m = st->m;
+    for (size_t i = 0; i < P; ++i) {
+      int* o = nbr + i * m;
+      std::copy(st->nbr_host + i * m, st->nbr_host + i * m + st->deg_host[i], o);
+      std::sort(o, o + st->deg_host[i]);
+      std::fill(o + st->deg_host[i], o + m, -1);
+    }
+  }
+  if (deg) std::copy(st->deg_host, st->deg_host + st->P(), deg);
   if (solve_steps) *solve_steps = static_cast<int>(st->cheb_a.size());
   return SHF_OK;
 }
@@ -986,12 +1290,13 @@ int nl_admm_get(nl_state* st, int what, void* dst, int on_host) {
     case SEG_W: return nl_copy(st, dst, st->w, sizeof(float) * P * K, kind, on_host);
     case SEG_BW: return nl_copy(st, dst, st->bw, sizeof(float) * P * K, kind, on_host);
     case SEG_S: return nl_copy(st, dst, st->s, sizeof(float) * P * K, kind, on_host);
-    case SEG_BV: return nl_copy(st, dst, st->bv, sizeof(float) * m * P * K, kind, on_host);
-    case SEG_V: {  // v = d + b_v
+    case SEG_BV:
+    case SEG_V: {  // b_v, or v = d + b_v, label-major
       const size_t n = m * P * K;
       float* tgt = static_cast<float*>(dst);
       if (on_host) NL_CK(cudaMallocAsync(reinterpret_cast<void**>(&tgt), sizeof(float) * n, st->stream));
-      k_nl_axpb<<<grid_for(n), kThreads, 0, st->stream>>>(st->d, st->bv, tgt, 1.f, n);
+      k_nl_unpack<<<grid_for(m * P * st->Q), kThreads, 0, st->stream>>>(
+          what == SEG_V ? st->d : st->bv, what == SEG_V ? st->bv : nullptr, tgt, 1.f, st->K, st->Q, m * P);
       cudaError_t e = cudaGetLastError();
       if (on_host) {
         if (e == cudaSuccess) e = cudaMemcpyAsync(dst, tgt, sizeof(float) * n, cudaMemcpyDeviceToHost, st->stream);
@@ -1043,13 +1348,26 @@ int nl_admm_set(nl_state* st, int what, const void* src, int on_host) {
     case SEG_W: rc = nl_copy(st, st->w, src, sizeof(float) * P * K, kind, false); break;
     case SEG_BW: rc = nl_copy(st, st->bw, src, sizeof(float) * P * K, kind, false); break;
     case SEG_U: rc = nl_copy(st, st->u, src, sizeof(float) * P * K, kind, false); break;
-    case SEG_BV: rc = nl_copy(st, st->bv, src, sizeof(float) * m * P * K, kind, false); break;
-    case SEG_V: {
-      rc = nl_copy(st, st->d, src, sizeof(float) * m * P * K, kind, false);
-      if (rc == SHF_OK) {
-        k_nl_axpb<<<grid_for(m * P * K), kThreads, 0, st->stream>>>(st->d, st->bv, st->d, -1.f, m * P * K);
-        NL_CK(cudaGetLastError());
+    case SEG_BV:
+    case SEG_V: {  // b_v, or d = v - b_v with the current b_v
+      const size_t n = m * P * K;
+      const float* from = static_cast<const float*>(src);
+      float* tmp = nullptr;
+      if (on_host) {
+        NL_CK(cudaMallocAsync(reinterpret_cast<void**>(&tmp), sizeof(float) * n, st->stream));
+        from = tmp;
       }
+      cudaError_t e = on_host ? cudaMemcpyAsync(tmp, src, sizeof(float) * n, cudaMemcpyHostToDevice, st->stream) : cudaSuccess;
+      if (e == cudaSuccess) {
+        k_nl_pack<<<grid_for(m * P * st->Q), kThreads, 0, st->stream>>>(
+            from, what == SEG_V ? st->bv : nullptr, what == SEG_V ? st->d : st->bv, -1.f, st->K, st->Q, m * P);
+        e = cudaGetLastError();
+      }
+      if (tmp) {
+        const cudaError_t e2 = cudaFreeAsync(tmp, st->stream);
+        if (e == cudaSuccess) e = e2;
+      }
+      NL_CK(e);
       break;
     }
     default: return nl_fail(SHF_ERR_ARG, "nl_admm_set: accepts SEG_W, SEG_BW, SEG_U, SEG_BV and SEG_V");
