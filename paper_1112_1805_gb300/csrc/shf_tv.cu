@@ -326,6 +326,7 @@ cudaError_t rebuild_rhs(tv_state* st) {
 // Data term and the zero state v = b_v = w = b_w = 0.
 int tv_restart(tv_state* st) {
   const size_t P = st->P(), K = st->K;
+  TV_CK(cudaMemsetAsync(st->flag, 0, sizeof(int), st->stream));
   TV_CK(shf::launch_count_nonfinite(st->f, static_cast<long>(P * st->C), st->flag, st->stream));
   int bad = 0;
   TV_CK(cudaMemcpyAsync(&bad, st->flag, sizeof(int), cudaMemcpyDeviceToHost, st->stream));
