@@ -74,6 +74,12 @@ struct shf_bank {
   // mapping it again (a 64 x 64 analysis: 256 us against 30 us in a row).
   cudaMemPool_t pool = nullptr;
   static constexpr unsigned long long kPoolKeep = 512ull << 20;
+  // Heights with register-FFT column kernels: the work list of one channel's
+  // filters, used by the transforms for every channel (its device arrays in
+  // `chan_mem`).
+  bool chan_ok = false;
+  shf::FastPlan chan;
+  int* chan_mem = nullptr;
 };
 
 struct seg_state {
@@ -170,6 +176,40 @@ void make_pool(shf_bank* b) {
   cudaGetLastError();
 }
 
+// The single-channel work list of a bank whose ranges are known; synchronous.
+int build_channel_plan(shf_bank* b, const std::vector<int2>& ranges) {
+  const Geo& g = b->g;
+  shf::FastPlan& p = b->chan;
+  p.col_ctas = shf::fast_col_ctas(g, 0);
+  p.fan_ctas = shf::fast_fan_ctas(g);
+  if (p.col_ctas < 1 || p.fan_ctas < 1) return fail(SHF_ERR_CUDA, "shfilters_build: no resident CTA");
+  std::vector<shf::WorkItem> items;
+  std::vector<int> cta_begin, tile_begin, tile_slots;
+  shf::build_fast_plan(g, ranges.data(), 1, &p, &items, &cta_begin, &tile_begin, &tile_slots);
+  // one upload: the items (four ints each), then the ranges and slot lists
+  std::vector<int> all(4 * items.size());
+  std::memcpy(all.data(), items.data(), sizeof(shf::WorkItem) * items.size());
+  const size_t at0 = all.size(), at1 = at0 + cta_begin.size(), at2 = at1 + tile_begin.size();
+  for (const std::vector<int>* v : {&cta_begin, &tile_begin, &tile_slots}) all.insert(all.end(), v->begin(), v->end());
+  int rc = dev_alloc(&b->chan_mem, all.size(), "work list");
+  if (rc) return rc;
+  SHF_CK(cudaMemcpy(b->chan_mem, all.data(), sizeof(int) * all.size(), cudaMemcpyHostToDevice));
+  p.items = reinterpret_cast<const shf::WorkItem*>(b->chan_mem);
+  p.cta_begin = b->chan_mem + at0;
+  p.tile_begin = b->chan_mem + at1;
+  p.tile_slots = b->chan_mem + at2;
+  b->chan_ok = true;
+  return SHF_OK;
+}
+
+// Channels of a launch over the single-channel plan: as many as keep the wave's
+// spectra within the plan's budget.
+int channels_per_launch(const shf_bank* b, int nch) {
+  const size_t plane = sizeof(float2) * static_cast<size_t>(b->g.H) * b->g.Wy;
+  const size_t per = plane * static_cast<size_t>(b->chan.y_planes);
+  return static_cast<int>(std::max<size_t>(1, std::min<size_t>(nch, (static_cast<size_t>(b->chan.wave_mib) << 20) / per)));
+}
+
 }  // namespace
 
 extern "C" {
@@ -188,8 +228,8 @@ int shfilters_build(int H, int W, int J, void* stream, shf_bank** out) {
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   int device = 0, optin = 0;
   SHF_CK(cudaGetDevice(&device));
-  SHF_CK(shf::prepare_kernels());
-  SHF_CK(shf::prepare_fast_kernels());
+  SHF_CK(shf::prepare_kernels(g));
+  SHF_CK(shf::prepare_fast_kernels(g));
   SHF_CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device));
   if (shf::max_dynamic_smem_needed(g, shf::kMaxK) > optin)
     return fail(SHF_ERR_SIZE, "tile does not fit in shared memory");
@@ -216,10 +256,18 @@ int shfilters_build(int H, int W, int J, void* stream, shf_bank** out) {
   if (e == cudaSuccess) e = shf::launch_pass_tables(&b->g, b->pt, st);
   if (e == cudaSuccess) e = shf::launch_build_bank(b->bank, b->g, b->descs, st);
   if (e == cudaSuccess) e = shf::launch_filter_ranges(b->bank, b->g, b->ranges, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // d is a host temporary
+  std::vector<int2> ranges(g.eta);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(ranges.data(), b->ranges, sizeof(int2) * g.eta, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // d and ranges are host temporaries
   if (e != cudaSuccess) {
     shfilters_destroy(b);
     return fail(SHF_ERR_CUDA, std::string("shfilters_build: ") + cudaGetErrorString(e));
+  }
+  if (shf::fast_columns_ok(b->g) && (rc = build_channel_plan(b, ranges))) {
+    const std::string m = g_err;
+    shfilters_destroy(b);
+    return fail(rc, m);
   }
   *out = b;
   return SHF_OK;
@@ -232,6 +280,7 @@ int shfilters_destroy(shf_bank* b) {
   cudaFree(b->twH);
   cudaFree(b->twW);
   cudaFree(b->pt);
+  cudaFree(b->chan_mem);
   if (b->pool) cudaMemPoolDestroy(b->pool);
   cudaFree(b->descs);
   cudaFree(b->ranges);
@@ -261,6 +310,28 @@ int shearlet_analyze(const shf_bank* b, const float* u, int nch, float* coef, vo
   const Geo& g = b->g;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const size_t ph = static_cast<size_t>(g.H) * g.Wh;
+  const float scale = 1.f / (static_cast<float>(g.H) * g.W);
+  if (b->chan_ok) {
+    const size_t php = static_cast<size_t>(g.H) * g.Wy;
+    const int nc = channels_per_launch(b, nch);
+    const size_t ny = php * b->chan.y_planes * static_cast<size_t>(nc);
+    float2* tmp = nullptr;
+    cudaError_t e = scratch_alloc(b, &tmp, ny + (php + ph) * static_cast<size_t>(nch), st);
+    if (e != cudaSuccess) return fail(SHF_ERR_OOM, std::string("shearlet_analyze: ") + cudaGetErrorString(e));
+    float2 *Y = tmp, *uhat = tmp + ny, *Ur = uhat + php * nch;
+    e = shf::run_row_r2c(g, u, Ur, nch, 1.f, st);
+    if (e == cudaSuccess) e = shf::run_channel_fwd(g, Ur, uhat, nch, st);
+    for (int w = 0; w < static_cast<int>(b->chan.wave_f0.size()); ++w)
+      for (int c = 0; c < nch && e == cudaSuccess; c += nc) {
+        const shf::FilterWave wv{c, std::min(nc, nch - c), b->chan.wave_f0[w], b->chan.wave_nf[w]};
+        e = shf::run_channel_fan(g, b->chan, w, uhat, Y, wv, st);
+        if (e == cudaSuccess) e = shf::run_wave_c2r(g, Y, coef, wv, scale, st);
+      }
+    cudaError_t e2 = cudaFreeAsync(tmp, st);
+    if (e != cudaSuccess || e2 != cudaSuccess)
+      return fail(SHF_ERR_CUDA, std::string("shearlet_analyze: ") + cudaGetErrorString(e != cudaSuccess ? e : e2));
+    return SHF_OK;
+  }
   const std::vector<shf::FilterWave> waves = shf::general_waves(g, nch, shf::default_groups(g, nch));
   float2* tmp = nullptr;
   cudaError_t e = scratch_alloc(b, &tmp, ph * nch + shf::wave_planes(waves) * g.H * g.Wy, st);
@@ -271,7 +342,7 @@ int shearlet_analyze(const shf_bank* b, const float* u, int nch, float* coef, vo
   if (e == cudaSuccess) e = shf::run_col_fwd(g, Ur, nch, st);
   for (const shf::FilterWave& wv : waves) {
     if (e == cudaSuccess) e = shf::run_wave_fan(g, Ur, Y, wv, st);
-    if (e == cudaSuccess) e = shf::run_wave_c2r(g, Y, coef, wv, 1.f / (static_cast<float>(g.H) * g.W), st);
+    if (e == cudaSuccess) e = shf::run_wave_c2r(g, Y, coef, wv, scale, st);
   }
   cudaError_t e2 = cudaFreeAsync(tmp, st);
   if (e != cudaSuccess || e2 != cudaSuccess)
@@ -283,6 +354,25 @@ namespace {
 // T[nch][H][Wh] = column-inverse of sum_f W_f * fft2(coef_f) (unscaled).
 cudaError_t synthesis_spectrum(const shf_bank* b, const Geo& g, const float* coef, int nch, float2* T,
                                cudaStream_t st) {
+  if (b->chan_ok) {
+    const size_t php = static_cast<size_t>(g.H) * g.Wy;
+    const int nc = channels_per_launch(b, nch);
+    const size_t ny = php * b->chan.y_planes * static_cast<size_t>(nc);
+    const size_t np = static_cast<size_t>(std::max(b->chan.nslots, 1)) * g.H * shf::fast_tile(g);
+    float2* tmp = nullptr;
+    cudaError_t e = scratch_alloc(b, &tmp, ny + np * static_cast<size_t>(nch), st);
+    if (e != cudaSuccess) return e;
+    float2 *Z = tmp, *part = tmp + ny;
+    for (int w = 0; w < static_cast<int>(b->chan.wave_f0.size()); ++w)
+      for (int c = 0; c < nch && e == cudaSuccess; c += nc) {
+        const shf::FilterWave wv{c, std::min(nc, nch - c), b->chan.wave_f0[w], b->chan.wave_nf[w]};
+        e = shf::run_wave_r2c(g, coef, Z, wv, st);
+        if (e == cudaSuccess) e = shf::run_channel_gather(g, b->chan, w, Z, part, wv, st);
+      }
+    if (e == cudaSuccess) e = shf::run_channel_reduce(g, b->chan, part, T, nch, st);
+    cudaError_t e2 = cudaFreeAsync(tmp, st);
+    return e != cudaSuccess ? e : e2;
+  }
   const size_t ph = static_cast<size_t>(g.H) * g.Wh;
   const int groups = shf::default_groups(g, nch);
   const std::vector<shf::FilterWave> waves = shf::general_waves(g, nch, groups);

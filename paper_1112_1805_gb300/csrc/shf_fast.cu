@@ -31,7 +31,7 @@ bool fast_path_ok(const Geo& g) { return reg::supported_col(g.H) && reg::support
 int fast_tile(const Geo& g) { return reg::col_batch(g.H); }
 
 bool fast_ustep_ok(const Geo& g, int K) {
-  if (!fast_path_ok(g) || K > 8) return false;
+  if (!reg::supported(g.L) || K > 8) return false;  // the row transforms only: any height
   int dev = 0, optin = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return false;
   if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) return false;
@@ -39,9 +39,9 @@ bool fast_ustep_ok(const Geo& g, int K) {
   return need > 0 && need <= static_cast<size_t>(optin);
 }
 
-cudaError_t prepare_fast_kernels() {
-  cudaError_t e = fast::prepare_col_kernels();
-  if (e == cudaSuccess) e = fast::prepare_row_kernels();
+cudaError_t prepare_fast_kernels(const Geo& g) {
+  cudaError_t e = fast::prepare_col_kernels(g.H);
+  if (e == cudaSuccess) e = fast::prepare_row_kernels(g.L);
   return e;
 }
 
@@ -104,6 +104,8 @@ int fast_row_ctas(const Geo& g, int row_kernel, int sms) {
 }
 
 int fast_fan_ctas(const Geo& g, int col_kernel, int sms) { return fast::fan_ctas_per_sm(g.H, col_kernel) * sms_for(sms); }
+
+bool fast_shrink_ok(const Geo& g) { return g.ranges && reg::supported(g.L); }
 
 bool fast_row_kernel_ok(const Geo& g, int row_kernel) { return fast::row_kernel_ok(g.L, row_kernel); }
 
@@ -226,6 +228,35 @@ cudaError_t run_fast_iteration_body(const Geo& g, const FastPlan& plan, const fl
   hook.mark(kKindReduce);
   if (e == cudaSuccess) e = fast::col_reduce(g, partial, plan.tile_begin, plan.tile_slots, T, K, st);
   return e;
+}
+
+bool fast_columns_ok(const Geo& g) { return reg::supported_col(g.H); }
+
+cudaError_t run_channel_fwd(const Geo& g, const float2* Ur, float2* uhat, int nch, cudaStream_t st) {
+  return fast::col_fwd(g, Ur, uhat, nch, fast_pitch(g), st);
+}
+
+cudaError_t run_channel_fan(const Geo& g, const FastPlan& plan, int w, const float2* uhat, float2* Y,
+                            const FilterWave& wv, cudaStream_t st) {
+  const int c0 = plan.wave_fcta0[w], nc = plan.wave_fcta0[w + 1] - c0;
+  if (nc < 1) return cudaSuccess;
+  return fast::col_fan(g, nc, uhat + static_cast<size_t>(g.H) * fast_pitch(g) * wv.c0, plan.items,
+                       plan.cta_begin + c0 + w, Y, fast_pitch(g), fast::Wave{0, wv.f0, wv.nf, wv.nf}, plan.col_kernel, st,
+                       wv.nc);
+}
+
+cudaError_t run_channel_gather(const Geo& g, const FastPlan& plan, int w, const float2* Y, float2* partial,
+                               const FilterWave& wv, cudaStream_t st) {
+  const int c0 = plan.wave_cta0[w], nc = plan.wave_cta0[w + 1] - c0;
+  if (nc < 1) return cudaSuccess;
+  return fast::col_gather(g, nc, Y, plan.items, plan.cta_begin + c0 + w,
+                          partial + static_cast<size_t>(plan.nslots) * g.H * fast_tile(g) * wv.c0, fast_pitch(g),
+                          fast::Wave{0, wv.f0, wv.nf, wv.nf}, plan.col_kernel, st, wv.nc, plan.nslots);
+}
+
+cudaError_t run_channel_reduce(const Geo& g, const FastPlan& plan, const float2* partial, float2* T, int nch,
+                               cudaStream_t st) {
+  return fast::col_reduce(g, partial, plan.tile_begin, plan.tile_slots, T, nch, st, std::max(plan.nslots, 1));
 }
 
 cudaError_t run_fast_adjoint_body(const Geo& g, const FastPlan& plan, const float2* Qr, float2* uhat, float2* Y,

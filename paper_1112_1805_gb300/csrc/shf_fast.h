@@ -96,7 +96,7 @@ struct Wave {
 // thread, or 16 (radix-16 passes; heights 512, 1024, 2048); 0 is the default
 // for the height.
 bool col_kernel_ok(int H, int variant);
-cudaError_t prepare_col_kernels();
+cudaError_t prepare_col_kernels(int H);  // shared-memory limits (any other height: nothing to set)
 int col_ctas_per_sm(int H, int variant = 0);  // resident CTAs per SM of the gather kernel
 int fan_ctas_per_sm(int H, int variant = 0);  // resident CTAs per SM of the fan kernel
 // Ur [K][H][Wh] -> uhat [K][H][Whp]: column-forward of the row spectra of u.
@@ -104,16 +104,32 @@ cudaError_t col_fwd(const Geo& g, const float2* Ur, float2* uhat, int K, int Whp
 // Y_v = column-inverse(W_f * uhat_label) on the (label, tile, filter) items of
 // CTA ranges cta_begin[0..nc] of wave wv.
 cudaError_t col_fan(const Geo& g, int nc, const float2* uhat, const WorkItem* items, const int* cta_begin,
-                    float2* Y, int Whp, const Wave& wv, int variant, cudaStream_t st);
+                    float2* Y, int Whp, const Wave& wv, int variant, cudaStream_t st, int chans = 1);
 // partial[slot] = sum over runs of items of W_f * column-forward(Y_v).
 cudaError_t col_gather(const Geo& g, int nc, const float2* Y, const WorkItem* items, const int* cta_begin,
-                       float2* partial, int Whp, const Wave& wv, int variant, cudaStream_t st);
+                       float2* partial, int Whp, const Wave& wv, int variant, cudaStream_t st, int chans = 1,
+                       int cslots = 0);
 // T [K][H][Wh] = column-inverse of the per-(label, tile) sums of the partial slots.
 cudaError_t col_reduce(const Geo& g, const float2* partial, const int* tile_begin, const int* tile_slots, float2* T,
-                       int K, cudaStream_t st);
+                       int K, cudaStream_t st, int cslots = 0);
+
+// `chans` > 1 (fan, gather): the same items for that many channels, whose uhat
+// and Y follow one another; `cslots`: a channel's slots in `partial` (gather,
+// and reduce over K channels of a single-channel plan).
+
+// Single row transforms (shf_fast_half.cu) for the half widths half_rows_ok(L):
+// planes of wave wv at row pitch `pitch`, real planes channel eta + f; with
+// `ranges` only the filters' columns are read (rows_inv) or their column tiles
+// written (rows_fwd).
+bool half_rows_ok(int L);
+cudaError_t prepare_half_kernels(int L);
+cudaError_t rows_inv(const Geo& g, const float2* X, int pitch, float* out, const int2* ranges, int eta, const Wave& wv,
+                     float scale, cudaStream_t st);
+cudaError_t rows_fwd(const Geo& g, const float* in, float2* X, int pitch, const int2* ranges, int eta, const Wave& wv,
+                     cudaStream_t st);
 
 // Row kernels (shf_fast_row.cu).
-cudaError_t prepare_row_kernels();
+cudaError_t prepare_row_kernels(int L);
 // Resident CTAs per SM and rows in flight per CTA of the v-step kernel
 // (mode 0) or of its adjoint (mode 1).
 // `variant` (RowKernel, shf_internal.h) selects the forward v-step: 8 values

@@ -105,6 +105,8 @@ __global__ void __launch_bounds__(ColGeo<H>::NT, col_min_blocks(H, ColGeo<H>::NT
   constexpr int KB = ColGeo<H>::KB;
   const int b = threadIdx.x % KB, tt = threadIdx.x / KB;
   const size_t Pb = static_cast<size_t>(H) * Wh, Pp = static_cast<size_t>(H) * Whp;
+  uhat += Pp * blockIdx.y;  // the launch's channels
+  Y += Pp * nf * blockIdx.y;
   WorkItem it = items[ib];
   int col = it.tile * KB + b;
   bool ok = col < Wh;
@@ -172,6 +174,8 @@ __global__ void __launch_bounds__(Col16Geo<H>::NT, H == 512 ? 2 : 1)
   if (ib >= ie) return;
   const int b = threadIdx.x % KB, tt = threadIdx.x / KB;
   const size_t Pb = static_cast<size_t>(H) * Wh, Pp = static_cast<size_t>(H) * Whp;
+  uhat += Pp * blockIdx.y;  // the launch's channels
+  Y += Pp * nf * blockIdx.y;
   WorkItem it = items[ib];
   int col = it.tile * KB + b;
   bool ok = col < Wh;
@@ -226,7 +230,7 @@ template <int H>
 __global__ void __launch_bounds__(ColGeo<H>::NT, gather_min_blocks(H, ColGeo<H>::NT))
     k_fcol_gather(const float2* __restrict__ Y, const float* __restrict__ bank, const WorkItem* __restrict__ items,
                   const int* __restrict__ cta_begin, float2* __restrict__ partial, int Wh, int Whp, int l0, int f0,
-                  int nf, const float2* __restrict__ twH) {
+                  int nf, const float2* __restrict__ twH, int cslots) {
   extern __shared__ float2 sm[];
   float2* tw = sm;  // per-pass twiddles
   float2* b0 = sm + reg::Passes<H>::TWSIZE;
@@ -236,6 +240,8 @@ __global__ void __launch_bounds__(ColGeo<H>::NT, gather_min_blocks(H, ColGeo<H>:
   constexpr int KB = ColGeo<H>::KB;
   const int b = threadIdx.x % KB, tt = threadIdx.x / KB;
   const size_t Pb = static_cast<size_t>(H) * Wh, Pp = static_cast<size_t>(H) * Whp;
+  Y += Pp * nf * blockIdx.y;  // the launch's channels
+  partial += static_cast<size_t>(cslots) * H * KB * blockIdx.y;
   WorkItem it = items[ib];
   int col = it.tile * KB + b;
   bool ok = col < Wh;
@@ -292,7 +298,7 @@ __global__ void __launch_bounds__(Col16Geo<H>::NT, H == 512 ? 2 : 1)
     k_fcol_gather16(const float2* __restrict__ Y, const float* __restrict__ bank,
                     const WorkItem* __restrict__ items, const int* __restrict__ cta_begin,
                     float2* __restrict__ partial, int Wh, int Whp, int l0, int f0, int nf,
-                    const float2* __restrict__ twH) {
+                    const float2* __restrict__ twH, int cslots) {
   using G = Col16Geo<H>;
   constexpr int KB = G::KB, T = G::T;
   extern __shared__ __align__(16) float2 sm[];
@@ -303,6 +309,8 @@ __global__ void __launch_bounds__(Col16Geo<H>::NT, H == 512 ? 2 : 1)
   if (ib >= ie) return;
   const int b = threadIdx.x % KB, tt = threadIdx.x / KB;
   const size_t Pb = static_cast<size_t>(H) * Wh, Pp = static_cast<size_t>(H) * Whp;
+  Y += Pp * nf * blockIdx.y;  // the launch's channels
+  partial += static_cast<size_t>(cslots) * H * KB * blockIdx.y;
   WorkItem it = items[ib];
   int col = it.tile * KB + b;
   bool ok = col < Wh;
@@ -391,6 +399,8 @@ __global__ void __launch_bounds__(ColVGeo<H>::NT, ColVGeo<H>::MINB)
   if (ib >= ie) return;
   const int b = threadIdx.x % KB, tt = threadIdx.x / KB;
   const size_t Pb = static_cast<size_t>(H) * Wh, Pp = static_cast<size_t>(H) * Whp;
+  uhat += Pp * blockIdx.y;  // the launch's channels
+  Y += Pp * nf * blockIdx.y;
   WorkItem it = items[ib];
   int col = it.tile * KB + b;
   bool ok = col < Wh;
@@ -441,7 +451,7 @@ template <int H>
 __global__ void __launch_bounds__(ColVGeo<H>::NT, ColVGeo<H>::MINB)
     k_fcol_gatherv(const float2* __restrict__ Y, const float* __restrict__ bank, const WorkItem* __restrict__ items,
                    const int* __restrict__ cta_begin, float2* __restrict__ partial, int Wh, int Whp, int l0, int f0,
-                   int nf, const float2* __restrict__ twH) {
+                   int nf, const float2* __restrict__ twH, int cslots) {
   using G = ColVGeo<H>;
   constexpr int KB = G::KB, T = G::T, V = G::V;
   constexpr bool PREFETCH = V <= 12;
@@ -453,6 +463,8 @@ __global__ void __launch_bounds__(ColVGeo<H>::NT, ColVGeo<H>::MINB)
   if (ib >= ie) return;
   const int b = threadIdx.x % KB, tt = threadIdx.x / KB;
   const size_t Pb = static_cast<size_t>(H) * Wh, Pp = static_cast<size_t>(H) * Whp;
+  Y += Pp * nf * blockIdx.y;  // the launch's channels
+  partial += static_cast<size_t>(cslots) * H * KB * blockIdx.y;
   WorkItem it = items[ib];
   int col = it.tile * KB + b;
   bool ok = col < Wh;
@@ -537,7 +549,7 @@ struct ReduceGeo {
 template <int H>
 __global__ void __launch_bounds__(ReduceGeo<H>::RG * ColGeo<H>::NT) k_fcol_reduce_inv(
     const float2* __restrict__ partial, const int* __restrict__ tile_begin, const int* __restrict__ tile_slots,
-    float2* __restrict__ T, int Wh, const float2* __restrict__ twH) {
+    float2* __restrict__ T, int Wh, const float2* __restrict__ twH, int cslots) {
   using RGeo = ReduceGeo<H>;
   constexpr int KB = ColGeo<H>::KB;
   constexpr int NT = ColGeo<H>::NT;
@@ -557,7 +569,10 @@ __global__ void __launch_bounds__(ReduceGeo<H>::RG * ColGeo<H>::NT) k_fcol_reduc
   load_pass_table<H, 1>(tw, twH);
   pdl_wait();
   pdl_trigger();
-  const int lt0 = label * gridDim.x + tile;  // the (label, tile) slot list
+  // the (label, tile) slot list; with cslots > 0 every label (channel) has the
+  // one list of a single-channel plan over slots of its own
+  const int lt0 = cslots > 0 ? tile : label * gridDim.x + tile;
+  partial += static_cast<size_t>(cslots) * label * H * KB;
   const int s0 = tile_begin[lt0], s1 = tile_begin[lt0 + 1], ns = s1 - s0;
   const int a0 = s0 + ns * grp / RGeo::RG, a1 = s0 + ns * (grp + 1) / RGeo::RG;
   for (int si = a0; si < a1; ++si) {
@@ -624,13 +639,15 @@ cudaError_t prepare_col_t() {
 
 }  // namespace
 
-cudaError_t prepare_col_kernels() {
-#define SHF_PREP(N) \
-  if (e == cudaSuccess) e = prepare_col_t<N>();
-  cudaError_t e = cudaSuccess;
-  SHF_COL_SIZES(SHF_PREP)
-#undef SHF_PREP
-  return e;
+cudaError_t prepare_col_kernels(int N) {
+  switch (N) {
+#define SHF_CASE(M) \
+  case M:           \
+    return prepare_col_t<M>();
+    SHF_COL_SIZES(SHF_CASE)
+#undef SHF_CASE
+    default: return cudaSuccess;
+  }
 }
 
 // The column transform a plan's variant selects at height H: radix-16 (16
@@ -701,17 +718,17 @@ cudaError_t col_fwd(const Geo& g, const float2* Ur, float2* uhat, int K, int Whp
 }
 
 cudaError_t col_fan(const Geo& g, int nc, const float2* uhat, const WorkItem* items, const int* cta_begin,
-                    float2* Y, int Whp, const Wave& wv, int variant, cudaStream_t st) {
+                    float2* Y, int Whp, const Wave& wv, int variant, cudaStream_t st, int chans) {
   switch (g.H) {
 #define SHF_CASE(N)                                                                                              \
   case N:                                                                                                        \
     if (use16(N, variant))                                                                                       \
-      return launch_pdl(k_fcol_fan16<fan16_len(N)>, dim3(nc), dim3(Col16Geo<fan16_len(N)>::NT), fan16_smem<N>(),  \
+      return launch_pdl(k_fcol_fan16<fan16_len(N)>, dim3(nc, chans), dim3(Col16Geo<fan16_len(N)>::NT), fan16_smem<N>(),  \
                         st, uhat, g.bank, items, cta_begin, Y, g.Wh, Whp, wv.l0, wv.f0, wv.nf, g.twH);           \
     if (usev(N, variant))                                                                                        \
-      return launch_pdl(k_fcol_fanv<colv_len(N)>, dim3(nc), dim3(ColVGeo<colv_len(N)>::NT), colv_smem<N>(), st,  \
+      return launch_pdl(k_fcol_fanv<colv_len(N)>, dim3(nc, chans), dim3(ColVGeo<colv_len(N)>::NT), colv_smem<N>(), st,  \
                         uhat, g.bank, items, cta_begin, Y, g.Wh, Whp, wv.l0, wv.f0, wv.nf, g.twH);               \
-    return launch_pdl(k_fcol_fan<N>, dim3(nc), dim3(ColGeo<N>::NT), col_smem<N>(), st, uhat, g.bank, items, cta_begin, Y, \
+    return launch_pdl(k_fcol_fan<N>, dim3(nc, chans), dim3(ColGeo<N>::NT), col_smem<N>(), st, uhat, g.bank, items, cta_begin, Y, \
                       g.Wh, Whp, wv.l0, wv.f0, wv.nf, g.twH);
     SHF_COL_SIZES(SHF_CASE)
 #undef SHF_CASE
@@ -720,19 +737,20 @@ cudaError_t col_fan(const Geo& g, int nc, const float2* uhat, const WorkItem* it
 }
 
 cudaError_t col_gather(const Geo& g, int nc, const float2* Y, const WorkItem* items, const int* cta_begin,
-                       float2* partial, int Whp, const Wave& wv, int variant, cudaStream_t st) {
+                       float2* partial, int Whp, const Wave& wv, int variant, cudaStream_t st, int chans,
+                       int cslots) {
   switch (g.H) {
 #define SHF_CASE(N)                                                                                           \
   case N:                                                                                                     \
     if (use16(N, variant))                                                                                    \
-      return launch_pdl(k_fcol_gather16<fan16_len(N)>, dim3(nc), dim3(Col16Geo<fan16_len(N)>::NT),           \
+      return launch_pdl(k_fcol_gather16<fan16_len(N)>, dim3(nc, chans), dim3(Col16Geo<fan16_len(N)>::NT),           \
                         fan16_smem<N>(), st, Y, g.bank, items, cta_begin, partial, g.Wh, Whp, wv.l0, wv.f0,   \
-                        wv.nf, g.twH);                                                                        \
+                        wv.nf, g.twH, cslots);                                                                        \
     if (usev(N, variant))                                                                                     \
-      return launch_pdl(k_fcol_gatherv<colv_len(N)>, dim3(nc), dim3(ColVGeo<colv_len(N)>::NT), colv_smem<N>(), \
-                        st, Y, g.bank, items, cta_begin, partial, g.Wh, Whp, wv.l0, wv.f0, wv.nf, g.twH);      \
-    return launch_pdl(k_fcol_gather<N>, dim3(nc), dim3(ColGeo<N>::NT), col_smem<N>(), st, Y, g.bank, items, cta_begin, \
-                      partial, g.Wh, Whp, wv.l0, wv.f0, wv.nf, g.twH);
+      return launch_pdl(k_fcol_gatherv<colv_len(N)>, dim3(nc, chans), dim3(ColVGeo<colv_len(N)>::NT), colv_smem<N>(), \
+                        st, Y, g.bank, items, cta_begin, partial, g.Wh, Whp, wv.l0, wv.f0, wv.nf, g.twH, cslots);      \
+    return launch_pdl(k_fcol_gather<N>, dim3(nc, chans), dim3(ColGeo<N>::NT), col_smem<N>(), st, Y, g.bank, items, cta_begin, \
+                      partial, g.Wh, Whp, wv.l0, wv.f0, wv.nf, g.twH, cslots);
     SHF_COL_SIZES(SHF_CASE)
 #undef SHF_CASE
     default: return cudaErrorInvalidValue;
@@ -740,14 +758,14 @@ cudaError_t col_gather(const Geo& g, int nc, const float2* Y, const WorkItem* it
 }
 
 cudaError_t col_reduce(const Geo& g, const float2* partial, const int* tile_begin, const int* tile_slots, float2* T,
-                       int K, cudaStream_t st) {
+                       int K, cudaStream_t st, int cslots) {
   const int tw = reg::col_batch(g.H), ntiles = (g.Wh + tw - 1) / tw;
   switch (g.H) {
 #define SHF_CASE(N)                                                                                          \
   case N:                                                                                                    \
     return launch_pdl(k_fcol_reduce_inv<N>, dim3(ntiles, K), dim3(ReduceGeo<N>::RG * ColGeo<N>::NT),             \
                       sizeof(float2) * ReduceGeo<N>::TOTAL, st, partial, tile_begin,                                  \
-                      tile_slots, T, g.Wh, g.twH);
+                      tile_slots, T, g.Wh, g.twH, cslots);
     SHF_COL_SIZES(SHF_CASE)
 #undef SHF_CASE
     default: return cudaErrorInvalidValue;

@@ -332,13 +332,15 @@ bool half_rows_ok(int L) {
   }
 }
 
-cudaError_t prepare_half_kernels() {
-#define SHF_PREP(N) \
-  if (e == cudaSuccess) e = prepare_half_t<N>();
-  cudaError_t e = cudaSuccess;
-  SHF_FAST_SIZES(SHF_PREP)
-#undef SHF_PREP
-  return e;
+cudaError_t prepare_half_kernels(int N) {
+  switch (N) {
+#define SHF_CASE(M) \
+  case M:           \
+    return prepare_half_t<M>();
+    SHF_FAST_SIZES(SHF_CASE)
+#undef SHF_CASE
+    default: return cudaSuccess;
+  }
 }
 
 cudaError_t rows_inv(const Geo& g, const float2* X, int pitch, float* out, const int2* ranges, int eta, const Wave& wv,

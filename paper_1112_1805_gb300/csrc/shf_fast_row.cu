@@ -1140,13 +1140,15 @@ cudaError_t ustep_t(const Geo& g, const float2* T, const float* s, float* w, flo
 
 }  // namespace
 
-cudaError_t prepare_row_kernels() {
-#define SHF_PREP(N) \
-  if (e == cudaSuccess) e = prepare_row_t<N>();
-  cudaError_t e = cudaSuccess;
-  SHF_FAST_SIZES(SHF_PREP)
-#undef SHF_PREP
-  return e;
+cudaError_t prepare_row_kernels(int N) {
+  switch (N) {
+#define SHF_CASE(M) \
+  case M:           \
+    return prepare_row_t<M>();
+    SHF_FAST_SIZES(SHF_CASE)
+#undef SHF_CASE
+    default: return cudaSuccess;
+  }
 }
 
 // The forward v-step a plan's variant selects at half width L (the default:

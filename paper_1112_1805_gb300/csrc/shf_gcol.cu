@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(kColThreads, 2)
 // W_f times uhat [nch][H][Wh], fg filters per CTA (uhat's tile then comes from
 // L1 after the first).
 __global__ void __launch_bounds__(kColThreads, 2)
-    k_gcol_fan(const __grid_constant__ Geo g, const float2* __restrict__ uhat, float2* __restrict__ Y, int fg,
+    k_gcol_fan(const __grid_constant__ Geo g, const float2* __restrict__ uhat, float2* __restrict__ Y, int fg, int mask,
                const FilterWave wv, const __grid_constant__ gf::Batch ba, int bufn) {
   extern __shared__ float2 sm[];
   gf::Exchange x{{sm, sm + bufn}};
@@ -92,9 +92,13 @@ __global__ void __launch_bounds__(kColThreads, 2)
   pdl_trigger();
   const float2* src = uhat + static_cast<size_t>(wv.c0 + blockIdx.y) * H * Wh + col0;
   for (int f = fb; f < fe; ++f) {
+    // columns b0..b1 of the tile are in the range; s0..s1 are stored: the range
+    // widened to whole tiles of mask + 1 columns (0: not widened)
     const int2 r = range_of(g, f);
+    if (r.x > r.y) continue;
     const int b0 = max(r.x - col0, 0), b1 = min(min(r.y, g.L) - col0, g.TC - 1);
-    if (b0 > b1) continue;
+    const int s0 = max((r.x & ~mask) - col0, 0), s1 = min(min(r.y | mask, g.L) - col0, g.TC - 1);
+    if (s0 > s1) continue;
     const float* wf = g.bank + static_cast<size_t>(f) * H * Wh + col0;
     float2* dst = Y + static_cast<size_t>(blockIdx.y * wv.nf + (f - wv.f0)) * H * Wy + col0;
     gf::fft<+1, true>(
@@ -105,7 +109,7 @@ __global__ void __launch_bounds__(kColThreads, 2)
           return c_scale(src[e], __ldg(wf + e));
         },
         [&](int i, int b, float2 v) {
-          if (b >= b0 && b <= b1) dst[static_cast<size_t>(i) * Wy + b] = v;
+          if (b >= s0 && b <= s1) dst[static_cast<size_t>(i) * Wy + b] = v;
         });
   }
 }
@@ -340,7 +344,7 @@ cudaError_t run_wave_fan(const Geo& g, const float2* uhat, float2* Y, const Filt
   const long all = static_cast<long>(g.ntiles) * wv.nc * wv.nf;
   const int fg = static_cast<int>(std::max<long>(1, std::min<long>(4, all / (8 * 152))));
   return launch_pdl(k_gcol_fan, dim3(g.ntiles, wv.nc, (wv.nf + fg - 1) / fg), dim3(kColThreads), s.smem, st, g, uhat, Y,
-                    fg, wv, s.ba, s.bufn);
+                    fg, fast_shrink_ok(g) ? reg::col_batch(g.H) - 1 : 0, wv, s.ba, s.bufn);
 }
 
 cudaError_t run_wave_gather(const Geo& g, const float2* Y, float2* partial, int nch, int groups, const FilterWave& wv,

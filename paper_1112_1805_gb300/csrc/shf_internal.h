@@ -86,7 +86,8 @@ cudaError_t run_col_fwd(const Geo& g, float2* U, int nch, cudaStream_t st);
 // out = column-inverse( g.bank * column-forward(in) ), planes [nch][H][Wh], one
 // filter [H][Wh].
 cudaError_t run_col_filter(const Geo& g, const float2* in, float2* out, int nch, cudaStream_t st);
-// Y = column-inverse( W_f * uhat[c] ) over the wave.
+// Y = column-inverse( W_f * uhat[c] ) over the wave; with fast_shrink_ok(g) the
+// rest of the column tiles that a range touches is written too (as zero).
 cudaError_t run_wave_fan(const Geo& g, const float2* uhat, float2* Y, const FilterWave& wv, cudaStream_t st);
 // Row transforms of the wave's coefficient planes, both ways.
 cudaError_t run_wave_r2c(const Geo& g, const float* coef, float2* Y, const FilterWave& wv, cudaStream_t st);
@@ -94,6 +95,7 @@ cudaError_t run_wave_c2r(const Geo& g, const float2* Y, float* coef, const Filte
                          cudaStream_t st);
 // ADMM v-step on the wave's spectra (in place) and b_v [nch][eta][H][W].
 // gout (optional): receives g = b_v + S u before the clipping, laid out as b_v.
+bool fast_shrink_ok(const Geo& g);  // whether run_wave_shrink (without gout) takes the register-FFT v-step
 cudaError_t run_wave_shrink(const Geo& g, float2* Y, float* bv, const float* thr, const FilterWave& wv, float scale,
                             cudaStream_t st, float* gout = nullptr);
 // lam[f] * ||row-inverse of Y||_1 of the wave's planes, one FP64 partial per
@@ -116,7 +118,7 @@ int default_groups(const Geo& g, int nch);
 // row block RB) in g when the kernels support it and their shared memory for
 // K labels fits in `smem_limit` bytes; false (g unchanged) otherwise.
 bool set_generic_tiles(Geo* g, int TC, int RB, int K, int smem_limit);
-cudaError_t prepare_kernels();
+cudaError_t prepare_kernels(const Geo& g);
 int max_dynamic_smem_needed(const Geo& g, int K);
 cudaError_t launch_sub(const float* a, const float* b, float* out, long n, cudaStream_t st);  // out = a - b
 
@@ -206,7 +208,7 @@ struct PdlScope {
 // Fast path for power-of-two sizes (shf_fast.cu).
 bool fast_path_ok(const Geo& g);
 int fast_tile(const Geo& g);  // columns per tile of the fast column kernels (8, or 4 for H > 1024)
-cudaError_t prepare_fast_kernels();
+cudaError_t prepare_fast_kernels(const Geo& g);  // the shared-memory limits of g's sizes
 int fast_wave(const Geo& g, int wave_mib);  // filters per wave of one label (at most eta)
 int fast_wave_labels(const Geo& g, int wave_mib, int K);  // labels per wave (1: waves of filters)
 int fast_pitch(const Geo& g);       // row pitch (complex) of the internal spectra: Wh rounded up to 8
@@ -221,6 +223,18 @@ cudaError_t run_fast_ustep(const Geo& g, const float2* T, const float* s, float*
 cudaError_t run_fast_iteration_body(const Geo& g, const FastPlan& plan, const float2* Ur, float2* uhat, float2* Y,
                                     float* bv, const float* thr, float2* partial, float2* T, int K, float scale,
                                     cudaStream_t st, const LaunchHook& hook, signed char* code = nullptr);
+// The column kernels over a single-channel plan (built for one label), every
+// launch for the channels of wave wv: heights with fast_columns_ok(g).  uhat
+// [nch][H][fast_pitch(g)]; `w`: the plan's wave wv comes from; partial: nslots
+// slots per channel.
+bool fast_columns_ok(const Geo& g);
+cudaError_t run_channel_fwd(const Geo& g, const float2* Ur, float2* uhat, int nch, cudaStream_t st);
+cudaError_t run_channel_fan(const Geo& g, const FastPlan& plan, int w, const float2* uhat, float2* Y,
+                            const FilterWave& wv, cudaStream_t st);
+cudaError_t run_channel_gather(const Geo& g, const FastPlan& plan, int w, const float2* Y, float2* partial,
+                               const FilterWave& wv, cudaStream_t st);
+cudaError_t run_channel_reduce(const Geo& g, const FastPlan& plan, const float2* partial, float2* T, int nch,
+                               cudaStream_t st);
 // Adjoint of the analysis - v-step - synthesis part of an iteration (reverse
 // mode): Qr [K][H][Wh] the row spectra of Qbar; bvbar [K][eta][H][W] updated in
 // place with the codes of the forward iteration; Tbar [K][H][Wh] receives the

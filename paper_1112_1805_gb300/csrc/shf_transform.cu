@@ -108,8 +108,13 @@ __global__ void __launch_bounds__(kRowThreads, 2)
   const int L = g.L, row0 = blockIdx.x * RB, rows = min(RB, g.H - row0);
   pdl_wait();
   pdl_trigger();
-  const Plane p = plane_of<FILT>(g, wv);
+  Plane p = plane_of<FILT>(g, wv);
   if (p.c1 < p.c0) return;  // an empty filter: nothing reads its spectrum
+  if (FILT) {  // whole column tiles: the register-FFT gather reads those
+    const int mask = reg::col_batch(g.H) - 1;
+    p.c0 &= ~mask;
+    p.c1 = min(g.L, p.c1 | mask);
+  }
   const float2* src = reinterpret_cast<const float2*>(in) + p.data * g.H * L + static_cast<size_t>(row0) * L;
   const auto ld = [&](int i, int b) { return b < rows ? src[static_cast<size_t>(b) * L + i] : make_float2(0.f, 0.f); };
   const float2* y = gf::fft_head<-1, false>(g.planL, ba, x, g.ptL, ld);
@@ -404,9 +409,10 @@ RowShape row_shape(const FftPlan& p, int rb) {
 
 cudaError_t prepare_col_general(int optin);
 
-// Raises the dynamic shared-memory limit of every kernel to the device's
-// opt-in maximum (an upper bound only), once per device, outside any capture.
-cudaError_t prepare_kernels() {
+// Raises the dynamic shared-memory limits of the kernels that g's transforms
+// launch, outside any capture: the staged kernels' to the device's opt-in
+// maximum (an upper bound only), the single row transforms' of g's width.
+cudaError_t prepare_kernels(const Geo& g) {
   int dev = 0, optin = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
@@ -416,7 +422,8 @@ cudaError_t prepare_kernels() {
       set_smem(k_row_r2c<false>, optin), set_smem(k_row_r2c<true>, optin), set_smem(k_row_c2r<false>, optin),
       set_smem(k_row_c2r<true>, optin),  set_smem(k_row_shrink, optin),
       set_smem(k_row_l1, optin - static_cast<int>(sizeof(double)) * kL1Threads),
-      set_smem(k_row_ustep, optin),      prepare_col_general(optin)};
+      set_smem(k_row_ustep, optin),      prepare_col_general(optin),
+      fast::prepare_half_kernels(g.L)};
   for (cudaError_t x : errs)
     if (x != cudaSuccess) return x;
   return cudaSuccess;
@@ -446,19 +453,28 @@ bool set_generic_tiles(Geo* g, int TC, int RB, int K, int smem_limit) {
   return true;
 }
 
+namespace {
+// A plain launch's planes as one wave of single-filter channels.
+fast::Wave plain(int planes) { return fast::Wave{0, 0, 1, planes}; }
+fast::Wave fast_wave_of(const FilterWave& wv) { return fast::Wave{wv.c0, wv.f0, wv.nf, wv.nc * wv.nf}; }
+}  // namespace
+
 cudaError_t run_row_r2c(const Geo& g, const float* in, float2* out, int planes, float scale, cudaStream_t st) {
+  if (scale == 1.f && fast::half_rows_ok(g.L)) return fast::rows_fwd(g, in, out, g.Wh, nullptr, 1, plain(planes), st);
   const RowShape s = row_shape(g.planL, g.RB);
   return launch_pdl(k_row_r2c<false>, dim3((g.H + g.RB - 1) / g.RB, planes), dim3(kRowThreads), s.smem, st, g, in, out,
                     g.Wh, g.RB, s.ba, s.bufn, FilterWave{}, scale);
 }
 
 cudaError_t run_row_c2r(const Geo& g, const float2* in, float* out, int planes, float scale, cudaStream_t st) {
+  if (fast::half_rows_ok(g.L)) return fast::rows_inv(g, in, g.Wh, out, nullptr, 1, plain(planes), scale, st);
   const RowShape s = row_shape(g.planL, g.RB);
   return launch_pdl(k_row_c2r<false>, dim3((g.H + g.RB - 1) / g.RB, planes), dim3(kRowThreads), s.smem, st, g, in, out,
                     g.Wh, g.RB, s.ba, s.bufn, FilterWave{}, scale);
 }
 
 cudaError_t run_wave_r2c(const Geo& g, const float* coef, float2* Y, const FilterWave& wv, cudaStream_t st) {
+  if (fast::half_rows_ok(g.L)) return fast::rows_fwd(g, coef, Y, g.Wy, g.ranges, g.eta, fast_wave_of(wv), st);
   const RowShape s = row_shape(g.planL, g.RB);
   return launch_pdl(k_row_r2c<true>, dim3((g.H + g.RB - 1) / g.RB, wv.nc * wv.nf), dim3(kRowThreads), s.smem, st, g,
                     coef, Y, g.Wy, g.RB, s.ba, s.bufn, wv, 1.f);
@@ -466,6 +482,7 @@ cudaError_t run_wave_r2c(const Geo& g, const float* coef, float2* Y, const Filte
 
 cudaError_t run_wave_c2r(const Geo& g, const float2* Y, float* coef, const FilterWave& wv, float scale,
                          cudaStream_t st) {
+  if (fast::half_rows_ok(g.L)) return fast::rows_inv(g, Y, g.Wy, coef, g.ranges, g.eta, fast_wave_of(wv), scale, st);
   const RowShape s = row_shape(g.planL, g.RB);
   return launch_pdl(k_row_c2r<true>, dim3((g.H + g.RB - 1) / g.RB, wv.nc * wv.nf), dim3(kRowThreads), s.smem, st, g, Y,
                     coef, g.Wy, g.RB, s.ba, s.bufn, wv, scale);
@@ -473,6 +490,11 @@ cudaError_t run_wave_c2r(const Geo& g, const float2* Y, float* coef, const Filte
 
 cudaError_t run_wave_shrink(const Geo& g, float2* Y, float* bv, const float* thr, const FilterWave& wv, float scale,
                             cudaStream_t st, float* gout) {
+  if (fast_shrink_ok(g) && !gout) {  // the register-FFT v-step of this half width
+    const fast::Wave f = fast_wave_of(wv);
+    const int rpc = fast::row_groups_per_cta(g.L), groups = (f.nv * g.H + rpc - 1) / rpc;
+    return fast::row_shrink(g, std::min(groups, std::max(1, fast_row_ctas(g))), Y, bv, thr, g.Wy, f, scale, nullptr, 0, st);
+  }
   const RowShape s = row_shape(g.planL, g.RB), r = row_shape(g.planLr, g.RB);
   const int bufn = std::max(s.bufn, r.bufn);
   return launch_pdl(k_row_shrink, dim3((g.H + g.RB - 1) / g.RB, wv.nc * wv.nf), dim3(kRowThreads),

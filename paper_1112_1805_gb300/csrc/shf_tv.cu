@@ -374,7 +374,7 @@ int tv_admm_init(int H, int W, const float* f, int C, const float* codebook, int
   g.eta = 1;
   int device = 0, optin = 0;
   TV_CK(cudaGetDevice(&device));
-  TV_CK(shf::prepare_kernels());
+  TV_CK(shf::prepare_kernels(g));
   TV_CK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device));
   if (shf::max_dynamic_smem_needed(g, K) > optin) return tv_fail(SHF_ERR_SIZE, "tile does not fit in shared memory");
   auto* st = new tv_state();
