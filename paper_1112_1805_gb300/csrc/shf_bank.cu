@@ -278,6 +278,7 @@ bool make_geo(int H, int W, int J, Geo* g) {
   g->twH = nullptr;
   g->twW = nullptr;
   g->ptH = g->ptL = g->ptLr = nullptr;
+  g->staged = 0;
   g->bank = nullptr;
   g->ranges = nullptr;
   return true;

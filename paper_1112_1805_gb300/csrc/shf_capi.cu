@@ -129,6 +129,8 @@ struct seg_state {
   float2* un_partial = nullptr;  // [un_groups][K][H][Wh]
   int un_groups = 0;
   std::vector<shf::FilterWave> un_waves;
+  Geo un_g;                      // general path: the geometry on sweep plans
+  float2* un_pt = nullptr;       // ... and their pass tables
   std::vector<float*> ck_bv, ck_w, ck_bw;
   std::vector<float2*> ck_T;
   // the forward and reverse sweeps captured as graphs for (T, ckpt) = un_key;
@@ -202,6 +204,15 @@ int build_channel_plan(shf_bank* b, const std::vector<int2>& ranges) {
   return SHF_OK;
 }
 
+// Transforms on whole planes in shared memory: small images, and no more CTAs
+// (one per channel and filter) than a few per SM; an analysis CTA repeats the
+// forward transform of its channel, a synthesis ends in one CTA per channel.
+// Up to 5000 half-spectrum values a synthesis takes 30 us (four channels), less
+// than four launches in a row; at 8320 57 us, more.
+bool small_transform(const Geo& g, int nch, bool analysis) {
+  return shf::small_ok(g) && static_cast<long long>(nch) * g.eta <= 4 * 152 && (analysis || g.H * g.Wh <= 5000);
+}
+
 // Channels of a launch over the single-channel plan: as many as keep the wave's
 // spectra within the plan's budget.
 int channels_per_launch(const shf_bank* b, int nch) {
@@ -248,6 +259,10 @@ int shfilters_build(int H, int W, int J, void* stream, shf_bank** out) {
   }
   b->g.bank = b->bank;
   b->g.ranges = b->ranges;
+  if (cudaError_t es = shf::prepare_small(b->g); es != cudaSuccess) {
+    shfilters_destroy(b);
+    return fail(SHF_ERR_CUDA, std::string("shfilters_build: ") + cudaGetErrorString(es));
+  }
   b->g.twH = b->twH;
   b->g.twW = b->twW;
   cudaError_t e = cudaMemcpyAsync(b->descs, d.data(), sizeof(shf::FilterDesc) * g.eta, cudaMemcpyHostToDevice, st);
@@ -311,6 +326,11 @@ int shearlet_analyze(const shf_bank* b, const float* u, int nch, float* coef, vo
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const size_t ph = static_cast<size_t>(g.H) * g.Wh;
   const float scale = 1.f / (static_cast<float>(g.H) * g.W);
+  if (small_transform(g, nch, true)) {
+    const cudaError_t e = shf::run_small_analyze(g, u, coef, nch, scale, st);
+    if (e != cudaSuccess) return fail(SHF_ERR_CUDA, std::string("shearlet_analyze: ") + cudaGetErrorString(e));
+    return SHF_OK;
+  }
   if (b->chan_ok) {
     const size_t php = static_cast<size_t>(g.H) * g.Wy;
     const int nc = channels_per_launch(b, nch);
@@ -398,6 +418,16 @@ int shearlet_synthesize(const shf_bank* b, const float* coef, int nch, float* u,
     return fail(SHF_ERR_ARG, "shearlet_synthesize: pointers must be 8-byte aligned");
   const Geo& g = b->g;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  if (small_transform(g, nch, false)) {
+    float2* part = nullptr;
+    cudaError_t e = scratch_alloc(b, &part, shf::small_partials(g, nch), st);
+    if (e != cudaSuccess) return fail(SHF_ERR_OOM, std::string("shearlet_synthesize: ") + cudaGetErrorString(e));
+    e = shf::run_small_synthesize(g, coef, u, part, nch, 1.f / (static_cast<float>(g.H) * g.W), st);
+    cudaError_t e2 = cudaFreeAsync(part, st);
+    if (e == cudaSuccess) e = e2;
+    if (e != cudaSuccess) return fail(SHF_ERR_CUDA, std::string("shearlet_synthesize: ") + cudaGetErrorString(e));
+    return SHF_OK;
+  }
   const size_t ph = static_cast<size_t>(g.H) * g.Wh;
   float2* T = nullptr;
   cudaError_t e = scratch_alloc(b, &T, ph * nch, st);
@@ -428,6 +458,7 @@ void free_state(seg_state* s) {
   cudaFree(s->d_tile_slots);
   cudaFree(s->un_Y);
   cudaFree(s->un_partial);
+  cudaFree(s->un_pt);
   if (s->un_fwd_exec) cudaGraphExecDestroy(s->un_fwd_exec);
   if (s->un_bwd_exec) cudaGraphExecDestroy(s->un_bwd_exec);
   cudaFree(s->un_mem);
@@ -556,10 +587,10 @@ cudaError_t enqueue_iteration(seg_state* st, bool timed, signed char* code = nul
   return e;
 }
 
-// One iteration on the generic kernels with the full coefficient scratch of
-// the unrolled mode; gout (optional) records g = b_v + S u.
+// One iteration on the general path's sweep plans with the unrolled mode's
+// scratch; gout (optional) records g = b_v + S u.
 cudaError_t enqueue_generic_iteration(seg_state* st, float* gout) {
-  const Geo& g = st->g;
+  const Geo& g = st->un_g;
   const float scale = 1.f / (static_cast<float>(g.H) * g.W);
   cudaStream_t s = st->stream;
   cudaError_t e =
@@ -1567,11 +1598,29 @@ int seg_admm_unrolled_fwd(seg_state* st, int T, int ckpt_every) {
   // the general path keeps the spectra of every filter; the fast path
   // iterates with its own wave scratch
   if (!st->fast && !st->un_Y) {
-    st->un_waves = shf::general_waves(g, st->K, st->groups);
-    if ((rc = dev_alloc(&st->un_Y, shf::wave_planes(st->un_waves) * g.H * g.Wy, "unrolled scratch")) ||
-        (rc = dev_alloc(&st->un_partial, Ph * st->K * st->groups, "unrolled partials")))
+    // filter groups for four CTAs per SM over all labels, unless the plan says otherwise
+    int groups = st->groups;
+    if (groups == shf::default_groups(g, st->K)) {
+      const int base = g.ntiles * st->K;
+      groups = normalise_groups(g.eta, (4 * 152 + base - 1) / base);
+    }
+    st->un_g = g;
+    st->un_g.staged = 1;
+    if (!shf::make_sweep_plan(g.H, &st->un_g.planH) || !shf::make_sweep_plan(g.L, &st->un_g.planL))
+      return fail(SHF_ERR_SIZE, "unsupported geometry");
+    st->un_g.planLr = st->un_g.planL;
+    st->un_waves = shf::general_waves(g, st->K, groups);
+    if ((rc = dev_alloc(&st->un_pt, shf::pass_table_entries(st->un_g), "pass tables")) ||
+        (rc = dev_alloc(&st->un_Y, shf::wave_planes(st->un_waves) * g.H * g.Wy, "unrolled scratch")) ||
+        (rc = dev_alloc(&st->un_partial, Ph * st->K * static_cast<size_t>(groups), "unrolled partials"))) {
+      cudaFree(st->un_pt);
+      cudaFree(st->un_Y);
+      st->un_pt = nullptr;
+      st->un_Y = nullptr;
       return rc;
-    st->un_groups = st->groups;
+    }
+    SHF_CK(shf::launch_pass_tables(&st->un_g, st->un_pt, st->stream));
+    st->un_groups = groups;
   }
   const int nseg = (T + ckpt_every - 1) / ckpt_every;
   while (static_cast<int>(st->ck_bv.size()) < nseg) {

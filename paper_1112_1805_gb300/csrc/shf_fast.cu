@@ -105,7 +105,7 @@ int fast_row_ctas(const Geo& g, int row_kernel, int sms) {
 
 int fast_fan_ctas(const Geo& g, int col_kernel, int sms) { return fast::fan_ctas_per_sm(g.H, col_kernel) * sms_for(sms); }
 
-bool fast_shrink_ok(const Geo& g) { return g.ranges && reg::supported(g.L); }
+bool fast_shrink_ok(const Geo& g) { return !g.staged && g.ranges && reg::supported(g.L); }
 
 bool fast_row_kernel_ok(const Geo& g, int row_kernel) { return fast::row_kernel_ok(g.L, row_kernel); }
 

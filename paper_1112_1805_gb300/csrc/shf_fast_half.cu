@@ -25,7 +25,6 @@ namespace {
 
 __host__ __device__ constexpr bool half16(int L) { return L == 64 || L == 128 || L == 256 || L == 512; }
 __host__ __device__ constexpr bool half_ok(int L) { return half16(L) || rv::supported(L); }
-__host__ __device__ constexpr int half_len(int L) { return half_ok(L) ? L : 64; }
 __host__ __device__ constexpr int even2(int n) { return (n + 1) & ~1; }
 
 // The transform of one row: 16 values per thread or V.

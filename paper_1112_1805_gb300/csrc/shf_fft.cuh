@@ -10,7 +10,7 @@
 
 namespace shf {
 
-constexpr int kMaxStages = 6;
+constexpr int kMaxStages = 8;
 
 // One Stockham stage of a transform of length L: radix, span (product of the
 // radices before it), butterflies L / radix, the offset of its twiddles in the
@@ -222,6 +222,24 @@ __host__ __device__ __forceinline__ float2 r2c_unpack(const float2* Z, int L, in
   return unpack_combine(s, d, twW[k]);
 }
 
+// Fills a plan from its radices in order.
+inline void set_stages(FftPlan* p, int L, const int* radix, int n) {
+  p->L = L;
+  p->nst = n;
+  int Ns = 1, off = 0;
+  for (int s = 0; s < n; ++s) {
+    FftStage& g = p->st[s];
+    g.R = radix[s];
+    g.Ns = Ns;
+    g.nb = L / g.R;
+    g.off = off;
+    g.mNs = fdiv_mul(static_cast<unsigned>(Ns));
+    g.mNb = fdiv_mul(static_cast<unsigned>(g.nb));
+    if (s > 0) off += (g.R - 1) * Ns;
+    Ns *= g.R;
+  }
+}
+
 // Stage plan for L = 2^a 3^b 5^c: the fewest stages of radices up to 16, then
 // the smallest sum of radices (registers and twiddles), in increasing order or,
 // for `reversed`, in decreasing order (the forward transform of the v-step,
@@ -249,20 +267,29 @@ inline bool make_plan(int L, FftPlan* p, bool reversed = false) {
   };
   search(search, L, 0, 0, 0);
   if (nbest > kMaxStages) return false;
-  p->L = L;
-  p->nst = nbest;
-  int Ns = 1, off = 0;
-  for (int s = 0; s < nbest; ++s) {
-    FftStage& g = p->st[s];
-    g.R = best[reversed ? nbest - 1 - s : s];
-    g.Ns = Ns;
-    g.nb = L / g.R;
-    g.off = off;
-    g.mNs = fdiv_mul(static_cast<unsigned>(Ns));
-    g.mNb = fdiv_mul(static_cast<unsigned>(g.nb));
-    if (s > 0) off += (g.R - 1) * Ns;
-    Ns *= g.R;
-  }
+  if (reversed)
+    for (int i = 0; i < nbest / 2; ++i) {
+      const int t = best[i];
+      best[i] = best[nbest - 1 - i];
+      best[nbest - 1 - i] = t;
+    }
+  set_stages(p, L, best, nbest);
+  return true;
+}
+
+// The radices 8 (as many as fit), then 4 or 2, then 3s and 5s: the sequence of
+// the unrolled sweeps, whose gradients hang on which side of the clip threshold
+// a rounded coefficient falls, so that their iterates stay bit for bit what
+// they have been.  False when L has another prime factor.
+inline bool make_sweep_plan(int L, FftPlan* p) {
+  int radix[16], n = 0, rest = L, a = 0;
+  for (; rest % 2 == 0; rest /= 2) ++a;
+  for (int i = 0; i < a / 3; ++i) radix[n++] = 8;
+  if (a % 3) radix[n++] = a % 3 == 2 ? 4 : 2;
+  for (; rest % 3 == 0; rest /= 3) radix[n++] = 3;
+  for (; rest % 5 == 0; rest /= 5) radix[n++] = 5;
+  if (rest != 1 || n < 1 || n > kMaxStages) return false;
+  set_stages(p, L, radix, n);
   return true;
 }
 

@@ -25,6 +25,7 @@ struct Geo {
   int L;   // W / 2, length of the packed complex row transform
   int Wh;  // W / 2 + 1, columns of the half spectrum
   int Wy;  // row pitch (complex) of the coefficient spectra of a wave
+  int staged;  // 1: only the staged kernels, on sweep plans (the unrolled sweeps of the general path)
   // stage plans: columns, rows, and the rows' reversed one with their pass tables
   FftPlan planH, planL, planLr;
   const float2 *ptH, *ptL, *ptLr;
@@ -110,6 +111,14 @@ cudaError_t run_wave_gather(const Geo& g, const float2* Y, float2* partial, int 
 // out[nch][H][Wh] = column-inverse( sum_grp partial[grp] ).
 cudaError_t run_col_reduce_inv(const Geo& g, const float2* partial, float2* out, int nch, int groups,
                                cudaStream_t st);
+// Transforms of small images (shf_small.cu), planes in shared memory; partial:
+// small_partials(g, channels) elements.
+bool small_ok(const Geo& g);
+cudaError_t prepare_small(const Geo& g);
+size_t small_partials(const Geo& g, int nch);
+cudaError_t run_small_analyze(const Geo& g, const float* u, float* coef, int nch, float scale, cudaStream_t st);
+cudaError_t run_small_synthesize(const Geo& g, const float* coef, float* u, float2* partial, int nch, float scale,
+                                 cudaStream_t st);
 // ADMM u-step and w-step per row block over all K labels.
 cudaError_t run_row_ustep(const Geo& g, const float2* T, const float* s, float* w, float* bw, float* u, float2* Ur,
                           float* stv, int K, float gamma, float scale, cudaStream_t st);

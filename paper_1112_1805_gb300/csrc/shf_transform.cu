@@ -284,15 +284,69 @@ __global__ void __launch_bounds__(kRowThreads, 2)
   if (threadIdx.x == 0) partial[p.data * gridDim.x + blockIdx.x] = red[0];
 }
 
+// The v-step with its transforms apart (sweep plans, whose forward transform
+// starts with another radix than the inverse one ends with).
+__global__ void __launch_bounds__(kRowThreads, 2)
+    k_row_shrink_apart(const __grid_constant__ Geo g, float2* __restrict__ Y, float* __restrict__ bv,
+                       const float* __restrict__ thr, int pitch, int RB, const __grid_constant__ gf::Batch ba, int bufn,
+                       const FilterWave wv, float scale, float* __restrict__ gout) {
+  extern __shared__ float2 sm[];
+  gf::Exchange x{{sm, sm + bufn}};
+  const int L = g.L, row0 = blockIdx.x * RB, rows = min(RB, g.H - row0);
+  pdl_wait();
+  pdl_trigger();
+  const Plane p = plane_of<true>(g, wv);
+  float2* X = Y + (static_cast<size_t>(blockIdx.y) * g.H + row0) * pitch;
+  const size_t off = (p.data * g.H + row0) * L;
+  float2* b2 = reinterpret_cast<float2*>(bv) + off;
+  float2* g2 = gout ? reinterpret_cast<float2*>(gout) + off : nullptr;
+  const float t = thr[p.f];
+  const auto ldx = [&](int i, int b) {
+    return b < rows ? packed(X + static_cast<size_t>(b) * pitch, L, i, p.c0, p.c1, g.twW) : make_float2(0.f, 0.f);
+  };
+  const float2* y = gf::fft_head<+1, false>(g.planL, ba, x, g.ptL, ldx);
+  float2* D = x.next();
+  const auto shrink = [&](int i, int b, float2 v) {
+    float2 d = make_float2(0.f, 0.f);
+    if (b < rows) {
+      const int e = b * L + i;
+      const float2 gv = c_fma2(make_float2(scale, scale), v, b2[e]);
+      const float2 c = make_float2(fminf(fmaxf(gv.x, -t), t), fminf(fmaxf(gv.y, -t), t));
+      b2[e] = c;
+      if (g2) g2[e] = gv;
+      d = c_fma2(make_float2(-2.f, -2.f), c, gv);  // g - 2 clip(g)
+    }
+    D[b * L + i] = d;
+  };
+  gf::NoLd nl;
+  if (g.planL.nst == 1)
+    gf::run_stage<+1, false, gf::kOnly>(g.planL, 0, ba, nullptr, nullptr, g.ptL, ldx, shrink, threadIdx.x, blockDim.x);
+  else
+    gf::run_stage<+1, false, gf::kLast>(g.planL, g.planL.nst - 1, ba, y, nullptr, g.ptL, nl, shrink, threadIdx.x, blockDim.x);
+  __syncthreads();
+  const auto ldd = [&](int i, int b) { return D[b * L + i]; };
+  y = gf::fft_head<-1, false>(g.planL, ba, x, g.ptL, ldd);
+  float2* Z = x.next();
+  const auto st = [&](int i, int b, float2 v) { Z[b * L + i] = v; };
+  if (g.planL.nst == 1)
+    gf::run_stage<-1, false, gf::kOnly>(g.planL, 0, ba, nullptr, nullptr, g.ptL, ldd, st, threadIdx.x, blockDim.x);
+  else
+    gf::run_stage<-1, false, gf::kLast>(g.planL, g.planL.nst - 1, ba, y, nullptr, g.ptL, nl, st, threadIdx.x, blockDim.x);
+  __syncthreads();
+  store_half(Z, X - static_cast<size_t>(row0) * pitch, pitch, L, row0, rows, p.c0, p.c1, 1.f, g.twW);
+}
+
 // u-step (u = 1/2 [S^T(v - b_v) + (w - b_w) - gamma s], A^T A = 2I), w-step
 // (pixelwise projection of g_w = b_w + u onto the simplex), b_w = g_w - w,
-// and the row-forward transform of u for the next analysis.  Shared memory:
-// the exchange buffers and U (K x RB x L complex).
+// and the row-forward transform of u for the next analysis.  KG labels' RB rows
+// are transformed as one batch (all labels where shared memory allows: label
+// after label the K transforms were a chain of 2 K times the barriers).  Shared
+// memory: the exchange buffers and U (K x RB x L complex).
 __global__ void __launch_bounds__(kRowThreads)
     k_row_ustep(const __grid_constant__ Geo g, const float2* __restrict__ T, const float* __restrict__ s,
                 float* __restrict__ w, float* __restrict__ bw, float* __restrict__ u, float2* __restrict__ Ur,
-                float* __restrict__ stv, int K, int RB, const __grid_constant__ gf::Batch ba, int bufn, float scale,
-                float gamma) {
+                float* __restrict__ stv, int K, int RB, int KG, unsigned mRB, const __grid_constant__ gf::Batch ba, int bufn,
+                float scale, float gamma) {
   extern __shared__ float2 sm[];
   gf::Exchange x{{sm, sm + bufn}};
   float2* U = sm + 2 * bufn;
@@ -300,15 +354,27 @@ __global__ void __launch_bounds__(kRowThreads)
   const size_t HL = static_cast<size_t>(g.H) * L, HWh = static_cast<size_t>(g.H) * Wh;
   pdl_wait();
   pdl_trigger();
-  for (int k = 0; k < K; ++k) {
-    const float2* src = T + k * HWh + static_cast<size_t>(row0) * Wh;
-    float2* Uk = U + k * E;
+  // sequence b of a batch: row r of label k0 + kk
+  const auto split = [&](int b, int& kk) {
+    kk = static_cast<int>(fdiv(static_cast<unsigned>(b), mRB));
+    return b - kk * RB;
+  };
+  for (int k0 = 0; k0 < K; k0 += KG) {
+    const float2* src = T + k0 * HWh + static_cast<size_t>(row0) * Wh;
+    float2* Uk = U + k0 * E;
     gf::fft<+1, false>(
         g.planL, ba, x, g.ptL,
         [&](int i, int b) {
-          return b < rows ? packed(src + static_cast<size_t>(b) * Wh, L, i, 0, L, g.twW) : make_float2(0.f, 0.f);
+          int kk;
+          const int r = split(b, kk);
+          return r < rows && k0 + kk < K ? packed(src + kk * HWh + static_cast<size_t>(r) * Wh, L, i, 0, L, g.twW)
+                                         : make_float2(0.f, 0.f);
         },
-        [&](int i, int b, float2 v) { Uk[b * L + i] = c_scale(v, scale); });
+        [&](int i, int b, float2 v) {
+          int kk;
+          const int r = split(b, kk);
+          if (k0 + kk < K) Uk[kk * E + r * L + i] = c_scale(v, scale);
+        });
   }
   __syncthreads();
   const float2* s2 = reinterpret_cast<const float2*>(s);
@@ -357,9 +423,14 @@ __global__ void __launch_bounds__(kRowThreads)
     }
   }
   __syncthreads();
-  for (int k = 0; k < K; ++k) {
-    const float2* Uk = U + k * E;
-    const auto ld = [&](int i, int b) { return Uk[b * L + i]; };
+  for (int k0 = 0; k0 < K; k0 += KG) {
+    const float2* Uk = U + k0 * E;
+    const int nk = min(KG, K - k0);
+    const auto ld = [&](int i, int b) {
+      int kk;
+      const int r = split(b, kk);
+      return kk < nk ? Uk[kk * E + r * L + i] : make_float2(0.f, 0.f);
+    };
     const float2* y = gf::fft_head<-1, false>(g.planL, ba, x, g.ptL, ld);
     float2* Z = x.next();
     const auto st = [&](int i, int b, float2 v) { Z[b * L + i] = v; };
@@ -370,7 +441,8 @@ __global__ void __launch_bounds__(kRowThreads)
       gf::run_stage<-1, false, gf::kLast>(g.planL, g.planL.nst - 1, ba, y, nullptr, g.ptL, nl, st, threadIdx.x,
                                           blockDim.x);
     __syncthreads();
-    store_half(Z, Ur + k * HWh, Wh, L, row0, rows, 0, L, 1.f, g.twW);
+    for (int kk = 0; kk < nk; ++kk)
+      store_half(Z + kk * E, Ur + (k0 + kk) * HWh, Wh, L, row0, rows, 0, L, 1.f, g.twW);
   }
 }
 
@@ -379,6 +451,7 @@ cudaError_t set_smem(K kernel, int bytes) {
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
+// Rows of a u/w-step CTA that a tile shape is accepted by.
 int ustep_rows(const Geo& g, int K) {
   int rb = 65536 / (g.L * (8 * K + 16));
   if (rb < 1) rb = 1;
@@ -421,6 +494,7 @@ cudaError_t prepare_kernels(const Geo& g) {
   const cudaError_t errs[] = {
       set_smem(k_row_r2c<false>, optin), set_smem(k_row_r2c<true>, optin), set_smem(k_row_c2r<false>, optin),
       set_smem(k_row_c2r<true>, optin),  set_smem(k_row_shrink, optin),
+      set_smem(k_row_shrink_apart, optin),
       set_smem(k_row_l1, optin - static_cast<int>(sizeof(double)) * kL1Threads),
       set_smem(k_row_ustep, optin),      prepare_col_general(optin),
       fast::prepare_half_kernels(g.L)};
@@ -456,25 +530,26 @@ bool set_generic_tiles(Geo* g, int TC, int RB, int K, int smem_limit) {
 namespace {
 // A plain launch's planes as one wave of single-filter channels.
 fast::Wave plain(int planes) { return fast::Wave{0, 0, 1, planes}; }
+bool half_rows(const Geo& g) { return !g.staged && fast::half_rows_ok(g.L); }
 fast::Wave fast_wave_of(const FilterWave& wv) { return fast::Wave{wv.c0, wv.f0, wv.nf, wv.nc * wv.nf}; }
 }  // namespace
 
 cudaError_t run_row_r2c(const Geo& g, const float* in, float2* out, int planes, float scale, cudaStream_t st) {
-  if (scale == 1.f && fast::half_rows_ok(g.L)) return fast::rows_fwd(g, in, out, g.Wh, nullptr, 1, plain(planes), st);
+  if (scale == 1.f && half_rows(g)) return fast::rows_fwd(g, in, out, g.Wh, nullptr, 1, plain(planes), st);
   const RowShape s = row_shape(g.planL, g.RB);
   return launch_pdl(k_row_r2c<false>, dim3((g.H + g.RB - 1) / g.RB, planes), dim3(kRowThreads), s.smem, st, g, in, out,
                     g.Wh, g.RB, s.ba, s.bufn, FilterWave{}, scale);
 }
 
 cudaError_t run_row_c2r(const Geo& g, const float2* in, float* out, int planes, float scale, cudaStream_t st) {
-  if (fast::half_rows_ok(g.L)) return fast::rows_inv(g, in, g.Wh, out, nullptr, 1, plain(planes), scale, st);
+  if (half_rows(g)) return fast::rows_inv(g, in, g.Wh, out, nullptr, 1, plain(planes), scale, st);
   const RowShape s = row_shape(g.planL, g.RB);
   return launch_pdl(k_row_c2r<false>, dim3((g.H + g.RB - 1) / g.RB, planes), dim3(kRowThreads), s.smem, st, g, in, out,
                     g.Wh, g.RB, s.ba, s.bufn, FilterWave{}, scale);
 }
 
 cudaError_t run_wave_r2c(const Geo& g, const float* coef, float2* Y, const FilterWave& wv, cudaStream_t st) {
-  if (fast::half_rows_ok(g.L)) return fast::rows_fwd(g, coef, Y, g.Wy, g.ranges, g.eta, fast_wave_of(wv), st);
+  if (half_rows(g)) return fast::rows_fwd(g, coef, Y, g.Wy, g.ranges, g.eta, fast_wave_of(wv), st);
   const RowShape s = row_shape(g.planL, g.RB);
   return launch_pdl(k_row_r2c<true>, dim3((g.H + g.RB - 1) / g.RB, wv.nc * wv.nf), dim3(kRowThreads), s.smem, st, g,
                     coef, Y, g.Wy, g.RB, s.ba, s.bufn, wv, 1.f);
@@ -482,7 +557,7 @@ cudaError_t run_wave_r2c(const Geo& g, const float* coef, float2* Y, const Filte
 
 cudaError_t run_wave_c2r(const Geo& g, const float2* Y, float* coef, const FilterWave& wv, float scale,
                          cudaStream_t st) {
-  if (fast::half_rows_ok(g.L)) return fast::rows_inv(g, Y, g.Wy, coef, g.ranges, g.eta, fast_wave_of(wv), scale, st);
+  if (half_rows(g)) return fast::rows_inv(g, Y, g.Wy, coef, g.ranges, g.eta, fast_wave_of(wv), scale, st);
   const RowShape s = row_shape(g.planL, g.RB);
   return launch_pdl(k_row_c2r<true>, dim3((g.H + g.RB - 1) / g.RB, wv.nc * wv.nf), dim3(kRowThreads), s.smem, st, g, Y,
                     coef, g.Wy, g.RB, s.ba, s.bufn, wv, scale);
@@ -494,6 +569,11 @@ cudaError_t run_wave_shrink(const Geo& g, float2* Y, float* bv, const float* thr
     const fast::Wave f = fast_wave_of(wv);
     const int rpc = fast::row_groups_per_cta(g.L), groups = (f.nv * g.H + rpc - 1) / rpc;
     return fast::row_shrink(g, std::min(groups, std::max(1, fast_row_ctas(g))), Y, bv, thr, g.Wy, f, scale, nullptr, 0, st);
+  }
+  if (g.staged) {
+    const RowShape s = row_shape(g.planL, g.RB);
+    return launch_pdl(k_row_shrink_apart, dim3((g.H + g.RB - 1) / g.RB, wv.nc * wv.nf), dim3(kRowThreads), s.smem, st, g, Y,
+                      bv, thr, g.Wy, g.RB, s.ba, s.bufn, wv, scale, gout);
   }
   const RowShape s = row_shape(g.planL, g.RB), r = row_shape(g.planLr, g.RB);
   const int bufn = std::max(s.bufn, r.bufn);
@@ -511,12 +591,31 @@ cudaError_t run_wave_l1(const Geo& g, const float2* Y, const float* lam, const F
 
 int l1_blocks(const Geo& g, int nch) { return ((g.H + g.RB - 1) / g.RB) * nch * g.eta; }
 
+namespace {
+// Rows and labels per batch of a u/w-step CTA: rows for two CTAs per SM, all
+// labels as one batch while that takes at most half of the shared memory.
+struct UstepShape {
+  int rb, kg, pad, bufn;
+  size_t smem;
+};
+UstepShape ustep_shape(const Geo& g, int K) {
+  UstepShape u{std::max(1, std::min(ustep_rows(g, K), g.H / (2 * 152))), K, 0, 0, 0};
+  for (;; --u.kg) {
+    const int B = u.kg * u.rb;
+    u.pad = row_pad(g.planL, B, K * u.rb * g.L);
+    u.bufn = gf::buf_elems(g.planL, B, u.pad);
+    u.smem = sizeof(float2) * (2 * static_cast<size_t>(u.bufn) + static_cast<size_t>(K) * u.rb * g.L);
+    if (u.kg == 1 || u.smem <= 113 * 1024) return u;
+  }
+}
+}  // namespace
+
 cudaError_t run_row_ustep(const Geo& g, const float2* T, const float* s, float* w, float* bw, float* u, float2* Ur,
                           float* stv, int K, float gamma, float scale, cudaStream_t st) {
-  const int rb = ustep_rows(g, K), pad = row_pad(g.planL, rb, K * rb * g.L), n = gf::buf_elems(g.planL, rb, pad);
-  return launch_pdl(k_row_ustep, dim3((g.H + rb - 1) / rb), dim3(kRowThreads),
-                    sizeof(float2) * (2 * static_cast<size_t>(n) + static_cast<size_t>(K) * rb * g.L), st, g, T, s, w, bw,
-                    u, Ur, stv, K, rb, gf::make_batch(g.planL, rb, pad), n, scale, gamma);
+  const UstepShape us = ustep_shape(g, K);
+  return launch_pdl(k_row_ustep, dim3((g.H + us.rb - 1) / us.rb), dim3(kRowThreads), us.smem, st, g, T, s, w, bw, u, Ur,
+                    stv, K, us.rb, us.kg, fdiv_mul(static_cast<unsigned>(us.rb)),
+                    gf::make_batch(g.planL, us.kg * us.rb, us.pad), us.bufn, scale, gamma);
 }
 
 }  // namespace shf
