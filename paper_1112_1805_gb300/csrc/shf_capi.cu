@@ -7,6 +7,7 @@
 #include <cstdio>
 #include <algorithm>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -63,17 +64,13 @@ struct shf_bank {
   Geo g;
   float* bank = nullptr;
   int2* ranges = nullptr;
+  std::vector<int2> ranges_host;  // the filters' column ranges
   float2* twH = nullptr;
   float2* twW = nullptr;
   float2* pt = nullptr;  // the plans' pass tables
   shf::FilterDesc* descs = nullptr;
   int device = 0;
-  // Temporaries of the transforms.  A pool of the bank's own keeps up to
-  // kPoolKeep bytes between calls: the device's default pool gives its memory
-  // back whenever the device is waited for, and a call after that pays for
-  // mapping it again (a 64 x 64 analysis: 256 us against 30 us in a row).
-  cudaMemPool_t pool = nullptr;
-  static constexpr unsigned long long kPoolKeep = 512ull << 20;
+  cudaMemPool_t pool = nullptr;  // the device's (DevicePool), shared by its banks
   // Heights with register-FFT column kernels: the work list of one channel's
   // filters, used by the transforms for every channel (its device arrays in
   // `chan_mem`).
@@ -84,6 +81,8 @@ struct shf_bank {
 
 struct seg_state {
   const shf_bank* bank = nullptr;
+  cudaMemPool_t pool = nullptr;  // the device's, shared
+  int device = 0;
   seg_batch* batch = nullptr;  // the batch whose graphs replay this state, if any
   Geo g;
   int K = 0, C = 0;
@@ -110,9 +109,7 @@ struct seg_state {
   bool fast = false;          // power-of-two sizes: the shf_fast.cu kernels
   bool fast_ustep = false;    // ... including the u/w-step (K <= 8)
   shf::FastPlan plan;         // fast path: static per-wave work list
-  std::vector<int2> ranges_host;  // fast path: the filters' column ranges
-  shf::WorkItem* d_items = nullptr;
-  int *d_cta_begin = nullptr, *d_tile_begin = nullptr, *d_tile_slots = nullptr;
+  int* d_lists = nullptr;     // fast path: the plan's work lists
   float2* uhat = nullptr;     // fast path: 2-D spectra of u [K][H][Wh]
   // Events recorded before every launch of an iteration (graph event nodes),
   // with the kind of the launch that follows each.
@@ -161,21 +158,73 @@ cudaError_t scratch_alloc(const shf_bank* b, float2** p, size_t count, cudaStrea
                  : cudaMallocAsync(reinterpret_cast<void**>(p), bytes, st);
 }
 
-// The bank's pool; without one (an older driver) the default pool serves.
-void make_pool(shf_bank* b) {
-  cudaMemPoolProps props = {};
-  props.allocType = cudaMemAllocationTypePinned;
-  props.handleTypes = cudaMemHandleTypeNone;
-  props.location.type = cudaMemLocationTypeDevice;
-  props.location.id = b->device;
-  unsigned long long keep = shf_bank::kPoolKeep;
-  if (cudaMemPoolCreate(&b->pool, &props) != cudaSuccess) {
-    b->pool = nullptr;
-  } else if (cudaMemPoolSetAttribute(b->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
-    cudaMemPoolDestroy(b->pool);
-    b->pool = nullptr;
+// The library's memory pool of a device, for the transforms' temporaries and the
+// states' buffers: made with the first bank there and destroyed with the last
+// bank or state.  It keeps up to kPoolKeep bytes between calls: the device's default pool
+// gives its memory back whenever the device is waited for, and a call after that
+// pays for mapping it again (a 64 x 64 analysis: 256 us against 30 us in a row).
+// Without one (an older driver) the default pool and cudaMalloc serve.
+constexpr unsigned long long kPoolKeep = 512ull << 20;
+constexpr int kMaxDevices = 64;
+struct DevicePool {
+  cudaMemPool_t pool = nullptr;
+  int users = 0;
+};
+std::mutex g_pool_mu;
+DevicePool g_pools[kMaxDevices];
+
+cudaMemPool_t acquire_pool(int device) {
+  if (device < 0 || device >= kMaxDevices) return nullptr;
+  std::lock_guard<std::mutex> lock(g_pool_mu);
+  DevicePool& d = g_pools[device];
+  if (!d.pool) {
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.handleTypes = cudaMemHandleTypeNone;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = device;
+    unsigned long long keep = kPoolKeep;
+    if (cudaMemPoolCreate(&d.pool, &props) != cudaSuccess) {
+      d.pool = nullptr;
+    } else if (cudaMemPoolSetAttribute(d.pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+      cudaMemPoolDestroy(d.pool);
+      d.pool = nullptr;
+    }
+    cudaGetLastError();
+    if (!d.pool) return nullptr;
   }
-  cudaGetLastError();
+  ++d.users;
+  return d.pool;
+}
+
+// After the device has been waited for.
+void release_pool(int device) {
+  std::lock_guard<std::mutex> lock(g_pool_mu);
+  DevicePool& d = g_pools[device];
+  if (--d.users > 0) return;
+  cudaStreamSynchronize(nullptr);  // the states' frees
+  cudaMemPoolDestroy(d.pool);
+  d.pool = nullptr;
+}
+
+// A work list's four arrays one after another (the items as four ints each);
+// at[i]: where array i starts.
+std::vector<int> pack_lists(const std::vector<shf::WorkItem>& items, const std::vector<int>& cta_begin,
+                            const std::vector<int>& tile_begin, const std::vector<int>& tile_slots, size_t (&at)[3]) {
+  std::vector<int> all(4 * items.size());
+  std::memcpy(all.data(), items.data(), sizeof(shf::WorkItem) * items.size());
+  const std::vector<int>* parts[] = {&cta_begin, &tile_begin, &tile_slots};
+  for (int i = 0; i < 3; ++i) {
+    at[i] = all.size();
+    all.insert(all.end(), parts[i]->begin(), parts[i]->end());
+  }
+  return all;
+}
+void set_lists(shf::FastPlan* p, const int* mem, const size_t (&at)[3]) {
+  p->items = reinterpret_cast<const shf::WorkItem*>(mem);
+  p->cta_begin = mem + at[0];
+  p->tile_begin = mem + at[1];
+  p->tile_slots = mem + at[2];
 }
 
 // The single-channel work list of a bank whose ranges are known; synchronous.
@@ -188,18 +237,12 @@ int build_channel_plan(shf_bank* b, const std::vector<int2>& ranges) {
   std::vector<shf::WorkItem> items;
   std::vector<int> cta_begin, tile_begin, tile_slots;
   shf::build_fast_plan(g, ranges.data(), 1, &p, &items, &cta_begin, &tile_begin, &tile_slots);
-  // one upload: the items (four ints each), then the ranges and slot lists
-  std::vector<int> all(4 * items.size());
-  std::memcpy(all.data(), items.data(), sizeof(shf::WorkItem) * items.size());
-  const size_t at0 = all.size(), at1 = at0 + cta_begin.size(), at2 = at1 + tile_begin.size();
-  for (const std::vector<int>* v : {&cta_begin, &tile_begin, &tile_slots}) all.insert(all.end(), v->begin(), v->end());
+  size_t at[3];
+  const std::vector<int> all = pack_lists(items, cta_begin, tile_begin, tile_slots, at);
   int rc = dev_alloc(&b->chan_mem, all.size(), "work list");
   if (rc) return rc;
   SHF_CK(cudaMemcpy(b->chan_mem, all.data(), sizeof(int) * all.size(), cudaMemcpyHostToDevice));
-  p.items = reinterpret_cast<const shf::WorkItem*>(b->chan_mem);
-  p.cta_begin = b->chan_mem + at0;
-  p.tile_begin = b->chan_mem + at1;
-  p.tile_slots = b->chan_mem + at2;
+  set_lists(&p, b->chan_mem, at);
   b->chan_ok = true;
   return SHF_OK;
 }
@@ -247,7 +290,7 @@ int shfilters_build(int H, int W, int J, void* stream, shf_bank** out) {
   auto* b = new shf_bank();
   b->g = g;
   b->device = device;
-  make_pool(b);
+  b->pool = acquire_pool(device);
   std::vector<shf::FilterDesc> d(g.eta);
   shf::filter_descs(J, d.data());
   if ((rc = dev_alloc(&b->bank, static_cast<size_t>(g.eta) * H * g.Wh, "bank")) ||
@@ -271,7 +314,8 @@ int shfilters_build(int H, int W, int J, void* stream, shf_bank** out) {
   if (e == cudaSuccess) e = shf::launch_pass_tables(&b->g, b->pt, st);
   if (e == cudaSuccess) e = shf::launch_build_bank(b->bank, b->g, b->descs, st);
   if (e == cudaSuccess) e = shf::launch_filter_ranges(b->bank, b->g, b->ranges, st);
-  std::vector<int2> ranges(g.eta);
+  std::vector<int2>& ranges = b->ranges_host;
+  ranges.resize(g.eta);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(ranges.data(), b->ranges, sizeof(int2) * g.eta, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // d and ranges are host temporaries
@@ -296,7 +340,7 @@ int shfilters_destroy(shf_bank* b) {
   cudaFree(b->twW);
   cudaFree(b->pt);
   cudaFree(b->chan_mem);
-  if (b->pool) cudaMemPoolDestroy(b->pool);
+  if (b->pool) release_pool(b->device);
   cudaFree(b->descs);
   cudaFree(b->ranges);
   delete b;
@@ -446,36 +490,45 @@ int shearlet_synthesize(const shf_bank* b, const float* coef, int nch, float* u,
 
 namespace {
 
+// Returns a state's buffer; the caller has waited for its users.  (To the pool in
+// the order of the legacy stream: the state's own stream may be gone by now.)
+void state_free(const seg_state* st, void* p) {
+  if (!p) return;
+  if (st->pool)
+    cudaFreeAsync(p, nullptr);
+  else
+    cudaFree(p);
+}
+
 void free_state(seg_state* s) {
+  cudaDeviceSynchronize();
   if (s->exec) cudaGraphExecDestroy(s->exec);
   if (s->exec_timed) cudaGraphExecDestroy(s->exec_timed);
   for (cudaEvent_t e : s->ev)
     if (e) cudaEventDestroy(e);
-  cudaFree(s->uhat);
-  cudaFree(s->d_items);
-  cudaFree(s->d_cta_begin);
-  cudaFree(s->d_tile_begin);
-  cudaFree(s->d_tile_slots);
-  cudaFree(s->un_Y);
-  cudaFree(s->un_partial);
-  cudaFree(s->un_pt);
+  state_free(s, s->uhat);
+  state_free(s, s->d_lists);
+  state_free(s, s->un_Y);
+  state_free(s, s->un_partial);
+  state_free(s, s->un_pt);
   if (s->un_fwd_exec) cudaGraphExecDestroy(s->un_fwd_exec);
   if (s->un_bwd_exec) cudaGraphExecDestroy(s->un_bwd_exec);
-  cudaFree(s->un_mem);
-  for (float* p : s->ck_bv) cudaFree(p);
-  for (float* p : s->ck_w) cudaFree(p);
-  for (float* p : s->ck_bw) cudaFree(p);
-  for (float2* p : s->ck_T) cudaFree(p);
+  state_free(s, s->un_mem);
+  for (float* p : s->ck_bv) state_free(s, p);
+  for (float* p : s->ck_w) state_free(s, p);
+  for (float* p : s->ck_bw) state_free(s, p);
+  for (float2* p : s->ck_T) state_free(s, p);
   float* fl[] = {s->f, s->s, s->bv, s->w, s->bw, s->u, s->stv, s->thr, s->lam, s->gap};
-  for (float* p : fl) cudaFree(p);
-  cudaFree(s->Ur);
-  cudaFree(s->Y);
-  cudaFree(s->partial);
-  cudaFree(s->T);
-  cudaFree(s->labels);
-  cudaFree(s->flag);
-  cudaFree(s->red);
+  for (float* p : fl) state_free(s, p);
+  state_free(s, s->Ur);
+  state_free(s, s->Y);
+  state_free(s, s->partial);
+  state_free(s, s->T);
+  state_free(s, s->labels);
+  state_free(s, s->flag);
+  state_free(s, s->red);
   if (s->own_stream && s->stream) cudaStreamDestroy(s->stream);
+  if (s->pool) release_pool(s->device);
   delete s;
 }
 
@@ -670,6 +723,23 @@ cudaGraphExec_t capture_work(seg_state* st, F enqueue) {
   return exec;
 }
 
+// A state's buffers come from the device's pool in the order of its stream: a training step that makes a state per image then
+// maps no memory.
+extern "C++" template <typename T>
+int state_alloc(seg_state* st, T** p, size_t count, const char* what) {
+  if (!st->pool) return dev_alloc(p, count, what);
+  *p = nullptr;
+  if (count == 0) return SHF_OK;
+  cudaError_t e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(p), count * sizeof(T), st->pool, st->stream);
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    *p = nullptr;
+    return fail(e == cudaErrorMemoryAllocation ? SHF_ERR_OOM : SHF_ERR_CUDA,
+                std::string("cudaMallocFromPoolAsync(") + what + "): " + cudaGetErrorString(e));
+  }
+  return SHF_OK;
+}
+
 // Fast path: builds the work list for (wave_mib, col_ctas_per_sm) and
 // allocates what depends on it (one wave of coefficient spectra Y, the
 // partial tiles, the device work list); the previous buffers are released
@@ -691,60 +761,40 @@ int install_fast_plan(seg_state* st, int wave_mib, int col_ctas_per_sm, int row_
     return fail(SHF_ERR_CUDA, "install_fast_plan: no resident CTA");
   std::vector<shf::WorkItem> h_items;
   std::vector<int> h_cta_begin, h_tile_begin, h_tile_slots;
-  shf::build_fast_plan(g, st->ranges_host.data(), st->K, &plan, &h_items, &h_cta_begin, &h_tile_begin,
+  shf::build_fast_plan(g, st->bank->ranges_host.data(), st->K, &plan, &h_items, &h_cta_begin, &h_tile_begin,
                        &h_tile_slots);
   const size_t Phs = static_cast<size_t>(g.H) * shf::fast_pitch(g);
   const size_t y_elems = Phs * static_cast<size_t>(std::max(plan.y_planes, 1));
   const size_t partial_elems = static_cast<size_t>(std::max(plan.nslots, 1)) * g.H * shf::fast_tile(g);
+  size_t at[3];
+  const std::vector<int> lists = pack_lists(h_items, h_cta_begin, h_tile_begin, h_tile_slots, at);
   float2 *Y = nullptr, *partial = nullptr;
-  shf::WorkItem* items = nullptr;
-  int *cta_begin = nullptr, *tile_begin = nullptr, *tile_slots = nullptr;
+  int* d_lists = nullptr;
   auto release = [&]() {
-    cudaFree(Y);
-    cudaFree(partial);
-    cudaFree(items);
-    cudaFree(cta_begin);
-    cudaFree(tile_begin);
-    cudaFree(tile_slots);
+    state_free(st, Y);
+    state_free(st, partial);
+    state_free(st, d_lists);
   };
   int rc;
-  if ((rc = dev_alloc(&Y, y_elems, "Y")) || (rc = dev_alloc(&partial, partial_elems, "partial")) ||
-      (rc = dev_alloc(&items, h_items.size(), "work items")) ||
-      (rc = dev_alloc(&cta_begin, h_cta_begin.size(), "work ranges")) ||
-      (rc = dev_alloc(&tile_begin, h_tile_begin.size(), "tile_begin")) ||
-      (rc = dev_alloc(&tile_slots, h_tile_slots.size(), "tile_slots"))) {
+  if ((rc = state_alloc(st, &Y, y_elems, "Y")) || (rc = state_alloc(st, &partial, partial_elems, "partial")) ||
+      (rc = state_alloc(st, &d_lists, lists.size(), "work lists"))) {
     release();
     return rc;
   }
-  cudaError_t e = cudaMemcpy(items, h_items.data(), sizeof(shf::WorkItem) * h_items.size(), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess)
-    e = cudaMemcpy(cta_begin, h_cta_begin.data(), sizeof(int) * h_cta_begin.size(), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess)
-    e = cudaMemcpy(tile_begin, h_tile_begin.data(), sizeof(int) * h_tile_begin.size(), cudaMemcpyHostToDevice);
-  if (e == cudaSuccess)
-    e = cudaMemcpy(tile_slots, h_tile_slots.data(), sizeof(int) * h_tile_slots.size(), cudaMemcpyHostToDevice);
+  cudaError_t e = cudaMemcpyAsync(d_lists, lists.data(), sizeof(int) * lists.size(), cudaMemcpyHostToDevice, st->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st->stream);  // the old buffers may still be in use
   if (e != cudaSuccess) {
     release();
     return fail(SHF_ERR_CUDA, std::string("install_fast_plan: ") + cudaGetErrorString(e));
   }
   drop_graphs(st);
-  cudaFree(st->Y);
-  cudaFree(st->partial);
-  cudaFree(st->d_items);
-  cudaFree(st->d_cta_begin);
-  cudaFree(st->d_tile_begin);
-  cudaFree(st->d_tile_slots);
+  state_free(st, st->Y);
+  state_free(st, st->partial);
+  state_free(st, st->d_lists);
   st->Y = Y;
   st->partial = partial;
-  st->d_items = items;
-  st->d_cta_begin = cta_begin;
-  st->d_tile_begin = tile_begin;
-  st->d_tile_slots = tile_slots;
-  plan.items = items;
-  plan.cta_begin = cta_begin;
-  plan.tile_begin = tile_begin;
-  plan.tile_slots = tile_slots;
+  st->d_lists = d_lists;
+  set_lists(&plan, d_lists, at);
   st->plan = plan;
   return SHF_OK;
 }
@@ -770,21 +820,21 @@ int install_generic_plan(seg_state* st, int TC, int RB, int groups) {
   groups = normalise_groups(g.eta, groups);
   std::vector<shf::FilterWave> waves = shf::general_waves(g, st->K, groups);
   float2 *partial = nullptr, *Y = nullptr;
-  int rc = dev_alloc(&partial, st->Ph() * st->K * static_cast<size_t>(groups), "partial");
-  if (!rc) rc = dev_alloc(&Y, shf::wave_planes(waves) * g.H * g.Wy, "Y");
+  int rc = state_alloc(st, &partial, st->Ph() * st->K * static_cast<size_t>(groups), "partial");
+  if (!rc) rc = state_alloc(st, &Y, shf::wave_planes(waves) * g.H * g.Wy, "Y");
   if (rc) {
-    cudaFree(partial);
+    state_free(st, partial);
     return rc;
   }
   cudaError_t e = cudaStreamSynchronize(st->stream);
   if (e != cudaSuccess) {
-    cudaFree(partial);
-    cudaFree(Y);
+    state_free(st, partial);
+    state_free(st, Y);
     return fail(SHF_ERR_CUDA, std::string("install_generic_plan: ") + cudaGetErrorString(e));
   }
   drop_graphs(st);
-  cudaFree(st->partial);
-  cudaFree(st->Y);
+  state_free(st, st->partial);
+  state_free(st, st->Y);
   st->partial = partial;
   st->Y = Y;
   st->g = g;
@@ -868,6 +918,8 @@ int seg_admm_init(const shf_bank* b, const float* f, int C, const float* codeboo
       return fail(SHF_ERR_ARG, "Lambda must be finite and non-negative");
   auto* st = new seg_state();
   st->bank = b;
+  st->device = b->device;
+  st->pool = acquire_pool(b->device);
   st->g = b->g;
   st->K = K;
   st->C = C;
@@ -882,7 +934,7 @@ int seg_admm_init(const shf_bank* b, const float* f, int C, const float* codeboo
   } else {
     cudaError_t e = cudaStreamCreateWithFlags(&st->stream, cudaStreamNonBlocking);
     if (e != cudaSuccess) {
-      delete st;
+      free_state(st);
       return fail(SHF_ERR_CUDA, std::string("cudaStreamCreate: ") + cudaGetErrorString(e));
     }
     st->own_stream = true;
@@ -892,31 +944,22 @@ int seg_admm_init(const shf_bank* b, const float* f, int C, const float* codeboo
   st->groups = shf::default_groups(g, K);
   st->fast = shf::fast_path_ok(g);
   st->fast_ustep = shf::fast_ustep_ok(g, K);
-  // the fast path's work list is built from the filters' column ranges
-  if (st->fast) {
-    st->ranges_host.resize(g.eta);
-    cudaError_t e = cudaMemcpy(st->ranges_host.data(), g.ranges, sizeof(int2) * g.eta, cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) {
-      free_state(st);
-      return fail(SHF_ERR_CUDA, std::string("seg_admm_init: ") + cudaGetErrorString(e));
-    }
-  }
   if (!st->fast) st->waves = shf::general_waves(g, K, st->groups);
   int rc;
-  if ((rc = dev_alloc(&st->f, P * C, "f")) || (rc = dev_alloc(&st->s, P * K, "s")) ||
-      (rc = dev_alloc(&st->bv, P * K * g.eta, "b_v")) || (rc = dev_alloc(&st->w, P * K, "w")) ||
-      (rc = dev_alloc(&st->bw, P * K, "b_w")) || (rc = dev_alloc(&st->u, P * K, "u")) ||
-      (rc = dev_alloc(&st->stv, P * K, "stv")) || (rc = dev_alloc(&st->Ur, Ph * K, "Ur")) ||
-      (rc = dev_alloc(&st->T, Ph * K, "T")) ||
-      (st->fast && (rc = dev_alloc(&st->uhat, static_cast<size_t>(g.H) * shf::fast_pitch(g) * K, "uhat"))) ||
+  if ((rc = state_alloc(st, &st->f, P * C, "f")) || (rc = state_alloc(st, &st->s, P * K, "s")) ||
+      (rc = state_alloc(st, &st->bv, P * K * g.eta, "b_v")) || (rc = state_alloc(st, &st->w, P * K, "w")) ||
+      (rc = state_alloc(st, &st->bw, P * K, "b_w")) || (rc = state_alloc(st, &st->u, P * K, "u")) ||
+      (rc = state_alloc(st, &st->stv, P * K, "stv")) || (rc = state_alloc(st, &st->Ur, Ph * K, "Ur")) ||
+      (rc = state_alloc(st, &st->T, Ph * K, "T")) ||
+      (st->fast && (rc = state_alloc(st, &st->uhat, static_cast<size_t>(g.H) * shf::fast_pitch(g) * K, "uhat"))) ||
       // one wave's coefficient spectra and one partial sum per filter group on
       // the general path (the fast path's come with its plan)
-      (!st->fast && (rc = dev_alloc(&st->Y, shf::wave_planes(st->waves) * g.H * g.Wy, "Y"))) ||
-      (!st->fast && (rc = dev_alloc(&st->partial, Ph * K * static_cast<size_t>(st->groups), "partial"))) ||
+      (!st->fast && (rc = state_alloc(st, &st->Y, shf::wave_planes(st->waves) * g.H * g.Wy, "Y"))) ||
+      (!st->fast && (rc = state_alloc(st, &st->partial, Ph * K * static_cast<size_t>(st->groups), "partial"))) ||
       (st->fast && (rc = install_fast_plan(st, shf::kDefaultWaveMiB, 0))) ||
-      (rc = dev_alloc(&st->thr, g.eta, "thr")) || (rc = dev_alloc(&st->lam, g.eta, "lam")) ||
-      (rc = dev_alloc(&st->gap, P, "gap")) || (rc = dev_alloc(&st->labels, P, "labels")) ||
-      (rc = dev_alloc(&st->flag, 1, "flag")) || (rc = dev_alloc(&st->red, 2 + 512, "red"))) {
+      (rc = state_alloc(st, &st->thr, g.eta, "thr")) || (rc = state_alloc(st, &st->lam, g.eta, "lam")) ||
+      (rc = state_alloc(st, &st->gap, P, "gap")) || (rc = state_alloc(st, &st->labels, P, "labels")) ||
+      (rc = state_alloc(st, &st->flag, 1, "flag")) || (rc = state_alloc(st, &st->red, 2 + 512, "red"))) {
     free_state(st);
     return rc;
   }
@@ -1610,11 +1653,11 @@ int seg_admm_unrolled_fwd(seg_state* st, int T, int ckpt_every) {
       return fail(SHF_ERR_SIZE, "unsupported geometry");
     st->un_g.planLr = st->un_g.planL;
     st->un_waves = shf::general_waves(g, st->K, groups);
-    if ((rc = dev_alloc(&st->un_pt, shf::pass_table_entries(st->un_g), "pass tables")) ||
-        (rc = dev_alloc(&st->un_Y, shf::wave_planes(st->un_waves) * g.H * g.Wy, "unrolled scratch")) ||
-        (rc = dev_alloc(&st->un_partial, Ph * st->K * static_cast<size_t>(groups), "unrolled partials"))) {
-      cudaFree(st->un_pt);
-      cudaFree(st->un_Y);
+    if ((rc = state_alloc(st, &st->un_pt, shf::pass_table_entries(st->un_g), "pass tables")) ||
+        (rc = state_alloc(st, &st->un_Y, shf::wave_planes(st->un_waves) * g.H * g.Wy, "unrolled scratch")) ||
+        (rc = state_alloc(st, &st->un_partial, Ph * st->K * static_cast<size_t>(groups), "unrolled partials"))) {
+      state_free(st, st->un_pt);
+      state_free(st, st->un_Y);
       st->un_pt = nullptr;
       st->un_Y = nullptr;
       return rc;
@@ -1626,12 +1669,12 @@ int seg_admm_unrolled_fwd(seg_state* st, int T, int ckpt_every) {
   while (static_cast<int>(st->ck_bv.size()) < nseg) {
     float *bv = nullptr, *w = nullptr, *bw = nullptr;
     float2* Tt = nullptr;
-    if ((rc = dev_alloc(&bv, NC, "checkpoint")) || (rc = dev_alloc(&w, KP, "checkpoint")) ||
-        (rc = dev_alloc(&bw, KP, "checkpoint")) || (rc = dev_alloc(&Tt, Ph * st->K, "checkpoint"))) {
-      cudaFree(bv);
-      cudaFree(w);
-      cudaFree(bw);
-      cudaFree(Tt);
+    if ((rc = state_alloc(st, &bv, NC, "checkpoint")) || (rc = state_alloc(st, &w, KP, "checkpoint")) ||
+        (rc = state_alloc(st, &bw, KP, "checkpoint")) || (rc = state_alloc(st, &Tt, Ph * st->K, "checkpoint"))) {
+      state_free(st, bv);
+      state_free(st, w);
+      state_free(st, bw);
+      state_free(st, Tt);
       return rc;
     }
     st->ck_bv.push_back(bv);
@@ -1639,13 +1682,18 @@ int seg_admm_unrolled_fwd(seg_state* st, int T, int ckpt_every) {
     st->ck_bw.push_back(bw);
     st->ck_T.push_back(Tt);
   }
-  // one graph per (T, ckpt), replayed by later calls
-  if (!(st->un_fwd_exec && st->un_fwd_key[0] == T && st->un_fwd_key[1] == ckpt_every)) {
-    if (st->un_fwd_exec) cudaGraphExecDestroy(st->un_fwd_exec);
-    st->un_fwd_exec = capture_work(st, [&]() { return enqueue_unrolled_fwd(st, T, ckpt_every); });
-    st->un_fwd_key[0] = T;
-    st->un_fwd_key[1] = ckpt_every;
+  // the first sweep of a (T, ckpt) is launched directly (a state made for one
+  // training step never pays for a graph: capturing and instantiating takes the
+  // host longer than launching), the second one captured, later ones replayed
+  const bool again = st->un_fwd_key[0] == T && st->un_fwd_key[1] == ckpt_every;
+  if (!again && st->un_fwd_exec) {
+    cudaGraphExecDestroy(st->un_fwd_exec);
+    st->un_fwd_exec = nullptr;
   }
+  if (again && !st->un_fwd_exec)
+    st->un_fwd_exec = capture_work(st, [&]() { return enqueue_unrolled_fwd(st, T, ckpt_every); });
+  st->un_fwd_key[0] = T;
+  st->un_fwd_key[1] = ckpt_every;
   if (st->un_fwd_exec)
     SHF_CK(cudaGraphLaunch(st->un_fwd_exec, st->stream));
   else
@@ -1666,21 +1714,23 @@ int seg_admm_unrolled_bwd_enqueue(seg_state* st, const float* dL_dw) {
     SHF_CK(cudaStreamSynchronize(s));
     if (st->un_bwd_exec) cudaGraphExecDestroy(st->un_bwd_exec);
     st->un_bwd_exec = nullptr;
-    cudaFree(st->un_mem);
+    state_free(st, st->un_mem);
     st->un_mem = nullptr;
     st->un_mem_bytes = 0;
-    int rc = dev_alloc(&st->un_mem, U.total, "reverse-sweep scratch");
+    int rc = state_alloc(st, &st->un_mem, U.total, "reverse-sweep scratch");
     if (rc) return rc;
     st->un_mem_bytes = U.total;
   }
   SHF_CK(cudaMemcpyAsync(st->un_mem + U.wbar, dL_dw, sizeof(float) * KP, cudaMemcpyDeviceToDevice, s));
-  // one graph per (T, ckpt), replayed by later calls
-  if (!(st->un_bwd_exec && st->un_bwd_key[0] == st->un_T && st->un_bwd_key[1] == st->un_ck)) {
-    if (st->un_bwd_exec) cudaGraphExecDestroy(st->un_bwd_exec);
-    st->un_bwd_exec = capture_work(st, [&]() { return enqueue_unrolled_bwd(st, U); });
-    st->un_bwd_key[0] = st->un_T;
-    st->un_bwd_key[1] = st->un_ck;
+  // as the forward sweep: directly, then captured, then replayed
+  const bool again = st->un_bwd_key[0] == st->un_T && st->un_bwd_key[1] == st->un_ck;
+  if (!again && st->un_bwd_exec) {
+    cudaGraphExecDestroy(st->un_bwd_exec);
+    st->un_bwd_exec = nullptr;
   }
+  if (again && !st->un_bwd_exec) st->un_bwd_exec = capture_work(st, [&]() { return enqueue_unrolled_bwd(st, U); });
+  st->un_bwd_key[0] = st->un_T;
+  st->un_bwd_key[1] = st->un_ck;
   SHF_CK(st->un_bwd_exec ? cudaGraphLaunch(st->un_bwd_exec, s) : enqueue_unrolled_bwd(st, U));
   st->un_bwd_pending = true;
   return SHF_OK;
