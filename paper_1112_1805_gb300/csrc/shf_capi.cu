@@ -82,6 +82,7 @@ struct shf_bank {
 struct seg_state {
   const shf_bank* bank = nullptr;
   cudaMemPool_t pool = nullptr;  // the device's, shared
+  std::vector<void*> direct;     // buffers too large for it (cudaMalloc)
   int device = 0;
   seg_batch* batch = nullptr;  // the batch whose graphs replay this state, if any
   Geo g;
@@ -231,6 +232,7 @@ void set_lists(shf::FastPlan* p, const int* mem, const size_t (&at)[3]) {
 int build_channel_plan(shf_bank* b, const std::vector<int2>& ranges) {
   const Geo& g = b->g;
   shf::FastPlan& p = b->chan;
+  p.wave_mib = shf::default_fast_plan(g).wave_mib;
   p.col_ctas = shf::fast_col_ctas(g, 0);
   p.fan_ctas = shf::fast_fan_ctas(g);
   if (p.col_ctas < 1 || p.fan_ctas < 1) return fail(SHF_ERR_CUDA, "shfilters_build: no resident CTA");
@@ -492,12 +494,15 @@ namespace {
 
 // Returns a state's buffer; the caller has waited for its users.  (To the pool in
 // the order of the legacy stream: the state's own stream may be gone by now.)
-void state_free(const seg_state* st, void* p) {
+void state_free(seg_state* st, void* p) {
   if (!p) return;
-  if (st->pool)
+  const auto it = std::find(st->direct.begin(), st->direct.end(), p);
+  if (it == st->direct.end()) {
     cudaFreeAsync(p, nullptr);
-  else
+  } else {
+    st->direct.erase(it);
     cudaFree(p);
+  }
 }
 
 void free_state(seg_state* s) {
@@ -724,12 +729,18 @@ cudaGraphExec_t capture_work(seg_state* st, F enqueue) {
 }
 
 // A state's buffers come from the device's pool in the order of its stream: a training step that makes a state per image then
-// maps no memory.
+// maps no memory.  Buffers that the pool would not keep anyway are mapped by
+// cudaMalloc, which takes fewer and larger pages (the 17 GB of a 2048 x 2048, K =
+// 8 state: 43 ms of preparation against 59).
 extern "C++" template <typename T>
 int state_alloc(seg_state* st, T** p, size_t count, const char* what) {
-  if (!st->pool) return dev_alloc(p, count, what);
   *p = nullptr;
   if (count == 0) return SHF_OK;
+  if (!st->pool || count * sizeof(T) > kPoolKeep / 2) {
+    const int rc = dev_alloc(p, count, what);
+    if (!rc) st->direct.push_back(*p);
+    return rc;
+  }
   cudaError_t e = cudaMallocFromPoolAsync(reinterpret_cast<void**>(p), count * sizeof(T), st->pool, st->stream);
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -945,6 +956,7 @@ int seg_admm_init(const shf_bank* b, const float* f, int C, const float* codeboo
   st->fast = shf::fast_path_ok(g);
   st->fast_ustep = shf::fast_ustep_ok(g, K);
   if (!st->fast) st->waves = shf::general_waves(g, K, st->groups);
+  const shf::FastPlan def = shf::default_fast_plan(g);
   int rc;
   if ((rc = state_alloc(st, &st->f, P * C, "f")) || (rc = state_alloc(st, &st->s, P * K, "s")) ||
       (rc = state_alloc(st, &st->bv, P * K * g.eta, "b_v")) || (rc = state_alloc(st, &st->w, P * K, "w")) ||
@@ -956,7 +968,7 @@ int seg_admm_init(const shf_bank* b, const float* f, int C, const float* codeboo
       // the general path (the fast path's come with its plan)
       (!st->fast && (rc = state_alloc(st, &st->Y, shf::wave_planes(st->waves) * g.H * g.Wy, "Y"))) ||
       (!st->fast && (rc = state_alloc(st, &st->partial, Ph * K * static_cast<size_t>(st->groups), "partial"))) ||
-      (st->fast && (rc = install_fast_plan(st, shf::kDefaultWaveMiB, 0))) ||
+      (st->fast && (rc = install_fast_plan(st, def.wave_mib, 0, def.row_kernel, def.col_kernel, def.serial))) ||
       (rc = state_alloc(st, &st->thr, g.eta, "thr")) || (rc = state_alloc(st, &st->lam, g.eta, "lam")) ||
       (rc = state_alloc(st, &st->gap, P, "gap")) || (rc = state_alloc(st, &st->labels, P, "labels")) ||
       (rc = state_alloc(st, &st->flag, 1, "flag")) || (rc = state_alloc(st, &st->red, 2 + 512, "red"))) {
@@ -1098,7 +1110,7 @@ std::vector<seg_plan> plan_candidates(const seg_state* st, const seg_plan& base,
       // wave budgets that give distinct waves (filters per wave of one label,
       // or labels per wave)
       std::vector<int> seen;
-      for (int mib : {16, 32, 64, 96, 128, 192, 256, 384}) {
+      for (int mib : {16, 32, 64, 96, 128, 192, 256, 384, 512, 1024}) {
         const int w = shf::fast_wave(g, mib), nl = shf::fast_wave_labels(g, mib, st->K);
         const int sig = nl > 1 ? -nl : (g.eta + w - 1) / w;
         if (std::find(seen.begin(), seen.end(), sig) != seen.end()) continue;

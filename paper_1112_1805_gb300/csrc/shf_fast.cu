@@ -26,6 +26,28 @@ namespace shf {
 
 int fast_pitch(const Geo& g) { return (g.Wh + 7) & ~7; }
 
+// Waves beyond the L2 pay where the column kernels read whole 64-byte row
+// segments (tiles of 8 columns, H <= 1024): the spectra's trips to DRAM cost less
+// than the launches' tails, which every wave has.  An iteration in us with waves
+// of 128 / 512 / 1024 MiB: 512 x 512, K = 4 285 / 271 / 270, K = 8 562 / 512 / 514;
+// 384 x 640, K = 5 488 / 452 / 452; 768 x 1024, K = 3 836 / 737 / 734; 1024 x
+// 1024, K = 4, J = 5 2630 / 2421 / 2216; 1024 x 2048 5846 / 5569 / 5468.  With
+// tiles of 4 columns 128 MiB stays (2048 x 2048, K = 8 27.5 / 33.4 ms; 2048 x
+// 1024 5.90 / 6.67), but for up to 2^20 pixels 512 (1536 x 512 931 / 888; 2048 x
+// 512 1458 / 1406).  At half width 1024 and from 2^20 pixels on, the 32-value
+// v-step in plain stream order: 512 x 2048 1307 -> 1217, 1024 x 2048 5468 -> 5156
+// (at 512 MiB), 2048 x 2048, K = 8 27.5 -> 24.9 ms.
+FastPlan default_fast_plan(const Geo& g) {
+  FastPlan p;
+  const long pixels = static_cast<long>(g.H) * g.W;
+  p.wave_mib = fast_tile(g) == 8 ? 1024 : (pixels <= (1l << 20) ? 512 : kWaveMiB);
+  if (g.L == 1024 && pixels >= (1l << 20)) {
+    p.row_kernel = kRowV;
+    p.serial = 1;
+  }
+  return p;
+}
+
 bool fast_path_ok(const Geo& g) { return reg::supported_col(g.H) && reg::supported(g.L); }
 
 int fast_tile(const Geo& g) { return reg::col_batch(g.H); }

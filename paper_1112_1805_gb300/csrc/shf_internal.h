@@ -171,12 +171,12 @@ struct WorkItem {
   int slot;    // partial-sum slot of the item's run
   int label;
 };
-constexpr int kDefaultWaveMiB = 128;  // coefficient spectra per wave
+constexpr int kWaveMiB = 128;  // coefficient spectra per wave, unless default_fast_plan says otherwise
 // FFT kernel variants of a plan (0: the default for the size).
 enum RowKernel { kRowDefault = 0, kRow8 = 1, kRow16 = 2, kRowPair = 3, kRowV = 4 };
 enum ColKernel { kColDefault = 0, kCol8 = 1, kCol16 = 2, kColV = 3 };
 struct FastPlan {
-  int wave_mib = kDefaultWaveMiB;
+  int wave_mib = kWaveMiB;
   int col_ctas_per_sm = 0;  // CTAs per SM of the column launches (0: as many as fit)
   int row_kernel = kRowDefault;  // forward v-step transform (RowKernel)
   int col_kernel = kColDefault;  // fan and gather transforms (ColKernel)
@@ -213,6 +213,9 @@ struct PdlScope {
   PdlScope(const PdlScope&) = delete;
   PdlScope& operator=(const PdlScope&) = delete;
 };
+
+// The plan fields a state starts with (wave budget, v-step kernel, launches).
+FastPlan default_fast_plan(const Geo& g);
 
 // Fast path for power-of-two sizes (shf_fast.cu).
 bool fast_path_ok(const Geo& g);
