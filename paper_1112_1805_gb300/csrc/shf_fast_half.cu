@@ -1,6 +1,6 @@
 // Single row transforms on the register FFTs of the v-step: half spectra ->
 // real rows and real rows -> half spectra, for the half widths with 16 values
-// per thread (64, 128, 256, 512) and with 12, 20 or 32 (shf_fftv.cuh: 3 2^a,
+// per thread (32, 64, 128, 256, 512) and with 12, 20 or 32 (shf_fftv.cuh: 3 2^a,
 // 5 2^a and 1024 with groups inside a warp).  The analysis, the synthesis, the
 // reverse sweep's S Qbar and S^T and the readouts use them; other half widths
 // take the staged kernels of shf_transform.cu.
@@ -16,58 +16,11 @@
 #include <algorithm>
 
 #include "shf_fast.h"
-#include "shf_fft16.cuh"
-#include "shf_fftv.cuh"
+#include "shf_rows.cuh"
 
 namespace shf {
 namespace fast {
 namespace {
-
-__host__ __device__ constexpr bool half16(int L) { return L == 64 || L == 128 || L == 256 || L == 512; }
-__host__ __device__ constexpr bool half_ok(int L) { return half16(L) || rv::supported(L); }
-__host__ __device__ constexpr int even2(int n) { return (n + 1) & ~1; }
-
-// The transform of one row: 16 values per thread or V.
-template <int L, bool R16 = half16(L)>
-struct Rows;
-template <int L>
-struct Rows<L, true> {
-  static constexpr int V = 16;
-  static constexpr int BUF = even2(reg::row_buf(L));
-  static constexpr int PT = even2(r16::Passes<L>::TWSIZE);
-  __device__ static void tables(float2* pt, const float2* tw) {
-    r16::build_pass_twiddles<L, 2>(pt, tw, threadIdx.x, blockDim.x);
-  }
-  template <int S>
-  __device__ static void fft(float2 (&v)[16], int tt, float2* fb, const float2* pt) {
-    r16::row_fft<L, S>(v, tt, fb, pt, 0);
-  }
-  __device__ static void pack(float2 (&v)[16], int k, int tt, float2 ra, float2 rb, float2& prev, const float2* tw) {
-    r16::pack_step<L>(v, k, tt, ra, rb, prev, tw);
-  }
-  __device__ static float2 unpack(const float2 (&v)[16], int q, int tt, float2 r, const float2* tw) {
-    return r16::unpack_value<L>(v, q, tt, r, tw);
-  }
-};
-template <int L>
-struct Rows<L, false> {
-  static constexpr int V = rv::vals_for(L);
-  static constexpr int BUF = even2(rv::row_buf(L));
-  static constexpr int PT = even2(rv::Passes<L>::TWSIZE);
-  __device__ static void tables(float2* pt, const float2* tw) {
-    rv::build_pass_twiddles<L, 2>(pt, tw, threadIdx.x, blockDim.x);
-  }
-  template <int S>
-  __device__ static void fft(float2 (&v)[V], int tt, float2* fb, const float2* pt) {
-    rv::row_fft<L, S>(v, tt, fb, pt);
-  }
-  __device__ static void pack(float2 (&v)[V], int k, int tt, float2 ra, float2 rb, float2& prev, const float2* tw) {
-    rv::pack_step<L>(v, k, tt, ra, rb, prev, tw);
-  }
-  __device__ static float2 unpack(const float2 (&v)[V], int q, int tt, float2 r, const float2* tw) {
-    return rv::unpack_value<L>(v, q, tt, r, tw);
-  }
-};
 
 template <int L>
 struct HalfGeo {
@@ -178,16 +131,8 @@ __global__ void __launch_bounds__(256, HalfGeo<L>::MINB)
       const int n = tt + k * T;
       v[k] = live && n >= c0 && n <= c1 ? __ldca(x + n) : make_float2(0.f, 0.f);
     }
-    float2 prev = live && c1 >= L ? __ldca(x + L) : make_float2(0.f, 0.f);
-#pragma unroll
-    for (int k = 0; k < V / 2; ++k) {
-      float2 ra, rb;
-      ra.x = __shfl_sync(0xffffffffu, v[V - 1 - k].x, wk.partner);
-      ra.y = __shfl_sync(0xffffffffu, v[V - 1 - k].y, wk.partner);
-      rb.x = __shfl_sync(0xffffffffu, v[k].x, wk.partner);
-      rb.y = __shfl_sync(0xffffffffu, v[k].y, wk.partner);
-      Rows<L>::pack(v, k, tt, ra, rb, prev, tw);
-    }
+    const float2 prev = live && c1 >= L ? __ldca(x + L) : make_float2(0.f, 0.f);
+    pack_row<L>(v, tt, wk.partner, prev, tw);
     Rows<L>::template fft<+1>(v, tt, fb, pt);
     if (live) {
       int ch;

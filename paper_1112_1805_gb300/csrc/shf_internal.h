@@ -302,6 +302,13 @@ cudaError_t tv_fast_rows_fwd(const float* q, const float* d, float2* Ur, int K, 
 // column transform, times the inverse symbol sym [H][W/2+1], inverse column transform: Ur -> Y.
 cudaError_t tv_fast_cols(const float2* Ur, const float* sym, float2* Y, int K, int H, int W, const float2* twH,
                          cudaStream_t st);
+// The row half of an iteration in one kernel (shf_tv_rows.cu): spectra Y of u ->
+// b_v (bv_in -> bv_out, different buffers), b_w (in place) and the spectra Ur of
+// the next right-hand side; sizes and label counts with tv_band_ok.
+bool tv_band_ok(int H, int W, int K);
+cudaError_t tv_band_prepare(int W);
+cudaError_t tv_band(const float2* Y, float2* Ur, int pitch, const float* bv_in, float* bv_out, float* bw, const float* s,
+                    int K, int H, int W, float t, float gamma, int per_label, const float2* twW, cudaStream_t st);
 // inverse row transforms times scale -> u [K][H][W].
 cudaError_t tv_fast_rows_inv(const float2* Y, float* u, int K, int H, int W, float scale, const float2* twW,
                              cudaStream_t st);

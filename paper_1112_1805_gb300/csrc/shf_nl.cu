@@ -644,7 +644,7 @@ __global__ void __launch_bounds__(kThreads) k_nl_prox(const float4* __restrict__
         wk[k + c] = gw[k + c];
       }
     }
-    shf::simplex_project<KM>(wk, K);
+    shf::simplex_project_sorted<KM>(wk, K);
 #pragma unroll
     for (int k = 0; k < KM; k += 4) {
       float qv[4] = {0.f, 0.f, 0.f, 0.f};

@@ -36,6 +36,7 @@ struct tv_state {
   bool own_stream = false;
   float *f = nullptr, *s = nullptr, *u = nullptr, *bv = nullptr, *d = nullptr, *w = nullptr, *bw = nullptr;
   float *q = nullptr, *rhs = nullptr, *sym = nullptr, *gap = nullptr;
+  float* bv_other = nullptr;  // b_v's second buffer (sizes with tv_band_ok)
   float2 *twH = nullptr, *twW = nullptr, *pt = nullptr, *Ur = nullptr, *Y = nullptr;
   int* labels = nullptr;
   int* flag = nullptr;
@@ -61,12 +62,13 @@ __global__ void k_poisson_symbol(float* __restrict__ sym, int H, int W, int Wh) 
   sym[i] = static_cast<float>(1.0 / (1.0 + 4.0 * s1 * s1 + 4.0 * s2 * s2));
 }
 
-// The v-, w- and b-updates after the u-step, per pixel over the K labels:
+// The v-, w- and b-updates after the u-step, per pixel over the K labels (b_v
+// from bv_in, which may be bv itself):
 // g = b_v + grad u (forward differences, periodic), b_v <- g min(1, t/|g|)
 // (the group clip; v = g - b_v is the shrinkage), d = g - 2 b_v;
 // g_w = b_w + u, w = P_C(g_w), b_w = g_w - w; q = (w - b_w) - gamma s.
 template <int KM>
-__global__ void __launch_bounds__(kThreads) k_tv_prox(const float* __restrict__ u, float* __restrict__ bv,
+__global__ void __launch_bounds__(kThreads) k_tv_prox(const float* __restrict__ u, const float* bv_in, float* bv,
                                                       float* __restrict__ d, float* __restrict__ w,
                                                       float* __restrict__ bw, const float* __restrict__ s,
                                                       float* __restrict__ q, int K, int H, int W, float t,
@@ -84,8 +86,8 @@ __global__ void __launch_bounds__(kThreads) k_tv_prox(const float* __restrict__ 
       if (k < K) {
         const float* up = u + k * P;
         uk[k] = up[x];
-        g0[k] = bv[(2 * k) * P + x] + (up[xr] - uk[k]);
-        g1[k] = bv[(2 * k + 1) * P + x] + (up[xc] - uk[k]);
+        g0[k] = bv_in[(2 * k) * P + x] + (up[xr] - uk[k]);
+        g1[k] = bv_in[(2 * k + 1) * P + x] + (up[xc] - uk[k]);
         n2 = fmaf(g0[k], g0[k], n2);
         n2 = fmaf(g1[k], g1[k], n2);
       }
@@ -113,7 +115,7 @@ __global__ void __launch_bounds__(kThreads) k_tv_prox(const float* __restrict__ 
     float wk[KM];
 #pragma unroll
     for (int k = 0; k < KM; ++k) wk[k] = gw[k];
-    shf::simplex_project<KM>(wk, K);
+    shf::simplex_project_sorted<KM>(wk, K);
 #pragma unroll
     for (int k = 0; k < KM; ++k) {
       if (k < K) {
@@ -245,7 +247,7 @@ void free_tv(tv_state* st) {
   if (!st) return;
   if (st->stream) cudaStreamSynchronize(st->stream);
   if (st->exec) cudaGraphExecDestroy(st->exec);
-  void* bufs[] = {st->f, st->s, st->u, st->bv, st->d, st->w, st->bw, st->q, st->rhs, st->sym, st->gap,
+  void* bufs[] = {st->f, st->s, st->u, st->bv, st->bv_other, st->d, st->w, st->bw, st->q, st->rhs, st->sym, st->gap,
                   st->twH, st->twW, st->pt, st->Ur, st->Y, st->labels, st->flag, st->red};
   for (void* b : bufs) cudaFree(b);
   if (st->own_stream && st->stream) cudaStreamDestroy(st->stream);
@@ -256,19 +258,19 @@ void free_tv(tv_state* st) {
 enum TvKind { kTvRowFwd = 0, kTvCol = 1, kTvRowInv = 2, kTvProx = 3, kTvRhs = 4, kTvKinds = 5 };
 const char* const kTvNames[kTvKinds] = {"tv_row_fwd", "tv_col_solve", "tv_row_inv", "tv_prox", "tv_rhs"};
 
-cudaError_t launch_prox(tv_state* st) {
+cudaError_t launch_prox(tv_state* st, const float* bv_in) {
   const Geo& g = st->g;
   const size_t P = st->P();
   const float t = st->gamma * st->lambda;
   const int grid = grid_for(P);
   if (st->K <= 4)
-    k_tv_prox<4><<<grid, kThreads, 0, st->stream>>>(st->u, st->bv, st->d, st->w, st->bw, st->s, st->q, st->K, g.H,
+    k_tv_prox<4><<<grid, kThreads, 0, st->stream>>>(st->u, bv_in, st->bv, st->d, st->w, st->bw, st->s, st->q, st->K, g.H,
                                                      g.W, t, st->gamma, st->per_label);
   else if (st->K <= 8)
-    k_tv_prox<8><<<grid, kThreads, 0, st->stream>>>(st->u, st->bv, st->d, st->w, st->bw, st->s, st->q, st->K, g.H,
+    k_tv_prox<8><<<grid, kThreads, 0, st->stream>>>(st->u, bv_in, st->bv, st->d, st->w, st->bw, st->s, st->q, st->K, g.H,
                                                      g.W, t, st->gamma, st->per_label);
   else
-    k_tv_prox<16><<<grid, kThreads, 0, st->stream>>>(st->u, st->bv, st->d, st->w, st->bw, st->s, st->q, st->K,
+    k_tv_prox<16><<<grid, kThreads, 0, st->stream>>>(st->u, bv_in, st->bv, st->d, st->w, st->bw, st->s, st->q, st->K,
                                                       g.H, g.W, t, st->gamma, st->per_label);
   return cudaGetLastError();
 }
@@ -296,7 +298,7 @@ cudaError_t enqueue_tv_iteration(tv_state* st, cudaEvent_t* ev) {
     if (e == cudaSuccess) e = mark(kTvRowInv);
     if (e == cudaSuccess) e = shf::tvfast::tv_fast_rows_inv(st->Y, st->u, st->K, g.H, g.W, scale, g.twW, ss);
     if (e == cudaSuccess) e = mark(kTvProx);
-    if (e == cudaSuccess) e = launch_prox(st);
+    if (e == cudaSuccess) e = launch_prox(st, st->bv);
     if (e == cudaSuccess) e = mark(kTvRhs);
     if (e == cudaSuccess) e = mark(kTvKinds);
     return e;
@@ -308,10 +310,40 @@ cudaError_t enqueue_tv_iteration(tv_state* st, cudaEvent_t* ev) {
   if (e == cudaSuccess) e = mark(kTvRowInv);
   if (e == cudaSuccess) e = shf::run_row_c2r(g, st->Y, st->u, st->K, 1.f / (static_cast<float>(g.H) * g.W), ss);
   if (e == cudaSuccess) e = mark(kTvProx);
-  if (e == cudaSuccess) e = launch_prox(st);
+  if (e == cudaSuccess) e = launch_prox(st, st->bv);
   if (e == cudaSuccess) e = mark(kTvRhs);
   if (e == cudaSuccess) e = launch_rhs(st);
   if (e == cudaSuccess) e = mark(kTvKinds);
+  return e;
+}
+
+// n > 1 iterations: the first one's right-hand side comes from d and q, the
+// last one leaves u, w, d and q behind as a single iteration does, and those in
+// between are two launches each (shf_tv_rows.cu; b_v alternates between two
+// buffers).  Launched directly, as programmatic dependents: two launches cost
+// the host less than the GPU takes for them.
+cudaError_t enqueue_tv_iterations(tv_state* st, int n) {
+  const Geo& g = st->g;
+  cudaStream_t ss = st->stream;
+  const float scale = 1.f / (static_cast<float>(g.H) * g.W), t = st->gamma * st->lambda;
+  cudaError_t e = st->fast ? shf::tvfast::tv_fast_rows_fwd(st->q, st->d, st->Ur, st->K, g.H, g.W, g.twW, ss)
+                           : shf::run_row_r2c(g, st->rhs, st->Ur, st->K, 1.f, ss);
+  const float* in = st->bv;
+  float* out = st->bv_other;
+  for (int i = 0; i < n && e == cudaSuccess; ++i) {
+    e = st->fast ? shf::tvfast::tv_fast_cols(st->Ur, st->sym, st->Y, st->K, g.H, g.W, g.twH, ss)
+                 : shf::run_col_filter(g, st->Ur, st->Y, st->K, ss);
+    if (e != cudaSuccess || i == n - 1) break;
+    e = shf::tvfast::tv_band(st->Y, st->Ur, st->pitch, in, out, st->bw, st->s, st->K, g.H, g.W, t, st->gamma, st->per_label,
+                            g.twW, ss);
+    in = out;
+    out = in == st->bv ? st->bv_other : st->bv;
+  }
+  if (e == cudaSuccess)
+    e = st->fast ? shf::tvfast::tv_fast_rows_inv(st->Y, st->u, st->K, g.H, g.W, scale, g.twW, ss)
+                 : shf::run_row_c2r(g, st->Y, st->u, st->K, scale, ss);
+  if (e == cudaSuccess) e = launch_prox(st, in);
+  if (e == cudaSuccess && !st->fast) e = launch_rhs(st);
   return e;
 }
 
@@ -403,12 +435,21 @@ int tv_admm_init(int H, int W, const float* f, int C, const float* codebook, int
       return tv_fail(SHF_ERR_CUDA, std::string("tv_admm_init: ") + cudaGetErrorString(e));
     }
   }
+  const bool band = shf::tvfast::tv_band_ok(H, W, K);
+  if (band) {
+    cudaError_t e = shf::tvfast::tv_band_prepare(W);
+    if (e != cudaSuccess) {
+      free_tv(st);
+      return tv_fail(SHF_ERR_CUDA, std::string("tv_admm_init: ") + cudaGetErrorString(e));
+    }
+  }
   st->pitch = st->fast ? shf::tvfast::tv_fast_pitch(W) : g.Wh;
   const size_t P = static_cast<size_t>(H) * W, Ph = static_cast<size_t>(H) * g.Wh;
   const size_t Phs = static_cast<size_t>(H) * st->pitch;  // spectra of the u-step at the path's pitch
   int rc;
   if ((rc = tv_alloc(&st->f, P * C, "f")) || (rc = tv_alloc(&st->s, P * K, "s")) ||
       (rc = tv_alloc(&st->u, P * K, "u")) || (rc = tv_alloc(&st->bv, 2 * P * K, "b_v")) ||
+      (band && (rc = tv_alloc(&st->bv_other, 2 * P * K, "b_v"))) ||
       (rc = tv_alloc(&st->d, 2 * P * K, "d")) || (rc = tv_alloc(&st->w, P * K, "w")) ||
       (rc = tv_alloc(&st->bw, P * K, "b_w")) || (rc = tv_alloc(&st->q, P * K, "q")) ||
       (rc = tv_alloc(&st->rhs, P * K, "rhs")) || (rc = tv_alloc(&st->sym, Ph, "symbol")) ||
@@ -457,6 +498,11 @@ int tv_admm_reset(tv_state* st, const float* f, int f_on_host) {
 int tv_admm_step(tv_state* st, int n) {
   if (!st || n < 0) return tv_fail(SHF_ERR_ARG, "tv_admm_step: bad argument");
   if (n == 0) return SHF_OK;
+  if (n > 1 && st->bv_other) {
+    TV_CK(enqueue_tv_iterations(st, n));
+    st->iter += n;
+    return SHF_OK;
+  }
   if (!st->graph_tried) {
     // one iteration captured as a CUDA graph when the stream allows capture
     st->graph_tried = true;

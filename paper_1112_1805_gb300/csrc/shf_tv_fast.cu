@@ -200,10 +200,19 @@ __global__ void __launch_bounds__(ColGeo<H>::NT, H == 512 ? 2 : 1)
   float2* b0 = sm + G::PT;
   float2* b1 = b0 + G::BR;
   const int b = threadIdx.x % KB, tt = threadIdx.x / KB;
+  const int ntiles = (Wh + KB - 1) / KB, items = K * ntiles;
+  // the symbol's column does not depend on the previous kernel: it is on its way
+  // while that one drains
+  float sy[16];
+  const auto load_sym = [&](int item) {
+    const int col = (item % ntiles) * KB + b;
+#pragma unroll
+    for (int j = 0; j < 16; ++j) sy[j] = col < Wh ? __ldg(sym + static_cast<size_t>(tt + j * T) * Wh + col) : 0.f;
+  };
+  load_sym(blockIdx.x);
   r16::build_pass_twiddles<H, 1>(pt, twH, threadIdx.x, blockDim.x);
   pdl_wait();
   pdl_trigger();
-  const int ntiles = (Wh + KB - 1) / KB, items = K * ntiles;
   for (int item = blockIdx.x; item < items; item += gridDim.x) {
     const int k = item / ntiles, col = (item - k * ntiles) * KB + b;
     const bool ok = col < Wh;
@@ -213,7 +222,8 @@ __global__ void __launch_bounds__(ColGeo<H>::NT, H == 512 ? 2 : 1)
     for (int j = 0; j < 16; ++j) v[j] = ok ? src[static_cast<size_t>(tt + j * T) * Whp] : make_float2(0.f, 0.f);
     r16::batch_fft<H, -1, KB>(v, tt, b, b0, b1, pt);  // starts with a CTA barrier
 #pragma unroll
-    for (int j = 0; j < 16; ++j) v[j] = c_scale(v[j], ok ? sym[static_cast<size_t>(tt + j * T) * Wh + col] : 0.f);
+    for (int j = 0; j < 16; ++j) v[j] = c_scale(v[j], sy[j]);
+    if (item + gridDim.x < items) load_sym(item + gridDim.x);
     r16::batch_fft<H, +1, KB>(v, tt, b, b0, b1, pt);
     if (ok) {
       float2* dst = Y + static_cast<size_t>(k) * H * Whp + col;
