@@ -6,6 +6,7 @@
 // scaling function varphi, discretised as in "Finite Discrete Shearlets" with
 // the glued seam shearlets for |k| = 2^j.  They are evaluated in FP64 on the
 // device and rounded once to FP32.
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 
@@ -151,6 +152,42 @@ __global__ void k_data_term(const float* __restrict__ f, int C, Codebook cb, int
       s[static_cast<size_t>(k) * P + r] = acc;
     }
   }
+}
+
+// The start of a solve in one launch: the data term s as above, w = b_w = u = 0
+// [K][P], T = 0 (nT values), and *bad = 1 (host memory) when f holds a NaN or
+// infinity.  Its parts were seven launches, memsets and copies, each a few
+// microseconds of host time and latency (a reset of a 64 x 64 state 84 us).
+__global__ void k_restart(const float* __restrict__ f, int C, Codebook cb, int K, float* __restrict__ s,
+                          float* __restrict__ w, float* __restrict__ bw, float* __restrict__ u, int P,
+                          float2* __restrict__ T, long long nT, int* bad) {
+  const long long i0 = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x, step = static_cast<long long>(gridDim.x) * blockDim.x;
+  bool nan = false;
+  for (long long r = i0; r < P; r += step) {
+    float fv[kMaxC];
+#pragma unroll
+    for (int ch = 0; ch < kMaxC; ++ch) {
+      fv[ch] = ch < C ? f[static_cast<size_t>(ch) * P + r] : 0.f;
+      nan = nan || !isfinite(fv[ch]);
+    }
+    for (int k = 0; k < K; ++k) {
+      float acc = 0.f;
+#pragma unroll
+      for (int ch = 0; ch < kMaxC; ++ch) {
+        if (ch < C) {
+          const float d = fv[ch] - cb.c[k * C + ch];
+          acc = fmaf(d, d, acc);
+        }
+      }
+      const size_t e = static_cast<size_t>(k) * P + r;
+      s[e] = acc;
+      w[e] = 0.f;
+      bw[e] = 0.f;
+      u[e] = 0.f;
+    }
+  }
+  for (long long e = i0; e < nT; e += step) T[e] = make_float2(0.f, 0.f);
+  if (nan) *static_cast<volatile int*>(bad) = 1;
 }
 
 // Label = argmax_k w[k] (ties: lowest k), gap = largest - second largest.
@@ -340,6 +377,14 @@ cudaError_t launch_data_term(const float* f, int C, const float* codebook_host, 
   Codebook cb{};
   for (int i = 0; i < K * C; ++i) cb.c[i] = codebook_host[i];
   k_data_term<<<grid_for(P, 256), 256, 0, st>>>(f, C, cb, K, s, P);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_restart(const float* f, int C, const float* codebook_host, int K, float* s, float* w, float* bw,
+                           float* u, int P, float2* T, long long nT, int* bad, cudaStream_t st) {
+  Codebook cb{};
+  for (int i = 0; i < K * C; ++i) cb.c[i] = codebook_host[i];
+  k_restart<<<grid_for(std::max<long long>(P, nT), 256), 256, 0, st>>>(f, C, cb, K, s, w, bw, u, P, T, nT, bad);
   return cudaGetLastError();
 }
 

@@ -99,7 +99,7 @@ struct seg_state {
   float2 *Ur = nullptr, *Y = nullptr, *partial = nullptr, *T = nullptr;
   float *thr = nullptr, *lam = nullptr, *gap = nullptr;
   int* labels = nullptr;
-  int* flag = nullptr;
+  int* bad = nullptr;  // pinned host memory, written by the restart kernel
   double* red = nullptr;
   int groups = 1;
   std::vector<shf::FilterWave> waves;  // general path: the waves of `groups` filter groups
@@ -170,7 +170,11 @@ constexpr int kMaxDevices = 64;
 struct DevicePool {
   cudaMemPool_t pool = nullptr;
   int users = 0;
+  // pinned host integers for the states' flags (one page for kFlags of them)
+  int* flags = nullptr;
+  std::vector<int*> free_flags;
 };
+constexpr int kFlags = 1024;
 std::mutex g_pool_mu;
 DevicePool g_pools[kMaxDevices];
 
@@ -206,6 +210,40 @@ void release_pool(int device) {
   cudaStreamSynchronize(nullptr);  // the states' frees
   cudaMemPoolDestroy(d.pool);
   d.pool = nullptr;
+  cudaFreeHost(d.flags);
+  d.flags = nullptr;
+  d.free_flags.clear();
+}
+
+// A pinned host integer: from the device's page, or its own allocation.
+int acquire_flag(int device, int** flag) {
+  if (device >= 0 && device < kMaxDevices) {
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    DevicePool& d = g_pools[device];
+    if (d.pool && !d.flags && cudaMallocHost(reinterpret_cast<void**>(&d.flags), sizeof(int) * kFlags) == cudaSuccess)
+      for (int i = 0; i < kFlags; ++i) d.free_flags.push_back(d.flags + i);
+    cudaGetLastError();
+    if (!d.free_flags.empty()) {
+      *flag = d.free_flags.back();
+      d.free_flags.pop_back();
+      return SHF_OK;
+    }
+  }
+  SHF_CK(cudaMallocHost(reinterpret_cast<void**>(flag), sizeof(int)));
+  return SHF_OK;
+}
+
+void release_flag(int device, int* flag) {
+  if (!flag) return;
+  if (device >= 0 && device < kMaxDevices) {
+    std::lock_guard<std::mutex> lock(g_pool_mu);
+    DevicePool& d = g_pools[device];
+    if (d.flags && flag >= d.flags && flag < d.flags + kFlags) {
+      d.free_flags.push_back(flag);
+      return;
+    }
+  }
+  cudaFreeHost(flag);
 }
 
 // A work list's four arrays one after another (the items as four ints each);
@@ -530,7 +568,7 @@ void free_state(seg_state* s) {
   state_free(s, s->partial);
   state_free(s, s->T);
   state_free(s, s->labels);
-  state_free(s, s->flag);
+  release_flag(s->device, s->bad);
   state_free(s, s->red);
   if (s->own_stream && s->stream) cudaStreamDestroy(s->stream);
   if (s->pool) release_pool(s->device);
@@ -541,19 +579,13 @@ void free_state(seg_state* s) {
 int restart(seg_state* st, const float* codebook) {
   const Geo& g = st->g;
   const size_t P = st->P();
-  SHF_CK(cudaMemsetAsync(st->flag, 0, sizeof(int), st->stream));
-  SHF_CK(shf::launch_count_nonfinite(st->f, static_cast<long>(P * st->C), st->flag, st->stream));
-  if (codebook) SHF_CK(shf::launch_data_term(st->f, st->C, codebook, st->K, st->s, static_cast<int>(P), st->stream));
+  *st->bad = 0;
+  SHF_CK(shf::launch_restart(st->f, st->C, codebook, st->K, st->s, st->w, st->bw, st->u, static_cast<int>(P), st->T,
+                             static_cast<long long>(st->Ph()) * st->K, st->bad, st->stream));
   SHF_CK(cudaMemsetAsync(st->bv, 0, sizeof(float) * P * st->K * g.eta, st->stream));
-  SHF_CK(cudaMemsetAsync(st->w, 0, sizeof(float) * P * st->K, st->stream));
-  SHF_CK(cudaMemsetAsync(st->bw, 0, sizeof(float) * P * st->K, st->stream));
-  SHF_CK(cudaMemsetAsync(st->u, 0, sizeof(float) * P * st->K, st->stream));
-  SHF_CK(cudaMemsetAsync(st->T, 0, sizeof(float2) * st->Ph() * st->K, st->stream));
-  int bad = 0;
-  SHF_CK(cudaMemcpyAsync(&bad, st->flag, sizeof(int), cudaMemcpyDeviceToHost, st->stream));
   SHF_CK(cudaStreamSynchronize(st->stream));
   st->iter = 0;
-  if (bad) return fail(SHF_ERR_NONFINITE, "image contains NaN or Inf");
+  if (*st->bad) return fail(SHF_ERR_NONFINITE, "image contains NaN or Inf");
   return SHF_OK;
 }
 
@@ -971,7 +1003,7 @@ int seg_admm_init(const shf_bank* b, const float* f, int C, const float* codeboo
       (st->fast && (rc = install_fast_plan(st, def.wave_mib, 0, def.row_kernel, def.col_kernel, def.serial))) ||
       (rc = state_alloc(st, &st->thr, g.eta, "thr")) || (rc = state_alloc(st, &st->lam, g.eta, "lam")) ||
       (rc = state_alloc(st, &st->gap, P, "gap")) || (rc = state_alloc(st, &st->labels, P, "labels")) ||
-      (rc = state_alloc(st, &st->flag, 1, "flag")) || (rc = state_alloc(st, &st->red, 2 + 512, "red"))) {
+      (rc = acquire_flag(st->device, &st->bad)) || (rc = state_alloc(st, &st->red, 2 + 512, "red"))) {
     free_state(st);
     return rc;
   }
@@ -1007,9 +1039,32 @@ int seg_admm_reset(seg_state* st, const float* f, int f_on_host) {
   return restart(st, st->codebook.data());
 }
 
+}  // extern "C"
+
+namespace {
+// Whether a state's iterations are launched one by one instead of as graphs: then
+// an iteration's first kernel overlaps the end of the iteration before (graph
+// launches follow one another with a gap) and a new state pays for no capture.
+// In us per iteration and for the first 20 of a state: 64 x 64, K = 3 27.7 -> 25.2
+// and 606 -> 489; 128 x 128, K = 4 37.2 -> 34.6; 256 x 256, K = 4 58.1 -> 55.5; the
+// general path 1-2% (480 x 640, K = 5 755 -> 753).  Where the iteration is long
+// the graph is ahead (512 x 512, K = 4 257.8 against 262.8).
+bool launched_directly(const seg_state* st) {
+  return !st->fast || static_cast<double>(st->P()) * st->K * st->g.eta <= 3.3e7;
+}
+}  // namespace
+
+extern "C" {
+
 int seg_admm_step(seg_state* st, int n) {
   if (!st || n < 0) return fail(SHF_ERR_ARG, "seg_admm_step: bad argument");
   if (n == 0) return SHF_OK;
+  if (launched_directly(st)) {
+    ensure_marks(st);
+    for (int i = 0; i < n; ++i) SHF_CK(enqueue_iteration(st, i == n - 1 && !st->untimed));
+    st->iter += n;
+    return SHF_OK;
+  }
   if (!st->graph_tried) try_capture(st);
   // the last iteration of the call records the per-kernel timing events
   for (int i = 0; i < n; ++i) {

@@ -57,6 +57,10 @@ cudaError_t launch_build_bank(float* bank, const Geo& g, const FilterDesc* descs
 cudaError_t launch_filter_ranges(const float* bank, const Geo& g, int2* ranges, cudaStream_t st);
 cudaError_t launch_data_term(const float* f, int C, const float* codebook_host, int K, float* s, int P,
                              cudaStream_t st);
+// Data term and zero state in one launch; *bad (pinned host memory) becomes 1 for
+// an image with a NaN or infinity.
+cudaError_t launch_restart(const float* f, int C, const float* codebook_host, int K, float* s, float* w, float* bw,
+                           float* u, int P, float2* T, long long nT, int* bad, cudaStream_t st);
 cudaError_t launch_labels(const float* w, int K, int P, int* labels, float* gap, cudaStream_t st);
 cudaError_t launch_count_nonfinite(const float* x, long n, int* count, cudaStream_t st);
 // Deterministic sums: partial[block] in FP64 then one ordered final pass.
