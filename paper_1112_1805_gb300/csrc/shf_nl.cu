@@ -8,11 +8,11 @@
 // every candidate j of the varpi x varpi search window (clipped to the image)
 // is computed on the GPU (in FP32, and in FP64 with every product and sum
 // rounded separately where that decides the order), and each pixel's
-// candidates are ranked by (distance, raster index).  The selection itself is sequential in the paper (pixels in
+// candidates are ranked by (distance, raster index).  The selection is sequential in the paper (pixels in
 // raster order pick min(mt, 2 mt - l) new neighbours, l the neighbours they
-// already have, and links are symmetric), so it runs on the host over the
-// ranked lists; a candidate already linked or holding 2 mt neighbours is
-// passed over.
+// already have, and links are symmetric); a candidate already linked or holding
+// 2 mt neighbours is passed over.  Pixels whose windows are apart don't see one
+// another, so it runs as a wavefront over the image with the same result.
 //
 // ADMM (Sec. 3 with S replaced by D, per iteration):
 //   u   = (I + D^T D)^(-1) [ D^T (v - b_v) + (w - b_w) - gamma s ]
@@ -39,9 +39,8 @@ struct nl_state {
   float gamma = 1.f, lambda = 0.f;
   nl_params prm{};
   std::vector<float> codebook;
-  // pinned: the links [P][m] in the order of selection, their counts, the first ranks
-  int* nbr_host = nullptr;
-  unsigned char *deg_host = nullptr, *head_host = nullptr;
+  // pinned: the links as window codes [P][kMaxM] in the order of selection, their counts
+  unsigned char *codes_host = nullptr, *deg_host = nullptr;
   std::vector<float> cheb_a, cheb_c;    // Chebyshev coefficients per step
   cudaStream_t stream = nullptr;
   bool own_stream = false;
@@ -55,10 +54,11 @@ struct nl_state {
   int* nbr = nullptr;                   // [m][P]
   short* off = nullptr;                 // [m][P] neighbour minus pixel index (|off| <= 7 W + 7)
   unsigned char *rev = nullptr, *deg = nullptr;
-  // the graph's construction: patch weights, the first ranks, the selected links
+  // the graph's construction: patch weights, the ranks of rank_rows rows, the selected links
   double* gw = nullptr;
-  unsigned char* head = nullptr;
-  int* list = nullptr;
+  unsigned char* rank = nullptr;
+  int rank_rows = 0;
+  uint4* codes = nullptr;
   int* labels = nullptr;
   int* flag = nullptr;
   double* red = nullptr;
@@ -109,10 +109,11 @@ constexpr int kMaxHalo = kMaxWin / 2 + kMaxPatch / 2;
 constexpr int kRankRows = kRankTY + 2 * kMaxHalo, kRankCols = kRankTX + 2 * kMaxHalo;
 constexpr float kRankMax = 1e4f;  // largest |f| of a tile for the FP32 distances
 constexpr float kTiny = 1e-36f;
-// ranks copied to the host for every pixel; a pixel needs more only when its
-// nearest 64 candidates are nearly all full (1 pixel in 10^4 of the textured
-// images, 3 in 10^3 would need more than 32)
-constexpr int kRankHead = 64;
+// ranks of a pixel, padded to whole words, and the bytes of them held at a time
+// (512 x 512 takes 67 MB, in one go)
+constexpr int kRankPitch = 256;
+constexpr size_t kRankBytes = size_t{256} << 20;
+constexpr size_t kRingBytes = 200 * 1024;  // shared memory for the selection's counts
 
 // FP64 distance of the pixel at tile position (y, x) to the candidate (dy, dx).
 __device__ __forceinline__ double nl_exact(const float (*tile)[kRankRows][kRankCols], int C, const double* __restrict__ G,
@@ -132,20 +133,21 @@ __device__ __forceinline__ double nl_exact(const float (*tile)[kRankRows][kRankC
   return acc;
 }
 
-// The rows from ystrip on.  rank (optional) holds every code of those rows'
-// pixels in order, 255 for the unused positions at the end; head[i] (optional)
-// the first kRankHead of pixel i.  G: the patch weights [(2h+1)^2].
+// The rows from ystrip up to yend.  rank [pixels][kRankPitch] holds every code of
+// those rows' pixels in order, 255 for the unused positions at the end; word w of
+// the pixel's 64 holds the positions 64 (w / 16) + w % 16 + {0, 16, 32, 48}.  G: the patch weights [(2h+1)^2].
 // Bound by instruction issue (about 3000 warp instructions a pixel: distances
 // 900, sort 1500); 512 x 512, 5 x 5 patches, 15 x 15 window: 79.3 ms with FP64
 // distances and ranks counted over all pairs, 1.2 ms so.
 template <int C>
 __global__ void __launch_bounds__(32 * kRankWarps)
     k_nl_rank(const float* __restrict__ f, int H, int W, const double* __restrict__ G, int h, int r, float delta,
-              int ystrip, unsigned char* __restrict__ rank, unsigned char* __restrict__ head) {
+              int ystrip, int yend, unsigned char* __restrict__ rank) {
   __shared__ float tile[C][kRankRows][kRankCols];
   __shared__ float sG[kMaxPatch * kMaxPatch];
   __shared__ double ex[kRankWarps][256];
-  __shared__ unsigned char code[kRankWarps][256], out[kRankWarps][256], list[kRankWarps][256], near_next[kRankWarps][256];
+  __shared__ __align__(8) unsigned char out[kRankWarps][kRankPitch];
+  __shared__ unsigned char code[kRankWarps][256], list[kRankWarps][256], near_next[kRankWarps][256];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int side = 2 * r + 1, NW = side * side, cen = NW / 2, n = 2 * h + 1, halo = r + h;
   const size_t P = static_cast<size_t>(H) * W;
@@ -177,7 +179,7 @@ __global__ void __launch_bounds__(32 * kRankWarps)
   }
   for (int px = wid; px < kRankTX * kRankTY; px += kRankWarps) {
     const int ri = y0 + px / kRankTX, ci = x0 + px % kRankTX;
-    if (ri >= H || ci >= W) continue;  // the whole warp
+    if (ri >= yend || ci >= W) continue;  // the whole warp
     const int y = px / kRankTX + halo, x = px % kRankTX + halo;
     float acc[7];
     const float* base[7];
@@ -288,24 +290,179 @@ __global__ void __launch_bounds__(32 * kRankWarps)
     }
     __syncwarp();
     const size_t i = static_cast<size_t>(ri) * W + ci;
-    if (rank)
-      for (int c = lane; c < NW; c += 32) rank[(i - static_cast<size_t>(ystrip) * W) * NW + c] = out[wid][c];
-    if (head)
-      for (int c = lane; c < kRankHead; c += 32) head[i * kRankHead + c] = c < NW ? out[wid][c] : 255;
+    unsigned word[2];
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int w = 2 * lane + q;
+      const unsigned char* o = out[wid] + (w & ~15) * 4 + (w & 15);
+      word[q] = o[0] | static_cast<unsigned>(o[16]) << 8 | static_cast<unsigned>(o[32]) << 16 |
+                static_cast<unsigned>(o[48]) << 24;
+    }
+    reinterpret_cast<uint2*>(rank + (i - static_cast<size_t>(ystrip) * W) * kRankPitch)[lane] = make_uint2(word[0], word[1]);
     __syncwarp();
   }
 }
 
-// The device tables of the selected links, list [P][m] with deg[i] entries:
+// The selection for the rows [y0, y0 + rows), whose ranks are in `rank`, after
+// every row above: codes [P][kMaxM] holds the window codes of a pixel's links in the
+// order they were made (255 for none), deg [P] their number.
+//
+// A pixel reads and changes the state of its window only, and two pixels can
+// meet in a window only if their columns are at most 2 r apart.  So at step t one
+// CTA takes the pixel (y, t - S y) of every row y, S = 2 r + 1: pixels of one step
+// have disjoint windows, and of any two pixels that meet the earlier one in
+// raster order comes in an earlier step (its row is d rows up, its column at
+// most 2 r < S d further right).  The links, their order included, are those of
+// the raster loop.  A half warp takes a pixel, 16 candidates at a time in the
+// order of rank; with more rows than half warps a step takes several turns.
+//
+// Bound by one SM's latency and issue slots, W + S (rows - 1) steps of two
+// dependent shared-memory reads, the votes and a barrier.  Hence
+//  - RING: the counts of the rows in reach live in shared memory, row y in slot
+//    y mod R; a row enters with the first row that reaches it, when the row R above,
+//    which no pixel reaches any more, goes to memory (R >= 2 r + (W - 1) / S + 1).
+//    Otherwise (images too wide for that) the counts are read from L2.
+//  - the next pixel's first 64 candidates and own links are read a step ahead; of the
+//    pixels that can link to it in between, there is only the current one.
+// A step takes about 1.1 us (512 x 512, window 15: 8177 steps, 9 ms).  The graph of an
+// image, with the raster loop on the host and the copies of ranks and links, and so:
+// 256 x 256 4.5 and 4.5 ms, 512 x 512 17.6 and 11.2, 1024 x 1024 68 and 42, 1800 x
+// 1800 212 and 105, 2048 x 2048 (counts in L2) 274 and 146; a 64 x 64 image, 0.56 and
+// 1.13, is the price of one path.  64 candidates at a time (four per lane) took 25 ms
+// at 512 x 512: the step is bound by instructions as much as by its chain.
+template <bool RING>
+__global__ void __launch_bounds__(1024) k_nl_select(const unsigned* __restrict__ rank, int H, int W, int r, int m,
+                                                    int mt, int y0, int rows, int R, unsigned char* codes,
+                                                    unsigned char* deg) {
+  __shared__ int step[256];
+  extern __shared__ unsigned char ring[];
+  constexpr unsigned kAll = 0xffffffffu;
+  constexpr int kWords = kRankPitch / 4;
+  const int side = 2 * r + 1, NW = side * side;
+  const int lane = threadIdx.x & 31, gl = lane & 15, grp = threadIdx.x >> 4, ngrp = blockDim.x >> 4;
+  const int turns = (min(rows, (W + side - 1) / side) + ngrp - 1) / ngrp, slots = turns * ngrp;
+  const int right = NW / 2 + 1, left_code = NW / 2 - 1;  // the codes of the row's next and previous pixel
+  for (int c = threadIdx.x; c < NW; c += blockDim.x) step[c] = (c / side - r) * W + (c % side - r);
+  const int first = max(0, y0 - r), RW = R * W;
+  if (RING)
+    for (int y = first; y < min(H, y0 + r); ++y)
+      for (int x = threadIdx.x; x < W; x += blockDim.x) ring[(y % R) * W + x] = deg[y * W + x];
+  __syncthreads();
+  unsigned char* const count = RING ? ring : deg;
+  const int steps = W + side * (rows - 1);
+  int yn = -1, xn = 0;  // the pixel that was read ahead: candidates, own links, linked by the one before
+  unsigned cn = kAll;
+  uint4 on = make_uint4(0u, 0u, 0u, 0u);
+  bool ln = false;
+  // the rows [ylo, yhi] of the step; ymod = ylo mod slots
+  int ylo = 0, yhi = -1, ymod = 0, start = 0, end = W;
+  for (int t = 0; t < steps; ++t) {
+    if (t == end) {  // the first row is done
+      ++ylo;
+      end += side;
+      ymod = ymod + 1 == slots ? 0 : ymod + 1;
+    }
+    if (t == start && yhi + 1 < rows) {  // a row starts
+      ++yhi;
+      start += side;
+      const int e = y0 + yhi + r;
+      if (RING && e < H) {  // row e enters
+        for (int x = threadIdx.x; x < W; x += blockDim.x) {
+          unsigned char* at = ring + (e % R) * W + x;
+          if (e - R >= first) deg[(e - R) * W + x] = *at;
+          *at = 0;
+        }
+        __syncthreads();
+      }
+    }
+    for (int turn = 0; turn < turns; ++turn) {
+      const int slot = turn * ngrp + grp;
+      const int y = ylo + slot - ymod + (slot < ymod ? slots : 0), x = t - side * y;
+      const bool act = y <= yhi;
+      const int i = act ? (y0 + y) * W + x : 0;                       // the pixel
+      const int ci = RING ? (act ? ((y0 + y) % R) * W + x : 0) : i;   // where its count is
+      const unsigned* rk = rank + (act ? static_cast<size_t>(y * W + x) * kWords : 0) + gl;
+      int left = 0, dgi = 0;
+      unsigned cw = kAll;  // the lane's next four candidates, 255 for none
+      uint4 own = make_uint4(0u, 0u, 0u, 0u);
+      bool link_left = false;
+      if (act) {
+        dgi = count[ci];
+        left = min(mt, m - dgi);
+        if (y == yn && x == xn) {
+          cw = cn;
+          own = on;
+          link_left = ln;
+        } else {
+          cw = rk[0];
+          own = reinterpret_cast<const uint4*>(codes)[i];
+        }
+        if (x + 1 < W) {
+          yn = y;
+          xn = x + 1;
+          cn = rk[kWords];
+          on = reinterpret_cast<const uint4*>(codes)[i + 1];
+          ln = false;
+        }
+        if (x + 8 < W && (gl == 0 || gl == 8)) asm volatile("prefetch.global.L1 [%0];" ::"l"(rk + 8 * kWords));
+      }
+      for (int pass = 0;; ++pass) {
+        const int c = static_cast<int>(cw & 255u);
+        bool ok = false;
+        int at = 0, dj = 0, st = 0;
+        if (c != 255 && left > 0) {
+          st = step[c];
+          at = ci + st;
+          if (RING) at += at < 0 ? RW : at >= RW ? -RW : 0;
+          dj = count[at];
+          const unsigned cc = 0x01010101u * static_cast<unsigned>(c);
+          const bool linked = (__vcmpeq4(own.x, cc) | __vcmpeq4(own.y, cc) | __vcmpeq4(own.z, cc) |
+                               __vcmpeq4(own.w, cc)) != 0u || (link_left && c == left_code);
+          ok = dj < m && !linked;
+        }
+        const unsigned free16 = __ballot_sync(kAll, ok) >> (lane & 16) & 0xffffu;
+        const int n = __popc(free16 & ((1u << gl) - 1u));
+        const bool take = ok && n < left;
+        if (take) {
+          count[at] = static_cast<unsigned char>(dj + 1);
+          codes[(i + st) * kMaxM + dj] = static_cast<unsigned char>(NW - 1 - c);  // the way back
+          codes[i * kMaxM + dgi + n] = static_cast<unsigned char>(c);
+        }
+        const unsigned next_linked = __ballot_sync(kAll, take && c == right) >> (lane & 16) & 0xffffu;
+        const int last = __shfl_sync(kAll, c, lane | 15);
+        ln = ln || next_linked != 0u;
+        const int took = min(__popc(free16), left);
+        dgi += took;
+        left -= took;
+        if (last == 255 || pass == kRankPitch / 16 - 1) left = 0;  // the list's end
+        if (!__any_sync(kAll, left > 0)) break;
+        cw = (pass & 3) != 3 ? cw >> 8 : left > 0 ? rk[(pass + 1) * 4] : kAll;
+      }
+      if (act && gl == 0) count[ci] = static_cast<unsigned char>(dgi);
+    }
+    __syncthreads();
+  }
+  if (RING) {
+    const int last = min(H - 1, y0 + rows - 1 + r);
+    for (int y = max(first, last - R + 1); y <= last; ++y)
+      for (int x = threadIdx.x; x < W; x += blockDim.x) deg[y * W + x] = ring[(y % R) * W + x];
+  }
+}
+
+// The device tables of the selected links, codes [P][kMaxM] with deg[i] entries:
 // sorted neighbour lists nbr [m][P] (-1 padded) and offsets off [m][P].
-__global__ void __launch_bounds__(kThreads) k_nl_tables(const int* __restrict__ list, const unsigned char* __restrict__ deg,
-                                                        int m, size_t P, int* __restrict__ nbr, short* __restrict__ off) {
+__global__ void __launch_bounds__(kThreads) k_nl_tables(const unsigned char* __restrict__ codes,
+                                                        const unsigned char* __restrict__ deg, int W, int r, int m,
+                                                        size_t P, int* __restrict__ nbr, short* __restrict__ off) {
   const size_t i = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x;
   if (i >= P) return;
-  const int dg = deg[i];
+  const int dg = deg[i], side = 2 * r + 1;
   int v[kMaxM];
 #pragma unroll
-  for (int b = 0; b < kMaxM; ++b) v[b] = b < dg ? list[i * m + b] : 0x7fffffff;
+  for (int b = 0; b < kMaxM; ++b) {
+    const int c = codes[i * kMaxM + b];
+    v[b] = b < dg ? static_cast<int>(i) + (c / side - r) * W + (c % side - r) : 0x7fffffff;
+  }
   // odd-even transposition
 #pragma unroll
   for (int t = 0; t < kMaxM; ++t)
@@ -835,13 +992,12 @@ void free_nl(nl_state* st) {
   if (st->stream) cudaStreamSynchronize(st->stream);
   if (st->exec) cudaGraphExecDestroy(st->exec);
   void* bufs[] = {st->f, st->s, st->u, st->xa, st->xb, st->cd, st->bv, st->d, st->w, st->bw, st->q, st->rhs,
-                  st->gap, st->nbr, st->off, st->rev, st->deg, st->gw, st->head, st->list, st->labels, st->flag,
+                  st->gap, st->nbr, st->off, st->rev, st->deg, st->gw, st->rank, st->codes, st->labels, st->flag,
                   st->red,
                   st->cbar, st->cerr, st->cheb_ac};
   for (void* b : bufs) cudaFree(b);
-  cudaFreeHost(st->nbr_host);
+  cudaFreeHost(st->codes_host);
   cudaFreeHost(st->deg_host);
-  cudaFreeHost(st->head_host);
   if (st->own_stream && st->stream) cudaStreamDestroy(st->stream);
   delete st;
 }
@@ -861,12 +1017,12 @@ std::vector<double> patch_weights(int h, double a) {
   return G;
 }
 
-// The graph of st->f: ranks on the GPU, the sequential selection here; then
-// the device tables (neighbours [m][P], reverse positions, counts) and the
-// Chebyshev coefficients.  Synchronises.
+// The graph of st->f: ranks and selection, the device tables (neighbours [m][P],
+// reverse positions, counts), the links on the host, and the Chebyshev
+// coefficients.  Synchronises.
 int build_graph(nl_state* st) {
   const int H = st->H, W = st->W, mt = st->prm.neighbours, m = st->m;
-  const int h = st->prm.patch / 2, r = st->prm.window / 2, side = 2 * r + 1, NW = side * side;
+  const int h = st->prm.patch / 2, r = st->prm.window / 2, side = 2 * r + 1;
   const size_t P = st->P();
   const auto G = patch_weights(h, st->prm.a);
   // twice the FP32 distances' relative error bound; negative when a weight is
@@ -875,74 +1031,40 @@ int build_graph(nl_state* st) {
   for (double g : G) gmin = std::min(gmin, g);
   const float bound = gmin < 1e-30 ? -1.f : static_cast<float>(2.02 * (static_cast<double>(G.size()) * st->C + 4) / 16777216.0);
   NL_CK(cudaMemcpyAsync(st->gw, G.data(), sizeof(double) * G.size(), cudaMemcpyHostToDevice, st->stream));
-  auto launch_rank = [&](int y, int strips, unsigned char* rank, unsigned char* head) {
-    const dim3 grid((W + kRankTX - 1) / kRankTX, strips);
+  auto* codes = reinterpret_cast<unsigned char*>(st->codes);
+  const auto* rank = reinterpret_cast<const unsigned*>(st->rank);
+  NL_CK(cudaMemsetAsync(codes, 255, P * kMaxM, st->stream));
+  NL_CK(cudaMemsetAsync(st->deg, 0, P, st->stream));
+  for (int y = 0; y < H; y += st->rank_rows) {
+    const int rows = std::min(st->rank_rows, H - y);
+    const dim3 grid((W + kRankTX - 1) / kRankTX, (rows + kRankTY - 1) / kRankTY);
     if (st->C == 1)
-      k_nl_rank<1><<<grid, 32 * kRankWarps, 0, st->stream>>>(st->f, H, W, st->gw, h, r, bound, y, rank, head);
+      k_nl_rank<1><<<grid, 32 * kRankWarps, 0, st->stream>>>(st->f, H, W, st->gw, h, r, bound, y, y + rows, st->rank);
     else
-      k_nl_rank<3><<<grid, 32 * kRankWarps, 0, st->stream>>>(st->f, H, W, st->gw, h, r, bound, y, rank, head);
-    return cudaGetLastError();
-  };
-  // every rank of the strip of kRankTY rows that holds row y (for the few
-  // pixels that need more than the first ones)
-  std::vector<unsigned char> strip;
-  int strip_y = -1;
-  auto fetch_strip = [&](int y) -> int {
-    const int y0 = y / kRankTY * kRankTY;
-    if (y0 == strip_y) return SHF_OK;
-    const size_t bytes = static_cast<size_t>(std::min(kRankTY, H - y0)) * W * NW;
-    unsigned char* drank = nullptr;
-    strip.resize(bytes);
-    NL_CK(cudaMallocAsync(reinterpret_cast<void**>(&drank), bytes, st->stream));
-    cudaError_t e = launch_rank(y0, 1, drank, nullptr);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(strip.data(), drank, bytes, cudaMemcpyDeviceToHost, st->stream);
-    const cudaError_t e2 = cudaFreeAsync(drank, st->stream);
-    if (e == cudaSuccess) e = e2;
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st->stream);
-    NL_CK(e);
-    strip_y = y0;
-    return SHF_OK;
-  };
-  NL_CK(launch_rank(0, (H + kRankTY - 1) / kRankTY, nullptr, st->head));
-  NL_CK(cudaMemcpyAsync(st->head_host, st->head, P * kRankHead, cudaMemcpyDeviceToHost, st->stream));
-  NL_CK(cudaStreamSynchronize(st->stream));
-  // selection in raster order over the ranked candidates
-  int* const nb = st->nbr_host;
-  unsigned char* const dg = st->deg_host;
-  std::fill(dg, dg + P, static_cast<unsigned char>(0));
-  std::vector<int> step(NW);
-  for (int c = 0; c < NW; ++c) step[c] = (c / side - r) * W + (c % side - r);
-  for (size_t i = 0; i < P; ++i) {
-    int left = std::min(mt, m - static_cast<int>(dg[i]));
-    int* mine = nb + i * m;
-    const unsigned char* rk = st->head_host + i * kRankHead;
-    for (int pos = 0; pos < NW && left > 0; ++pos) {
-      if (pos == kRankHead) {  // beyond the ranks copied for every pixel (rare)
-        const int rc = fetch_strip(static_cast<int>(i / W));
-        if (rc) return rc;
-        rk = strip.data() + (i - static_cast<size_t>(strip_y) * W) * NW;
-      }
-      const int c = rk[pos];
-      if (c == 255) break;  // the rest lie outside the image
-      const int j = static_cast<int>(i) + step[c];
-      if (dg[j] >= m) continue;
-      bool linked = false;
-      for (int b = 0; b < dg[i]; ++b) linked = linked || mine[b] == j;
-      if (linked) continue;
-      mine[dg[i]++] = j;
-      nb[static_cast<size_t>(j) * m + dg[j]++] = static_cast<int>(i);
-      --left;
+      k_nl_rank<3><<<grid, 32 * kRankWarps, 0, st->stream>>>(st->f, H, W, st->gw, h, r, bound, y, y + rows, st->rank);
+    NL_CK(cudaGetLastError());
+    // a half warp for every row of a step
+    const int threads = std::min(1024, (std::min(rows, (W + side - 1) / side) + 1) / 2 * 32);
+    const int R = 2 * r + (W - 1) / side + 1;
+    if (static_cast<size_t>(R) * W <= kRingBytes) {
+      NL_CK(cudaFuncSetAttribute(k_nl_select<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kRingBytes)));
+      k_nl_select<true><<<1, threads, static_cast<size_t>(R) * W, st->stream>>>(rank, H, W, r, m, mt, y, rows, R, codes, st->deg);
+    } else {
+      k_nl_select<false><<<1, threads, 0, st->stream>>>(rank, H, W, r, m, mt, y, rows, R, codes, st->deg);
     }
+    NL_CK(cudaGetLastError());
   }
-  st->deg_max = 0;
-  for (size_t i = 0; i < P; ++i) st->deg_max = std::max(st->deg_max, static_cast<int>(dg[i]));
-  NL_CK(cudaMemcpyAsync(st->list, nb, sizeof(int) * P * m, cudaMemcpyHostToDevice, st->stream));
-  NL_CK(cudaMemcpyAsync(st->deg, dg, P, cudaMemcpyHostToDevice, st->stream));
   const unsigned tgrid = static_cast<unsigned>((P + kThreads - 1) / kThreads);
-  k_nl_tables<<<tgrid, kThreads, 0, st->stream>>>(st->list, st->deg, m, P, st->nbr, st->off);
+  k_nl_tables<<<tgrid, kThreads, 0, st->stream>>>(codes, st->deg, W, r, m, P, st->nbr, st->off);
   NL_CK(cudaGetLastError());
   k_nl_reverse<<<tgrid, kThreads, 0, st->stream>>>(st->nbr, st->deg, m, P, st->rev);
   NL_CK(cudaGetLastError());
+  NL_CK(cudaMemcpyAsync(st->codes_host, codes, P * kMaxM, cudaMemcpyDeviceToHost, st->stream));
+  NL_CK(cudaMemcpyAsync(st->deg_host, st->deg, P, cudaMemcpyDeviceToHost, st->stream));
+  NL_CK(cudaStreamSynchronize(st->stream));
+  const unsigned char* const dg = st->deg_host;
+  st->deg_max = 0;
+  for (size_t i = 0; i < P; ++i) st->deg_max = std::max(st->deg_max, static_cast<int>(dg[i]));
   // Chebyshev iteration on [1, 1 + 4 deg_max]: theta = centre, delta = half width
   const double lo = 1.0, hi = 1.0 + 4.0 * st->deg_max;
   const double theta = 0.5 * (hi + lo), delta = 0.5 * (hi - lo);
@@ -1170,6 +1292,8 @@ int nl_admm_init(int H, int W, const float* f, int C, const float* codebook, int
     st->own_stream = true;
   }
   const size_t P = static_cast<size_t>(H) * W, m = st->m;
+  const size_t rank_row = static_cast<size_t>(W) * kRankPitch;
+  st->rank_rows = static_cast<int>(std::min<size_t>(H, std::max<size_t>(kRankBytes / rank_row, kRankTY)));
   int rc;
   if ((rc = nl_alloc(&st->f, P * C, "f")) || (rc = nl_alloc(&st->s, P * K, "s")) ||
       (rc = nl_alloc(&st->u, P * K, "u")) || (rc = nl_alloc(&st->xa, P * st->Q, "chebyshev x")) ||
@@ -1180,9 +1304,8 @@ int nl_admm_init(int H, int W, const float* f, int C, const float* codebook, int
       (rc = nl_alloc(&st->rhs, P * st->Q, "rhs")) || (rc = nl_alloc(&st->gap, P, "gap")) ||
       (rc = nl_alloc(&st->nbr, P * m, "neighbours")) || (rc = nl_alloc(&st->off, P * m, "offsets")) ||
       (rc = nl_alloc(&st->rev, P * m, "reverse")) || (rc = nl_alloc(&st->gw, kMaxPatch * kMaxPatch, "weights")) ||
-      (rc = nl_alloc(&st->head, P * kRankHead, "ranks")) || (rc = nl_alloc(&st->list, P * m, "links")) ||
-      (rc = nl_alloc_host(&st->nbr_host, P * m, "links")) || (rc = nl_alloc_host(&st->deg_host, P, "counts")) ||
-      (rc = nl_alloc_host(&st->head_host, P * kRankHead, "ranks")) ||
+      (rc = nl_alloc(&st->rank, rank_row * st->rank_rows, "ranks")) || (rc = nl_alloc(&st->codes, P, "links")) ||
+      (rc = nl_alloc_host(&st->codes_host, P * kMaxM, "links")) || (rc = nl_alloc_host(&st->deg_host, P, "counts")) ||
       (rc = nl_alloc(&st->deg, P, "counts")) || (rc = nl_alloc(&st->labels, P, "labels")) ||
       (rc = nl_alloc(&st->flag, 1, "flag")) || (rc = nl_alloc(&st->red, 2 * kRedBlocks + 2, "red")) ||
       (rc = nl_alloc(&st->cbar, 1, "barrier")) || (rc = nl_alloc(&st->cerr, 1, "barrier flag"))) {
@@ -1219,9 +1342,13 @@ int nl_admm_graph(const nl_state* st, int* nbr, int* deg, int* solve_steps) {
   if (!st) return nl_fail(SHF_ERR_ARG, "nl_admm_graph: NULL state");
   if (nbr) {  // the selection's links, sorted, -1 padded
     const size_t P = st->P(), m = st->m;
+    const int side = 2 * (st->prm.window / 2) + 1, r = side / 2;
     for (size_t i = 0; i < P; ++i) {
       int* o = nbr + i * m;
-      std::copy(st->nbr_host + i * m, st->nbr_host + i * m + st->deg_host[i], o);
+      for (int b = 0; b < st->deg_host[i]; ++b) {
+        const int c = st->codes_host[i * kMaxM + b];
+        o[b] = static_cast<int>(i) + (c / side - r) * st->W + (c % side - r);
+      }
       std::sort(o, o + st->deg_host[i]);
       std::fill(o + st->deg_host[i], o + m, -1);
     }
