@@ -188,7 +188,8 @@ int seg_admm_step(seg_state* st, int n_iters);
  * FFT kernels: the v-step's (8, 16, 12, 20 or 32 values per thread, one row
  * or a pair of rows per thread group) and the fan's and gather's (8, 16, 12
  * or 20 values per thread), among those that exist for the size, and whether
- * the iteration's launches overlap (serial).  Fields of the other path
+ * the iteration's launches overlap (serial).  A new state starts with the
+ * plan for its size that measured best.  Fields of the other path
  * are 0 in seg_admm_get_plan and ignored by seg_admm_set_plan.  The plan
  * changes the grouping of the FP32 synthesis sums (wave_mib,
  * col_ctas_per_sm, groups) and the order of the FFT arithmetic (row_kernel,
@@ -212,7 +213,7 @@ typedef struct {
                         height, 1 8 values per thread, 2 16 values (heights
                         512, 1024, 2048), 3 12 or 20 values (heights 12 T or
                         20 T, T = 2..128)                                     */
-  int serial;        /* fast: 0 (default) each kernel of the iteration is
+  int serial;        /* fast: 0 each kernel of the iteration is
                         launched with programmatic dependent launch (its CTAs
                         start while the previous kernel drains), 1 plain
                         stream order; no effect on the results            */
@@ -473,8 +474,8 @@ typedef struct {
 } nl_params;
 
 /* f: device [C][H][W] (H, W in 8..2048); codebook: HOST [K][C].  Builds the
- * neighbour graph of f (patch distances and their ranking on the GPU, the
- * sequential selection on the host), the data term and the zero state.
+ * neighbour graph of f (patch distances, their ranking and the selection in
+ * raster order, on the GPU), the data term and the zero state.
  * Synchronises.  Errors: SHF_ERR_ARG, SHF_ERR_SIZE, SHF_ERR_NONFINITE,
  * SHF_ERR_OOM, SHF_ERR_CUDA. */
 int nl_admm_init(int H, int W, const float* f, int C, const float* codebook, int K, const nl_params* params,

@@ -158,7 +158,7 @@ struct LaunchHook {
 };
 
 // Static work list of the fast path.  A wave is a set of (label, filter)
-// pairs whose coefficient spectra stay in L2 between its three launches: the
+// pairs whose coefficient spectra are held between its three launches: the
 // filters [f0, f0 + nf) of one label when a label's spectra exceed the wave
 // budget, else whole labels [l0, l0 + nl) (nf = eta), so that small images
 // fill the GPU with fewer, larger launches.  The wave's spectra are indexed by
