@@ -475,7 +475,7 @@ def run_ours(args):
         if rank == 0:
             line["batched"] = b
     if rank == 0 and world == 1 and not args.no_differentiable and name == WORKLOAD:
-        line["differentiable"] = measure_differentiable(2, 1)
+        line["differentiable"] = measure_differentiable(2, 3)
     if rank == 0:
         print(json.dumps(line))
     if world > 1:
