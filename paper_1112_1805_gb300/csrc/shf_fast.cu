@@ -122,7 +122,7 @@ int fast_col_ctas(const Geo& g, int per_sm, int col_kernel, int sms) {
 }
 
 int fast_row_ctas(const Geo& g, int row_kernel, int sms) {
-  return fast::row_ctas_per_sm(g.L, 0, row_kernel) * sms_for(sms);
+  return fast::row_ctas_per_sm(g, 0, row_kernel) * sms_for(sms);
 }
 
 int fast_fan_ctas(const Geo& g, int col_kernel, int sms) { return fast::fan_ctas_per_sm(g.H, col_kernel) * sms_for(sms); }
@@ -225,7 +225,7 @@ cudaError_t run_fast_iteration_body(const Geo& g, const FastPlan& plan, const fl
                                     cudaStream_t st, const LaunchHook& hook, signed char* code) {
   const int Whp = fast_pitch(g);
   const int nw = static_cast<int>(plan.wave_f0.size());
-  const int rpc = fast::row_groups_per_cta(g.L, 0, plan.row_kernel);
+  const int rpc = fast::row_groups_per_cta(g, 0, plan.row_kernel);
   hook.mark(kKindColFwd);
   cudaError_t e = fast::col_fwd(g, Ur, uhat, K, Whp, st);
   for (int w = 0; w < nw && e == cudaSuccess; ++w) {
@@ -287,8 +287,8 @@ cudaError_t run_fast_adjoint_body(const Geo& g, const FastPlan& plan, const floa
   const PdlScope pdl(!plan.serial);
   const int Whp = fast_pitch(g);
   const int nw = static_cast<int>(plan.wave_f0.size());
-  const int rpc = fast::row_groups_per_cta(g.L, 1);
-  const int actas = fast::row_ctas_per_sm(g.L, 1) * sm_count();
+  const int rpc = fast::row_groups_per_cta(g, 1);
+  const int actas = fast::row_ctas_per_sm(g, 1) * sm_count();
   cudaError_t e = fast::col_fwd(g, Qr, uhat, K, Whp, st);
   for (int w = 0; w < nw && e == cudaSuccess; ++w) {
     const fast::Wave wv{plan.wave_l0[w], plan.wave_f0[w], plan.wave_nf[w], plan.wave_nl[w] * plan.wave_nf[w]};

@@ -134,11 +134,11 @@ cudaError_t prepare_row_kernels(int L);
 // (mode 0) or of its adjoint (mode 1).
 // `variant` (RowKernel, shf_internal.h) selects the forward v-step: 8 values
 // per thread, 16 (half widths 64..1024, powers of two) or pairs of rows (64,
-// 128); 0 is the default for the width; the adjoint (mode 1) always takes its
-// default.
+// 128, even heights); 0 is the default for the size; the adjoint (mode 1) always
+// takes its default.
 bool row_kernel_ok(int L, int variant);
-int row_ctas_per_sm(int L, int mode = 0, int variant = 0);
-int row_groups_per_cta(int L, int mode = 0, int variant = 0);
+int row_ctas_per_sm(const Geo& g, int mode = 0, int variant = 0);
+int row_groups_per_cta(const Geo& g, int mode = 0, int variant = 0);
 // v-step on the rows of wave wv: ctas resident CTAs; code (optional,
 // [K][eta][H][W] bytes) receives 0 where |g| < t, else sign g.
 cudaError_t row_shrink(const Geo& g, int ctas, float2* Y, float* bv, const float* thr, int Whp, const Wave& wv,

@@ -1151,12 +1151,16 @@ cudaError_t prepare_row_kernels(int N) {
   }
 }
 
-// The forward v-step a plan's variant selects at half width L (the default:
+// The forward v-step a plan's variant selects at g's half width (the default:
 // pairs of rows at 64 and 128, radix-16 rows at the other powers of two up to
-// 1024, 8 values per thread elsewhere).
-int row_variant(int L, int mode, int variant) {
+// 1024, 8 values per thread elsewhere).  The one place that chooses: a pair needs
+// an even height (the general path has odd ones too), an odd one takes single
+// rows of 16 values.
+int row_variant(const Geo& g, int mode, int variant) {
+  const int L = g.L;
   if (mode == 1) return use_r16(L) ? kRow16 : kRow8;
-  if (variant == kRowDefault) return use_pair(L) ? kRowPair : (use_r16(L) ? kRow16 : (use_v(L) ? kRowV : kRow8));
+  if (variant == kRowDefault) variant = use_pair(L) ? kRowPair : (use_r16(L) ? kRow16 : (use_v(L) ? kRowV : kRow8));
+  if (variant == kRowPair && (g.H & 1)) variant = kRow16;
   if (variant == kRowPair && !use_pair(L)) return kRow8;
   if (variant == kRow16 && !use_r16(L)) return kRow8;
   if (variant == kRowV && !use_v(L)) return kRow8;
@@ -1168,11 +1172,11 @@ bool row_kernel_ok(int L, int variant) {
          (variant == kRowPair && use_pair(L)) || (variant == kRowV && use_v(L));
 }
 
-int row_ctas_per_sm(int L, int mode, int variant) {
+int row_ctas_per_sm(const Geo& g, int mode, int variant) {
   int fit = 0;
   cudaError_t e = cudaErrorInvalidValue;
-  const int v = row_variant(L, mode, variant);
-  switch (L) {
+  const int v = row_variant(g, mode, variant);
+  switch (g.L) {
 #define SHF_OCC(N)                                                                                              \
   case N:                                                                                                       \
     if (v == kRowPair)                                                                                          \
@@ -1198,9 +1202,9 @@ int row_ctas_per_sm(int L, int mode, int variant) {
   return e == cudaSuccess ? fit : 0;
 }
 
-int row_groups_per_cta(int L, int mode, int variant) {
-  const int v = row_variant(L, mode, variant);
-  switch (L) {
+int row_groups_per_cta(const Geo& g, int mode, int variant) {
+  const int v = row_variant(g, mode, variant);
+  switch (g.L) {
 #define SHF_CASE(N)                                        \
   case N:                                                  \
     if (v == kRowPair) return 2 * PairGeo<pair_len(N)>::RPC; /* rows */ \
@@ -1214,7 +1218,7 @@ int row_groups_per_cta(int L, int mode, int variant) {
 
 cudaError_t row_shrink(const Geo& g, int ctas, float2* Y, float* bv, const float* thr, int Whp, const Wave& wv,
                        float scale, signed char* code, int variant, cudaStream_t st) {
-  const int v = row_variant(g.L, 0, variant);
+  const int v = row_variant(g, 0, variant);
   switch (g.L) {
 #define SHF_CASE(N)                                                                                                \
   case N:                                                                                                          \

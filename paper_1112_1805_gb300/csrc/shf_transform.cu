@@ -567,7 +567,7 @@ cudaError_t run_wave_shrink(const Geo& g, float2* Y, float* bv, const float* thr
                             cudaStream_t st, float* gout) {
   if (fast_shrink_ok(g) && !gout) {  // the register-FFT v-step of this half width
     const fast::Wave f = fast_wave_of(wv);
-    const int rpc = fast::row_groups_per_cta(g.L), groups = (f.nv * g.H + rpc - 1) / rpc;
+    const int rpc = fast::row_groups_per_cta(g), groups = (f.nv * g.H + rpc - 1) / rpc;
     return fast::row_shrink(g, std::min(groups, std::max(1, fast_row_ctas(g))), Y, bv, thr, g.Wy, f, scale, nullptr, 0, st);
   }
   if (g.staged) {
