@@ -530,46 +530,55 @@ int shearlet_synthesize(const shf_bank* b, const float* coef, int nch, float* u,
 
 namespace {
 
-// Returns a state's buffer; the caller has waited for its users.  (To the pool in
-// the order of the legacy stream: the state's own stream may be gone by now.)
-void state_free(seg_state* st, void* p) {
+// Returns a state's buffer in the order of `order`: what that stream has queued by
+// now runs before the pool hands the memory on.  A call that fails leaves no error
+// behind for a later launch's check (in a broken context those fail by themselves).
+void state_free_in(seg_state* st, void* p, cudaStream_t order) {
   if (!p) return;
   const auto it = std::find(st->direct.begin(), st->direct.end(), p);
+  cudaError_t e;
   if (it == st->direct.end()) {
-    cudaFreeAsync(p, nullptr);
+    e = cudaFreeAsync(p, order);
   } else {
     st->direct.erase(it);
-    cudaFree(p);
+    e = cudaFree(p);
   }
+  if (e != cudaSuccess) cudaGetLastError();
 }
+// ... of its own stream, in which pool memory is allocated and used: a buffer that
+// an unfinished call gives back has its allocation there, and maybe a user.
+void state_free(seg_state* st, void* p) { state_free_in(st, p, st->stream); }
 
 void free_state(seg_state* s) {
+  // The caller's stream may be gone by now: everything is waited for, and the
+  // buffers go back in the order of the legacy stream.
   cudaDeviceSynchronize();
+  const auto give = [s](void* p) { state_free_in(s, p, nullptr); };
   if (s->exec) cudaGraphExecDestroy(s->exec);
   if (s->exec_timed) cudaGraphExecDestroy(s->exec_timed);
   for (cudaEvent_t e : s->ev)
     if (e) cudaEventDestroy(e);
-  state_free(s, s->uhat);
-  state_free(s, s->d_lists);
-  state_free(s, s->un_Y);
-  state_free(s, s->un_partial);
-  state_free(s, s->un_pt);
+  give(s->uhat);
+  give(s->d_lists);
+  give(s->un_Y);
+  give(s->un_partial);
+  give(s->un_pt);
   if (s->un_fwd_exec) cudaGraphExecDestroy(s->un_fwd_exec);
   if (s->un_bwd_exec) cudaGraphExecDestroy(s->un_bwd_exec);
-  state_free(s, s->un_mem);
-  for (float* p : s->ck_bv) state_free(s, p);
-  for (float* p : s->ck_w) state_free(s, p);
-  for (float* p : s->ck_bw) state_free(s, p);
-  for (float2* p : s->ck_T) state_free(s, p);
+  give(s->un_mem);
+  for (float* p : s->ck_bv) give(p);
+  for (float* p : s->ck_w) give(p);
+  for (float* p : s->ck_bw) give(p);
+  for (float2* p : s->ck_T) give(p);
   float* fl[] = {s->f, s->s, s->bv, s->w, s->bw, s->u, s->stv, s->thr, s->lam, s->gap};
-  for (float* p : fl) state_free(s, p);
-  state_free(s, s->Ur);
-  state_free(s, s->Y);
-  state_free(s, s->partial);
-  state_free(s, s->T);
-  state_free(s, s->labels);
+  for (float* p : fl) give(p);
+  give(s->Ur);
+  give(s->Y);
+  give(s->partial);
+  give(s->T);
+  give(s->labels);
   release_flag(s->device, s->bad);
-  state_free(s, s->red);
+  give(s->red);
   if (s->own_stream && s->stream) cudaStreamDestroy(s->stream);
   if (s->pool) release_pool(s->device);
   delete s;

@@ -1,0 +1,94 @@
+// The library's states on the stand-in runtime of fake_cudart.h: every allocation
+// of every call is made to fail once.  A call that runs out of memory says so,
+// leaves the state usable, returns what it had taken in the order of the stream it
+// was taken on, and nothing is left when everything is destroyed.
+#include <cstdio>
+#include <string>
+#include <vector>
+
+#include "fake_cudart.h"
+#include "shearseg.h"
+
+namespace {
+
+int failures = 0;
+void expect(bool ok, const char* what, int n = 0) {
+  if (!ok) {
+    ++failures;
+    std::printf("FAILED: %s (%d): %s\n", what, n, shf_last_error());
+  }
+}
+
+struct Problem {
+  int H, W, K, J;
+  std::vector<float> f, cb, lam;
+  shf_bank* bank = nullptr;
+  Problem(int h, int w, int k, int j) : H(h), W(w), K(k), J(j), f(static_cast<size_t>(h) * w, 0.5f), lam(j + 1, 0.01f) {
+    for (int i = 0; i < k; ++i) cb.push_back(0.1f * (i + 1));
+    expect(shfilters_build(H, W, J, nullptr, &bank) == SHF_OK, "bank");
+  }
+  ~Problem() { shfilters_destroy(bank); }
+  int init(seg_state** st) {
+    seg_params p{};
+    p.gamma = 1.f;
+    p.Lambda = lam.data();
+    p.J = J;
+    p.max_iters = 10;
+    return seg_admm_init(bank, f.data(), 1, cb.data(), K, &p, nullptr, st);
+  }
+};
+
+// Calls `call` with its first, second, ... allocation failing, until none is left
+// to fail; the number of calls that ran out of memory.  A call may do without the
+// allocation that failed; `undo` then takes its result back.
+template <typename F, typename U>
+int exhaust(const char* what, F&& call, U&& undo) {
+  int out = 0;
+  for (int n = 1; n < 200; ++n) {
+    fake::fail_alloc_at = n;
+    const int rc = call();
+    const bool none_failed = fake::fail_alloc_at > 0;
+    fake::fail_alloc_at = 0;
+    expect(rc == SHF_OK || (!none_failed && rc == SHF_ERR_OOM), what, n);
+    if (none_failed) return out;
+    if (rc == SHF_OK)
+      undo();
+    else
+      ++out;
+  }
+  expect(false, what);
+  return out;
+}
+
+void plans_and_sweeps(int H, int W) {
+  Problem pb(H, W, 3, 2);
+  seg_state* st = nullptr;
+  expect(exhaust("init", [&] { return pb.init(&st); }, [&] { seg_admm_destroy(st); }) > 10, "init: failing allocations");
+  seg_plan plan{};
+  expect(seg_admm_get_plan(st, &plan) == SHF_OK, "get_plan");
+  if (plan.fast) {
+    plan.wave_mib = 1;
+  } else {
+    plan.groups = plan.groups > 1 ? 1 : 2;
+  }
+  expect(seg_admm_step(st, 2) == SHF_OK, "step");
+  const auto nothing = [] {};
+  expect(exhaust("set_plan", [&] { return seg_admm_set_plan(st, &plan); }, nothing) >= 2, "set_plan: failing allocations");
+  expect(seg_admm_step(st, 2) == SHF_OK, "step");
+  expect(exhaust("unrolled_fwd", [&] { return seg_admm_unrolled_fwd(st, 6, 2); }, nothing) >= 3, "unrolled_fwd: failing allocations");
+  std::vector<float> g(static_cast<size_t>(H) * W * 3, 0.f);
+  expect(exhaust("unrolled_bwd", [&] { return seg_admm_unrolled_bwd_enqueue(st, g.data()); }, nothing) >= 1,
+         "unrolled_bwd: failing allocations");
+  expect(seg_admm_destroy(st) == SHF_OK, "destroy");
+}
+
+}  // namespace
+
+int main() {
+  plans_and_sweeps(64, 64);  // register-FFT path
+  plans_and_sweeps(30, 50);  // general path
+  expect(fake::violations == 0, "buffers returned in order", fake::violations);
+  expect(fake::live() == 0, "buffers left", static_cast<int>(fake::live()));
+  std::printf("%s\n", failures ? "failed" : "all ok");
+  return failures ? 1 : 0;
+}
