@@ -1705,6 +1705,46 @@ cudaError_t enqueue_unrolled_bwd(seg_state* st, const UnLayout& U) {
   return e;
 }
 
+// The general path's sweep plans, their tables and scratch; the state has them all
+// or, after a failure, none.
+int make_sweep_scratch(seg_state* st) {
+  const Geo& g = st->g;
+  const size_t Ph = st->Ph();
+  // filter groups for four CTAs per SM over all labels, unless the plan says otherwise
+  int groups = st->groups;
+  if (groups == shf::default_groups(g, st->K)) {
+    const int base = g.ntiles * st->K;
+    groups = normalise_groups(g.eta, (4 * 152 + base - 1) / base);
+  }
+  Geo sg = g;
+  sg.staged = 1;
+  if (!shf::make_sweep_plan(g.H, &sg.planH) || !shf::make_sweep_plan(g.L, &sg.planL))
+    return fail(SHF_ERR_SIZE, "unsupported geometry");
+  sg.planLr = sg.planL;
+  std::vector<shf::FilterWave> waves = shf::general_waves(g, st->K, groups);
+  float2 *pt = nullptr, *Y = nullptr, *partial = nullptr;
+  int rc;
+  if (!(rc = state_alloc(st, &pt, shf::pass_table_entries(sg), "pass tables")) &&
+      !(rc = state_alloc(st, &Y, shf::wave_planes(waves) * g.H * g.Wy, "unrolled scratch")) &&
+      !(rc = state_alloc(st, &partial, Ph * st->K * static_cast<size_t>(groups), "unrolled partials"))) {
+    const cudaError_t e = shf::launch_pass_tables(&sg, pt, st->stream);
+    if (e != cudaSuccess) rc = fail(SHF_ERR_CUDA, std::string("pass tables: ") + cudaGetErrorString(e));
+  }
+  if (rc) {
+    state_free(st, pt);
+    state_free(st, Y);
+    state_free(st, partial);
+    return rc;
+  }
+  st->un_g = sg;
+  st->un_waves = std::move(waves);
+  st->un_groups = groups;
+  st->un_pt = pt;
+  st->un_Y = Y;
+  st->un_partial = partial;
+  return SHF_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -1714,33 +1754,9 @@ int seg_admm_unrolled_fwd(seg_state* st, int T, int ckpt_every) {
   const Geo& g = st->g;
   const size_t P = st->P(), Ph = st->Ph(), KP = P * st->K, NC = KP * g.eta;
   int rc;
-  // the general path keeps the spectra of every filter; the fast path
-  // iterates with its own wave scratch
-  if (!st->fast && !st->un_Y) {
-    // filter groups for four CTAs per SM over all labels, unless the plan says otherwise
-    int groups = st->groups;
-    if (groups == shf::default_groups(g, st->K)) {
-      const int base = g.ntiles * st->K;
-      groups = normalise_groups(g.eta, (4 * 152 + base - 1) / base);
-    }
-    st->un_g = g;
-    st->un_g.staged = 1;
-    if (!shf::make_sweep_plan(g.H, &st->un_g.planH) || !shf::make_sweep_plan(g.L, &st->un_g.planL))
-      return fail(SHF_ERR_SIZE, "unsupported geometry");
-    st->un_g.planLr = st->un_g.planL;
-    st->un_waves = shf::general_waves(g, st->K, groups);
-    if ((rc = state_alloc(st, &st->un_pt, shf::pass_table_entries(st->un_g), "pass tables")) ||
-        (rc = state_alloc(st, &st->un_Y, shf::wave_planes(st->un_waves) * g.H * g.Wy, "unrolled scratch")) ||
-        (rc = state_alloc(st, &st->un_partial, Ph * st->K * static_cast<size_t>(groups), "unrolled partials"))) {
-      state_free(st, st->un_pt);
-      state_free(st, st->un_Y);
-      st->un_pt = nullptr;
-      st->un_Y = nullptr;
-      return rc;
-    }
-    SHF_CK(shf::launch_pass_tables(&st->un_g, st->un_pt, st->stream));
-    st->un_groups = groups;
-  }
+  // the fast path iterates with its plan's wave scratch; the general path has a
+  // wave of its own (another number of filter groups, sweep plans)
+  if (!st->fast && !st->un_Y && (rc = make_sweep_scratch(st))) return rc;
   const int nseg = (T + ckpt_every - 1) / ckpt_every;
   while (static_cast<int>(st->ck_bv.size()) < nseg) {
     float *bv = nullptr, *w = nullptr, *bw = nullptr;

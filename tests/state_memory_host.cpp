@@ -82,11 +82,28 @@ void plans_and_sweeps(int H, int W) {
   expect(seg_admm_destroy(st) == SHF_OK, "destroy");
 }
 
+// The unrolled sweeps' tables of the general path: a launch that fails is reported,
+// and the next call makes them after all.
+void failed_tables() {
+  Problem pb(30, 50, 3, 2);
+  seg_state* st = nullptr;
+  expect(pb.init(&st) == SHF_OK, "init");
+  const std::size_t before = fake::live();
+  fake::fail_kernel = "k_pass_table";
+  expect(seg_admm_unrolled_fwd(st, 4, 2) == SHF_ERR_CUDA, "unrolled_fwd: tables fail");
+  expect(!fake::fail_kernel && fake::live() == before, "unrolled_fwd: buffers of a failed setup");
+  const int tables = fake::launched("k_pass_table");
+  expect(seg_admm_unrolled_fwd(st, 4, 2) == SHF_OK, "unrolled_fwd after a failed one");
+  expect(fake::launched("k_pass_table") == tables + 3, "unrolled_fwd: the tables of three plans");
+  expect(seg_admm_destroy(st) == SHF_OK, "destroy");
+}
+
 }  // namespace
 
 int main() {
   plans_and_sweeps(64, 64);  // register-FFT path
   plans_and_sweeps(30, 50);  // general path
+  failed_tables();
   expect(fake::violations == 0, "buffers returned in order", fake::violations);
   expect(fake::live() == 0, "buffers left", static_cast<int>(fake::live()));
   std::printf("%s\n", failures ? "failed" : "all ok");
