@@ -410,8 +410,10 @@ int tv_admm_init(int H, int W, const float* f, int C, const float* codebook, int
  * recomputed, state back to zero.  Synchronises. */
 int tv_admm_reset(tv_state* st, const float* f, int f_on_host);
 
-/* Enqueues n_iters iterations (replays of a CUDA graph of one iteration when
- * the stream can be captured). */
+/* Enqueues n_iters iterations: one as separate kernels (the replay of a CUDA
+ * graph when the stream can be captured), several as two kernels each between
+ * the separate ones of the first and the last, at most sizes.  The iterates do
+ * not depend on how the iterations are split over calls, bit for bit. */
 int tv_admm_step(tv_state* st, int n_iters);
 
 /* Readouts as seg_admm_get: SEG_U, SEG_W, SEG_BW, SEG_S ([K][H][W]), SEG_BV

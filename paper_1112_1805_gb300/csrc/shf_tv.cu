@@ -122,13 +122,16 @@ __global__ void __launch_bounds__(kThreads) k_tv_prox(const float* __restrict__ 
         const float bn = gw[k] - wk[k];
         w[k * P + x] = wk[k];
         bw[k * P + x] = bn;
-        q[k * P + x] = (wk[k] - bn) - gamma * s[k * P + x];
+        q[k * P + x] = fmaf(-gamma, s[k * P + x], wk[k] - bn);
       }
     }
   }
 }
 
-// rhs = q + grad^T d: (grad^T d)(r, c) = d0(r-1, c) - d0(r, c) + d1(r, c-1) - d1(r, c).
+// rhs = q + grad^T d: (grad^T d)(r, c) = d0(r-1, c) - d0(r, c) + d1(r, c-1) - d1(r, c),
+// summed in the order of shf_tv_rows.cu, so that iterates don't depend on how the
+// iterations are split over calls: what a column pair holds itself first, then what
+// comes from the row above and the pair to the left.
 __global__ void __launch_bounds__(kThreads) k_tv_rhs(const float* __restrict__ q, const float* __restrict__ d,
                                                      float* __restrict__ rhs, int K, int H, int W) {
   const size_t P = static_cast<size_t>(H) * W;
@@ -141,7 +144,8 @@ __global__ void __launch_bounds__(kThreads) k_tv_rhs(const float* __restrict__ q
     const float* d1 = d0 + P;
     const size_t xr = static_cast<size_t>(r == 0 ? H - 1 : r - 1) * W + c;
     const size_t xc = static_cast<size_t>(r) * W + (c == 0 ? W - 1 : c - 1);
-    rhs[i] = q[i] + ((d0[xr] - d0[x]) + (d1[xc] - d1[x]));
+    rhs[i] = (c & 1) == 0 ? (q[i] - (d0[x] + d1[x])) + (d0[xr] + d1[xc])
+                          : (q[i] + ((d1[xc] - d1[x]) - d0[x])) + d0[xr];
   }
 }
 

@@ -97,7 +97,8 @@ __global__ void __launch_bounds__(256, 2)
       const float2 am = *reinterpret_cast<const float2*>(d0m + c);
       const float2 b = *reinterpret_cast<const float2*>(d1r + c);
       const float bm = d1r[c == 0 ? W - 1 : c - 1];
-      v[j] = live ? make_float2(qq.x + ((am.x - a.x) + (bm - b.x)), qq.y + ((am.y - a.y) + (b.x - b.y)))
+      // the sums in the order of shf_tv_rows.cu (and k_tv_rhs)
+      v[j] = live ? make_float2((qq.x - (a.x + b.x)) + (am.x + bm), (qq.y + ((b.x - b.y) - a.y)) + am.y)
                   : make_float2(0.f, 0.f);
     }
     r16::row_fft<L, -1>(v, tt, fb, pt, bar);

@@ -13,6 +13,10 @@
 // item of its own: the CTA's loads are all in flight at once, where walking down
 // the rows with the row above in registers left one row's latency after the
 // other (with the staged transforms: 31 us a launch at 512 x 512, K = 4).
+//
+// Its arithmetic is that of the separate kernels, operation by operation (the row
+// transforms are the same functions, and the right-hand side is summed in this
+// kernel's order there too): n iterations in one call give the bits of n calls.
 #include <algorithm>
 
 #include "shf_fast.h"
@@ -144,7 +148,7 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_tv_band(const BandArgs a, cons
         if (k < K) {
           const float2 bn = make_float2(gx[k] - wx[k], gy[k] - wy[k]), sv = s2[k * HL + off];
           bw2[k * HL + off] = bn;
-          q[k] = make_float2((wx[k] - bn.x) - a.gamma * sv.x, (wy[k] - bn.y) - a.gamma * sv.y);
+          q[k] = make_float2(fmaf(-a.gamma, sv.x, wx[k] - bn.x), fmaf(-a.gamma, sv.y, wy[k] - bn.y));
         }
     }
 #pragma unroll
