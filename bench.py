@@ -557,10 +557,13 @@ def tv_kernel_bytes(H, W, K):
     transforms (right-hand side in, half spectra through, u out; the symbol
     read once) and the two pointwise kernels (the prox kernel reads u, b_v,
     b_w, s and writes b_v, d, w, b_w, q: 48 B per pixel and label; the
-    right-hand side reads q and d and writes rhs: 16 B)."""
+    right-hand side reads q and d and writes rhs: 16 B); and for the row half
+    of an iteration in one kernel the spectra in and out, b_v and b_w read and
+    written and s read (28 B per pixel and label)."""
     P, Ph = H * W, H * (W // 2 + 1)
     return {"tv_row_fwd": K * (P * 4 + Ph * 8), "tv_col_solve": K * 2 * Ph * 8 + Ph * 4,
-            "tv_row_inv": K * (Ph * 8 + P * 4), "tv_prox": K * P * 48, "tv_rhs": K * P * 16}
+            "tv_row_inv": K * (Ph * 8 + P * 4), "tv_prox": K * P * 48, "tv_rhs": K * P * 16,
+            "tv_band": K * (2 * Ph * 8 + P * 28)}
 
 
 def measure_tv(iters: int, steps: int, warmup: int, lam: float = 1.0 / 12.0):
@@ -595,7 +598,7 @@ def measure_tv(iters: int, steps: int, warmup: int, lam: float = 1.0 / 12.0):
     ev1.synchronize()
     ms = ev0.elapsed_time(ev1)
     label_error = float((labels_dev.cpu().numpy() != lab).mean())
-    kt = seg.kernel_times(5)
+    kt = seg.loop_kernel_times(20)
     seg.close()
     units = wl.H * wl.W * wl.K * iters * steps
     kb = tv_kernel_bytes(wl.H, wl.W, wl.K)

@@ -427,12 +427,22 @@ int tv_admm_get(tv_state* st, int what, void* dst, int dst_on_host);
  * rebuilds the next u-step's right-hand side.  Synchronises. */
 int tv_admm_set(tv_state* st, int what, const void* src, int src_on_host);
 
-/* Instrumentation (no counterpart in the paper): runs n iterations launched
- * one by one with CUDA events between the kernels and writes the mean
- * milliseconds of each of the iteration's 5 kernels to ms (room for 5), *nk
- * (may be NULL) = 5.  Advances the iterate by n.  Synchronises. */
+/* Instrumentation (no counterpart in the paper): runs n iterations of the
+ * separate kernels (those of a call of one iteration, and of the last one of a
+ * longer call) with CUDA events between them and writes the mean milliseconds
+ * of each of these 5 kernels to ms (room for 5), *nk (may be NULL) = 5.
+ * Advances the iterate by n.  Synchronises. */
 int tv_admm_kernel_times(tv_state* st, int n, float* ms, int* nk);
 const char* tv_admm_kernel_name(int i);
+
+/* The same for the iterations inside a call of several, where almost all the
+ * time of a long call goes: 2 kernels (the column solve, and the row half of
+ * the iteration in one), *nk = 2, the iterate advanced by n + 1; at the sizes
+ * where a call of several runs the separate kernels throughout, these, *nk = 5,
+ * advanced by n.  In the calls themselves the kernels overlap, so their sum is
+ * above the time of an iteration.  The name of kernel i of this state. */
+int tv_admm_loop_kernel_times(tv_state* st, int n, float* ms, int* nk);
+const char* tv_admm_loop_kernel_name(const tv_state* st, int i);
 
 int tv_admm_sync(tv_state* st);
 /* Releases the state (synchronises its stream).  NULL is accepted. */

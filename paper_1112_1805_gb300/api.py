@@ -377,8 +377,13 @@ class TVSegmenter:
         return self.get(B.SEG_LABELS)
 
     def kernel_times(self, n: int = 5) -> dict:
-        """Mean milliseconds per kernel over n iterations (advances the iterate)."""
+        """Mean milliseconds of the separate kernels of an iteration over n of them (advances the iterate)."""
         return B.tv_admm_kernel_times(self.handle, n)
+
+    def loop_kernel_times(self, n: int = 5) -> dict:
+        """Mean milliseconds per kernel over n iterations inside a call of several (advances the iterate by n + 1,
+        or by n at the sizes that run the separate kernels throughout)."""
+        return B.tv_admm_loop_kernel_times(self.handle, n)
 
 
 class NLSegmenter(TVSegmenter):
@@ -467,6 +472,9 @@ class NLSegmenter(TVSegmenter):
 
     def kernel_times(self, n: int = 5) -> dict:
         return B.nl_admm_kernel_times(self.handle, n)
+
+    def loop_kernel_times(self, n: int = 5) -> dict:
+        return self.kernel_times(n)  # every iteration runs the same kernels
 
 
 class UnrolledSegmentation(torch.autograd.Function):

@@ -121,6 +121,8 @@ _SIG = {
     "tv_admm_set": (_I, [_VP, _I, _VP, _I]),
     "tv_admm_kernel_times": (_I, [_VP, _I, ctypes.POINTER(ctypes.c_float), ctypes.POINTER(_I)]),
     "tv_admm_kernel_name": (ctypes.c_char_p, [_I]),
+    "tv_admm_loop_kernel_times": (_I, [_VP, _I, ctypes.POINTER(ctypes.c_float), ctypes.POINTER(_I)]),
+    "tv_admm_loop_kernel_name": (ctypes.c_char_p, [_VP, _I]),
     "tv_admm_sync": (_I, [_VP]),
     "tv_admm_destroy": (_I, [_VP]),
     "nl_admm_init": (_I, [_I, _I, _VP, _I, ctypes.POINTER(ctypes.c_float), _I, ctypes.POINTER(nl_params), _VP,
@@ -415,11 +417,19 @@ def tv_admm_set(state: int, what: int, src: int, src_on_host: bool) -> None:
 
 
 def tv_admm_kernel_times(state: int, n: int) -> dict:
-    """{kernel: mean milliseconds} over n iterations launched one by one."""
+    """{kernel: mean milliseconds} over n iterations of the separate kernels."""
     ms = (ctypes.c_float * 8)()
     nk = _I()
     _call("tv_admm_kernel_times", _VP(state), int(n), ms, ctypes.byref(nk))
     return {lib().tv_admm_kernel_name(i).decode(): float(ms[i]) for i in range(nk.value)}
+
+
+def tv_admm_loop_kernel_times(state: int, n: int) -> dict:
+    """{kernel: mean milliseconds} over n iterations inside a call of several."""
+    ms = (ctypes.c_float * 8)()
+    nk = _I()
+    _call("tv_admm_loop_kernel_times", _VP(state), int(n), ms, ctypes.byref(nk))
+    return {lib().tv_admm_loop_kernel_name(_VP(state), i).decode(): float(ms[i]) for i in range(nk.value)}
 
 
 def tv_admm_sync(state: int) -> None:

@@ -325,8 +325,9 @@ cudaError_t enqueue_tv_iteration(tv_state* st, cudaEvent_t* ev) {
 // last one leaves u, w, d and q behind as a single iteration does, and those in
 // between are two launches each (shf_tv_rows.cu; b_v alternates between two
 // buffers).  Launched directly, as programmatic dependents: two launches cost
-// the host less than the GPU takes for them.
-cudaError_t enqueue_tv_iterations(tv_state* st, int n) {
+// the host less than the GPU takes for them.  `ev` (optional, 2 n - 1 events):
+// recorded before each launch of those in between and after the last of them.
+cudaError_t enqueue_tv_iterations(tv_state* st, int n, cudaEvent_t* ev = nullptr) {
   const Geo& g = st->g;
   cudaStream_t ss = st->stream;
   const float scale = 1.f / (static_cast<float>(g.H) * g.W), t = st->gamma * st->lambda;
@@ -334,12 +335,19 @@ cudaError_t enqueue_tv_iterations(tv_state* st, int n) {
                            : shf::run_row_r2c(g, st->rhs, st->Ur, st->K, 1.f, ss);
   const float* in = st->bv;
   float* out = st->bv_other;
+  auto mark = [&](int i) {
+    if (ev && e == cudaSuccess) e = cudaEventRecord(ev[i], ss);
+  };
   for (int i = 0; i < n && e == cudaSuccess; ++i) {
+    mark(2 * i);
+    if (e != cudaSuccess) break;
     e = st->fast ? shf::tvfast::tv_fast_cols(st->Ur, st->sym, st->Y, st->K, g.H, g.W, g.twH, ss)
                  : shf::run_col_filter(g, st->Ur, st->Y, st->K, ss);
     if (e != cudaSuccess || i == n - 1) break;
-    e = shf::tvfast::tv_band(st->Y, st->Ur, st->pitch, in, out, st->bw, st->s, st->K, g.H, g.W, t, st->gamma, st->per_label,
-                            g.twW, ss);
+    mark(2 * i + 1);
+    if (e == cudaSuccess)
+      e = shf::tvfast::tv_band(st->Y, st->Ur, st->pitch, in, out, st->bw, st->s, st->K, g.H, g.W, t, st->gamma, st->per_label,
+                              g.twW, ss);
     in = out;
     out = in == st->bv ? st->bv_other : st->bv;
   }
@@ -551,6 +559,36 @@ int tv_admm_kernel_times(tv_state* st, int n, float* ms, int* nk) {
   if (rc == SHF_OK) st->iter += n;
   if (nk) *nk = kTvKinds;
   return rc;
+}
+
+int tv_admm_loop_kernel_times(tv_state* st, int n, float* ms, int* nk) {
+  if (!st || !ms || n < 1) return tv_fail(SHF_ERR_ARG, "tv_admm_loop_kernel_times: bad argument");
+  if (!st->bv_other) return tv_admm_kernel_times(st, n, ms, nk);
+  std::vector<cudaEvent_t> ev(2 * static_cast<size_t>(n) + 1, nullptr);
+  cudaError_t e = cudaSuccess;
+  for (cudaEvent_t& x : ev)
+    if (e == cudaSuccess) e = cudaEventCreate(&x);
+  // n iterations of the loop and the last one of a call
+  if (e == cudaSuccess) e = enqueue_tv_iterations(st, n + 1, ev.data());
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st->stream);
+  ms[0] = ms[1] = 0.f;
+  for (int i = 0; i < 2 * n && e == cudaSuccess; ++i) {
+    float t = 0.f;
+    e = cudaEventElapsedTime(&t, ev[i], ev[i + 1]);
+    ms[i & 1] += t / n;
+  }
+  for (cudaEvent_t x : ev)
+    if (x) cudaEventDestroy(x);
+  if (e != cudaSuccess)
+    return tv_fail(SHF_ERR_CUDA, std::string("tv_admm_loop_kernel_times: ") + cudaGetErrorString(e));
+  st->iter += n + 1;
+  if (nk) *nk = 2;
+  return SHF_OK;
+}
+
+const char* tv_admm_loop_kernel_name(const tv_state* st, int i) {
+  if (!st || !st->bv_other) return tv_admm_kernel_name(i);
+  return i == 0 ? kTvNames[kTvCol] : (i == 1 ? "tv_band" : "");
 }
 
 const char* tv_admm_kernel_name(int i) { return (i >= 0 && i < kTvKinds) ? kTvNames[i] : ""; }
