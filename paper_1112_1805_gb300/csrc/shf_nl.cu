@@ -1371,8 +1371,8 @@ int nl_admm_step(nl_state* st, int n) {
         if (cudaGraphInstantiate(&st->exec, graph, 0) != cudaSuccess) st->exec = nullptr;
       }
       if (graph) cudaGraphDestroy(graph);
-      cudaGetLastError();
     }
+    cudaGetLastError();  // also of a stream that can't be captured
   }
   for (int i = 0; i < n; ++i) {
     if (st->exec)

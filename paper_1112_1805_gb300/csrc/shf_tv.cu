@@ -526,8 +526,8 @@ int tv_admm_step(tv_state* st, int n) {
         if (cudaGraphInstantiate(&st->exec, graph, 0) != cudaSuccess) st->exec = nullptr;
       }
       if (graph) cudaGraphDestroy(graph);
-      cudaGetLastError();
     }
+    cudaGetLastError();  // also of a stream that can't be captured
   }
   for (int i = 0; i < n; ++i) {
     if (st->exec)
