@@ -851,6 +851,18 @@ int install_fast_plan(seg_state* st, int wave_mib, int col_ctas_per_sm, int row_
   return SHF_OK;
 }
 
+// The plan that a new state starts with; where its larger waves do not fit in
+// memory, waves of kWaveMiB.  (Waves of 1024 MiB hold all spectra of most states,
+// another b_v: a 512 x 512, K = 4, J = 4 state takes 570 MB in place of 430.)
+int install_default_plan(seg_state* st) {
+  const shf::FastPlan def = shf::default_fast_plan(st->g);
+  const auto install = [&](int mib) {
+    return install_fast_plan(st, mib, 0, def.row_kernel, def.col_kernel, def.serial);
+  };
+  const int rc = install(def.wave_mib);
+  return rc == SHF_ERR_OOM && def.wave_mib > shf::kWaveMiB ? install(shf::kWaveMiB) : rc;
+}
+
 // Filter groups as the general-path kernels use them: groups of ceil(eta/G)
 // filters, no group empty.
 int normalise_groups(int eta, int G) {
@@ -997,7 +1009,6 @@ int seg_admm_init(const shf_bank* b, const float* f, int C, const float* codeboo
   st->fast = shf::fast_path_ok(g);
   st->fast_ustep = shf::fast_ustep_ok(g, K);
   if (!st->fast) st->waves = shf::general_waves(g, K, st->groups);
-  const shf::FastPlan def = shf::default_fast_plan(g);
   int rc;
   if ((rc = state_alloc(st, &st->f, P * C, "f")) || (rc = state_alloc(st, &st->s, P * K, "s")) ||
       (rc = state_alloc(st, &st->bv, P * K * g.eta, "b_v")) || (rc = state_alloc(st, &st->w, P * K, "w")) ||
@@ -1009,10 +1020,11 @@ int seg_admm_init(const shf_bank* b, const float* f, int C, const float* codeboo
       // the general path (the fast path's come with its plan)
       (!st->fast && (rc = state_alloc(st, &st->Y, shf::wave_planes(st->waves) * g.H * g.Wy, "Y"))) ||
       (!st->fast && (rc = state_alloc(st, &st->partial, Ph * K * static_cast<size_t>(st->groups), "partial"))) ||
-      (st->fast && (rc = install_fast_plan(st, def.wave_mib, 0, def.row_kernel, def.col_kernel, def.serial))) ||
       (rc = state_alloc(st, &st->thr, g.eta, "thr")) || (rc = state_alloc(st, &st->lam, g.eta, "lam")) ||
       (rc = state_alloc(st, &st->gap, P, "gap")) || (rc = state_alloc(st, &st->labels, P, "labels")) ||
-      (rc = acquire_flag(st->device, &st->bad)) || (rc = state_alloc(st, &st->red, 2 + 512, "red"))) {
+      (rc = acquire_flag(st->device, &st->bad)) || (rc = state_alloc(st, &st->red, 2 + 512, "red")) ||
+      // last: its size depends on what is left
+      (st->fast && (rc = install_default_plan(st)))) {
     free_state(st);
     return rc;
   }

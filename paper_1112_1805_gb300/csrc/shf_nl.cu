@@ -1304,11 +1304,18 @@ int nl_admm_init(int H, int W, const float* f, int C, const float* codebook, int
       (rc = nl_alloc(&st->rhs, P * st->Q, "rhs")) || (rc = nl_alloc(&st->gap, P, "gap")) ||
       (rc = nl_alloc(&st->nbr, P * m, "neighbours")) || (rc = nl_alloc(&st->off, P * m, "offsets")) ||
       (rc = nl_alloc(&st->rev, P * m, "reverse")) || (rc = nl_alloc(&st->gw, kMaxPatch * kMaxPatch, "weights")) ||
-      (rc = nl_alloc(&st->rank, rank_row * st->rank_rows, "ranks")) || (rc = nl_alloc(&st->codes, P, "links")) ||
+      (rc = nl_alloc(&st->codes, P, "links")) ||
       (rc = nl_alloc_host(&st->codes_host, P * kMaxM, "links")) || (rc = nl_alloc_host(&st->deg_host, P, "counts")) ||
       (rc = nl_alloc(&st->deg, P, "counts")) || (rc = nl_alloc(&st->labels, P, "labels")) ||
       (rc = nl_alloc(&st->flag, 1, "flag")) || (rc = nl_alloc(&st->red, 2 * kRedBlocks + 2, "red")) ||
       (rc = nl_alloc(&st->cbar, 1, "barrier")) || (rc = nl_alloc(&st->cerr, 1, "barrier flag"))) {
+    free_nl(st);
+    return rc;
+  }
+  // as many rows' ranks at a time as there is memory for
+  while ((rc = nl_alloc(&st->rank, rank_row * st->rank_rows, "ranks")) == SHF_ERR_OOM && st->rank_rows > kRankTY)
+    st->rank_rows = std::max(kRankTY, st->rank_rows / 2);
+  if (rc) {
     free_nl(st);
     return rc;
   }

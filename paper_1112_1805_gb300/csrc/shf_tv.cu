@@ -461,7 +461,6 @@ int tv_admm_init(int H, int W, const float* f, int C, const float* codebook, int
   int rc;
   if ((rc = tv_alloc(&st->f, P * C, "f")) || (rc = tv_alloc(&st->s, P * K, "s")) ||
       (rc = tv_alloc(&st->u, P * K, "u")) || (rc = tv_alloc(&st->bv, 2 * P * K, "b_v")) ||
-      (band && (rc = tv_alloc(&st->bv_other, 2 * P * K, "b_v"))) ||
       (rc = tv_alloc(&st->d, 2 * P * K, "d")) || (rc = tv_alloc(&st->w, P * K, "w")) ||
       (rc = tv_alloc(&st->bw, P * K, "b_w")) || (rc = tv_alloc(&st->q, P * K, "q")) ||
       (rc = tv_alloc(&st->rhs, P * K, "rhs")) || (rc = tv_alloc(&st->sym, Ph, "symbol")) ||
@@ -469,7 +468,9 @@ int tv_admm_init(int H, int W, const float* f, int C, const float* codebook, int
       (rc = tv_alloc(&st->twW, W, "twW")) ||
       (rc = tv_alloc(&st->pt, shf::pass_table_entries(g), "pass tables")) || (rc = tv_alloc(&st->Ur, Phs * K, "Ur")) ||
       (rc = tv_alloc(&st->Y, Phs * K, "Y")) || (rc = tv_alloc(&st->labels, P, "labels")) ||
-      (rc = tv_alloc(&st->flag, 1, "flag")) || (rc = tv_alloc(&st->red, 2 * kRedBlocks + 2, "red"))) {
+      (rc = tv_alloc(&st->flag, 1, "flag")) || (rc = tv_alloc(&st->red, 2 * kRedBlocks + 2, "red")) ||
+      // without memory for it the separate kernels run throughout, with the same results
+      (band && (rc = tv_alloc(&st->bv_other, 2 * P * K, "b_v")) && rc != SHF_ERR_OOM)) {
     free_tv(st);
     return rc;
   }

@@ -125,6 +125,44 @@ void no_capture() {
   expect(nl_admm_step(nl, 3) == SHF_OK && nl_admm_destroy(nl) == SHF_OK, "nl: step, destroy");
 }
 
+// What a state takes only to be faster it does without when memory is short: the
+// larger waves of the default plans, TV's second b_v, NL-means ranks of all rows at
+// once.
+void short_of_memory() {
+  {
+    // coefficient spectra of all labels: 264 MB in one wave, b_v 256 MB
+    Problem pb(512, 512, 4, 4);
+    seg_state* st = nullptr;
+    seg_plan plan{};
+    expect(pb.init(&st) == SHF_OK && seg_admm_get_plan(st, &plan) == SHF_OK && plan.wave_mib > 128, "default waves");
+    expect(seg_admm_destroy(st) == SHF_OK, "destroy");
+    fake::fail_over = 260000000;
+    expect(pb.init(&st) == SHF_OK, "init with little memory");
+    fake::fail_over = 0;
+    if (st) {
+      expect(seg_admm_get_plan(st, &plan) == SHF_OK && plan.wave_mib == 128, "waves of 128 MiB", plan.wave_mib);
+      expect(seg_admm_step(st, 2) == SHF_OK && seg_admm_destroy(st) == SHF_OK, "step, destroy");
+    }
+  }
+  const auto served = [](const char* what, auto&& init, auto&& destroy) {  // without the n-th allocation
+    int out = 0;
+    exhaust(what, init, [&] {
+      ++out;
+      destroy();
+    });
+    destroy();
+    return out;
+  };
+  tv_state* tv = nullptr;
+  expect(served("tv_init", [&] { return tv_init(&tv); },
+                [&] { expect(tv_admm_step(tv, 3) == SHF_OK && tv_admm_destroy(tv) == SHF_OK, "tv step, destroy"); }) == 1,
+         "tv: without the second b_v");
+  nl_state* nl = nullptr;
+  expect(served("nl_init", [&] { return nl_init(&nl); },
+                [&] { expect(nl_admm_step(nl, 3) == SHF_OK && nl_admm_destroy(nl) == SHF_OK, "nl step, destroy"); }) == 1,
+         "nl: ranks of fewer rows at a time");
+}
+
 }  // namespace
 
 int main() {
@@ -132,6 +170,7 @@ int main() {
   plans_and_sweeps(30, 50);  // general path
   failed_tables();
   no_capture();
+  short_of_memory();
   expect(fake::violations == 0, "buffers returned in order", fake::violations);
   expect(fake::live() == 0, "buffers left", static_cast<int>(fake::live()));
   std::printf("%s\n", failures ? "failed" : "all ok");
