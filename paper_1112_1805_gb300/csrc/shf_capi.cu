@@ -20,8 +20,11 @@ namespace {
 
 thread_local std::string g_err;
 
+// An error of the runtime is reported once: left pending, it would be taken for
+// that of the next kernel launched.
 int fail(int code, const std::string& msg) {
   g_err = msg;
+  if (code == SHF_ERR_CUDA || code == SHF_ERR_OOM) cudaGetLastError();
   return code;
 }
 

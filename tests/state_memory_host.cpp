@@ -125,6 +125,31 @@ void no_capture() {
   expect(nl_admm_step(nl, 3) == SHF_OK && nl_admm_destroy(nl) == SHF_OK, "nl: step, destroy");
 }
 
+// An error is reported by the call that meets it and by no later one.
+void reported_once() {
+  Problem pb(270, 64, 3, 2);  // general path, more than one plane per CTA
+  seg_state* st = nullptr;
+  expect(pb.init(&st) == SHF_OK, "init");
+  std::vector<float> u(3ul * 270 * 64, 0.f), c(13 * u.size(), 0.f);
+  double energy = 0;
+  const auto once = [](const char* what, auto&& call) {
+    for (int n = 1; n <= 2; ++n) {
+      fake::fail_alloc_at = n;
+      const int rc = call();
+      const bool failed = fake::fail_alloc_at == 0;
+      fake::fail_alloc_at = 0;
+      expect((rc != SHF_OK) == failed && call() == SHF_OK, what, n);
+    }
+    fake::fail_kernel = "k_";
+    expect(call() == SHF_ERR_CUDA && call() == SHF_OK, what);
+  };
+  once("analyze", [&] { return shearlet_analyze(pb.bank, u.data(), 3, c.data(), nullptr); });
+  once("synthesize", [&] { return shearlet_synthesize(pb.bank, c.data(), 3, u.data(), nullptr); });
+  once("energy", [&] { return seg_admm_get(st, SEG_ENERGY, &energy, 1); });
+  once("set v", [&] { return seg_admm_set(st, SEG_V, c.data(), 1); });
+  expect(seg_admm_destroy(st) == SHF_OK, "destroy");
+}
+
 // What a state takes only to be faster it does without when memory is short: the
 // larger waves of the default plans, TV's second b_v, NL-means ranks of all rows at
 // once.
@@ -170,6 +195,7 @@ int main() {
   plans_and_sweeps(30, 50);  // general path
   failed_tables();
   no_capture();
+  reported_once();
   short_of_memory();
   expect(fake::violations == 0, "buffers returned in order", fake::violations);
   expect(fake::live() == 0, "buffers left", static_cast<int>(fake::live()));
