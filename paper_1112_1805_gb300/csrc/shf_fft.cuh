@@ -205,14 +205,9 @@ __host__ __device__ __forceinline__ void dft_small(float2* v) {
 // Inverse packing: from the half spectrum X[0..L] of a real row, the complex
 // sequence whose unscaled inverse DFT of length L has the even samples of the
 // unscaled length-W inverse in its real part and the odd samples in its
-// imaginary part:  Z[k] = (X[k] + conj X[L-k]) + i e^{+2 pi i k/W} (X[k] - conj X[L-k]).
-__host__ __device__ __forceinline__ float2 c2r_pack(const float2* X, int L, int k, const float2* twW) {
-  const float2 a = X[k];
-  const float2 b = c_conj(X[L - k]);
-  const float2 s = c_add(a, b), d = c_sub(a, b);
-  return pack_combine(s, d, twW[k]);
-}
-
+// imaginary part:  Z[k] = (X[k] + conj X[L-k]) + i e^{+2 pi i k/W} (X[k] - conj X[L-k])
+// (pack_combine, on what the row kernels load of X).
+//
 // Forward unpacking: Z = DFT_L(x[2n] + i x[2n+1]); returns X[k], k = 0..L,
 // X[k] = 1/2 [ (Z_k + conj Z_{L-k}) - i e^{-2 pi i k/W} (Z_k - conj Z_{L-k}) ] (indices mod L).
 __host__ __device__ __forceinline__ float2 r2c_unpack(const float2* Z, int L, int k, const float2* twW) {

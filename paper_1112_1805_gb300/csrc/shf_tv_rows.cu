@@ -27,6 +27,7 @@ namespace shf {
 namespace tvfast {
 namespace {
 
+using fast::even2;
 using fast::launch_pdl;
 using fast::load_table;
 using fast::pack_row;
@@ -35,7 +36,6 @@ using fast::pdl_wait;
 using fast::Rows;
 
 __host__ __device__ constexpr bool len_ok(int L) { return fast::half_ok(L) && L <= 640 && L >= 32; }
-__host__ __device__ constexpr int even2(int n) { return (n + 1) & ~1; }
 
 template <int L, int NT>
 struct BandGeo {
