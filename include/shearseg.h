@@ -105,9 +105,11 @@ int shfilters_copy(const shf_bank* bank, float* dst, void* stream);
  * Shearlet transform S (eq. wichtig: one fft2 per channel, then per filter a
  * pointwise product with the real spectrum and an ifft2).
  * u: device [nch][H][W]; coef: device [nch][eta][H][W] (must not alias u).
- * Temporary device memory is taken stream-ordered from the default pool and
- * returned before the call's work completes.  Errors: SHF_ERR_ARG,
- * SHF_ERR_OOM, SHF_ERR_CUDA. */
+ * Temporary device memory is taken in the stream's order from a memory pool
+ * that the library keeps per device while it has a bank or a state there (up
+ * to 512 MiB stay in it between calls), and returned before the call's work
+ * completes; an analysis of planes that fit one CTA takes none.  Errors:
+ * SHF_ERR_ARG, SHF_ERR_OOM, SHF_ERR_CUDA. */
 int shearlet_analyze(const shf_bank* bank, const float* u, int nch, float* coef, void* stream);
 
 /* Adjoint S^T (the synthesis paragraph after the Theorem: fft2 of every
@@ -166,10 +168,11 @@ int seg_admm_init(const shf_bank* bank, const float* f, int C, const float* code
  * data term and returns the state to v = b_v = w = b_w = 0, iteration 0. */
 int seg_admm_reset(seg_state* st, const float* f, int f_on_host);
 
-/* Enqueues n_iters ADMM iterations on the state's stream (replays of a CUDA
- * graph of one iteration, captured on first use when the stream allows it;
- * the last iteration of each call records the events of
- * seg_admm_kernel_times). */
+/* Enqueues n_iters ADMM iterations on the state's stream: launched one by one
+ * where an iteration is short (K eta H W up to 3.3e7) and for sizes without
+ * the register-FFT path, otherwise as replays of a CUDA graph of one
+ * iteration, captured on first use when the stream allows it.  The last
+ * iteration of each call records the events of seg_admm_kernel_times. */
 int seg_admm_step(seg_state* st, int n_iters);
 
 /* ---------------------------------------------------------------------------
@@ -287,8 +290,10 @@ int seg_admm_load(seg_state* st, const char* path);
  * Jacobian of the simplex projection on the active face, the 0/1 masks of the
  * clipping |g| < gamma Lambda, and S / S^T exchanged).
  * seg_admm_unrolled_fwd returns the state to v = b_v = w = b_w = 0, runs T
- * iterations on the general-size kernels and keeps the state of every
- * ckpt_every-th iteration on the device.  seg_admm_unrolled_bwd takes dL/dw_T
+ * iterations and keeps the state of every ckpt_every-th iteration on the
+ * device.  A state's first sweeps for a (T, ckpt_every) launch their kernels one
+ * by one, the second ones capture them as CUDA graphs (and take longer than
+ * the first where the launches are short), later ones replay these.  seg_admm_unrolled_bwd takes dL/dw_T
  * (device [K][H][W]) of a loss of the final w, recomputes each segment from
  * its checkpoint, runs the adjoint iterations backwards and returns
  * dL/dcodebook (HOST [K][C]), dL/dLambda (HOST [J+1]), and optionally dL/df

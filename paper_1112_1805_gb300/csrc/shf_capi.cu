@@ -856,7 +856,7 @@ int install_fast_plan(seg_state* st, int wave_mib, int col_ctas_per_sm, int row_
 
 // The plan that a new state starts with; where its larger waves do not fit in
 // memory, waves of kWaveMiB.  (Waves of 1024 MiB hold all spectra of most states,
-// another b_v: a 512 x 512, K = 4, J = 4 state takes 570 MB in place of 430.)
+// another b_v: a 512 x 512, K = 4, J = 4 state takes 570 MB in place of 440.)
 int install_default_plan(seg_state* st) {
   const shf::FastPlan def = shf::default_fast_plan(st->g);
   const auto install = [&](int mib) {
@@ -1791,7 +1791,12 @@ int seg_admm_unrolled_fwd(seg_state* st, int T, int ckpt_every) {
   }
   // the first sweep of a (T, ckpt) is launched directly (a state made for one
   // training step never pays for a graph: capturing and instantiating takes the
-  // host longer than launching), the second one captured, later ones replayed
+  // host longer than launching), the second one captured, later ones replayed.
+  // A forward and reverse pass in us, first / second / third, and with the capture
+  // in the first: 64 x 64, K = 3, T = 10 1029 / 1266 / 811 (1652 / 895 / 887); 256 x
+  // 256, K = 4, T = 10 2162 / 2153 / 1957 (3155 / 2142 / 2137), T = 50 9890 / 9933 /
+  // 9232 (13554 / 10144 / 10137).  So the second pass of a small state can take
+  // longer, but no number of passes does.
   const bool again = st->un_fwd_key[0] == T && st->un_fwd_key[1] == ckpt_every;
   if (!again && st->un_fwd_exec) {
     cudaGraphExecDestroy(st->un_fwd_exec);

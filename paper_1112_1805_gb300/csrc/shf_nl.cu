@@ -103,7 +103,9 @@ __device__ __forceinline__ int mirror_idx(int x, int n) {
 // such candidates is ordered.  The bound: with the weights and the image
 // in the range checked below, a distance is a sum of n positive terms, each
 // with four rounding errors, so its relative error is at most (n + 4) 2^-24
-// (the caller's `delta` doubles it) plus what underflow costs (kTiny).
+// (the caller's `delta` doubles it) plus what underflow costs (kTiny).  Rounding
+// the bound itself costs nothing: a distance above the rounded bound is at least
+// the next number up, which lies above the exact one.
 constexpr int kRankTX = 32, kRankTY = 4;  // pixels per CTA
 constexpr int kMaxHalo = kMaxWin / 2 + kMaxPatch / 2;
 constexpr int kRankRows = kRankTY + 2 * kMaxHalo, kRankCols = kRankTX + 2 * kMaxHalo;
