@@ -2203,6 +2203,8 @@ extern "C" {
 
 int seg_admm_batch_tune(seg_batch* b, int iters) {
   if (!b || iters < 1) return fail(SHF_ERR_ARG, "seg_admm_batch_tune: bad argument");
+  // the images' iterates are saved on their own streams: the batch's iterations end first
+  SHF_CK(cudaStreamSynchronize(b->stream));
   // every image back on grids for all SMs before its shape is tuned alone
   for (seg_state* st : b->states) {
     if (!st->fast || st->plan.sms == 0) continue;

@@ -12,6 +12,7 @@
 
 namespace fake {
 int violations = 0, fail_alloc_at = 0;
+bool capture = false;
 std::size_t fail_over = 0;
 const char* fail_kernel = nullptr;
 
@@ -36,6 +37,11 @@ std::map<std::string, int>& runs() {
   return *m;
 }
 std::set<cudaStream_t> busy;  // streams with work since they were waited for
+bool capturing = false;
+std::set<cudaStream_t> captured;                                // streams with work in the capture
+std::map<std::uintptr_t, std::set<cudaStream_t>> graphs;        // ... in a graph (or its executable)
+std::map<cudaStream_t, std::set<cudaStream_t>> flights;         // ... in the graphs running on a stream
+std::map<cudaEvent_t, cudaStream_t> recorded;
 cudaError_t last = cudaSuccess;
 std::uintptr_t next_handle = 0x1000;
 struct {
@@ -47,6 +53,27 @@ struct {
 template <typename T>
 T handle() {
   return reinterpret_cast<T>(next_handle += 16);
+}
+// Work on a stream: a copy or a kernel.
+void work_on(cudaStream_t st) {
+  if (capturing) {
+    captured.insert(st);
+    return;
+  }
+  busy.insert(st);
+  for (const auto& f : flights)
+    if (f.first != st && f.second.count(st)) {
+      std::printf("violation: work on a stream beside the graph that runs its work elsewhere\n");
+      ++violations;
+    }
+}
+void waited_for(cudaStream_t st) {
+  busy.erase(st);
+  flights.erase(st);
+}
+void all_waited_for() {
+  busy.clear();
+  flights.clear();
 }
 cudaError_t allocate(void** p, std::size_t n, Kind kind, cudaStream_t st) {
   *p = nullptr;
@@ -70,7 +97,6 @@ cudaError_t release(void* p, Kind kind, cudaStream_t st) {
     std::printf("violation: %zu bytes returned in another stream's order\n", it->second.bytes);
     ++violations;
   }
-  if (kind == kAsync) busy.insert(st);
   std::free(p);
   buffers().erase(it);
   return cudaSuccess;
@@ -82,7 +108,7 @@ cudaError_t run(const void* fun, cudaStream_t st) {
     return last = cudaErrorLaunchOutOfResources;
   }
   ++runs()[n];
-  busy.insert(st);
+  work_on(st);
   return cudaSuccess;
 }
 }  // namespace
@@ -154,7 +180,7 @@ cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr a, int) {
   return cudaSuccess;
 }
 cudaError_t cudaDeviceSynchronize() {
-  busy.clear();
+  all_waited_for();
   return cudaSuccess;
 }
 cudaError_t cudaGetLastError() {
@@ -167,7 +193,7 @@ const char* cudaGetErrorString(cudaError_t) { return "made to fail"; }
 // memory
 cudaError_t cudaMalloc(void** p, size_t n) { return allocate(p, n, kPlain, nullptr); }
 cudaError_t cudaFree(void* p) {
-  busy.clear();  // waits for the device
+  all_waited_for();  // waits for the device
   return release(p, kPlain, nullptr);
 }
 cudaError_t cudaMallocHost(void** p, size_t n) { return allocate(p, n, kHost, nullptr); }
@@ -187,40 +213,58 @@ cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) {
 }
 cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind, cudaStream_t st) {
   std::memcpy(d, s, n);
-  busy.insert(st);
+  work_on(st);
   return cudaSuccess;
 }
 cudaError_t cudaMemset(void*, int, size_t) { return cudaSuccess; }
 cudaError_t cudaMemsetAsync(void*, int, size_t, cudaStream_t st) {  // nothing reads the values
-  busy.insert(st);
+  work_on(st);
   return cudaSuccess;
 }
 
-// streams, events, graphs (no capture: the library then launches directly)
+// streams, events, graphs (without capture the library launches directly)
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) {
   *s = handle<cudaStream_t>();
   return cudaSuccess;
 }
 cudaError_t cudaStreamDestroy(cudaStream_t) { return cudaSuccess; }
 cudaError_t cudaStreamSynchronize(cudaStream_t s) {
-  busy.erase(s);
+  waited_for(s);
   return cudaSuccess;
 }
 cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
 cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* c) {
-  *c = cudaStreamCaptureStatusNone;
+  *c = capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
   return cudaSuccess;
 }
-cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) { return last = cudaErrorNotSupported; }
+cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) {
+  if (!capture || capturing) return last = cudaErrorNotSupported;
+  capturing = true;
+  captured.clear();
+  return cudaSuccess;
+}
 cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t* g) {
-  *g = nullptr;
-  return last = cudaErrorNotSupported;
+  *g = handle<cudaGraph_t>();
+  capturing = false;
+  graphs[reinterpret_cast<std::uintptr_t>(*g)] = captured;
+  return cudaSuccess;
 }
-cudaError_t cudaGraphInstantiate(cudaGraphExec_t* e, cudaGraph_t, unsigned long long) {
-  *e = nullptr;
-  return last = cudaErrorNotSupported;
+cudaError_t cudaGraphInstantiate(cudaGraphExec_t* e, cudaGraph_t g, unsigned long long) {
+  *e = handle<cudaGraphExec_t>();
+  graphs[reinterpret_cast<std::uintptr_t>(*e)] = graphs[reinterpret_cast<std::uintptr_t>(g)];
+  return cudaSuccess;
 }
-cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) { return last = cudaErrorNotSupported; }
+cudaError_t cudaGraphLaunch(cudaGraphExec_t e, cudaStream_t st) {
+  for (cudaStream_t x : graphs[reinterpret_cast<std::uintptr_t>(e)]) {
+    if (x != st && busy.count(x)) {
+      std::printf("violation: a graph launched beside work on a stream whose work it runs\n");
+      ++violations;
+    }
+    flights[st].insert(x);
+  }
+  work_on(st);
+  return cudaSuccess;
+}
 cudaError_t cudaGraphDestroy(cudaGraph_t) { return cudaSuccess; }
 cudaError_t cudaGraphExecDestroy(cudaGraphExec_t) { return cudaSuccess; }
 cudaError_t cudaEventCreate(cudaEvent_t* e) {
@@ -229,9 +273,15 @@ cudaError_t cudaEventCreate(cudaEvent_t* e) {
 }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) { return cudaEventCreate(e); }
 cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
-cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
-cudaError_t cudaEventRecordWithFlags(cudaEvent_t, cudaStream_t, unsigned) { return cudaSuccess; }
-cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t st) {
+  if (!capturing) recorded[e] = st;
+  return cudaSuccess;
+}
+cudaError_t cudaEventRecordWithFlags(cudaEvent_t e, cudaStream_t st, unsigned) { return cudaEventRecord(e, st); }
+cudaError_t cudaEventSynchronize(cudaEvent_t e) {
+  if (recorded.count(e)) waited_for(recorded[e]);
+  return cudaSuccess;
+}
 cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t, cudaEvent_t) {
   *ms = 0.f;
   return cudaSuccess;

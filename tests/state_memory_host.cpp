@@ -150,6 +150,37 @@ void reported_once() {
   expect(seg_admm_destroy(st) == SHF_OK, "destroy");
 }
 
+// A batch's iterations run as a graph on the batch's stream, tuning and readouts on
+// the images' own.
+struct Batch {
+  std::vector<float> f, cb{0.2f, 0.5f, 0.8f}, lam;
+  seg_batch* b = nullptr;
+  Batch() : f(64 * 64, 0.5f), lam(3, 0.01f) {
+    const int H[2] = {64, 30}, W[2] = {64, 50}, C[2] = {1, 1}, K[2] = {3, 3};
+    const float* fs[2] = {f.data(), f.data()};
+    const float* cbs[2] = {cb.data(), cb.data()};
+    seg_params p[2] = {};
+    for (seg_params& x : p) {
+      x.gamma = 1.f;
+      x.Lambda = lam.data();
+      x.J = 2;
+      x.max_iters = 10;
+    }
+    expect(seg_admm_batch_init(2, H, W, C, K, fs, cbs, p, nullptr, &b) == SHF_OK, "batch init");
+  }
+  ~Batch() { expect(seg_admm_batch_destroy(b) == SHF_OK, "batch destroy"); }
+};
+void batch_order() {
+  fake::capture = true;
+  {
+    Batch ba;
+    expect(seg_admm_batch_step(ba.b, 4) == SHF_OK && seg_admm_batch_tune(ba.b, 2) == SHF_OK, "tune after iterations");
+    expect(seg_admm_batch_step(ba.b, 2) == SHF_OK && seg_admm_batch_sync(ba.b) == SHF_OK, "iterations after tune");
+    expect(fake::violations == 0, "batch: streams in order", fake::violations);
+  }
+  fake::capture = false;
+}
+
 // What a state takes only to be faster it does without when memory is short: the
 // larger waves of the default plans, TV's second b_v, NL-means ranks of all rows at
 // once.
@@ -196,6 +227,7 @@ int main() {
   failed_tables();
   no_capture();
   reported_once();
+  batch_order();
   short_of_memory();
   expect(fake::violations == 0, "buffers returned in order", fake::violations);
   expect(fake::live() == 0, "buffers left", static_cast<int>(fake::live()));
