@@ -348,7 +348,9 @@ int seg_admm_batch_step(seg_batch* batch, int n_iters);
 
 /* Borrows image i's state for seg_admm_get/set/save/load/reset (owned by the
  * batch: do not destroy it).  Its work goes to the image's own stream; call
- * seg_admm_batch_sync first to order it after the batch's iterations. */
+ * seg_admm_batch_sync first to order it after the batch's iterations.  Each of
+ * these calls waits for that stream, so that the batch's next iterations come
+ * after it. */
 int seg_admm_batch_image(seg_batch* batch, int i, seg_state** out);
 
 /* Lanes of a batch iteration: with lanes = L in [1, n) the n images form L

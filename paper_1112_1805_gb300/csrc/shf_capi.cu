@@ -1387,8 +1387,18 @@ int seg_admm_solve(seg_state* st, int* iters_done, float* final_residual) {
   return SHF_OK;
 }
 
-int seg_admm_get(seg_state* st, int what, void* dst, int on_host) {
-  if (!st || !dst) return fail(SHF_ERR_ARG, "seg_admm_get: NULL argument");
+}  // extern "C"
+
+namespace {
+
+// An image of a batch: what a call left on the image's stream has ended before the
+// batch's next iterations, which run as a graph on the batch's.
+int settled(seg_state* st, int rc) {
+  if (!rc && st->batch) SHF_CK(cudaStreamSynchronize(st->stream));
+  return rc;
+}
+
+int get_component(seg_state* st, int what, void* dst, int on_host) {
   const Geo& g = st->g;
   const size_t P = st->P(), KP = P * st->K;
   switch (what) {
@@ -1424,8 +1434,7 @@ int seg_admm_get(seg_state* st, int what, void* dst, int on_host) {
   }
 }
 
-int seg_admm_set(seg_state* st, int what, const void* src, int on_host) {
-  if (!st || !src) return fail(SHF_ERR_ARG, "seg_admm_set: NULL argument");
+int set_component(seg_state* st, int what, const void* src, int on_host) {
   const Geo& g = st->g;
   const size_t P = st->P(), KP = P * st->K;
   switch (what) {
@@ -1454,6 +1463,20 @@ int seg_admm_set(seg_state* st, int what, const void* src, int on_host) {
     }
     default: return fail(SHF_ERR_ARG, "selector cannot be set");
   }
+}
+
+}  // namespace
+
+extern "C" {
+
+int seg_admm_get(seg_state* st, int what, void* dst, int on_host) {
+  if (!st || !dst) return fail(SHF_ERR_ARG, "seg_admm_get: NULL argument");
+  return settled(st, get_component(st, what, dst, on_host));
+}
+
+int seg_admm_set(seg_state* st, int what, const void* src, int on_host) {
+  if (!st || !src) return fail(SHF_ERR_ARG, "seg_admm_set: NULL argument");
+  return settled(st, set_component(st, what, src, on_host));
 }
 
 namespace {

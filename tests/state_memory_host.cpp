@@ -176,6 +176,20 @@ void batch_order() {
     Batch ba;
     expect(seg_admm_batch_step(ba.b, 4) == SHF_OK && seg_admm_batch_tune(ba.b, 2) == SHF_OK, "tune after iterations");
     expect(seg_admm_batch_step(ba.b, 2) == SHF_OK && seg_admm_batch_sync(ba.b) == SHF_OK, "iterations after tune");
+    // what a call leaves on an image's stream is not beside the next iterations
+    std::vector<float> x(3ul * 13 * 64 * 64, 0.f);
+    for (int i = 0; i < 2; ++i) {
+      seg_state* st = nullptr;
+      expect(seg_admm_batch_image(ba.b, i, &st) == SHF_OK, "image", i);
+      for (int what : {SEG_W, SEG_STV, SEG_V}) {
+        expect(seg_admm_set(st, what, x.data(), 0) == SHF_OK, "set", what);
+        expect(seg_admm_batch_step(ba.b, 1) == SHF_OK && seg_admm_batch_sync(ba.b) == SHF_OK, "iteration");
+      }
+      for (int what : {SEG_W, SEG_STV, SEG_LABELS}) {
+        expect(seg_admm_get(st, what, x.data(), 0) == SHF_OK, "get", what);
+        expect(seg_admm_batch_step(ba.b, 1) == SHF_OK && seg_admm_batch_sync(ba.b) == SHF_OK, "iteration");
+      }
+    }
     expect(fake::violations == 0, "batch: streams in order", fake::violations);
   }
   fake::capture = false;
