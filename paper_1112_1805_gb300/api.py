@@ -23,6 +23,18 @@ def _dev_f32(t: torch.Tensor, name: str) -> torch.Tensor:
     return t
 
 
+def _readout(shape, dt, stream) -> torch.Tensor:
+    """A tensor for `stream` to write (None: a stream that torch does not know).  Its
+    memory may be that of a freed tensor which work queued on the current stream
+    still reads; that work comes first."""
+    out = torch.empty(shape, dtype=dt, device="cuda")
+    if not torch.cuda.is_current_stream_capturing():
+        cur = torch.cuda.current_stream()
+        if not cur.query():
+            cur.synchronize() if stream is None else stream.wait_stream(cur)
+    return out
+
+
 class FilterBank:
     """Shearlet filter bank for one (H, W, J) (Sec. 2 of the paper)."""
 
@@ -141,7 +153,7 @@ class ShearletSegmenter:
             B.seg_admm_get(self.handle, what, buf.ctypes.data, True)
             return torch.tensor(int(buf[0]))
         shape, dt = self._shape(what)
-        out = torch.empty(shape, dtype=dt, device="cuda")
+        out = _readout(shape, dt, getattr(self, "stream", None))
         B.seg_admm_get(self.handle, what, out.data_ptr(), False)
         self.synchronize()
         return out
@@ -349,7 +361,7 @@ class TVSegmenter:
             B.tv_admm_get(self.handle, what, buf.ctypes.data, True)
             return torch.tensor(int(buf[0]))
         shape, dt = self._shape(what)
-        out = torch.empty(shape, dtype=dt, device="cuda")
+        out = _readout(shape, dt, getattr(self, "stream", None))
         B.tv_admm_get(self.handle, what, out.data_ptr(), False)
         self.synchronize()
         return out
@@ -449,7 +461,7 @@ class NLSegmenter(TVSegmenter):
             B.nl_admm_get(self.handle, what, buf.ctypes.data, True)
             return torch.tensor(int(buf[0]))
         shape, dt = self._shape(what)
-        out = torch.empty(shape, dtype=dt, device="cuda")
+        out = _readout(shape, dt, getattr(self, "stream", None))
         B.nl_admm_get(self.handle, what, out.data_ptr(), False)
         self.synchronize()
         return out
