@@ -272,6 +272,11 @@ int seg_admm_solve(seg_state* st, int* iters_done, float* final_residual);
  * SEG_ENERGY or SEG_ITER.  Errors: SHF_ERR_ARG for an unknown selector. */
 int seg_admm_get(seg_state* st, int what, void* dst, int dst_on_host);
 
+/* seg_admm_get into device memory, waited for, and ordered after the work that
+ * `earlier` has queued by now: for a dst whose memory that stream may still use
+ * (an allocator that hands freed memory on in a stream's order gives such). */
+int seg_admm_read(seg_state* st, int what, void* dst, void* earlier);
+
 /* Overwrites a state component from src (device, or host if src_on_host) --
  * used to resume or to start from a given state.  Accepts SEG_W, SEG_BW,
  * SEG_BV, SEG_STV and SEG_V. */
@@ -428,6 +433,7 @@ int tv_admm_step(tv_state* st, int n_iters);
  * <w, s> + lambda TV(w)), SEG_ITER (int, host only).  Host destinations and
  * SEG_ENERGY synchronise. */
 int tv_admm_get(tv_state* st, int what, void* dst, int dst_on_host);
+int tv_admm_read(tv_state* st, int what, void* dst, void* earlier); /* as seg_admm_read */
 
 /* Overwrites SEG_W, SEG_BW, SEG_BV or SEG_V (v itself; set SEG_BV first,
  * since the state keeps v - b_v, which setting SEG_BV leaves unchanged) and
@@ -518,6 +524,7 @@ int nl_admm_step(nl_state* st, int n_iters);
 
 /* Readouts as tv_admm_get, with SEG_BV and SEG_V of shape [K][m][H][W]. */
 int nl_admm_get(nl_state* st, int what, void* dst, int dst_on_host);
+int nl_admm_read(nl_state* st, int what, void* dst, void* earlier); /* as seg_admm_read */
 
 /* Overwrites SEG_W, SEG_BW, SEG_U (the u-step's starting point), SEG_BV or
  * SEG_V (set SEG_BV first) and rebuilds the right-hand side.  Synchronises. */

@@ -14,25 +14,14 @@ from . import binding as B
 
 
 def _cur_stream():
-    return torch.cuda.current_stream().cuda_stream
+    # the current stream's handle without a Stream object around it (0.1 against 2.9 us)
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _dev_f32(t: torch.Tensor, name: str) -> torch.Tensor:
     if not (t.is_cuda and t.dtype == torch.float32 and t.is_contiguous()):
         raise ValueError(f"{name} must be a contiguous float32 CUDA tensor")
     return t
-
-
-def _readout(shape, dt, stream) -> torch.Tensor:
-    """A tensor for `stream` to write (None: a stream that torch does not know).  Its
-    memory may be that of a freed tensor which work queued on the current stream
-    still reads; that work comes first."""
-    out = torch.empty(shape, dtype=dt, device="cuda")
-    if not torch.cuda.is_current_stream_capturing():
-        cur = torch.cuda.current_stream()
-        if not cur.query():
-            cur.synchronize() if stream is None else stream.wait_stream(cur)
-    return out
 
 
 class FilterBank:
@@ -153,9 +142,9 @@ class ShearletSegmenter:
             B.seg_admm_get(self.handle, what, buf.ctypes.data, True)
             return torch.tensor(int(buf[0]))
         shape, dt = self._shape(what)
-        out = _readout(shape, dt, getattr(self, "stream", None))
-        B.seg_admm_get(self.handle, what, out.data_ptr(), False)
-        self.synchronize()
+        # written on the state's stream, after what the current one still does with this memory
+        out = torch.empty(shape, dtype=dt, device="cuda")
+        B.seg_admm_read(self.handle, what, out.data_ptr(), _cur_stream())
         return out
 
     def get_host(self, what: int, out: torch.Tensor | None = None) -> torch.Tensor:
@@ -361,9 +350,9 @@ class TVSegmenter:
             B.tv_admm_get(self.handle, what, buf.ctypes.data, True)
             return torch.tensor(int(buf[0]))
         shape, dt = self._shape(what)
-        out = _readout(shape, dt, getattr(self, "stream", None))
-        B.tv_admm_get(self.handle, what, out.data_ptr(), False)
-        self.synchronize()
+        # written on the state's stream, after what the current one still does with this memory
+        out = torch.empty(shape, dtype=dt, device="cuda")
+        B.tv_admm_read(self.handle, what, out.data_ptr(), _cur_stream())
         return out
 
     def get_host(self, what: int, out: torch.Tensor | None = None) -> torch.Tensor:
@@ -461,9 +450,9 @@ class NLSegmenter(TVSegmenter):
             B.nl_admm_get(self.handle, what, buf.ctypes.data, True)
             return torch.tensor(int(buf[0]))
         shape, dt = self._shape(what)
-        out = _readout(shape, dt, getattr(self, "stream", None))
-        B.nl_admm_get(self.handle, what, out.data_ptr(), False)
-        self.synchronize()
+        # written on the state's stream, after what the current one still does with this memory
+        out = torch.empty(shape, dtype=dt, device="cuda")
+        B.nl_admm_read(self.handle, what, out.data_ptr(), _cur_stream())
         return out
 
     def get_host(self, what: int, out: torch.Tensor | None = None) -> torch.Tensor:

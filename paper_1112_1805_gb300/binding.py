@@ -88,6 +88,7 @@ _SIG = {
     "seg_admm_reset": (_I, [_VP, _VP, _I]),
     "seg_admm_step": (_I, [_VP, _I]),
     "seg_admm_solve": (_I, [_VP, ctypes.POINTER(_I), ctypes.POINTER(ctypes.c_float)]),
+    "seg_admm_read": (_I, [_VP, _I, _VP, _VP]),
     "seg_admm_get": (_I, [_VP, _I, _VP, _I]),
     "seg_admm_set": (_I, [_VP, _I, _VP, _I]),
     "seg_admm_save": (_I, [_VP, ctypes.c_char_p]),
@@ -117,6 +118,7 @@ _SIG = {
                           ctypes.POINTER(_VP)]),
     "tv_admm_reset": (_I, [_VP, _VP, _I]),
     "tv_admm_step": (_I, [_VP, _I]),
+    "tv_admm_read": (_I, [_VP, _I, _VP, _VP]),
     "tv_admm_get": (_I, [_VP, _I, _VP, _I]),
     "tv_admm_set": (_I, [_VP, _I, _VP, _I]),
     "tv_admm_kernel_times": (_I, [_VP, _I, ctypes.POINTER(ctypes.c_float), ctypes.POINTER(_I)]),
@@ -130,6 +132,7 @@ _SIG = {
     "nl_admm_reset": (_I, [_VP, _VP, _I]),
     "nl_admm_graph": (_I, [_VP, _VP, _VP, ctypes.POINTER(_I)]),
     "nl_admm_step": (_I, [_VP, _I]),
+    "nl_admm_read": (_I, [_VP, _I, _VP, _VP]),
     "nl_admm_get": (_I, [_VP, _I, _VP, _I]),
     "nl_admm_set": (_I, [_VP, _I, _VP, _I]),
     "nl_admm_kernel_times": (_I, [_VP, _I, ctypes.POINTER(ctypes.c_float), ctypes.POINTER(_I)]),
@@ -252,6 +255,10 @@ def seg_admm_solve(state: int):
 
 def seg_admm_get(state: int, what: int, dst: int, dst_on_host: bool) -> None:
     _call("seg_admm_get", _VP(state), int(what), _VP(dst), int(bool(dst_on_host)))
+
+
+def seg_admm_read(state: int, what: int, dst: int, earlier: int) -> None:
+    _call("seg_admm_read", _VP(state), int(what), _VP(dst), _VP(earlier))
 
 
 def seg_admm_set(state: int, what: int, src: int, src_on_host: bool) -> None:
@@ -412,6 +419,10 @@ def tv_admm_get(state: int, what: int, dst: int, dst_on_host: bool) -> None:
     _call("tv_admm_get", _VP(state), int(what), _VP(dst), int(bool(dst_on_host)))
 
 
+def tv_admm_read(state: int, what: int, dst: int, earlier: int) -> None:
+    _call("tv_admm_read", _VP(state), int(what), _VP(dst), _VP(earlier))
+
+
 def tv_admm_set(state: int, what: int, src: int, src_on_host: bool) -> None:
     _call("tv_admm_set", _VP(state), int(what), _VP(src), int(bool(src_on_host)))
 
@@ -474,6 +485,10 @@ def nl_admm_step(state: int, n_iters: int) -> None:
 
 def nl_admm_get(state: int, what: int, dst: int, dst_on_host: bool) -> None:
     _call("nl_admm_get", _VP(state), int(what), _VP(dst), int(bool(dst_on_host)))
+
+
+def nl_admm_read(state: int, what: int, dst: int, earlier: int) -> None:
+    _call("nl_admm_read", _VP(state), int(what), _VP(dst), _VP(earlier))
 
 
 def nl_admm_set(state: int, what: int, src: int, src_on_host: bool) -> None:

@@ -321,6 +321,9 @@ cudaError_t tv_fast_rows_inv(const float2* Y, float* u, int K, int H, int W, flo
 // C ABI layer (shf_capi.cu): the geometry and device tables of a bank, and the
 // thread-local message behind shf_last_error() (returns code).
 void bank_geo(const shf_bank* b, Geo* g);
+// Work queued on `st` from now on comes after what `earlier` has queued by now
+// (left alone while `earlier` is captured).
+cudaError_t order_after(cudaStream_t st, cudaStream_t earlier);
 int bank_device(const shf_bank* b);  // the device the bank's tables live on
 int set_error(int code, const std::string& msg);
 

@@ -1475,6 +1475,13 @@ int nl_admm_get(nl_state* st, int what, void* dst, int on_host) {
   }
 }
 
+int nl_admm_read(nl_state* st, int what, void* dst, void* earlier) {
+  if (!st || !dst) return nl_fail(SHF_ERR_ARG, "nl_admm_read: NULL argument");
+  NL_CK(shf::order_after(st->stream, static_cast<cudaStream_t>(earlier)));
+  const int rc = nl_admm_get(st, what, dst, 0);
+  return rc ? rc : nl_admm_sync(st);
+}
+
 int nl_admm_set(nl_state* st, int what, const void* src, int on_host) {
   if (!st || !src) return nl_fail(SHF_ERR_ARG, "nl_admm_set: NULL argument");
   const size_t P = st->P(), K = st->K, m = st->m;

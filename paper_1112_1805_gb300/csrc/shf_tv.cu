@@ -651,6 +651,13 @@ int tv_admm_get(tv_state* st, int what, void* dst, int on_host) {
   }
 }
 
+int tv_admm_read(tv_state* st, int what, void* dst, void* earlier) {
+  if (!st || !dst) return tv_fail(SHF_ERR_ARG, "tv_admm_read: NULL argument");
+  TV_CK(shf::order_after(st->stream, static_cast<cudaStream_t>(earlier)));
+  const int rc = tv_admm_get(st, what, dst, 0);
+  return rc ? rc : tv_admm_sync(st);
+}
+
 int tv_admm_set(tv_state* st, int what, const void* src, int on_host) {
   if (!st || !src) return tv_fail(SHF_ERR_ARG, "tv_admm_set: NULL argument");
   const size_t P = st->P(), K = st->K;

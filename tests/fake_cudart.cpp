@@ -42,6 +42,7 @@ std::set<cudaStream_t> captured;                                // streams with 
 std::map<std::uintptr_t, std::set<cudaStream_t>> graphs;        // ... in a graph (or its executable)
 std::map<cudaStream_t, std::set<cudaStream_t>> flights;         // ... in the graphs running on a stream
 std::map<cudaEvent_t, cudaStream_t> recorded;
+int stream_waits = 0;
 cudaError_t last = cudaSuccess;
 std::uintptr_t next_handle = 0x1000;
 struct {
@@ -113,6 +114,7 @@ cudaError_t run(const void* fun, cudaStream_t st) {
 }
 }  // namespace
 
+int waits() { return stream_waits; }
 std::size_t live() { return buffers().size(); }
 std::size_t held() {
   std::size_t n = 0;
@@ -232,7 +234,10 @@ cudaError_t cudaStreamSynchronize(cudaStream_t s) {
   waited_for(s);
   return cudaSuccess;
 }
-cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
+cudaError_t cudaStreamWaitEvent(cudaStream_t st, cudaEvent_t e, unsigned) {
+  if (recorded.count(e) && recorded[e] != st) ++stream_waits;
+  return cudaSuccess;
+}
 cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus* c) {
   *c = capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
   return cudaSuccess;

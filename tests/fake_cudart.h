@@ -17,5 +17,6 @@ extern std::size_t fail_over;    // device allocations of more bytes fail (0: no
 extern const char* fail_kernel;  // the next kernel whose name contains this fails
 std::size_t live();              // buffers not given back
 std::size_t held();              // their bytes
+int waits();                     // streams made to wait for another one's event
 int launched(const char* name);  // kernels so far whose name contains `name`
 }  // namespace fake

@@ -2,6 +2,8 @@
 // of every call is made to fail once.  A call that runs out of memory says so,
 // leaves the state usable, returns what it had taken in the order of the stream it
 // was taken on, and nothing is left when everything is destroyed.
+#include <cuda_runtime_api.h>
+
 #include <cstdio>
 #include <string>
 #include <vector>
@@ -150,6 +152,29 @@ void reported_once() {
   expect(seg_admm_destroy(st) == SHF_OK, "destroy");
 }
 
+// A readout into memory that another stream may still use comes after that stream.
+void readouts() {
+  cudaStream_t other = nullptr;
+  cudaStreamCreateWithFlags(&other, cudaStreamNonBlocking);
+  std::vector<float> out(3ul * 64 * 128, 0.f), in(out);
+  Problem pb(64, 64, 3, 2);
+  seg_state* st = nullptr;
+  tv_state* tv = nullptr;
+  nl_state* nl = nullptr;
+  expect(pb.init(&st) == SHF_OK && tv_init(&tv) == SHF_OK && nl_init(&nl) == SHF_OK, "init");
+  const auto check = [&](const char* what, auto&& read) {
+    cudaMemcpyAsync(out.data(), in.data(), 4, cudaMemcpyDeviceToDevice, other);
+    const int n = fake::waits();
+    expect(read() == SHF_OK && fake::waits() == n + 1, what);
+    expect(cudaGetLastError() == cudaSuccess, what);
+  };
+  check("seg_admm_read", [&] { return seg_admm_read(st, SEG_W, out.data(), other); });
+  check("tv_admm_read", [&] { return tv_admm_read(tv, SEG_W, out.data(), other); });
+  check("nl_admm_read", [&] { return nl_admm_read(nl, SEG_W, out.data(), other); });
+  expect(seg_admm_read(st, 99, out.data(), other) == SHF_ERR_ARG, "unknown selector");
+  expect(seg_admm_destroy(st) == SHF_OK && tv_admm_destroy(tv) == SHF_OK && nl_admm_destroy(nl) == SHF_OK, "destroy");
+}
+
 // A batch's iterations run as a graph on the batch's stream, tuning and readouts on
 // the images' own.
 struct Batch {
@@ -241,6 +266,7 @@ int main() {
   failed_tables();
   no_capture();
   reported_once();
+  readouts();
   batch_order();
   short_of_memory();
   expect(fake::violations == 0, "buffers returned in order", fake::violations);
