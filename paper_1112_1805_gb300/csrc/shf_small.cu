@@ -11,8 +11,9 @@
 // and orientation (a few KB of code that the kernels share: instruction fetch
 // would otherwise cost as much as the arithmetic), with element-wise passes
 // between them.  One 64 x 64 channel, 13 filters: analysis 31 -> 22 us in a row
-// (17 where the caller has the stream's handle at hand) and 270 -> 85 us for the first on a bank (four launches on the staged or
-// register-FFT kernels: 33 us).  The ADMM iteration was tried the same way (a
+// (17 where the caller has the stream's handle at hand) and 270 -> 85 us for the
+// first on a bank (four launches on the staged or register-FFT kernels: 33 us).
+// The ADMM iteration was tried the same way (a
 // cluster of one CTA per label for the u/w-step, a CTA per label and filter for
 // the rest) and is slower than its six or seven short launches: 41 against 25 us
 // at 64 x 64, K = 3, 62 against 56 at 50 x 216, K = 5; a CTA needs about 20 us for
